@@ -178,34 +178,35 @@ class _State:
     pass
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
+    """The state of a pass without its handles, and the head's weights (None where the path has no head)."""
     dev = torch.device("cuda")
     gen = torch.Generator(device=dev).manual_seed(seed)
     s, kind, n = _State(), case["kind"], case["n"]
     s.kind = kind
     if kind == "host":
-        return _prepare_host(s, case, gen)
+        return s, _host_inputs(s, case, gen)
     s.feat = _features(n * case.get("rows", 1), case["d"], case["heavy"], gen)
     if kind == "calibrate":
         s.pool = torch.empty(case["pool"], device=dev).uniform_(0.0, math.log(case["d"]), generator=gen)
-        return s
+        return s, None
     s.tau = _threshold(_entropies(s.feat, case.get("rows", 1)), case["drop"])
     if kind == "blocks":
         s.rows, s.gamma = case["rows"], case["gamma"]
         s.r = torch.rand(n, device=dev, generator=gen)
         s.ratio = 0.5 + torch.rand(n, device=dev, generator=gen)
-        return s
+        return s, None
     s.mask = torch.zeros(n, dtype=torch.uint8, device=dev)
     s.idx = torch.zeros(n, dtype=torch.int32, device=dev)
     s.count = torch.zeros(1, dtype=torch.int32, device=dev)
     if kind == "gate":
         s.entropy = torch.zeros(n, device=dev)
-        return s
+        return s, None
     K = case["K"]
     s.cond = torch.randn((n, case["Dc"]), device=dev, generator=gen).to(torch.bfloat16)
     s.noise = torch.randn((n, case["C"]), device=dev, generator=gen)
     s.out = torch.zeros((n, case["C"]), device=dev)       # rows of dropped tokens are left as they are
-    s.head = ardiff.Head(case["C"], case["Dc"], case["W"], case["L"], TIME_FEATURES, K, n, _weights(case, gen))
+    weights = _weights(case, gen)
     if kind == "path":
         s.t = np.arange(K + 1, dtype=np.float32) / K
     else:
@@ -214,10 +215,10 @@ def prepare(case, seed):
         keep = (np.arange(K) + 1.0) / K
         s.coef = np.stack([np.zeros(K), np.sqrt(keep), np.sqrt(1.0 - keep)], axis=1).astype(np.float32)
         s.step_noise = torch.randn((K, n, case["C"]), device=dev, generator=gen)
-    return s
+    return s, weights
 
 
-def _prepare_host(s, case, gen):
+def _host_inputs(s, case, gen):
     n, K = case["n"], case["K"]
     s.slots, s.batches = case["slots"], []
     for _ in range(case["batches"]):
@@ -229,8 +230,15 @@ def _prepare_host(s, case, gen):
                               noise=noise.cpu().pin_memory(), tau=tau, out=torch.zeros((n, case["C"])).pin_memory(),
                               mask=torch.zeros(n, dtype=torch.uint8).pin_memory()))
     s.t = np.arange(K + 1, dtype=np.float32) / K
-    s.head = ardiff.Head(case["C"], case["Dc"], case["W"], case["L"], TIME_FEATURES, K, n, _weights(case, gen))
-    s.pipe = ardiff.Pipeline(s.head, n, case["d"], slots=s.slots)
+    return _weights(case, gen)
+
+
+def prepare(case, seed):
+    s, weights = _inputs(case, seed)
+    if weights is not None:
+        s.head = ardiff.Head(case["C"], case["Dc"], case["W"], case["L"], TIME_FEATURES, case["K"], case["n"], weights)
+    if s.kind == "host":
+        s.pipe = ardiff.Pipeline(s.head, case["n"], case["d"], slots=s.slots)
     return s
 
 
@@ -270,6 +278,83 @@ def _run_host(s):
     for i in range(len(s.batches) - min(s.slots, len(s.batches)), len(s.batches)):
         kept.append(s.pipe.ardiff_pipeline_wait(i % s.slots))
     return [kept] + [[b["out"], b["mask"]] for b in s.batches]
+
+
+# ---- the same in 64 bits -------------------------------------------------------------------------
+def _row_entropies(feat):
+    """Row entropies in fp64, whole batches in slices."""
+    n, d = feat.shape
+    step = max(1, (1 << 27) // d)
+    h = torch.empty(n, dtype=torch.float64, device="cuda")
+    for r0 in range(0, n, step):
+        lp = torch.log_softmax(feat[r0:r0 + step].cuda().double(), dim=1)
+        h[r0:r0 + step] = -(lp.exp() * lp).sum(dim=1)
+    return h
+
+
+def _threshold_statistics(h):
+    mean, std = h.double().mean(), h.double().std(unbiased=False)
+    return torch.stack([mean, std, 0.3 * mean - 0.1 * std])
+
+
+def _head64(case, weights, cond, noise, t, coef, step_noise):
+    """The head's sampler steps over the given rows: noise, one (ax, av, an) per step, fresh noise or None."""
+    def bf16(name):
+        return torch.from_numpy(weights[name].view(np.int16)).cuda().view(torch.bfloat16)
+
+    w = {name: bf16(name) for name in weights}
+    linear = lambda x, a, b: torch.nn.functional.linear(x, a.double(), b.double())
+    silu, W, F = torch.nn.functional.silu, case["W"], TIME_FEATURES
+    ln = lambda x: torch.nn.functional.layer_norm(x, (W,), eps=1e-6)
+    freq = torch.exp(-math.log(10000.0) * torch.arange(F // 2, dtype=torch.float64, device="cuda") / (F // 2))
+    c = linear(cond.cuda().double(), w["Wc"], w["bc"])
+    x = noise.cuda().double()
+    for k in range(len(coef)):
+        arg = 1000.0 * float(t[k]) * freq
+        temb = linear(silu(linear(torch.cat([arg.cos(), arg.sin()]), w["Wt1"], w["bt1"])), w["Wt2"], w["bt2"])
+        s = silu(c + temb)
+        h = linear(x, w["Win"], w["bin"])
+        for b in range(case["L"]):
+            shift, scale, gate = linear(s, w["Wmod"][b], w["bmod"][b]).chunk(3, dim=1)
+            u = ln(h) * (1.0 + scale) + shift
+            h = h + gate * linear(silu(linear(u, w["W1"][b], w["b1"][b])), w["W2"][b], w["b2"][b])
+        shift, scale = linear(s, w["Wfm"], w["bfm"]).chunk(2, dim=1)
+        v = linear(ln(h) * (1.0 + scale) + shift, w["Wout"], w["bout"])
+        ax, av, an = (float(a) for a in coef[k])
+        x = ax * x + av * v
+        if step_noise is not None:
+            x = x + an * step_noise[k].cuda().double()
+    return x
+
+
+def exact(case, seed):
+    """What run() returns, in fp64 torch; None in the place of masks, ids, counts and lengths."""
+    s, weights = _inputs(case, seed)
+    kind = case["kind"]
+    if kind == "gate":
+        return [None, None, None, _row_entropies(s.feat)]
+    if kind == "calibrate":
+        h = _row_entropies(s.feat)
+        return [None, None, None, h, _threshold_statistics(h), _threshold_statistics(s.pool)]
+    if kind == "blocks":
+        return [None, None, None, _row_entropies(s.feat).reshape(-1, s.rows).mean(dim=1), None]
+    if kind == "sampler":
+        coef, batches = s.coef.astype(np.float64), [s.__dict__]
+    else:
+        t = s.t.astype(np.float64)
+        coef = np.stack([np.ones(case["K"]), np.diff(t), np.zeros(case["K"])], axis=1)
+        batches = s.batches if kind == "host" else [s.__dict__]
+    outs = []
+    for b in batches:
+        keep = (_row_entropies(b["feat"]) >= b["tau"]).nonzero()[:, 0]
+        at = keep.to(b["cond"].device)
+        out = torch.zeros((case["n"], case["C"]), dtype=torch.float64, device="cuda")
+        fresh = s.step_noise[:, at] if kind == "sampler" else None
+        out[keep] = _head64(case, weights, b["cond"][at], b["noise"][at], s.t, coef, fresh)
+        outs.append(out)
+    if kind != "host":
+        return [None, None, None, outs[0]]
+    return [outs[0], None, None] if s.slots == 1 else [None] + [[out, None] for out in outs]
 
 
 # ---- what a pass cannot do without ---------------------------------------------------------------
