@@ -648,51 +648,60 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
         while (have) {
             const bool have_nx = next_item(nx);
             bool ok = true;
-            if (lane == 0 && !pre_ok) {
-                const int* ctr = P.counters + (size_t)it.abs_m * CTRS;
-                ok = wait_counters(ctr, it.needA, it.needB ? ctr + it.gsel : nullptr, it.needB, P);
+            const int src_stage = stage;
+            const uint32_t src_phase = phase;
+            int seen = 0;
+            if (ptx::elect_one()) {
+                if (!pre_ok) {
+                    const int* ctr = P.counters + (size_t)it.abs_m * CTRS;
+                    ok = wait_counters(ctr, it.needA, it.needB ? ctr + it.gsel : nullptr, it.needB, P);
+                }
+                TRACE(0, 0);
+                if (ok) {
+                    ptx::mbar_arrive(dep_bar(seq));      // the epilogue may now load this item's inputs
+                    // operands that other CTAs wrote with plain stores (z, xb) cross from the generic to the async
+                    // proxy; everything else was written by TMA stores and is read by TMA loads
+                    if (it.type == OP_COND || it.type == OP_IN) ptx::fence_proxy_async();
+                    const void* map_a = P.maps + it.map_a;
+                    const void* map_b = P.maps + it.map_b;
+                    const int b_rows = it.umma_n / 2;                         // rows of B this CTA stages
+                    const uint32_t tx = 2u * (A_BYTES + (uint32_t)b_rows * BK * 2);
+                    const int b_row = it.b_row + rank * b_rows;
+                    const int peek_kb = it.kblocks > 3 ? it.kblocks - 3 : 0;
+                    int pv1 = 0, pv2 = 0;      // the next item's counters, read while this item still streams
+                    int st = src_stage;
+                    uint32_t ph = src_phase;
+                    for (int kb = 0; kb < it.kblocks; ++kb) {
+                        ok = wait_mbar(empty_bar(st), ph ^ 1u, P);
+                        if (!ok) break;
+                        if (kb == 0) TRACE(0, 1);
+                        TRACE_STAGE(0, kb);
+                        const uint32_t sa = smem_base + st * STAGE_BYTES;
+                        // the even CTA arms its barrier for the bytes of both CTAs
+                        if (rank == 0) ptx::mbar_arrive_expect_tx(full_bar(st), tx);
+                        ptx::tma_load_2d_pair(sa, map_a, full_bar(st), kb * BK, it.a_row0);
+                        ptx::tma_load_2d_pair(sa + A_BYTES, map_b, full_bar(st), kb * BK, b_row);
+                        if (kb == peek_kb && have_nx) {
+                            // issued here, looked at only after the last slice went out
+                            const int* ctr = P.counters + (size_t)nx.abs_m * CTRS;
+                            pv1 = ptx::ld_acquire_gpu(ctr);
+                            pv2 = nx.needB ? ptx::ld_acquire_gpu(ctr + nx.gsel) : 0;
+                        }
+                        issued |= 1u << st;
+                        issued_parity = (issued_parity & ~(1u << st)) | (ph << st);
+                        if (++st == STAGES) { st = 0; ph ^= 1u; }
+                    }
+                    seen = (have_nx && pv1 >= nx.needA && pv2 >= nx.needB) ? 1 : 0;
+                }
+                TRACE(0, 2); TRACE_TYPE(0);
             }
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) { aborted = true; break; }
-            TRACE(0, 0);
-            if (lane == 0) ptx::mbar_arrive(dep_bar(seq));      // the epilogue may now load this item's inputs
+            TRACE_NEXT();
             ++seq;
-            // operands that other CTAs wrote with plain stores (z, xb) cross from the generic to the async proxy;
-            // everything else was written by TMA stores and is read by TMA loads
-            if (it.type == OP_COND || it.type == OP_IN) ptx::fence_proxy_async();
-            const void* map_a = P.maps + it.map_a;
-            const void* map_b = P.maps + it.map_b;
-            const int b_rows = it.umma_n / 2;                         // rows of B this CTA stages
-            const uint32_t tx = 2u * (A_BYTES + (uint32_t)b_rows * BK * 2);
-            const int peek_kb = it.kblocks > 3 ? it.kblocks - 3 : 0;
-            int pv1 = 0, pv2 = 0;      // the next item's counters, read while this item still streams
-            for (int kb = 0; kb < it.kblocks; ++kb) {
-                ok = wait_mbar(empty_bar(stage), phase ^ 1u, P);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
-                if (kb == 0) TRACE(0, 1);
-                TRACE_STAGE(0, kb);
-                if (lane == 0) {
-                    const uint32_t sa = smem_base + stage * STAGE_BYTES;
-                    // the even CTA arms its barrier for the bytes of both CTAs
-                    if (rank == 0) ptx::mbar_arrive_expect_tx(full_bar(stage), tx);
-                    ptx::tma_load_2d_pair(sa, map_a, full_bar(stage), kb * BK, it.a_row0);
-                    ptx::tma_load_2d_pair(sa + A_BYTES, map_b, full_bar(stage), kb * BK, it.b_row + rank * b_rows);
-                    if (kb == peek_kb && have_nx) {
-                        // issued here, looked at only after the last slice went out
-                        const int* ctr = P.counters + (size_t)nx.abs_m * CTRS;
-                        pv1 = ptx::ld_acquire_gpu(ctr);
-                        pv2 = nx.needB ? ptx::ld_acquire_gpu(ctr + nx.gsel) : 0;
-                    }
-                }
-                issued |= 1u << stage;
-                issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
-                if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-            }
-            TRACE(0, 2); TRACE_TYPE(0); TRACE_NEXT();
-            if (!ok) { aborted = true; break; }
-            const int pre = (have_nx && pv1 >= nx.needA && pv2 >= nx.needB) ? 1 : 0;
-            pre_ok = __shfl_sync(0xffffffffu, pre, 0) != 0;
+            stage += it.kblocks;
+            for (; stage >= STAGES; stage -= STAGES) phase ^= 1u;
+            pre_ok = __any_sync(0xffffffffu, seen);
             it = nx;
             have = have_nx;
         }
@@ -701,12 +710,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
         // the even CTA's barriers; after a normal run they were all consumed, after an abort it
         // simply waits out a bounded time that covers any TMA latency.
         if (rank == 0) {
+            // (the elected lane is the one that kept the record)
             for (int s = 0; s < STAGES; ++s)
                 if (issued & (1u << s)) drain_mbar(full_bar(s), (issued_parity >> s) & 1u);
         } else if (aborted) {
             const uint64_t t0 = ptx::globaltimer_ns();
             while (ptx::globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
         }
+        __syncwarp();
     } else if (warp == 1) {
         // ---------------- MMA issuer (the even CTA issues for the pair) ----------------
         if (rank == 0) {
@@ -720,41 +731,43 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                 if (it.type == OP_GATHER || it.type == OP_NOP) continue;
                 const uint32_t buf = acc_iter & 1u;
                 const uint32_t acc_phase = (acc_iter >> 1) & 1u;
-                bool ok = wait_mbar(tempty_bar(buf), acc_phase ^ 1u, P);
-                ok = __all_sync(0xffffffffu, ok);
-                TRACE(1, 0);
-                if (!ok) break;
-                ptx::tc_fence_after();
-                const uint32_t d_tmem = tmem_base + buf * BN;
-                const uint32_t idesc = ptx::idesc_bf16_f32(2 * BM, (uint32_t)it.umma_n);
-                for (int kb = 0; kb < it.kblocks; ++kb) {
-                    ok = wait_mbar(full_bar(stage), phase, P);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (kb == 0) TRACE(1, 1);
-                    TRACE_STAGE(1, kb);
-                    if (!ok) break;
+                bool ok = true;
+                if (ptx::elect_one()) {
+                    ok = wait_mbar(tempty_bar(buf), acc_phase ^ 1u, P);
+                    TRACE(1, 0);
                     ptx::tc_fence_after();
-                    if (lane == 0) {
-                        const uint32_t sa = smem_base + stage * STAGE_BYTES;
+                    const uint32_t d_tmem = tmem_base + buf * BN;
+                    const uint32_t idesc = ptx::idesc_bf16_f32(2 * BM, (uint32_t)it.umma_n);
+                    int st = stage;
+                    uint32_t ph = phase;
+                    for (int kb = 0; ok && kb < it.kblocks; ++kb) {
+                        ok = wait_mbar(full_bar(st), ph, P);
+                        if (kb == 0) TRACE(1, 1);
+                        TRACE_STAGE(1, kb);
+                        if (!ok) break;
+                        ptx::tc_fence_after();
+                        const uint32_t sa = smem_base + st * STAGE_BYTES;
                         const uint64_t da = ptx::smem_desc_sw128(sa);
                         const uint64_t db = ptx::smem_desc_sw128(sa + A_BYTES);
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k)
                             ptx::mma_f16_ss_pair(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc,
                                                  (kb | k) != 0 ? 1u : 0u);
-                        ptx::mma_commit_pair_mc(empty_bar(stage), 3);   // frees the stage in both CTAs
+                        ptx::mma_commit_pair_mc(empty_bar(st), 3);   // frees the stage in both CTAs
+                        if (++st == STAGES) { st = 0; ph ^= 1u; }
                     }
-                    __syncwarp();
-                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                    if (ok) ptx::mma_commit_pair_mc(tfull_bar(buf), 3);
+                    TRACE(1, 2); TRACE_TYPE(1);
                 }
+                ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                if (lane == 0) ptx::mma_commit_pair_mc(tfull_bar(buf), 3);
-                __syncwarp();
+                stage += it.kblocks;
+                for (; stage >= STAGES; stage -= STAGES) phase ^= 1u;
                 ++acc_iter;
-                TRACE(1, 2); TRACE_TYPE(1); TRACE_NEXT();
+                TRACE_NEXT();
             }
             // all MMAs this thread issued must be done before TMEM is freed
-            if (lane == 0) ptx::mma_commit_pair(drain_bar);
+            if (ptx::elect_one()) ptx::mma_commit_pair(drain_bar);
             __syncwarp();
             drain_mbar(drain_bar, 0);
         }
@@ -835,13 +848,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                 const uint32_t tacc = tmem_base + buf * BN + ((uint32_t)(quarter * 32) << 16);
                 // a slab may be rewritten once the TMA store that read it last (two stores back) is done reading
                 auto slab_ready = [&]() {
-                    if (lane == 0) ptx::bulk_wait_read<EPI_NB - 1>();
+                    if (ptx::elect_one()) ptx::bulk_wait_read<EPI_NB - 1>();
                     __syncwarp();
                 };
                 auto slab_store = [&](int map, uint32_t slab, int col, int grow0) {
                     ptx::fence_proxy_async_smem();
                     __syncwarp();
-                    if (lane == 0) {
+                    if (ptx::elect_one()) {
                         ptx::tma_store_2d(P.maps + map, slab, col, grow0);
                         ptx::bulk_commit();
                     }
@@ -971,7 +984,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive_even_cta(tempty_bar(buf));
                 ++acc_iter;
-                if (lane == 0) ptx::bulk_wait<0>();   // this warp's TMA stores are performed
+                if (ptx::elect_one()) ptx::bulk_wait<0>();   // this warp's TMA stores are performed
                 __syncwarp();
             }
             if (fail) break;
@@ -989,7 +1002,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
             }
         }
         // own copies in flight: stores not yet done
-        if (lane == 0) ptx::bulk_wait<0>();
+        if (ptx::elect_one()) ptx::bulk_wait<0>();
         __syncwarp();
     }
 

@@ -42,6 +42,21 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
+// One lane of a converged warp, the same one every time. Asynchronous instructions (tcgen05.mma, commits, TMA
+// copies) take their operands from uniform registers: under `lane == 0` the compiler cannot know that one thread
+// is active and walks the active lanes one by one, under elect.sync it does not. Measured on a ring that is always
+// full, cycles per 64-wide slice (four products, one commit): 540 whatever the tile width under `lane == 0`,
+// 514 (256 columns, the tensor pipe's own pace) and 259 (128 columns and fewer) under elect.sync.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
 // ---- proxies / fences ---------------------------------------------------------------------
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async_smem() {
