@@ -50,12 +50,20 @@ namespace {
 using bf16 = __nv_bfloat16;
 
 constexpr int BM = 128;           // tokens per tile (one CTA)
-constexpr int BN = 256;           // output columns per item (UMMA N)
 constexpr int BK = 64;            // K slice per pipeline stage (128 bytes of bf16: one swizzle row)
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int B_ROWS = BN / 2;    // rows of the weight tile that one CTA of the pair stages
-constexpr int STAGES = 6;
-constexpr int STAGE_BYTES = A_BYTES + B_ROWS * BK * 2;   // 32 KB
+constexpr int N_WIDTHS = 3;       // item widths: width w has item_cols(w) output columns per item (UMMA N)
+__host__ __device__ constexpr int item_cols(int w) { return 256 >> w; }
+constexpr int ACC_COLS = 256;     // TMEM columns of one of the two accumulators
+constexpr int RING_BYTES = 192 * 1024;
+constexpr int MAX_STAGES = 9;
+// The operand ring of items of BN columns: a CTA of the pair stages its token tile and half of the weight tile.
+template <int BN>
+struct Ring {
+    static constexpr int STAGE_BYTES = A_BYTES + BN / 2 * BK * 2;       // 32, 24, 20 KB
+    static constexpr int FIT = RING_BYTES / STAGE_BYTES;
+    static constexpr int STAGES = FIT < MAX_STAGES ? FIT : MAX_STAGES;  // 6, 8, 9
+};
 // epilogue staging: every epilogue warp owns EPI_NB bf16 slabs (32 rows x 64 B, 64-byte swizzle) for the
 // results that later GEMMs read as operands (s, u, a): written by the lanes, drained by TMA stores.
 // Everything else an epilogue reads or writes (h, gate values, x) moves between registers and global memory
@@ -64,9 +72,9 @@ constexpr int EPI_WARPS = 8;
 constexpr int EPI_NB = 2;
 constexpr int SLAB_H = 32 * 64;
 constexpr int EPI_BYTES = EPI_WARPS * EPI_NB * SLAB_H;
-constexpr int DEP_BARS = 8;       // the producer runs at most 6 items ahead of the epilogue
-constexpr int NUM_BARS = 2 * STAGES + 5 + DEP_BARS;
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_BYTES + 1024 /*align slack*/ + 8 * NUM_BARS + 16;
+constexpr int DEP_BARS = 16;      // items that the producer may be ahead of the epilogue (see ardiff_head_create)
+constexpr int NUM_BARS = 2 * MAX_STAGES + 5 + DEP_BARS;
+constexpr int SMEM_BYTES = RING_BYTES + EPI_BYTES + 1024 /*align slack*/ + 8 * NUM_BARS + 16;
 constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS;  // warp 0: TMA producer, warp 1: MMA issuer, warps 2-9: epilogue
 constexpr int XB_COLS = 64;       // x is fed to the in-projection as bf16, K padded to one slice
 constexpr int KMAX = 64;
@@ -95,9 +103,10 @@ constexpr int TRACE_ITEMS = 4096;
 
 enum OpType : int { OP_GATHER = 0, OP_COND, OP_IN, OP_SS, OP_GATE, OP_G1, OP_G2, OP_FSS, OP_OUT, OP_NOP, OP_END = 15 };
 enum MapId : int {
-    MAP_Z = 0, MAP_XB, MAP_S, MAP_U, MAP_A, MAP_WC, MAP_WIN, MAP_WCAT, MAP_WOUT,   // GEMM operands
-    EMAP_S, EMAP_U, EMAP_A,                                                 // epilogue output slabs
-    MAP_COUNT
+    MAP_Z = 0, MAP_XB, MAP_S, MAP_U, MAP_A, MAP_WOUT,   // GEMM operands
+    EMAP_S, EMAP_U, EMAP_A,                             // epilogue output slabs
+    MAP_B,                                              // weights, one set of boxes per item width: + 3 w + W_C ..
+    MAP_COUNT = MAP_B + 3 * N_WIDTHS
 };
 
 // One phase of the per-step program: `ntiles` column tiles (tile0 ..) of one layer for every token
@@ -113,14 +122,23 @@ struct Phase {
     int kplus;     // OP_GATE: 1 when the gate belongs to block `block` of the NEXT step
 };
 
-struct HeadParams {
-    int C, Dc, W, L, K, NT, TGu, slots;     // NT = W/256, TGu = largest group in units, slots = scratch tiles
-    int T_pro, T_step, T_chain;             // items per unit: prologue, one step, whole call
-    int C_pro, C_step, C_total;             // chain-counter items per token tile: prologue, one step, whole call
-    int R;                                  // rows of the scratch arrays (slots * 128)
-    int max_tokens;
+enum WeightId : int { W_C = 0, W_IN, W_CAT };
+
+// The item list of one item width.
+struct Program {
+    int NT;                                 // column tiles of a W-wide layer
+    int T_pro, T_step;                      // items per unit: prologue, one step
+    int C_pro, C_step;                      // chain-counter items per token tile: prologue, one step
+    int max_units;                          // most pairs of token tiles this width serves
     const Phase* phases;
     const uint16_t* cum2phase;              // [T_step]: phase that holds the c-th column tile of a step
+};
+
+struct HeadParams {
+    int C, Dc, W, L, K, TGu, slots;         // TGu = largest group in units, slots = scratch tiles
+    int R;                                  // rows of the scratch arrays (slots * 128)
+    int max_tokens;
+    Program prog[N_WIDTHS];
     const CUtensorMap* maps;
     const bf16* cond;
     const float* noise;
@@ -148,8 +166,9 @@ struct Packed { uint32_t w0, w1, w2, w3, w4; };
 
 struct Item {
     int type, abs_m, slot_row0, a_row0, nt, k, block, gsel;   // a_row0: first row of the A operand in its tensor
-    int needA, needB;
-    int map_a, map_b, b_row, kblocks, umma_n;
+    int needA, needB;            // counters the operands wait for (chain; gates: G2 only)
+    int needE;                   // modulation items: chain counter the epilogue waits for (the residual stream)
+    int map_a, map_b, b_row, b_step, kblocks, umma_n;   // CTA r of the pair stages weight rows b_row + r b_step ..
 };
 
 // ------------------------------------------------------------------------------------------
@@ -190,13 +209,17 @@ __device__ __forceinline__ void drain_mbar(uint32_t bar, uint32_t parity) {
     }
 }
 
-// bounded wait until *c1 >= n1 and (c2 == nullptr or *c2 >= n2) (acquire); one thread calls it
-__device__ __forceinline__ bool wait_counters(const int* c1, int n1, const int* c2, int n2, const HeadParams& P) {
+// bounded wait until *c1 >= n1 and (c2 == nullptr or *c2 >= n2) (acquire); one thread calls it. While the
+// counters are short `meanwhile` is called; as long as it returns true it has done something useful.
+template <typename F>
+__device__ __forceinline__ bool wait_counters(const int* c1, int n1, const int* c2, int n2, const HeadParams& P,
+                                              F&& meanwhile) {
     uint64_t t0 = 0;
     for (uint32_t it = 0;; ++it) {
         const int v1 = ptx::ld_acquire_gpu(c1);
         const int v2 = c2 ? ptx::ld_acquire_gpu(c2) : n2;
         if (v1 >= n1 && v2 >= n2) return true;
+        if (meanwhile()) continue;
         if (it > 8) __nanosleep(64);
         if ((it & 63u) == 63u) {
             if (ptx::ld_relaxed_gpu(P.abort_flag) != 0) return false;
@@ -208,6 +231,10 @@ __device__ __forceinline__ bool wait_counters(const int* c1, int n1, const int* 
             }
         }
     }
+}
+
+__device__ __forceinline__ bool wait_counters(const int* c1, int n1, const int* c2, int n2, const HeadParams& P) {
+    return wait_counters(c1, n1, c2, n2, P, [] { return false; });
 }
 
 // SiLU(a) = a * sigmoid(a) = h + h * tanh(h) with h = a / 2: one special-function instruction per element
@@ -229,49 +256,52 @@ __device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w &
 
 // Item `item` of the static list, for the CTA of rank `rank` within its unit. MTu = units (pairs of
 // token tiles) of this call, tgu = units per group (balanced over the groups).
+template <int WI>
 __device__ __forceinline__ Packed decode_packed(const HeadParams& P, int MTu, int tgu, int rank, long long item,
                                                 long long total) {
+    constexpr int BN = item_cols(WI);
+    const Program& V = P.prog[WI];
     Packed pk{(uint32_t)OP_END << 24, 0u, 0u, 0u, 0u};
     if (item >= total) return pk;
-    const long long per_group = (long long)tgu * P.T_chain;
+    const long long per_group = (long long)tgu * (V.T_pro + P.K * V.T_step);
     const int grp = (int)(item / per_group);
     int r = (int)(item - (long long)grp * per_group);
     const int m0 = grp * tgu;
     const int mtg = min(tgu, MTu - m0);
-    const int pro = mtg * P.T_pro;
+    const int pro = mtg * V.T_pro;
     int m, type, nt = 0, k = 0, block = 0, gsel = 0;
     int needA = 0, needB = 0, b_row = 0;
     if (r < pro) {
         if (r < mtg) {
             type = OP_GATHER; m = r;
-        } else if (r < mtg + mtg * P.NT) {
+        } else if (r < mtg + mtg * V.NT) {
             r -= mtg;
-            m = r / P.NT;
-            nt = r - m * P.NT;
+            m = r / V.NT;
+            nt = r - m * V.NT;
             type = OP_COND;
             needA = EPI_WARPS;            // the gather of this token tile
             b_row = nt * BN;
         } else {
             // the gate of step 0, block 0 (gate number 0): needs s_0, i.e. the conditioning items
-            r -= mtg + mtg * P.NT;
-            m = r / P.NT;
-            nt = r - m * P.NT;
+            r -= mtg + mtg * V.NT;
+            m = r / V.NT;
+            nt = r - m * V.NT;
             type = OP_GATE; gsel = 1;
-            needA = EPI_WARPS * P.C_pro;
+            needA = EPI_WARPS * V.C_pro;
             b_row = 2 * P.W + nt * BN;
         }
     } else {
         r -= pro;
-        const int per_step = mtg * P.T_step;
+        const int per_step = mtg * V.T_step;
         k = r / per_step;
         r -= k * per_step;
         const int c = r / mtg;
-        const Phase p = P.phases[__ldg(P.cum2phase + c)];
+        const Phase p = V.phases[__ldg(V.cum2phase + c)];
         const int q = r - p.cum * mtg;
         m = q / p.ntiles;
         nt = p.tile0 + (q - m * p.ntiles);
         type = p.type; block = p.block;
-        needA = EPI_WARPS * (P.C_pro + k * P.C_step + p.offA);
+        needA = EPI_WARPS * (V.C_pro + k * V.C_step + p.offA);
         b_row = p.b_row0 + nt * BN;
         // gates are numbered q = step * L + block over the whole call; gate q lives in buffer q & 1 and
         // ticks counter 1 + (q & 1), so the (q >> 1) + 1 -th gate of that parity is complete at NT * that many ticks
@@ -282,7 +312,18 @@ __device__ __forceinline__ Packed decode_packed(const HeadParams& P, int MTu, in
         } else if (type == OP_G2) {
             const int q = k * P.L + block;
             gsel = 1 + (q & 1);
-            needB = EPI_WARPS * P.NT * ((q >> 1) + 1);
+            needB = EPI_WARPS * V.NT * ((q >> 1) + 1);
+        } else if (type == OP_SS || type == OP_FSS) {
+            // The operands (s_k and weights) exist once the conditioning items are done; only the epilogue needs the
+            // residual stream. Narrow items serve few tokens, where the chain of dependent layers is what a call
+            // takes: there the products run ahead of it and the epilogue waits. The widest items keep the one
+            // wait of the producer (16384-row batches run at the power cap and lose 1 % to the extra polling).
+            if (BN < ACC_COLS) {
+                needB = needA;
+                needA = EPI_WARPS * V.C_pro;
+            }
+            // 128 channels' shift rows, then their scale rows: this item's BN / 2 channels of both
+            b_row = p.b_row0 + (nt * (BN / 2) / 128) * 256 + nt * (BN / 2) % 128;
         }
     }
     const int abs_m = (m0 + m) * 2 + rank;
@@ -293,7 +334,9 @@ __device__ __forceinline__ Packed decode_packed(const HeadParams& P, int MTu, in
     return pk;
 }
 
+template <int WI>
 __device__ __forceinline__ void unpack_item(const HeadParams& P, const Packed& pk, Item& it) {
+    constexpr int BN = item_cols(WI);
     it.type = (int)(pk.w0 >> 24);
     it.abs_m = (int)(pk.w0 & 0xffffffu);
     it.slot_row0 = (it.abs_m % P.slots) * BM;
@@ -301,31 +344,37 @@ __device__ __forceinline__ void unpack_item(const HeadParams& P, const Packed& p
     it.k = (int)((pk.w1 >> 8) & 0xffu);
     it.block = (int)((pk.w1 >> 16) & 0xffu);
     it.gsel = (int)(pk.w1 >> 24);
-    it.needA = (int)pk.w2; it.needB = (int)pk.w3; it.b_row = (int)pk.w4;
-    it.kblocks = P.W / BK; it.umma_n = BN; it.map_b = MAP_WCAT; it.map_a = MAP_S;
+    it.needA = (int)pk.w2; it.needB = (int)pk.w3; it.needE = 0; it.b_row = (int)pk.w4;
+    it.kblocks = P.W / BK; it.umma_n = BN; it.map_b = MAP_B + 3 * WI + W_CAT; it.map_a = MAP_S;
+    it.b_step = BN / 2;
     it.a_row0 = it.slot_row0;
     switch (it.type) {
         case OP_SS:
-        case OP_GATE:
-        case OP_FSS: it.a_row0 = it.k * P.R + it.slot_row0; break;     // s of step k
-        case OP_COND: it.map_a = MAP_Z; it.map_b = MAP_WC; it.kblocks = P.Dc / BK; break;
-        case OP_IN: it.map_a = MAP_XB; it.map_b = MAP_WIN; it.kblocks = 1; break;
+        case OP_FSS:
+            if (BN < ACC_COLS) { it.needE = it.needB; it.needB = 0; }
+            it.b_step = 128;                                           // shift rows, scale rows
+            it.a_row0 = it.k * P.R + it.slot_row0;                     // s of step k
+            break;
+        case OP_GATE: it.a_row0 = it.k * P.R + it.slot_row0; break;
+        case OP_COND: it.map_a = MAP_Z; it.map_b = MAP_B + 3 * WI + W_C; it.kblocks = P.Dc / BK; break;
+        case OP_IN: it.map_a = MAP_XB; it.map_b = MAP_B + 3 * WI + W_IN; it.kblocks = 1; break;
         case OP_G1: it.map_a = MAP_U; break;
         case OP_G2: it.map_a = MAP_A; break;
-        case OP_OUT: it.map_a = MAP_U; it.map_b = MAP_WOUT; it.umma_n = P.C; break;
+        case OP_OUT: it.map_a = MAP_U; it.map_b = MAP_WOUT; it.umma_n = P.C; it.b_step = P.C / 2; break;
         default: break;
     }
 }
 
 // The items of one CTA, decoded 32 at a time (lane l decodes the l-th of the next 32) and handed
 // out by shuffle. Every lane of the warp calls next() together.
+template <int WI>
 struct ItemStream {
     Packed mine;
     int n = 0;
     __device__ __forceinline__ bool next(const HeadParams& P, int MTu, int tgu, int rank, int unit_id, int n_units,
                                          long long total, int lane, Item& it) {
         if ((n & 31) == 0)
-            mine = decode_packed(P, MTu, tgu, rank, (long long)unit_id + (long long)(n + lane) * n_units, total);
+            mine = decode_packed<WI>(P, MTu, tgu, rank, (long long)unit_id + (long long)(n + lane) * n_units, total);
         Packed cur;
         const int src = n & 31;
         cur.w0 = __shfl_sync(0xffffffffu, mine.w0, src);
@@ -335,7 +384,7 @@ struct ItemStream {
         cur.w4 = __shfl_sync(0xffffffffu, mine.w4, src);
         ++n;
         if ((cur.w0 >> 24) == (uint32_t)OP_END) return false;
-        unpack_item(P, cur, it);
+        unpack_item<WI>(P, cur, it);
         return true;
     }
 };
@@ -451,10 +500,11 @@ __device__ __forceinline__ void unit_g_values(const UnitG& d, float (&v)[16]) {
     }
 }
 
-// LayerNorm statistics of one row from its 2*NT partials (mean, M2 over 128 columns each). One pass:
+// LayerNorm statistics of one row from its partials (mean, M2 over COLS columns each). One pass:
 // the first partial's mean serves as pivot, so nothing cancels.
+template <int COLS>
 __device__ __forceinline__ void row_mean_rstd(const HeadParams& P, int grow, float& mean, float& rstd) {
-    const int np = 2 * P.NT;
+    const int np = P.W / COLS;
     const float2* sp = P.stats + (size_t)grow * np;
     const float2 v0 = ptx::ldcg_f2(sp);
     float sd = 0.f, m2 = v0.y;
@@ -463,7 +513,7 @@ __device__ __forceinline__ void row_mean_rstd(const HeadParams& P, int grow, flo
         const float2 v = ptx::ldcg_f2(sp + t);
         const float dm = v.x - v0.x;
         sd += dm;
-        m2 += fmaf(128.0f * dm, dm, v.y);
+        m2 += fmaf((float)COLS * dm, dm, v.y);
     }
     const float dmean = sd / (float)np;                       // mean - pivot
     mean = v0.x + dmean;
@@ -562,70 +612,32 @@ __device__ __forceinline__ void gather_rows(const HeadParams& P, const Item& it,
     }
 }
 
-// ------------------------------------------------------------------------------------------
-// the persistent kernel: clusters of two CTAs. Both load their own token tile (A) and half of the
-// weight tile (B); the even CTA issues cta_group::2 MMAs that read both CTAs' shared memory and
-// write 128 accumulator rows into each CTA's TMEM; every CTA runs the epilogue of its own token tile.
-// ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_constant__ HeadParams P) {
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const uint32_t smem_base = ptx::smem_u32(smem);
-    const uint32_t epi_base = smem_base + STAGES * STAGE_BYTES;      // 1024-aligned
-    const uint32_t bars = epi_base + EPI_BYTES;
+// What the roles of a CTA share: its place in the grid and the item list of the call.
+struct Place {
+    uint32_t smem_base, bars, tmem_base;
+    int rank, unit_id, n_units;             // token tile of the unit this CTA owns, its unit, all units
+    int count, MTu, tgu;                    // survivors; pairs of token tiles: of the call, of one group
+    long long total;                        // items of the call
+};
+
+// The three roles of a CTA over the call's items, which are item_cols(WI) columns wide.
+template <int WI>
+__device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, int warp, int lane) {
+    constexpr int BN = item_cols(WI);
+    constexpr int STAGES = Ring<BN>::STAGES, STAGE_BYTES = Ring<BN>::STAGE_BYTES;
+    constexpr int SPAN = BN / 2;                                 // accumulator columns of one epilogue warp
+    constexpr int UNITS = SPAN / 16;
+    constexpr int MOD_UNITS = UNITS / 2 < 2 ? 2 : UNITS / 2;     // of shift, and of scale
+    const Program& V = P.prog[WI];
+    const uint32_t smem_base = X.smem_base, bars = X.bars;
+    const uint32_t epi_base = smem_base + RING_BYTES;            // 1024-aligned
+    const int rank = X.rank;
     auto full_bar = [&](int s) { return bars + 8u * s; };
-    auto empty_bar = [&](int s) { return bars + 8u * (STAGES + s); };
-    auto tfull_bar = [&](int b) { return bars + 8u * (2 * STAGES + b); };
-    auto tempty_bar = [&](int b) { return bars + 8u * (2 * STAGES + 2 + b); };
-    const uint32_t drain_bar = bars + 8u * (2 * STAGES + 4);
-    auto dep_bar = [&](uint32_t i) { return bars + 8u * (2 * STAGES + 5 + (i % DEP_BARS)); };
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + STAGES * STAGE_BYTES + EPI_BYTES + 8 * NUM_BARS);
-    const int warp = threadIdx.x >> 5;
-    const int lane = threadIdx.x & 31;
-    const int rank = (int)ptx::cluster_ctarank();                  // token tile of the unit this CTA owns
-    const int unit_id = (int)blockIdx.x / 2;
-    const int n_units = (int)gridDim.x / 2;
-
-    int count = __ldg(P.count);
-    if (count > P.max_tokens) {
-        count = P.max_tokens;
-        if (threadIdx.x == 0 && blockIdx.x == 0) atomicCAS(P.status, 0, ARDIFF_ERR_SHAPE);
-    }
-    if (count < 0) count = 0;
-    const int MT = (count + BM - 1) / BM;
-    const int MTu = (MT + 1) / 2;                  // an odd last tile gets an all-padding partner
-    const int n_groups = (MTu + P.TGu - 1) / P.TGu;
-    const int tgu = n_groups > 0 ? (MTu + n_groups - 1) / n_groups : 1;   // balanced group size
-    const long long total = (long long)MTu * P.T_chain;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            ptx::mbar_init(full_bar(s), 1);
-            ptx::mbar_init(empty_bar(s), 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            ptx::mbar_init(tfull_bar(b), 1);
-            ptx::mbar_init(tempty_bar(b), 2 * EPI_WARPS);   // epilogue warps of both CTAs of the unit
-        }
-        ptx::mbar_init(drain_bar, 1);
-        for (int i = 0; i < DEP_BARS; ++i) ptx::mbar_init(dep_bar(i), 1);
-        ptx::fence_mbar_init();
-    }
-    if (warp == 1) {
-        ptx::tmem_alloc_pair(ptx::smem_u32(tmem_slot), 512);
-        ptx::tmem_relinquish_pair();
-    }
-    ptx::tc_fence_before();
-    ptx::cluster_sync_all();
-    ptx::tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
-    long long probe_c0 = 0;
-    unsigned long long probe_g0 = 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        probe_c0 = clock64();
-        probe_g0 = ptx::globaltimer_ns();
-    }
-
+    auto empty_bar = [&](int s) { return bars + 8u * (MAX_STAGES + s); };
+    auto tfull_bar = [&](int b) { return bars + 8u * (2 * MAX_STAGES + b); };
+    auto tempty_bar = [&](int b) { return bars + 8u * (2 * MAX_STAGES + 2 + b); };
+    const uint32_t drain_bar = bars + 8u * (2 * MAX_STAGES + 4);
+    auto dep_bar = [&](uint32_t i) { return bars + 8u * (2 * MAX_STAGES + 5 + (i % DEP_BARS)); };
     if (warp == 0) {
         // ---------------- TMA producer ----------------
         int stage = 0;
@@ -633,13 +645,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
         uint32_t issued = 0, issued_parity = 0;
         uint32_t seq = 0;
         bool aborted = false;
-        ItemStream ist;
+        ItemStream<WI> ist;
         Item it, nx;
         TRACE_DECL
         // next item with operands to load (gather items have none)
         auto next_item = [&](Item& dst) {
             bool have;
-            do have = ist.next(P, MTu, tgu, rank, unit_id, n_units, total, lane, dst);
+            do have = ist.next(P, X.MTu, X.tgu, rank, X.unit_id, X.n_units, X.total, lane, dst);
             while (have && (dst.type == OP_GATHER || dst.type == OP_NOP));
             return have;
         };
@@ -652,9 +664,33 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
             const uint32_t src_phase = phase;
             int seen = 0;
             if (ptx::elect_one()) {
+                const void* map_a = P.maps + it.map_a;
+                const void* map_b = P.maps + it.map_b;
+                const uint32_t tx = 2u * (A_BYTES + (uint32_t)(it.umma_n / 2) * BK * 2);
+                const int b_row = it.b_row + rank * it.b_step;
+                // weights of slice kb into stage st: the even CTA arms its barrier for the bytes of both CTAs
+                auto load_weights = [&](int st, int kb) {
+                    if (rank == 0) ptx::mbar_arrive_expect_tx(full_bar(st), tx);
+                    ptx::tma_load_2d_pair(smem_base + st * STAGE_BYTES + A_BYTES, map_b, full_bar(st), kb * BK, b_row);
+                };
+                int pre = 0;        // slices whose weights were sent for before the item's inputs were complete
                 if (!pre_ok) {
                     const int* ctr = P.counters + (size_t)it.abs_m * CTRS;
-                    ok = wait_counters(ctr, it.needA, it.needB ? ctr + it.gsel : nullptr, it.needB, P);
+                    // few tokens: the chain of dependent layers is what the call takes, so the weights (which depend
+                    // on nothing) come in while it is waited for
+                    int pst = src_stage;
+                    uint32_t pph = src_phase;
+                    ok = wait_counters(ctr, it.needA, it.needB ? ctr + it.gsel : nullptr, it.needB, P, [&] {
+                        if (BN == ACC_COLS || pre >= it.kblocks || pre >= STAGES ||
+                            !ptx::mbar_test_wait(empty_bar(pst), pph ^ 1u))
+                            return false;
+                        load_weights(pst, pre);
+                        issued |= 1u << pst;
+                        issued_parity = (issued_parity & ~(1u << pst)) | (pph << pst);
+                        ++pre;
+                        if (++pst == STAGES) { pst = 0; pph ^= 1u; }
+                        return true;
+                    });
                 }
                 TRACE(0, 0);
                 if (ok) {
@@ -662,25 +698,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                     // operands that other CTAs wrote with plain stores (z, xb) cross from the generic to the async
                     // proxy; everything else was written by TMA stores and is read by TMA loads
                     if (it.type == OP_COND || it.type == OP_IN) ptx::fence_proxy_async();
-                    const void* map_a = P.maps + it.map_a;
-                    const void* map_b = P.maps + it.map_b;
-                    const int b_rows = it.umma_n / 2;                         // rows of B this CTA stages
-                    const uint32_t tx = 2u * (A_BYTES + (uint32_t)b_rows * BK * 2);
-                    const int b_row = it.b_row + rank * b_rows;
                     const int peek_kb = it.kblocks > 3 ? it.kblocks - 3 : 0;
                     int pv1 = 0, pv2 = 0;      // the next item's counters, read while this item still streams
                     int st = src_stage;
                     uint32_t ph = src_phase;
                     for (int kb = 0; kb < it.kblocks; ++kb) {
-                        ok = wait_mbar(empty_bar(st), ph ^ 1u, P);
-                        if (!ok) break;
+                        if (BN == ACC_COLS || kb >= pre) {
+                            ok = wait_mbar(empty_bar(st), ph ^ 1u, P);
+                            if (!ok) break;
+                            load_weights(st, kb);
+                        }
                         if (kb == 0) TRACE(0, 1);
                         TRACE_STAGE(0, kb);
-                        const uint32_t sa = smem_base + st * STAGE_BYTES;
-                        // the even CTA arms its barrier for the bytes of both CTAs
-                        if (rank == 0) ptx::mbar_arrive_expect_tx(full_bar(st), tx);
-                        ptx::tma_load_2d_pair(sa, map_a, full_bar(st), kb * BK, it.a_row0);
-                        ptx::tma_load_2d_pair(sa + A_BYTES, map_b, full_bar(st), kb * BK, b_row);
+                        ptx::tma_load_2d_pair(smem_base + st * STAGE_BYTES, map_a, full_bar(st), kb * BK, it.a_row0);
                         if (kb == peek_kb && have_nx) {
                             // issued here, looked at only after the last slice went out
                             const int* ctr = P.counters + (size_t)nx.abs_m * CTRS;
@@ -724,10 +754,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
             int stage = 0;
             uint32_t phase = 0;
             uint32_t acc_iter = 0;
-            ItemStream ist;
+            ItemStream<WI> ist;
             Item it;
             TRACE_DECL
-            while (ist.next(P, MTu, tgu, rank, unit_id, n_units, total, lane, it)) {
+            while (ist.next(P, X.MTu, X.tgu, rank, X.unit_id, X.n_units, X.total, lane, it)) {
                 if (it.type == OP_GATHER || it.type == OP_NOP) continue;
                 const uint32_t buf = acc_iter & 1u;
                 const uint32_t acc_phase = (acc_iter >> 1) & 1u;
@@ -736,7 +766,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                     ok = wait_mbar(tempty_bar(buf), acc_phase ^ 1u, P);
                     TRACE(1, 0);
                     ptx::tc_fence_after();
-                    const uint32_t d_tmem = tmem_base + buf * BN;
+                    const uint32_t d_tmem = X.tmem_base + buf * ACC_COLS;
                     const uint32_t idesc = ptx::idesc_bf16_f32(2 * BM, (uint32_t)it.umma_n);
                     int st = stage;
                     uint32_t ph = phase;
@@ -780,21 +810,21 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
         const uint32_t my_buf = epi_base + (uint32_t)ew * EPI_NB * SLAB_H;
         uint32_t acc_iter = 0;
         uint32_t seq = 0;
-        ItemStream ist;
+        ItemStream<WI> ist;
         Item it;
         TRACE_DECL
-        while (ist.next(P, MTu, tgu, rank, unit_id, n_units, total, lane, it)) {
+        while (ist.next(P, X.MTu, X.tgu, rank, X.unit_id, X.n_units, X.total, lane, it)) {
             bool fail = false;
             if (it.type == OP_NOP) continue;
             if (it.type == OP_GATHER) {
                 bool ok = true;
                 // the scratch slot is free once the token tile that used it before has run its whole chain
                 if (lane == 0 && it.abs_m >= P.slots)
-                    ok = wait_counters(P.counters + (size_t)(it.abs_m - P.slots) * CTRS, EPI_WARPS * P.C_total,
+                    ok = wait_counters(P.counters + (size_t)(it.abs_m - P.slots) * CTRS, EPI_WARPS * (V.C_pro + P.K * V.C_step),
                                        nullptr, 0, P);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                gather_rows(P, it, ew, lane, count);
+                gather_rows(P, it, ew, lane, X.count);
             } else {
                 // the producer has seen this item's dependencies complete
                 bool ok = wait_mbar(dep_bar(seq), (seq / DEP_BARS) & 1u, P);
@@ -803,9 +833,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                 if (!ok) break;
                 if (ew == 0) TRACE(2, 0);
                 const bool mod = (it.type == OP_SS || it.type == OP_FSS);
-                // this warp's span: 128 accumulator columns (64 of shift and 64 of scale for a modulation item)
-                const int acc0 = mod ? half * 64 : half * 128;
-                const int col0 = mod ? it.nt * 128 + half * 64 : it.nt * BN + half * 128;   // column of the layer's output
+                // this warp's span: half of the item's columns; a modulation item holds BN / 2 shift columns and the
+                // BN / 2 scale columns of the same channels, and a warp takes MOD_UNITS * 16 of either (the narrowest
+                // item has work for one warp of the two only: a slab is 32 columns wide)
+                const int acc0 = mod ? half * (MOD_UNITS * 16) : half * SPAN;
+                const int col0 = mod ? it.nt * (BN / 2) + acc0 : it.nt * BN + acc0;   // column of the layer's output
+                const bool mod_idle = mod && acc0 >= BN / 2;
                 const int row0 = it.slot_row0 + quarter * 32;
                 const int grow = it.slot_row0 + row;
                 const size_t chunk0 = chunk_of(P, row0, col0);
@@ -816,28 +849,39 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                 const bf16* gsrc = it.gsel == 2 ? P.g1 : P.g0;
                 if (it.type == OP_G2) {
 #pragma unroll
-                    for (int u = 0; u < 3; ++u) {
+                    for (int u = 0; u < (UNITS < 3 ? UNITS : 3); ++u) {
                         load_unit_h(P.h, chunk0, u, lane, hin[u]);
                         load_unit_g(gsrc, chunk0, u, lane, gin[u]);
                     }
                 } else if (mod) {
+                    // the products did not wait for the residual stream: this warp does, before it reads it
+                    if (BN < ACC_COLS) {
+                        if (lane == 0) ok = wait_counters(P.counters + (size_t)it.abs_m * CTRS, it.needE, nullptr, 0, P);
+                        ok = __all_sync(0xffffffffu, ok);
+                        if (!ok) break;
+                    }
+                    if (!mod_idle) {
 #pragma unroll
-                    for (int u = 0; u < 3; ++u) load_unit_h(P.h, chunk0, u, lane, hin[u]);
+                        for (int u = 0; u < (MOD_UNITS < 3 ? MOD_UNITS : 3); ++u)
+                            load_unit_h(P.h, chunk0, u, lane, hin[u]);
+                    }
                 }
-                // bias values of the warp's chunks, one column per lane (modulation items: shift in bq[0..1], scale in bq[2..3])
+                // bias values of the warp's 32-column chunks, one column per lane (modulation items: shift in bq[0..1],
+                // scale, 128 rows further in the packed weights, in bq[2..3])
                 float bq[4] = {0.f, 0.f, 0.f, 0.f};
                 {
                     const float* bb = it.type == OP_IN     ? P.bin + col0
                                       : it.type == OP_COND ? P.bc + col0
                                                            : P.bias_cat + it.b_row + acc0;
-                    if (it.type != OP_OUT) {
+                    if (it.type != OP_OUT && !mod_idle) {
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
-                            bq[q] = __ldg(bb + (mod ? (q & 1) * 32 + (q >> 1) * 128 : q * 32) + lane);
+                            if (mod ? (q & 1) < MOD_UNITS / 2 : q < SPAN / 32)
+                                bq[q] = __ldg(bb + (mod ? (q & 1) * 32 + (q >> 1) * 128 : q * 32) + lane);
                     }
                 }
                 float mean = 0.f, rstd = 0.f;
-                if (mod) row_mean_rstd(P, grow, mean, rstd);
+                if (mod && !mod_idle) row_mean_rstd<SPAN>(P, grow, mean, rstd);
                 const uint32_t buf = acc_iter & 1u;
                 const uint32_t acc_phase = (acc_iter >> 1) & 1u;
                 ok = wait_mbar(tfull_bar(buf), acc_phase, P);
@@ -845,7 +889,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                 fail = !ok;
                 if (ew == 0) TRACE(2, 1);
                 ptx::tc_fence_after();
-                const uint32_t tacc = tmem_base + buf * BN + ((uint32_t)(quarter * 32) << 16);
+                const uint32_t tacc = X.tmem_base + buf * ACC_COLS + ((uint32_t)(quarter * 32) << 16);
                 // a slab may be rewritten once the TMA store that read it last (two stores back) is done reading
                 auto slab_ready = [&]() {
                     if (ptx::elect_one()) ptx::bulk_wait_read<EPI_NB - 1>();
@@ -862,12 +906,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                 if (fail) {
                     // aborted: nothing valid to work on
                 } else if (it.type == OP_OUT) {
-                    if (half == 0) epi_out(P, it, tacc, grow, it.abs_m * BM + row, count);
+                    if (half == 0) epi_out(P, it, tacc, grow, it.abs_m * BM + row, X.count);
                 } else if (it.type == OP_COND) {
                     // c = acc + bc stays in registers; s_k = SiLU(c + temb_k) leaves as one bf16 slab per step
                     int n_st = 0;
 #pragma unroll 1
-                    for (int j = 0; j < 4; ++j) {
+                    for (int j = 0; j < SPAN / 32; ++j) {
                         float cv[32];
                         {
                             float lo[16], hi[16];
@@ -898,10 +942,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                         }
                     }
                 } else if (it.type == OP_IN) {
-                    // h = acc + bin, straight to global memory; LayerNorm partials of the 128 columns
+                    // h = acc + bin, straight to global memory; LayerNorm partials of the span's columns
                     Stats st;
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
+                    for (int u = 0; u < UNITS; ++u) {
                         float v[16];
                         load_acc16(tacc + acc0 + 16 * u, v);
                         add_bias16(v, (u >> 1) == 0 ? bq[0] : (u >> 1) == 1 ? bq[1] : (u >> 1) == 2 ? bq[2] : bq[3], 16 * (u & 1));
@@ -910,12 +954,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                         for (int i = 0; i < 16; ++i) st.add(v[i]);
                         store_unit_h(P.h, chunk0, u, lane, v);
                     }
-                    P.stats[(size_t)grow * (2 * P.NT) + it.nt * 2 + half] = st.finish(128);
+                    P.stats[(size_t)grow * (2 * V.NT) + it.nt * 2 + half] = st.finish(SPAN);
                 } else if (it.type == OP_GATE) {
                     // g = acc + bias, as bf16 straight to global memory
                     bf16* gdst = it.gsel == 2 ? P.g1 : P.g0;
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
+                    for (int u = 0; u < UNITS; ++u) {
                         float v[16];
                         load_acc16(tacc + acc0 + 16 * u, v);
                         add_bias16(v, (u >> 1) == 0 ? bq[0] : (u >> 1) == 1 ? bq[1] : (u >> 1) == 2 ? bq[2] : bq[3], 16 * (u & 1));
@@ -924,7 +968,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                 } else if (it.type == OP_G1) {
                     // a = SiLU(acc + b1): operand of the next GEMM, leaves as bf16 slabs
 #pragma unroll 1
-                    for (int j = 0; j < 4; ++j) {
+                    for (int j = 0; j < SPAN / 32; ++j) {
                         const uint32_t sl = my_buf + (uint32_t)(j & 1) * SLAB_H;
                         const float bj = j == 0 ? bq[0] : j == 1 ? bq[1] : j == 2 ? bq[2] : bq[3];
                         slab_ready();
@@ -941,14 +985,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                     }
                 } else if (mod) {
                     // u = LN(h) * (1 + scale) + shift: operand of the next GEMM, leaves as bf16 slabs
+                    const int n_mod = mod_idle ? 0 : MOD_UNITS;
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
+                    for (int u = 0; u < MOD_UNITS; ++u) {
+                        if (u >= n_mod) break;
                         const uint32_t sl = my_buf + (uint32_t)((u >> 1) & 1) * SLAB_H;
-                        if (u + 3 < 4) load_unit_h(P.h, chunk0, u + 3, lane, hin[(u + 3) & 3]);
+                        if (u + 3 < MOD_UNITS) load_unit_h(P.h, chunk0, u + 3, lane, hin[(u + 3) & 3]);
                         if ((u & 1) == 0) slab_ready();
                         float sh[16], sc[16], hv[16];
                         load_acc16(tacc + acc0 + 16 * u, sh);
-                        load_acc16(tacc + acc0 + 128 + 16 * u, sc);
+                        load_acc16(tacc + acc0 + BN / 2 + 16 * u, sc);
                         add_bias16(sh, (u >> 1) == 0 ? bq[0] : bq[1], 16 * (u & 1));
                         add_bias16(sc, (u >> 1) == 0 ? bq[2] : bq[3], 16 * (u & 1));
                         unit_h_values(hin[u & 3], hv);
@@ -958,11 +1004,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                         if (u & 1) slab_store(EMAP_U, sl, col0 + 32 * (u >> 1), row0);
                     }
                 } else {
-                    // OP_G2: h += g * (acc + b2), read and written in place; LayerNorm partials of the 128 columns
+                    // OP_G2: h += g * (acc + b2), read and written in place; LayerNorm partials of the span's columns
                     Stats st;
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        if (u + 3 < 8) {
+                    for (int u = 0; u < UNITS; ++u) {
+                        if (u + 3 < UNITS) {
                             load_unit_h(P.h, chunk0, u + 3, lane, hin[(u + 3) & 3]);
                             load_unit_g(gsrc, chunk0, u + 3, lane, gin[(u + 3) & 3]);
                         }
@@ -978,7 +1024,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
                         for (int i = 0; i < 16; ++i) st.add(hv[i]);
                         store_unit_h(P.h, chunk0, u, lane, hv);
                     }
-                    P.stats[(size_t)grow * (2 * P.NT) + it.nt * 2 + half] = st.finish(128);
+                    P.stats[(size_t)grow * (2 * V.NT) + it.nt * 2 + half] = st.finish(SPAN);
                 }
                 ptx::tc_fence_before();
                 __syncwarp();
@@ -1005,13 +1051,71 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
         if (ptx::elect_one()) ptx::bulk_wait<0>();
         __syncwarp();
     }
+}
+
+// ------------------------------------------------------------------------------------------
+// the persistent kernel: clusters of two CTAs. Both load their own token tile (A) and half of the
+// weight tile (B); the even CTA issues cta_group::2 MMAs that read both CTAs' shared memory and
+// write 128 accumulator rows into each CTA's TMEM; every CTA runs the epilogue of its own token tile.
+// ------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_constant__ HeadParams P) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const uint32_t smem_base = ptx::smem_u32(smem);
+    const uint32_t bars = smem_base + RING_BYTES + EPI_BYTES;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + RING_BYTES + EPI_BYTES + 8 * NUM_BARS);
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const int rank = (int)ptx::cluster_ctarank();                  // token tile of the unit this CTA owns
+    const int unit_id = (int)blockIdx.x / 2;
+    const int n_units = (int)gridDim.x / 2;
+
+    int count = __ldg(P.count);
+    if (count > P.max_tokens) {
+        count = P.max_tokens;
+        if (threadIdx.x == 0 && blockIdx.x == 0) atomicCAS(P.status, 0, ARDIFF_ERR_SHAPE);
+    }
+    if (count < 0) count = 0;
+    const int MT = (count + BM - 1) / BM;
+    const int MTu = (MT + 1) / 2;                  // an odd last tile gets an all-padding partner
+    const int n_groups = (MTu + P.TGu - 1) / P.TGu;
+    const int tgu = n_groups > 0 ? (MTu + n_groups - 1) / n_groups : 1;   // balanced group size
+    // the narrowest items that the number of token tiles allows (see width_limit)
+    const int width = MTu <= P.prog[2].max_units ? 2 : MTu <= P.prog[1].max_units ? 1 : 0;
+
+    if (threadIdx.x == 0) {
+        // full[MAX_STAGES], empty[MAX_STAGES], accumulator full[2], accumulator free[2], drain, inputs complete[DEP_BARS]
+        for (int i = 0; i < NUM_BARS; ++i)
+            // an accumulator is freed by the epilogue warps of both CTAs of the unit
+            ptx::mbar_init(bars + 8u * i, i == 2 * MAX_STAGES + 2 || i == 2 * MAX_STAGES + 3 ? 2 * EPI_WARPS : 1);
+        ptx::fence_mbar_init();
+    }
+    if (warp == 1) {
+        ptx::tmem_alloc_pair(ptx::smem_u32(tmem_slot), 512);
+        ptx::tmem_relinquish_pair();
+    }
+    ptx::tc_fence_before();
+    ptx::cluster_sync_all();
+    ptx::tc_fence_after();
+    const Place X{smem_base, bars, *tmem_slot, rank, unit_id, n_units, count, MTu, tgu,
+                  (long long)MTu * (P.prog[width].T_pro + P.K * P.prog[width].T_step)};
+    long long probe_c0 = 0;
+    unsigned long long probe_g0 = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        probe_c0 = clock64();
+        probe_g0 = ptx::globaltimer_ns();
+    }
+
+    if (width == 0) run_roles<0>(P, X, warp, lane);
+    else if (width == 1) run_roles<1>(P, X, warp, lane);
+    else run_roles<2>(P, X, warp, lane);
 
     ptx::tc_fence_before();
     // nobody leaves while its partner may still signal its barriers or read its shared memory
     ptx::cluster_sync_all();
     if (warp == 1) {
         ptx::tc_fence_after();
-        ptx::tmem_dealloc_pair(tmem_base, 512);
+        ptx::tmem_dealloc_pair(X.tmem_base, 512);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0 && P.clock_probe) {
         // SM cycles and wall time of this launch as seen by CTA 0: their ratio is the clock the SM really ran at
@@ -1151,7 +1255,8 @@ inline float bf16_bits_to_float(uint16_t b) {
 struct ardiff_head {
     ardiff_head_desc d;
     int device, n_sm, grid, coop;
-    int NT, TGu, slots, T_pro, T_step, C_pro, C_step, n_phases;
+    int TGu, slots;
+    Program prog[N_WIDTHS];
     int64_t max_tiles;
     std::vector<void*> allocs;
     // device
@@ -1162,8 +1267,6 @@ struct ardiff_head {
     float2* stats;
     int *counters, *status;  // status[0] = status word, status[1] = abort flag
     long long* trace;        // per-item time stamps (only with ARDIFF_HEAD_PROFILE)
-    Phase* phases;
-    uint16_t* cum2phase;
     CUtensorMap* maps;
     long long* clock_probe;  // [2]: SM cycles and nanoseconds of the last launch, stamped by CTA 0
     // optional timing of the persistent kernel (state of the last call, not of the head: mutable)
@@ -1213,6 +1316,25 @@ int env_int(const char* name, int dflt) {
 }
 #endif
 
+}  // namespace
+
+namespace {
+// Most pairs of token tiles that items of width `wi` serve. Narrow items shorten every link of the chain of
+// dependent layers (K loop and epilogue) and give more units something to do, but each of them reads its token tile
+// again: 128 columns win while a W-wide layer is at most two thirds of a grid of them, 64 columns up to a quarter.
+// Kernel time in us with 256 / 128 / 64 columns, K = 4, W = 1024, 3 blocks: 256 tokens 434 / 363 / 341; 730: 474 / 431 /
+// 447; 1434: 504 / 472 / 619; 2048: 524 / 520 / 757; 3072: 519 / 649 / 1035. W = 1536, 6 blocks, K = 2: 512 tokens
+// 519 / 473 / 543; 1024: 548 / 541 / 768; 2048: 592 / 766 / 1346.
+int width_limit(int wi, int W, int units, int TGu) {
+    int lim = (wi == 1 ? 2 * units / 3 : units / 4) * item_cols(wi) / W;
+#ifdef ARDIFF_TUNING
+    lim = env_int(wi == 1 ? "ARDIFF_HEAD_W1" : "ARDIFF_HEAD_W2", lim);
+#endif
+    // one group, and no longer run of single-slice items than the dependency barriers allow
+    lim = lim < TGu ? lim : TGu;
+    const int run = 3 * units * item_cols(wi) / W;
+    return lim < run ? lim : run;
+}
 }  // namespace
 
 #define TRY(expr)                   \
@@ -1287,12 +1409,6 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     H->device = dev;
     H->n_sm = prop.multiProcessorCount;
     const int W = d.W, C = d.C, Dc = d.Dc, L = d.L;
-    const int NT = W / BN;
-    H->NT = NT;
-    H->T_pro = 1 + 2 * NT;     // gather, conditioning items, the gate of step 0 / block 0
-    H->T_step = NT * (3 + 5 * L) + 1;
-    H->C_pro = 1 + NT;
-    H->C_step = NT * (3 + 4 * L) + 1;
     H->max_tiles = (d.max_tokens + BM - 1) / BM;
     if (H->max_tiles < 1) H->max_tiles = 1;
 
@@ -1330,7 +1446,8 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
 
     // largest group, in units (pairs of token tiles): a phase of NT column tiles per token tile should
     // span about 2.5 grids of items so that a dependent phase finds its producers long finished
-    int tgu = (5 * units / 2 + NT - 1) / NT;
+    const int NT0 = W / item_cols(0);
+    int tgu = (5 * units / 2 + NT0 - 1) / NT0;
 #ifdef ARDIFF_TUNING
     {
         const int tg_env = env_int("ARDIFF_HEAD_TGU", 0);
@@ -1338,10 +1455,12 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     }
 #endif
     // A unit gets r = ceil(tgu * NT / units) in-projection items in a row, each a single K slice: the producer can
-    // then be r + 1 items ahead of the MMA issuer, which with its two accumulators is up to 2 ahead of the
-    // epilogue; the dependency barriers are a ring of DEP_BARS phases, so r + 3 must stay below DEP_BARS
-    // (r = 3 with the group size chosen above).
-    while (tgu > 1 && ((int64_t)tgu * NT + units - 1) / units > DEP_BARS - 4) --tgu;
+    // then be r + 1 + MAX_STAGES / 4 items ahead of the MMA issuer (all other items have at least 4 slices), which
+    // with its two accumulators is up to 2 ahead of the epilogue; the dependency barriers are a ring of DEP_BARS
+    // phases, so r + 6 must stay below DEP_BARS (r = 3 with the group size chosen above).
+    constexpr int MAX_RUN = 4;
+    static_assert(MAX_RUN + 3 + MAX_STAGES / 4 < DEP_BARS, "dependency barriers");
+    while (tgu > 1 && ((int64_t)tgu * NT0 + units - 1) / units > MAX_RUN) --tgu;
     if (tgu < 1) tgu = 1;
     if ((int64_t)tgu * 2 > H->max_tiles + 1) tgu = (int)((H->max_tiles + 1) / 2);
     H->TGu = tgu;
@@ -1414,7 +1533,7 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     TRY(dev_alloc(H, &H->g1, R * W, true));
     TRY(dev_alloc(H, &H->x, R * C, true));
     TRY(dev_alloc(H, &H->h, R * W, true));
-    TRY(dev_alloc(H, &H->stats, R * 2 * NT, true));
+    TRY(dev_alloc(H, &H->stats, R * 2 * (W / item_cols(N_WIDTHS - 1)), true));
     TRY(dev_alloc(H, &H->counters, ((size_t)H->max_tiles + 2) * CTRS, true));
     TRY(dev_alloc(H, &H->status, 2, true));
     TRY(dev_alloc(H, &H->clock_probe, 2, true));
@@ -1422,8 +1541,16 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     TRY(dev_alloc(H, &H->trace, (size_t)TRACE_ITEMS * 12 + (size_t)TRACE_ITEMS * 16, true));
 #endif
 
-    // ---- the program of one step: phases in list order ----
-    {
+    // ---- the program of one step for every item width: phases in list order ----
+    for (int wi = 0; wi < N_WIDTHS; ++wi) {
+        Program& V = H->prog[wi];
+        const int NT = W / item_cols(wi);
+        V.NT = NT;
+        V.T_pro = 1 + 2 * NT;     // gather, conditioning items, the gate of step 0 / block 0
+        V.T_step = NT * (3 + 5 * L) + 1;
+        V.C_pro = 1 + NT;
+        V.C_step = NT * (3 + 4 * L) + 1;
+        V.max_units = wi == 0 ? 0x7fffffff : width_limit(wi, W, units, H->TGu);
         std::vector<Phase> ph;
         int cum = 0;
         auto add = [&](int type, int block, int tile0, int ntiles, size_t b_row0, int offA, int kplus) {
@@ -1453,7 +1580,7 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
         gate(0, 1, L - 1, 0, na);
         add(OP_OUT, -1, 0, 1, out_row0, NT + 4 * NT * L + 2 * NT, 0);
         gate(0, 1, L - 1, na, NT - na);
-        if (cum != H->T_step) {
+        if (cum != V.T_step) {
             free_all(H);
             delete H;
             return ARDIFF_ERR_UNSUPPORTED;
@@ -1461,11 +1588,14 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
         std::vector<uint16_t> c2p(cum);
         for (size_t i = 0; i < ph.size(); ++i)
             for (int t = 0; t < ph[i].ntiles; ++t) c2p[ph[i].cum + t] = (uint16_t)i;
-        H->n_phases = (int)ph.size();
-        TRY(dev_alloc(H, &H->phases, ph.size(), false));
-        TRY(upload(H->phases, ph.data(), ph.size() * sizeof(Phase)));
-        TRY(dev_alloc(H, &H->cum2phase, c2p.size(), false));
-        TRY(upload(H->cum2phase, c2p.data(), c2p.size() * sizeof(uint16_t)));
+        Phase* phases = nullptr;
+        uint16_t* cum2phase = nullptr;
+        TRY(dev_alloc(H, &phases, ph.size(), false));
+        TRY(upload(phases, ph.data(), ph.size() * sizeof(Phase)));
+        TRY(dev_alloc(H, &cum2phase, c2p.size(), false));
+        TRY(upload(cum2phase, c2p.data(), c2p.size() * sizeof(uint16_t)));
+        V.phases = phases;
+        V.cum2phase = cum2phase;
     }
 
     // ---- tensor maps ----
@@ -1478,9 +1608,12 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
         ok &= make_map(&maps[MAP_U], H->u, R, W, BM);
         ok &= make_map(&maps[MAP_A], H->a, R, W, BM);
         // a CTA of a pair stages half of the weight tile's rows
-        ok &= make_map(&maps[MAP_WC], H->Wc, W, Dc, B_ROWS);
-        ok &= make_map(&maps[MAP_WIN], H->Win, W, XB_COLS, B_ROWS);
-        ok &= make_map(&maps[MAP_WCAT], H->Wcat, cat_rows, W, B_ROWS);
+        for (int wi = 0; wi < N_WIDTHS; ++wi) {
+            const uint32_t b_rows = (uint32_t)item_cols(wi) / 2;
+            ok &= make_map(&maps[MAP_B + 3 * wi + W_C], H->Wc, W, Dc, b_rows);
+            ok &= make_map(&maps[MAP_B + 3 * wi + W_IN], H->Win, W, XB_COLS, b_rows);
+            ok &= make_map(&maps[MAP_B + 3 * wi + W_CAT], H->Wcat, cat_rows, W, b_rows);
+        }
         ok &= make_map(&maps[MAP_WOUT], H->Wcat, cat_rows, W, (uint32_t)C / 2);
         ok &= make_slab_map(&maps[EMAP_S], H->s, (uint64_t)kmax * R, W);
         ok &= make_slab_map(&maps[EMAP_U], H->u, R, W);
@@ -1552,12 +1685,11 @@ int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise,
 
     HeadParams P;
     memset(&P, 0, sizeof(P));
-    P.C = C; P.Dc = H->d.Dc; P.W = W; P.L = H->d.L; P.K = K; P.NT = H->NT; P.TGu = H->TGu; P.slots = H->slots;
-    P.T_pro = H->T_pro; P.T_step = H->T_step; P.T_chain = H->T_pro + K * H->T_step;
-    P.C_pro = H->C_pro; P.C_step = H->C_step; P.C_total = H->C_pro + K * H->C_step;
+    P.C = C; P.Dc = H->d.Dc; P.W = W; P.L = H->d.L; P.K = K; P.TGu = H->TGu; P.slots = H->slots;
+    for (int wi = 0; wi < N_WIDTHS; ++wi) P.prog[wi] = H->prog[wi];
     P.R = H->slots * BM;
     P.max_tokens = (int)H->d.max_tokens;
-    P.phases = H->phases; P.cum2phase = H->cum2phase; P.maps = H->maps;
+    P.maps = H->maps;
     P.cond = reinterpret_cast<const bf16*>(cond); P.noise = noise; P.idx = idx; P.count = count; P.out = out;
     P.z = H->z; P.xb = H->xb; P.s = H->s; P.u = H->u; P.a = H->a; P.g0 = H->g0; P.g1 = H->g1;
     P.x = H->x; P.h = H->h; P.stats = H->stats;

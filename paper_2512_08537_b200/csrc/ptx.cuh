@@ -42,6 +42,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
+// the same without suspending the thread
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // One lane of a converged warp, the same one every time. Asynchronous instructions (tcgen05.mma, commits, TMA
 // copies) take their operands from uniform registers: under `lane == 0` the compiler cannot know that one thread
 // is active and walks the active lanes one by one, under elect.sync it does not. Measured on a ring that is always
