@@ -206,7 +206,8 @@ typedef struct {
 
 /*
  * Packs the weights into the kernels' tile layout on the current device and allocates
- * the head's scratch (a fixed-size activation workspace for two groups of token tiles plus
+ * the head's scratch (a fixed-size activation workspace for two groups of token tiles, up to
+ * 128 MB of modulation values plus a smaller exchange buffer for calls of few tokens, and
  * max_tokens/128 progress counters). Synchronous; the only head call that allocates.
  * Side effect on the CUDA context: while at least one head exists on a device, the context's
  * cudaLimitPersistingL2CacheSize is at least the size of one token group's fp32 residual
@@ -236,8 +237,10 @@ int ardiff_head_destroy(ardiff_head* head);
  *                 status word as ARDIFF_ERR_SHAPE)
  *   out      dev  float [n][C]: rows idx[j] are written, all other rows are left untouched
  * One persistent cooperative kernel walks a static schedule of GEMM tiles; tiles wait for
- * their producers on device-side counters with bounded spins. If a wait runs out the
- * kernel finishes early, the results are invalid and ardiff_head_status reports
+ * their producers on device-side counters with bounded spins. Up to 64 survivors (as many as
+ * *count says, for widths up to 2048) the layers that depend on x leave that schedule and run with
+ * one exchange of values between SMs per layer; those waits are bounded the same way. If a wait
+ * runs out the kernel finishes early, the results are invalid and ardiff_head_status reports
  * ARDIFF_ERR_TIMEOUT. Calls on one head must not overlap on the device (they share its
  * scratch): enqueue them on one stream or order them with events.
  */

@@ -52,6 +52,8 @@ using bf16 = __nv_bfloat16;
 constexpr int BM = 128;           // tokens per tile (one CTA)
 constexpr int BK = 64;            // K slice per pipeline stage (128 bytes of bf16: one swizzle row)
 constexpr int A_BYTES = BM * BK * 2;
+constexpr int N_PROGRAMS = 4;     // item lists: one per item width, and what the chain (chain.cuh) leaves
+constexpr int MOD_PROGRAM = 3, MOD_WIDTH = 1;
 constexpr int N_WIDTHS = 3;       // item widths: width w has item_cols(w) output columns per item (UMMA N)
 __host__ __device__ constexpr int item_cols(int w) { return 256 >> w; }
 constexpr int ACC_COLS = 256;     // TMEM columns of one of the two accumulators
@@ -101,7 +103,7 @@ constexpr int TRACE_ITEMS = 4096;
 #define TRACE_NEXT()
 #endif
 
-enum OpType : int { OP_GATHER = 0, OP_COND, OP_IN, OP_SS, OP_GATE, OP_G1, OP_G2, OP_FSS, OP_OUT, OP_NOP, OP_END = 15 };
+enum OpType : int { OP_GATHER = 0, OP_COND, OP_IN, OP_SS, OP_GATE, OP_G1, OP_G2, OP_FSS, OP_OUT, OP_NOP, OP_MOD, OP_END = 15 };
 enum MapId : int {
     MAP_Z = 0, MAP_XB, MAP_S, MAP_U, MAP_A, MAP_WOUT,   // GEMM operands
     EMAP_S, EMAP_U, EMAP_A,                             // epilogue output slabs
@@ -138,7 +140,7 @@ struct HeadParams {
     int C, Dc, W, L, K, TGu, slots;         // TGu = largest group in units, slots = scratch tiles
     int R;                                  // rows of the scratch arrays (slots * 128)
     int max_tokens;
-    Program prog[N_WIDTHS];
+    Program prog[N_PROGRAMS];
     const CUtensorMap* maps;
     const bf16* cond;
     const float* noise;
@@ -157,6 +159,10 @@ struct HeadParams {
     long long step_stride;                  // n * C
     float ax[KMAX], av[KMAX], an[KMAX];     // sampler step k: x <- ax x + av v + an z_k
     unsigned long long wait_limit_ns;       // bound of every dependency wait
+    int chain_count;                        // up to this many survivors chain.cuh does what depends on x and h:
+    int grid_counter;                       // index of the grid barrier's counter
+    float* mods;                            // here only s_k and all modulations (into mods), and its exchange buffer
+    uint8_t* xch;                           // is set to "nothing there yet"
     int stall_tile;                         // self-test: conditioning items of this token tile wait for one
                                             // predecessor more than exists (-1: none)
     long long* clock_probe;                 // [4]: clock64 and globaltimer of CTA 0 at start and end
@@ -256,34 +262,38 @@ __device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w &
 
 // Item `item` of the static list, for the CTA of rank `rank` within its unit. MTu = units (pairs of
 // token tiles) of this call, tgu = units per group (balanced over the groups).
-template <int WI>
-__device__ __forceinline__ Packed decode_packed(const HeadParams& P, int MTu, int tgu, int rank, long long item,
+template <int WI, int PI>
+__device__ __forceinline__ Packed decode_packed(const HeadParams& P, int MTu, int tgu, int steps, int rank, long long item,
                                                 long long total) {
     constexpr int BN = item_cols(WI);
-    const Program& V = P.prog[WI];
+    const Program& V = P.prog[PI];
     Packed pk{(uint32_t)OP_END << 24, 0u, 0u, 0u, 0u};
     if (item >= total) return pk;
-    const long long per_group = (long long)tgu * (V.T_pro + P.K * V.T_step);
+    const long long per_group = (long long)tgu * (V.T_pro + steps * V.T_step);
     const int grp = (int)(item / per_group);
     int r = (int)(item - (long long)grp * per_group);
     const int m0 = grp * tgu;
     const int mtg = min(tgu, MTu - m0);
-    const int pro = mtg * V.T_pro;
+    // The modulations-only list has one pair of token tiles; its "token units" are pairs of steps, so that the items of
+    // one weight tile lie side by side in the list and the weights come from HBM once.
+    const int mtp = PI == MOD_PROGRAM ? 1 : mtg;
+    const int pro = mtp * V.T_pro;
     int m, type, nt = 0, k = 0, block = 0, gsel = 0;
     int needA = 0, needB = 0, b_row = 0;
     if (r < pro) {
-        if (r < mtg) {
+        const int mgath = PI == MOD_PROGRAM ? 0 : mtg;     // (there the rows are gathered before this kernel)
+        if (r < mgath) {
             type = OP_GATHER; m = r;
-        } else if (r < mtg + mtg * V.NT) {
-            r -= mtg;
+        } else if (r < mgath + mtp * V.NT) {
+            r -= mgath;
             m = r / V.NT;
             nt = r - m * V.NT;
             type = OP_COND;
-            needA = EPI_WARPS;            // the gather of this token tile
+            needA = PI == MOD_PROGRAM ? 0 : EPI_WARPS;   // the gather of this token tile
             b_row = nt * BN;
         } else {
             // the gate of step 0, block 0 (gate number 0): needs s_0, i.e. the conditioning items
-            r -= mtg + mtg * V.NT;
+            r -= mgath + mtp * V.NT;
             m = r / V.NT;
             nt = r - m * V.NT;
             type = OP_GATE; gsel = 1;
@@ -326,6 +336,10 @@ __device__ __forceinline__ Packed decode_packed(const HeadParams& P, int MTu, in
             b_row = p.b_row0 + (nt * (BN / 2) / 128) * 256 + nt * (BN / 2) % 128;
         }
     }
+    if (PI == MOD_PROGRAM) {
+        k = m;
+        m = 0;
+    }
     const int abs_m = (m0 + m) * 2 + rank;
     if (type == OP_COND && abs_m == P.stall_tile) needA += 1;   // self-test: never satisfied
     pk.w0 = (uint32_t)abs_m | ((uint32_t)type << 24);
@@ -360,6 +374,12 @@ __device__ __forceinline__ void unpack_item(const HeadParams& P, const Packed& p
         case OP_IN: it.map_a = MAP_XB; it.map_b = MAP_B + 3 * WI + W_IN; it.kblocks = 1; break;
         case OP_G1: it.map_a = MAP_U; break;
         case OP_G2: it.map_a = MAP_A; break;
+        case OP_MOD:
+            // the pair takes two steps of the one token tile: rank r of it step 2 k + r
+            it.k = 2 * it.k + it.abs_m;
+            it.abs_m = 0; it.slot_row0 = 0;
+            it.a_row0 = min(it.k, P.K - 1) * P.R;
+            break;
         case OP_OUT: it.map_a = MAP_U; it.map_b = MAP_WOUT; it.umma_n = P.C; it.b_step = P.C / 2; break;
         default: break;
     }
@@ -367,14 +387,14 @@ __device__ __forceinline__ void unpack_item(const HeadParams& P, const Packed& p
 
 // The items of one CTA, decoded 32 at a time (lane l decodes the l-th of the next 32) and handed
 // out by shuffle. Every lane of the warp calls next() together.
-template <int WI>
+template <int WI, int PI>
 struct ItemStream {
     Packed mine;
     int n = 0;
-    __device__ __forceinline__ bool next(const HeadParams& P, int MTu, int tgu, int rank, int unit_id, int n_units,
+    __device__ __forceinline__ bool next(const HeadParams& P, int MTu, int tgu, int steps, int rank, int unit_id, int n_units,
                                          long long total, int lane, Item& it) {
         if ((n & 31) == 0)
-            mine = decode_packed<WI>(P, MTu, tgu, rank, (long long)unit_id + (long long)(n + lane) * n_units, total);
+            mine = decode_packed<WI, PI>(P, MTu, tgu, steps, rank, (long long)unit_id + (long long)(n + lane) * n_units, total);
         Packed cur;
         const int src = n & 31;
         cur.w0 = __shfl_sync(0xffffffffu, mine.w0, src);
@@ -388,6 +408,8 @@ struct ItemStream {
         return true;
     }
 };
+
+#include "chain.cuh"
 
 // ------------------------------------------------------------------------------------------
 // epilogues. Two epilogue warps share each 32-row quarter of the tile (TMEM lane quarter*32 + lane);
@@ -616,19 +638,21 @@ __device__ __forceinline__ void gather_rows(const HeadParams& P, const Item& it,
 struct Place {
     uint32_t smem_base, bars, tmem_base;
     int rank, unit_id, n_units;             // token tile of the unit this CTA owns, its unit, all units
-    int count, MTu, tgu;                    // survivors; pairs of token tiles: of the call, of one group
+    int count, MTu, tgu;                    // survivors; pairs of token tiles (modulations only: of steps): of the call,
+                                            // of one group
+    int steps;                              // repetitions of the program's step
     long long total;                        // items of the call
 };
 
 // The three roles of a CTA over the call's items, which are item_cols(WI) columns wide.
-template <int WI>
+template <int WI, int PI = WI>
 __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, int warp, int lane) {
     constexpr int BN = item_cols(WI);
     constexpr int STAGES = Ring<BN>::STAGES, STAGE_BYTES = Ring<BN>::STAGE_BYTES;
     constexpr int SPAN = BN / 2;                                 // accumulator columns of one epilogue warp
     constexpr int UNITS = SPAN / 16;
     constexpr int MOD_UNITS = UNITS / 2 < 2 ? 2 : UNITS / 2;     // of shift, and of scale
-    const Program& V = P.prog[WI];
+    const Program& V = P.prog[PI];
     const uint32_t smem_base = X.smem_base, bars = X.bars;
     const uint32_t epi_base = smem_base + RING_BYTES;            // 1024-aligned
     const int rank = X.rank;
@@ -645,13 +669,13 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
         uint32_t issued = 0, issued_parity = 0;
         uint32_t seq = 0;
         bool aborted = false;
-        ItemStream<WI> ist;
+        ItemStream<WI, PI> ist;
         Item it, nx;
         TRACE_DECL
         // next item with operands to load (gather items have none)
         auto next_item = [&](Item& dst) {
             bool have;
-            do have = ist.next(P, X.MTu, X.tgu, rank, X.unit_id, X.n_units, X.total, lane, dst);
+            do have = ist.next(P, X.MTu, X.tgu, X.steps, rank, X.unit_id, X.n_units, X.total, lane, dst);
             while (have && (dst.type == OP_GATHER || dst.type == OP_NOP));
             return have;
         };
@@ -754,10 +778,10 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
             int stage = 0;
             uint32_t phase = 0;
             uint32_t acc_iter = 0;
-            ItemStream<WI> ist;
+            ItemStream<WI, PI> ist;
             Item it;
             TRACE_DECL
-            while (ist.next(P, X.MTu, X.tgu, rank, X.unit_id, X.n_units, X.total, lane, it)) {
+            while (ist.next(P, X.MTu, X.tgu, X.steps, rank, X.unit_id, X.n_units, X.total, lane, it)) {
                 if (it.type == OP_GATHER || it.type == OP_NOP) continue;
                 const uint32_t buf = acc_iter & 1u;
                 const uint32_t acc_phase = (acc_iter >> 1) & 1u;
@@ -810,17 +834,17 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
         const uint32_t my_buf = epi_base + (uint32_t)ew * EPI_NB * SLAB_H;
         uint32_t acc_iter = 0;
         uint32_t seq = 0;
-        ItemStream<WI> ist;
+        ItemStream<WI, PI> ist;
         Item it;
         TRACE_DECL
-        while (ist.next(P, X.MTu, X.tgu, rank, X.unit_id, X.n_units, X.total, lane, it)) {
+        while (ist.next(P, X.MTu, X.tgu, X.steps, rank, X.unit_id, X.n_units, X.total, lane, it)) {
             bool fail = false;
             if (it.type == OP_NOP) continue;
             if (it.type == OP_GATHER) {
                 bool ok = true;
                 // the scratch slot is free once the token tile that used it before has run its whole chain
                 if (lane == 0 && it.abs_m >= P.slots)
-                    ok = wait_counters(P.counters + (size_t)(it.abs_m - P.slots) * CTRS, EPI_WARPS * (V.C_pro + P.K * V.C_step),
+                    ok = wait_counters(P.counters + (size_t)(it.abs_m - P.slots) * CTRS, EPI_WARPS * (V.C_pro + X.steps * V.C_step),
                                        nullptr, 0, P);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
@@ -965,6 +989,24 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
                         add_bias16(v, (u >> 1) == 0 ? bq[0] : (u >> 1) == 1 ? bq[1] : (u >> 1) == 2 ? bq[2] : bq[3], 16 * (u & 1));
                         store_unit_g(gdst, chunk0, u, lane, v);
                     }
+                } else if (PI == MOD_PROGRAM && it.type == OP_MOD) {
+                    // acc + bias of step it.k in fp32, for the chain: tiles of 128 rows, shift and scale in turn,
+                    // then the gates
+                    const int which = it.nt < 2 * V.NT ? it.nt & 1 : 2;
+                    const int ch = (which == 2 ? it.nt - 2 * V.NT : it.nt >> 1) * BN + half * SPAN;
+                    float* dst = P.mods + mods_index(X.count, P.L, P.W, it.k, it.block, which) + (size_t)row * P.W + ch;
+                    const bool live = it.k < P.K && row < X.count;
+#pragma unroll
+                    for (int u = 0; u < UNITS; ++u) {
+                        float v[16];
+                        load_acc16(tacc + acc0 + 16 * u, v);
+                        add_bias16(v, (u >> 1) == 0 ? bq[0] : (u >> 1) == 1 ? bq[1] : (u >> 1) == 2 ? bq[2] : bq[3], 16 * (u & 1));
+                        if (live) {
+#pragma unroll
+                            for (int i = 0; i < 16; i += 4)
+                                ptx::st_f4(dst + 16 * u + i, make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]));
+                        }
+                    }
                 } else if (it.type == OP_G1) {
                     // a = SiLU(acc + b1): operand of the next GEMM, leaves as bf16 slabs
 #pragma unroll 1
@@ -1040,7 +1082,7 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
             // read by TMA (z, xb) additionally need the generic -> async proxy fence on the writer's side.
             if (it.type == OP_GATHER || it.type == OP_OUT) ptx::fence_proxy_async();
             __syncwarp();
-            if (lane == 0)
+            if (lane == 0 && !(PI == MOD_PROGRAM && it.type == OP_MOD))
                 ptx::red_release_gpu_add(P.counters + (size_t)it.abs_m * CTRS + (it.type == OP_GATE ? it.gsel : 0), 1);
             if (it.type != OP_GATHER) {
                 if (ew == 0) { TRACE(2, 2); TRACE_TYPE(2); }
@@ -1053,13 +1095,27 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
     }
 }
 
+// The modulations-only list, and the exchange buffer cleared, as a call: inlined beside the other three they made those
+// spill (730 tokens, W = 1024: 443 -> 454 us).
+__device__ __noinline__ void run_modulations(const HeadParams& P, const Place X, int warp, int lane) {
+    const ChainLayout lay(X.count, P.K, P.L, P.W, P.C);
+    for (size_t i = (size_t)blockIdx.x * NUM_THREADS + threadIdx.x; i < lay.total / 16; i += (size_t)gridDim.x * NUM_THREADS) {
+        const uint32_t v = i * 16 < lay.u ? 0u : CHAIN_EMPTY;
+        ptx::st_u4(P.xch + i * 16, make_uint4(v, v, v, v));
+    }
+    run_roles<MOD_WIDTH, MOD_PROGRAM>(P, X, warp, lane);
+}
+
 // ------------------------------------------------------------------------------------------
 // the persistent kernel: clusters of two CTAs. Both load their own token tile (A) and half of the
 // weight tile (B); the even CTA issues cta_group::2 MMAs that read both CTAs' shared memory and
 // write 128 accumulator rows into each CTA's TMEM; every CTA runs the epilogue of its own token tile.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_constant__ HeadParams P) {
+__global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_constant__ HeadParams P,
+                                                              const __grid_constant__ ChainParams Q) {
     extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t s_chain_bars[2 * CHAIN_MAX_SLOTS];
+    __shared__ int s_chain_abort;
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t smem_base = ptx::smem_u32(smem);
     const uint32_t bars = smem_base + RING_BYTES + EPI_BYTES;
@@ -1081,7 +1137,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
     const int n_groups = (MTu + P.TGu - 1) / P.TGu;
     const int tgu = n_groups > 0 ? (MTu + n_groups - 1) / n_groups : 1;   // balanced group size
     // the narrowest items that the number of token tiles allows (see width_limit)
-    const int width = MTu <= P.prog[2].max_units ? 2 : MTu <= P.prog[1].max_units ? 1 : 0;
+    const bool chained = count > 0 && count <= P.chain_count;
+    const int program = chained ? MOD_PROGRAM : MTu <= P.prog[2].max_units ? 2 : MTu <= P.prog[1].max_units ? 1 : 0;
+    const int pairs = chained ? (P.K + 1) / 2 : MTu;             // of steps, or of token tiles
+    const int steps = chained ? 1 : P.K;
 
     if (threadIdx.x == 0) {
         // full[MAX_STAGES], empty[MAX_STAGES], accumulator full[2], accumulator free[2], drain, inputs complete[DEP_BARS]
@@ -1097,8 +1156,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
     ptx::tc_fence_before();
     ptx::cluster_sync_all();
     ptx::tc_fence_after();
-    const Place X{smem_base, bars, *tmem_slot, rank, unit_id, n_units, count, MTu, tgu,
-                  (long long)MTu * (P.prog[width].T_pro + P.K * P.prog[width].T_step)};
+    const Place X{smem_base, bars, *tmem_slot, rank, unit_id, n_units, count, pairs, chained ? pairs : tgu, steps,
+                  (long long)MTu * P.prog[program].T_pro + (long long)pairs * steps * P.prog[program].T_step};
     long long probe_c0 = 0;
     unsigned long long probe_g0 = 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1106,9 +1165,41 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
         probe_g0 = ptx::globaltimer_ns();
     }
 
-    if (width == 0) run_roles<0>(P, X, warp, lane);
-    else if (width == 1) run_roles<1>(P, X, warp, lane);
-    else run_roles<2>(P, X, warp, lane);
+    if (program == 0) run_roles<0>(P, X, warp, lane);
+    else if (program == 1) run_roles<1>(P, X, warp, lane);
+    else if (program == 2) run_roles<2>(P, X, warp, lane);
+    else {
+        if (threadIdx.x == 0) {
+            s_chain_abort = 0;
+            for (int i = 0; i < 2 * CHAIN_MAX_SLOTS; ++i)
+                ptx::mbar_init(ptx::smem_u32(s_chain_bars + i), i < CHAIN_MAX_SLOTS ? 1 : CHAIN_WARPS);
+            ptx::fence_mbar_init();
+        }
+        run_modulations(P, X, warp, lane);
+        // grid barrier: every CTA's modulations and its share of the cleared exchange buffer are there
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int* arrived = P.counters + P.grid_counter;
+            ptx::red_release_gpu_add(arrived, 1);
+            if (!wait_counters(arrived, (int)gridDim.x, nullptr, 0, P)) s_chain_abort = 1;
+        }
+        __syncthreads();
+        if ((int)blockIdx.x < P.W / CHAIN_COLS && !s_chain_abort) {
+            const uint32_t cb = ptx::smem_u32(s_chain_bars);
+            switch (P.W / 256) {
+                case 1: chain_cta<1>(Q, count, smem, cb, &s_chain_abort); break;
+                case 2: chain_cta<2>(Q, count, smem, cb, &s_chain_abort); break;
+                case 3: chain_cta<3>(Q, count, smem, cb, &s_chain_abort); break;
+                case 4: chain_cta<4>(Q, count, smem, cb, &s_chain_abort); break;
+                case 5: chain_cta<5>(Q, count, smem, cb, &s_chain_abort); break;
+                case 6: chain_cta<6>(Q, count, smem, cb, &s_chain_abort); break;
+                case 7: chain_cta<7>(Q, count, smem, cb, &s_chain_abort); break;
+                case 8: chain_cta<8>(Q, count, smem, cb, &s_chain_abort); break;
+                default: break;
+            }
+        }
+        __syncthreads();
+    }
 
     ptx::tc_fence_before();
     // nobody leaves while its partner may still signal its barriers or read its shared memory
@@ -1131,12 +1222,43 @@ struct TimeArgs {
     float t[KMAX];
 };
 
-// hidden[k][o] = SiLU(Wt1[o] . e(t_k) + bt1[o]); one warp per output
-__global__ void __launch_bounds__(256) temb_hidden_kernel(const bf16* __restrict__ Wt1,
-                                                         const float* __restrict__ bt1, int W, int F,
-                                                         TimeArgs ta, float* __restrict__ hidden) {
+struct PrepArgs {
+    const bf16* Wt1;
+    const float* bt1;
+    float* hidden;
+    int W, F, K;
+    int* counters;              // zeroed
+    int n_counters;
+    int* abort_flag;            // zeroed
+    const bf16* cond;           // calls that the chain serves: z = cond[idx[j]]
+    bf16* z;
+    const int *idx, *count;
+    int Dc, max_tokens, chain_count;
+};
+constexpr int PREP_BLOCKS = 148;        // beside the time embedding's
+
+// Everything a call needs before the head kernel. The first blocks: hidden[k][o] = SiLU(Wt1[o] . e(t_k) + bt1[o]), one
+// warp per output. The others: counters to zero, and for few tokens the gather of their conditioning rows over the whole
+// GPU (as one item of the head kernel it took 150 of the 205 us before the first modulation of 29 rows of 5120; with
+// thousands of tokens there are enough items and the rows are gathered where they are used).
+__global__ void __launch_bounds__(256) prep_kernel(const __grid_constant__ PrepArgs A, TimeArgs ta) {
     extern __shared__ float e_s[];
-    const int k = blockIdx.y;
+    const int W = A.W, F = A.F;
+    const int per_step = (W + 7) / 8;
+    if ((int)blockIdx.x >= per_step * A.K) {
+        const int t0 = ((int)blockIdx.x - per_step * A.K) * blockDim.x + threadIdx.x, stride = PREP_BLOCKS * blockDim.x;
+        for (int i = t0; i < A.n_counters; i += stride) A.counters[i] = 0;
+        if (t0 == 0) *A.abort_flag = 0;
+        const int S = min(*A.count, A.max_tokens);
+        if (S > A.chain_count) return;
+        const int chunks = A.Dc / 8;
+        for (int i = t0; i < S * chunks; i += stride) {
+            const int j = i / chunks, c = i - j * chunks;
+            reinterpret_cast<uint4*>(A.z)[i] = __ldg(reinterpret_cast<const uint4*>(A.cond + (size_t)A.idx[j] * A.Dc) + c);
+        }
+        return;
+    }
+    const int k = blockIdx.x / per_step;
     const int half = F / 2;
     for (int f = threadIdx.x; f < half; f += blockDim.x) {
         const double w = exp(-log(10000.0) * (double)f / (double)half);
@@ -1148,16 +1270,16 @@ __global__ void __launch_bounds__(256) temb_hidden_kernel(const bf16* __restrict
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int o = blockIdx.x * 8 + warp;
+    const int o = (blockIdx.x - k * per_step) * 8 + warp;
     if (o >= W) return;
-    const bf16* wr = Wt1 + (size_t)o * F;
+    const bf16* wr = A.Wt1 + (size_t)o * F;
     float acc = 0.f;
     for (int i = lane; i < F; i += 32) acc = fmaf(__bfloat162float(wr[i]), e_s[i], acc);
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
     if (lane == 0) {
-        const float a = acc + bt1[o];
-        hidden[(size_t)k * W + o] = a / (1.0f + expf(-a));
+        const float a = acc + A.bt1[o];
+        A.hidden[(size_t)k * W + o] = a / (1.0f + expf(-a));
     }
 }
 
@@ -1256,7 +1378,12 @@ struct ardiff_head {
     ardiff_head_desc d;
     int device, n_sm, grid, coop;
     int TGu, slots;
-    Program prog[N_WIDTHS];
+    Program prog[N_PROGRAMS];
+    size_t chain_token_steps;   // survivors x steps that mods and xch hold; 0: no chain for this shape
+    size_t out_row0;
+    int chain_slots;
+    float* mods;
+    uint8_t* xch;
     int64_t max_tiles;
     std::vector<void*> allocs;
     // device
@@ -1319,6 +1446,19 @@ int env_int(const char* name, int dflt) {
 }  // namespace
 
 namespace {
+// survivors up to which the chain is used, of `fit` that its buffers hold
+int chain_limit(int fit) {
+#ifdef ARDIFF_TUNING
+    const int lim = env_int("ARDIFF_HEAD_CHAIN", CHAIN_MAX_TOKENS);
+    if (lim < fit) fit = lim;
+#endif
+    return fit;
+}
+// shared memory of the chain with `slots` weight tiles
+int chain_smem(int slots, int W) {
+    return 2 * chain_red_bytes(W / 256) + CHAIN_COLS * XB_COLS * 2 + slots * CHAIN_COLS * (W * 2 + 64);
+}
+
 // Most pairs of token tiles that items of width `wi` serve. Narrow items shorten every link of the chain of
 // dependent layers (K loop and epilogue) and give more units something to do, but each of them reads its token tile
 // again: 128 columns win while a W-wide layer is at most two thirds of a grid of them, 64 columns up to a quarter.
@@ -1534,6 +1674,22 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     TRY(dev_alloc(H, &H->x, R * C, true));
     TRY(dev_alloc(H, &H->h, R * W, true));
     TRY(dev_alloc(H, &H->stats, R * 2 * (W / item_cols(N_WIDTHS - 1)), true));
+    // the chain: its buffers hold token_steps survivors x steps (as many as K_max and max_tokens can ask for, up
+    // to 128 MB of modulations)
+    H->out_row0 = out_row0;
+    if (W / 256 <= CHAIN_MAX_NC && W / CHAIN_COLS <= H->grid && d.K_max > 0 && d.max_tokens > 0) {
+        const size_t per = mods_floats_per_token_step(L, W);
+        const size_t most = (size_t)d.K_max * (size_t)(d.max_tokens < CHAIN_MAX_TOKENS ? d.max_tokens : CHAIN_MAX_TOKENS);
+        const size_t fit = ((size_t)128 << 20) / (per * sizeof(float));
+        H->chain_token_steps = most < fit ? most : fit;
+        const int tile = CHAIN_COLS * (W * 2 + 64);
+        H->chain_slots = (RING_BYTES + EPI_BYTES - chain_smem(0, W)) / tile;
+        if (H->chain_slots > CHAIN_MAX_SLOTS) H->chain_slots = CHAIN_MAX_SLOTS;
+        if (H->chain_token_steps > 0) {
+            TRY(dev_alloc(H, &H->mods, H->chain_token_steps * per, false));
+            TRY(dev_alloc(H, &H->xch, chain_xch_bytes(H->chain_token_steps, d.K_max, L, W, C), false));
+        }
+    }
     TRY(dev_alloc(H, &H->counters, ((size_t)H->max_tiles + 2) * CTRS, true));
     TRY(dev_alloc(H, &H->status, 2, true));
     TRY(dev_alloc(H, &H->clock_probe, 2, true));
@@ -1542,15 +1698,16 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
 #endif
 
     // ---- the program of one step for every item width: phases in list order ----
-    for (int wi = 0; wi < N_WIDTHS; ++wi) {
-        Program& V = H->prog[wi];
-        const int NT = W / item_cols(wi);
+    for (int pi = 0; pi < N_PROGRAMS; ++pi) {
+        Program& V = H->prog[pi];
+        const bool mods_only = pi == MOD_PROGRAM;
+        const int NT = W / item_cols(mods_only ? MOD_WIDTH : pi);
         V.NT = NT;
-        V.T_pro = 1 + 2 * NT;     // gather, conditioning items, the gate of step 0 / block 0
-        V.T_step = NT * (3 + 5 * L) + 1;
-        V.C_pro = 1 + NT;
-        V.C_step = NT * (3 + 4 * L) + 1;
-        V.max_units = wi == 0 ? 0x7fffffff : width_limit(wi, W, units, H->TGu);
+        V.T_pro = mods_only ? NT : 1 + 2 * NT;      // gather, conditioning items, the gate of step 0 / block 0
+        V.T_step = mods_only ? NT * (3 * L + 2) : NT * (3 + 5 * L) + 1;
+        V.C_pro = mods_only ? NT : 1 + NT;
+        V.C_step = mods_only ? 0 : NT * (3 + 4 * L) + 1;
+        V.max_units = mods_only ? 0 : pi == 0 ? 0x7fffffff : width_limit(pi, W, units, H->TGu);
         std::vector<Phase> ph;
         int cum = 0;
         auto add = [&](int type, int block, int tile0, int ntiles, size_t b_row0, int offA, int kplus) {
@@ -1564,8 +1721,9 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
             add(OP_GATE, b, tile0, ntiles, b * blk_rows + 2 * (size_t)W, NT + 4 * NT * host, kplus);
         };
         const int na = NT / 2;
-        add(OP_IN, -1, 0, NT, 0, 0, 0);
-        for (int b = 0; b < L; ++b) {
+        for (int b = 0; mods_only && b <= L; ++b) add(OP_MOD, b, 0, b < L ? 3 * NT : 2 * NT, b * blk_rows, 0, 0);
+        if (!mods_only) add(OP_IN, -1, 0, NT, 0, 0, 0);
+        for (int b = 0; !mods_only && b < L; ++b) {
             const int base = NT + 4 * NT * b;
             add(OP_SS, b, 0, 2 * NT, b * blk_rows, base, 0);
             add(OP_G1, b, 0, NT, b * blk_rows + 3 * (size_t)W, base + 2 * NT, 0);
@@ -1576,10 +1734,12 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
         }
         // the last block hosts the first gate of the NEXT step, spread over the step boundary where the chain
         // (final modulation -> out-projection -> in-projection) has little else to overlap with
-        add(OP_FSS, -1, 0, 2 * NT, fm_row0, NT + 4 * NT * L, 0);
-        gate(0, 1, L - 1, 0, na);
-        add(OP_OUT, -1, 0, 1, out_row0, NT + 4 * NT * L + 2 * NT, 0);
-        gate(0, 1, L - 1, na, NT - na);
+        if (!mods_only) {
+            add(OP_FSS, -1, 0, 2 * NT, fm_row0, NT + 4 * NT * L, 0);
+            gate(0, 1, L - 1, 0, na);
+            add(OP_OUT, -1, 0, 1, out_row0, NT + 4 * NT * L + 2 * NT, 0);
+            gate(0, 1, L - 1, na, NT - na);
+        }
         if (cum != V.T_step) {
             free_all(H);
             delete H;
@@ -1675,18 +1835,23 @@ int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise,
 
     TimeArgs ta;
     for (int k = 0; k < K; ++k) ta.t[k] = t_sched[k];
-    temb_hidden_kernel<<<dim3((W + 7) / 8, K), 256, H->d.F * sizeof(float), st>>>(H->Wt1, H->bt1, W, H->d.F, ta,
-                                                                                  H->temb_hidden);
+    const size_t chain_fit = H->chain_token_steps / (size_t)K;
+    const int chain_count = chain_limit((int)(chain_fit < CHAIN_MAX_TOKENS ? chain_fit : CHAIN_MAX_TOKENS));
+    PrepArgs A;
+    A.Wt1 = H->Wt1; A.bt1 = H->bt1; A.hidden = H->temb_hidden; A.W = W; A.F = H->d.F; A.K = K;
+    A.counters = H->counters; A.n_counters = (int)((H->max_tiles + 2) * CTRS); A.abort_flag = H->status + 1;
+    A.cond = reinterpret_cast<const bf16*>(cond); A.z = H->z; A.idx = idx; A.count = count;
+    A.Dc = H->d.Dc; A.max_tokens = (int)H->d.max_tokens; A.chain_count = chain_count;
+    prep_kernel<<<(W + 7) / 8 * K + PREP_BLOCKS, 256, H->d.F * sizeof(float), st>>>(A, ta);
     temb_out_kernel<<<dim3((W + 7) / 8, K), 256, 0, st>>>(H->Wt2, H->bt2, W, H->temb_hidden, H->temb);
     launches += 2;
-    if (cudaMemsetAsync(H->counters, 0, sizeof(int) * ((size_t)H->max_tiles + 2) * CTRS, st) != cudaSuccess)
-        return ARDIFF_ERR_CUDA;
-    if (cudaMemsetAsync(H->status + 1, 0, sizeof(int), st) != cudaSuccess) return ARDIFF_ERR_CUDA;
-
     HeadParams P;
     memset(&P, 0, sizeof(P));
     P.C = C; P.Dc = H->d.Dc; P.W = W; P.L = H->d.L; P.K = K; P.TGu = H->TGu; P.slots = H->slots;
-    for (int wi = 0; wi < N_WIDTHS; ++wi) P.prog[wi] = H->prog[wi];
+    for (int pi = 0; pi < N_PROGRAMS; ++pi) P.prog[pi] = H->prog[pi];
+    P.chain_count = chain_count;
+    P.mods = H->mods; P.xch = H->xch;
+    P.grid_counter = (int)((H->max_tiles + 1) * CTRS);
     P.R = H->slots * BM;
     P.max_tokens = (int)H->d.max_tokens;
     P.maps = H->maps;
@@ -1710,6 +1875,14 @@ int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise,
         H->stall_tile = -1;
     }
 
+    ChainParams Q;
+    memset(&Q, 0, sizeof(Q));
+    Q.C = C; Q.W = W; Q.L = H->d.L; Q.K = K; Q.n_slots = H->chain_slots; Q.out_row0 = H->out_row0;
+    Q.idx = idx; Q.Wcat = H->Wcat; Q.Win = H->Win; Q.bias_cat = H->bias_cat; Q.bin = H->bin;
+    Q.noise = noise; Q.step_noise = step_noise; Q.step_stride = P.step_stride; Q.mods = H->mods; Q.out = out;
+    Q.xch = H->xch; Q.status = H->status; Q.abort_flag = P.abort_flag; Q.wait_limit_ns = P.wait_limit_ns;
+    memcpy(Q.ax, P.ax, sizeof(Q.ax)); memcpy(Q.av, P.av, sizeof(Q.av)); memcpy(Q.an, P.an, sizeof(Q.an));
+
     if (H->timing) cudaEventRecord(H->ev0, st);
     {
         cudaLaunchConfig_t cfg;
@@ -1727,16 +1900,16 @@ int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise,
         cfg.gridDim = dim3(H->grid); cfg.blockDim = dim3(NUM_THREADS);
         cfg.dynamicSmemBytes = SMEM_BYTES;
         cfg.stream = st; cfg.attrs = at; cfg.numAttrs = na;
-        if (cudaLaunchKernelEx(&cfg, head_kernel, P) != cudaSuccess) {
+        if (cudaLaunchKernelEx(&cfg, head_kernel, P, Q) != cudaSuccess) {
             (void)cudaGetLastError();
             return ARDIFF_ERR_CUDA;
         }
     }
+    launches += 1;
     if (H->timing) {
         cudaEventRecord(H->ev1, st);
         H->timed = 1;
     }
-    launches += 1;
     ardiff::set_launch_count(launches);
     return ARDIFF_OK;
 }

@@ -115,6 +115,54 @@ def test_item_width_boundaries(count):
     head.close()
 
 
+@pytest.mark.parametrize("W", [256, 512, 768, 1024, 1280, 1536, 1792, 2048, 2304])
+def test_few_tokens_at_every_width(W):
+    """Up to 64 survivors the chain of layers runs in its own kernel (one instance per W / 256 up to 8): one token, a
+    ragged token tile, a second pass, the last count it takes and the first that it does not; the same call twice gives
+    the same bits. Tolerance: the agreement bar of this file."""
+    wl = synth.workload("cfg1", n=80, W=W, L=2, K=3, C=32 if W % 512 else 64, Dc=192)
+    w, cond_bits, noise, t = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
+    order = np.random.default_rng(W).permutation(wl.n).astype(np.int32)
+    want = oracle.head_sample(w, cond_bits, noise, t, order[:65])
+    head = make_head(wl, w)
+    for count in (1, 9, 33, 64, 65):
+        idx = order[:count]
+        got = run_head(head, cond_bits, noise, t, idx)
+        assert_parity(got, want, idx, f"{count} tokens")
+        assert np.all(got[np.setdiff1d(np.arange(wl.n), idx)] == SENTINEL)
+        assert np.array_equal(run_head(head, cond_bits, noise, t, idx), got)
+    head.close()
+
+
+def test_few_tokens_with_fresh_noise_and_after_a_stall():
+    """The sampler form with step noise on few tokens, before and after a call whose conditioning never completes."""
+    dev = require_cuda()
+    wl = synth.workload("cfg1", n=50, W=512, K=2)
+    w, cond_bits, noise = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl)
+    idx_np = np.random.default_rng(3).permutation(wl.n)[:41].astype(np.int32)
+    t_in = np.array([0.95, 0.5], np.float32)
+    coef = np.array([[0.3, 0.7, 0.7], [0.0, 1.0, 0.1]], np.float32)
+    z = np.random.default_rng(8).standard_normal((2, wl.n, wl.C)).astype(np.float32)
+    want = oracle.head_sample_coef(w, cond_bits, noise, t_in, coef, idx_np, step_noise=z)
+    head = make_head(wl, w)
+    idx = torch.from_numpy(idx_np).to(dev)
+    count = torch.tensor([len(idx_np)], dtype=torch.int32, device=dev)
+    clean = None
+    for stall in (False, True, False):
+        if stall:
+            head.inject_stall(0, 3000)
+        out = torch.full(noise.shape, SENTINEL, dtype=torch.float32, device=dev)
+        head.ardiff_head_sample_coef(dev_bf16(cond_bits), dev_f32(noise), t_in, coef, idx, count, out,
+                                     step_noise=torch.from_numpy(z).to(dev))
+        assert head.status() == (ardiff.ARDIFF_ERR_TIMEOUT if stall else 0)
+        if not stall:
+            got = out.cpu().numpy()
+            assert_parity(got, want, idx_np)
+            assert clean is None or np.array_equal(got, clean)
+            clean = got
+    head.close()
+
+
 @pytest.mark.parametrize("std", [0.02, None])
 def test_velocity_parity_one_step(std):
     wl = synth.workload("cfg1", n=256, K=1)
