@@ -652,6 +652,7 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
     constexpr int SPAN = BN / 2;                                 // accumulator columns of one epilogue warp
     constexpr int UNITS = SPAN / 16;
     constexpr int MOD_UNITS = UNITS / 2 < 2 ? 2 : UNITS / 2;     // of shift, and of scale
+    constexpr bool HALF_IDLE = 2 * MOD_UNITS * 16 > BN / 2;
     const Program& V = P.prog[PI];
     const uint32_t smem_base = X.smem_base, bars = X.bars;
     const uint32_t epi_base = smem_base + RING_BYTES;            // 1024-aligned
@@ -862,7 +863,7 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
                 // item has work for one warp of the two only: a slab is 32 columns wide)
                 const int acc0 = mod ? half * (MOD_UNITS * 16) : half * SPAN;
                 const int col0 = mod ? it.nt * (BN / 2) + acc0 : it.nt * BN + acc0;   // column of the layer's output
-                const bool mod_idle = mod && acc0 >= BN / 2;
+                const bool mod_idle = HALF_IDLE && mod && half != 0;
                 const int row0 = it.slot_row0 + quarter * 32;
                 const int grow = it.slot_row0 + row;
                 const size_t chunk0 = chunk_of(P, row0, col0);
@@ -1030,7 +1031,7 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
                     const int n_mod = mod_idle ? 0 : MOD_UNITS;
 #pragma unroll
                     for (int u = 0; u < MOD_UNITS; ++u) {
-                        if (u >= n_mod) break;
+                        if (HALF_IDLE && u >= n_mod) break;
                         const uint32_t sl = my_buf + (uint32_t)((u >> 1) & 1) * SLAB_H;
                         if (u + 3 < MOD_UNITS) load_unit_h(P.h, chunk0, u + 3, lane, hin[(u + 3) & 3]);
                         if ((u & 1) == 0) slab_ready();
@@ -1134,7 +1135,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
     if (count < 0) count = 0;
     const int MT = (count + BM - 1) / BM;
     const int MTu = (MT + 1) / 2;                  // an odd last tile gets an all-padding partner
-    const int n_groups = (MTu + P.TGu - 1) / P.TGu;
+    // A lone group may be a tenth larger than the others: 12188 tokens at W = 1024 (48 pairs, groups of 47) take 1796 us as
+    // one group and 1848 us as two of 24, whose phases are too short for the latency of the chain. Much larger ones lose
+    // (56 pairs as one group 2161 us, as two 2090 us): their residual stream no longer fits the set-aside part of L2.
+    const int n_groups = MTu <= P.TGu + P.TGu / 10 ? 1 : (MTu + P.TGu - 1) / P.TGu;
     const int tgu = n_groups > 0 ? (MTu + n_groups - 1) / n_groups : 1;   // balanced group size
     // the narrowest items that the number of token tiles allows (see width_limit)
     const bool chained = count > 0 && count <= P.chain_count;
