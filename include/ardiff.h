@@ -56,9 +56,9 @@ int ardiff_version(void);
  *   count  dev  int32 [1]  out: number of kept tokens (stays on the device)
  *   entropy (the _ex form) dev float [n] out, or NULL: H_i as computed
  *
- * Rows are read once from HBM when d % 8 == 0 (d <= 8192: registers hold the row; longer rows:
- * a running maximum per lane with rescaled partial sums); other d take a slower two-pass kernel
- * with scalar loads. n == 0 is valid (writes *count = 0).
+ * Rows are read once from HBM (d up to about 8192: registers hold the row; longer rows: a running
+ * maximum per lane with rescaled partial sums), those of a width that is no multiple of 8 as the
+ * aligned 16-byte pieces that cover them. n == 0 is valid (writes *count = 0).
  *
  * Scratch and concurrency. The two kernels of a call hand per-block counts to each other
  * through a small per-device scratch (512 KB) that the library allocates on the first call on
@@ -97,9 +97,10 @@ int ardiff_entropy_gate_stats(const void* feat, int64_t n, int32_t d, float tau,
  *
  *   feat           dev bf16 [n * rows_per_token][d], alignment as for ardiff_entropy_gate
  *   row_entropy    dev float [n * rows_per_token]  out, or NULL. One pass over the features does all of it
- *                  (row entropies stay in shared memory) when d % 8 == 0, d <= 8192 and
- *                  gamma * rows_per_token <= 24576; other shapes go through row_entropy as scratch and
- *                  return ARDIFF_ERR_NULL without it
+ *                  (row entropies stay in shared memory) when d <= 8192 (8178 at widths that are no
+ *                  multiple of 8) and gamma * rows_per_token <= 24576; other shapes go through
+ *                  row_entropy as scratch. Those, and widths that are no multiple of 8, return
+ *                  ARDIFF_ERR_NULL without it
  *   token_entropy  dev float [n]  out, or NULL
  *   mask, idx, count   as for ardiff_entropy_gate (idx ascending)
  *   block_len      dev int32 [ceil(n / gamma)]  out, or NULL: tokens kept in each block
@@ -115,7 +116,7 @@ int ardiff_entropy_gate_blocks(const void* feat, int64_t n, int32_t rows_per_tok
 /* Threshold from entropy statistics (the tau equation of "Entropy-Based Early Stopping in Inference
  * Phase"): out3 = { mean(H), std(H), 0.3 * mean - 0.1 * std }, std with divisor n, all in fp64
  * with a fixed summation order (results are reproducible run to run).
- *   entropy dev float [n], n >= 1;  out3 dev double [3]. One CTA: meant for calibration, not the hot path. */
+ *   entropy dev float [n], n >= 1;  out3 dev double [3]. One cluster of CTAs: meant for calibration, not the hot path. */
 int ardiff_tau_calibrate(const float* entropy, int64_t n, double* out3, void* stream);
 
 /* Accepted draft length per block (Algorithm 1, Step 4):
@@ -147,8 +148,8 @@ int ardiff_accept_prefix(const float* r, const float* ratio, int64_t n, int32_t 
  * launched (the fixed number of blocks would otherwise each walk an ever longer token range).
  * The first call on each device looks up the array's device address (cudaGetSymbolAddress,
  * with that device current), and the first call for each feature-width class (d / 256 rounded up
- * to 1, 2, 4, 8, 12, 16, 20, 24, 32, or the generic path) loads that kernel and queries its
- * occupancy: make those first calls before any stream capture starts.
+ * to 1, 2, 4, 8, 12, 16, 20, 24, 32, or longer rows; multiples of 8 and other widths apart) loads
+ * that kernel and queries its occupancy: make those first calls before any stream capture starts.
  * All calls on one device share the one array. Every call overwrites the entries it uses
  * before it reads them, so nothing needs clearing between calls and back-to-back calls on one
  * stream are safe; two calls that can run on the GPU at the same time (different streams

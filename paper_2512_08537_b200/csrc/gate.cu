@@ -18,6 +18,7 @@
 #include <math_constants.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <mutex>
 #include <type_traits>
 
@@ -56,9 +57,11 @@ __device__ __forceinline__ uint32_t max_bf16x2_nan(uint32_t a, uint32_t b) {
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
+// over the G lanes that share a row
+template <int G = 32>
 __device__ __forceinline__ float warp_max_nan(float v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = G / 2; o > 0; o >>= 1) {
         float other = __shfl_xor_sync(0xffffffffu, v, o);
         // NaN-propagating max
         v = (v != v || other != other) ? CUDART_NAN_F : fmaxf(v, other);
@@ -66,9 +69,10 @@ __device__ __forceinline__ float warp_max_nan(float v) {
     return v;
 }
 
+template <int G = 32>
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
@@ -82,6 +86,77 @@ __device__ __forceinline__ void acc_word(uint32_t w, float mneg, float& S, float
     S += e1;
     T = fmaf(t0, e0, T);
     T = fmaf(t1, e1, T);
+}
+
+// the same for words that may hold -inf (fill, or a real channel): e is 0 there, and t, which e multiplies, stays finite.
+// NaN, +inf and rows of -inf alone still give S = NaN through the row maximum.
+__device__ __forceinline__ void acc_word_safe(uint32_t w, float mneg, float& S, float& T) {
+    float t0 = fmaf(bf16_lo(w), kLog2e, mneg);
+    float t1 = fmaf(bf16_hi(w), kLog2e, mneg);
+    float e0 = ex2_approx(t0);
+    float e1 = ex2_approx(t1);
+    S += e0;
+    S += e1;
+    T = fmaf(fmaxf(t0, -1e30f), e0, T);
+    T = fmaf(fmaxf(t1, -1e30f), e1, T);
+}
+
+// Rows of a width that is no multiple of 8 start at any even address. They are read as the 16-byte chunks that cover
+// them: the first chunk starts with `head` elements of the row before, the last one ends with elements of the row
+// after; both are replaced by -inf once the chunk has arrived. Scalar loads in two passes, as before, took
+// 57 us for 65536 x 777 (1.8 TB/s).
+constexpr uint32_t kFill = 0xff80ff80u;
+struct RowSpan {
+    const uint4* base;       // first chunk
+    int nch, head;
+};
+template <bool RAGGED>
+__device__ __forceinline__ RowSpan row_span(const void* feat, int64_t row, int32_t d) {
+    if (!RAGGED) return RowSpan{static_cast<const uint4*>(feat) + row * (int64_t)(d / 8), d / 8, 0};
+    const uintptr_t at = reinterpret_cast<uintptr_t>(feat) + (uintptr_t)row * (uintptr_t)d * 2;
+    const int head = (int)(at & 15u) / 2;
+    return RowSpan{reinterpret_cast<const uint4*>(at & ~(uintptr_t)15), (head + d + 7) / 8, head};
+}
+// Chunk c of a row. Rows at the edges of the matrix read their partial chunks element by element: nothing outside the
+// caller's array is touched.
+template <bool RAGGED>
+__device__ __forceinline__ uint4 load_chunk(const RowSpan& r, int c, int32_t d, bool edge) {
+    if (RAGGED && edge && (c == 0 || c == r.nch - 1)) {
+        const uint16_t* e = reinterpret_cast<const uint16_t*>(r.base + c);
+        uint32_t w[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            w[q] = kFill;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int i = 8 * c + 2 * q + h - r.head;
+                if (i >= 0 && i < d) w[q] = (w[q] & (h ? 0x0000ffffu : 0xffff0000u)) | ((uint32_t)e[2 * q + h] << (16 * h));
+            }
+        }
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    return ld_stream_v4(r.base + c);
+}
+// elements lo .. hi - 1 of a chunk kept, the others -inf
+__device__ __forceinline__ uint4 keep_elements(uint4 v, int lo, int hi) {
+    uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (2 * q < lo || 2 * q >= hi) w[q] = (w[q] & 0xffff0000u) | 0xff80u;
+        if (2 * q + 1 < lo || 2 * q + 1 >= hi) w[q] = (w[q] & 0x0000ffffu) | 0xff800000u;
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+template <bool RAGGED>
+__device__ __forceinline__ uint4 own_elements(uint4 v, const RowSpan& r, int c, int32_t d) {
+    if (RAGGED && (c == 0 || c == r.nch - 1)) return keep_elements(v, c == 0 ? r.head : 0, min(8, r.head + d - 8 * c));
+    return v;
+}
+
+// Whether a row's chunks may stick out of the matrix: fewer than 8 elements before it or after it.
+template <bool RAGGED>
+__device__ __forceinline__ bool edge_row(int64_t row, int64_t n, int32_t d) {
+    return RAGGED && (row * d < 8 || (n - 1 - row) * d < 8);
 }
 
 // Slow exact-semantics path for one row: used when the fast path meets a non-finite
@@ -107,51 +182,68 @@ __device__ __noinline__ float row_entropy_careful(const uint4* row, int nchunks,
     return logf(S) - kLn2 * (T / S);
 }
 
-// Entropy of the row held in v (NCH 16-byte chunks per lane). Each chunk is refilled with the warp's NEXT row
+// Entropy of the row held in v by G lanes (NCH 16-byte chunks per lane). Each chunk is refilled with the warp's NEXT row
 // as soon as the exponentials of the current row have consumed it, so a warp always has loads in flight while
 // it computes (with 128 registers per thread only 16 warps fit an SM: they cannot hide HBM latency by
-// switching alone).
-template <int NCH>
-__device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const uint4* row, const uint4* next_row,
-                                                      bool has_next, int32_t nchunks, int lane) {
+// switching alone). Up to 2048 channels a warp holds 32 / G rows: what a row costs beside its elements (three
+// reductions by shuffle, a logarithm, a division, the loop) is then paid once for all of them. One row per warp took
+// 243 us for 2^20 x 64 and 22 us for 65536 x 256.
+template <int NCH, int G, bool RAGGED>
+__device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const RowSpan& row, const RowSpan& next,
+                                                      bool has_next, bool next_edge, int32_t d, int l) {
+    constexpr bool SAFE = RAGGED || G < 32;
+    if (RAGGED) {
+#pragma unroll
+        for (int j = 0; j < NCH; ++j) v[j] = own_elements<true>(v[j], row, l + G * j, d);
+    }
     // row maximum (packed, exact in bf16)
-    uint32_t mx = 0xff80ff80u;
+    uint32_t mx = kFill;
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
         mx = max_bf16x2_nan(mx, max_bf16x2_nan(max_bf16x2_nan(v[j].x, v[j].y), max_bf16x2_nan(v[j].z, v[j].w)));
     }
     float ml = bf16_lo(mx), mh = bf16_hi(mx);
     float m = (ml != ml || mh != mh) ? CUDART_NAN_F : fmaxf(ml, mh);
-    m = warp_max_nan(m);
+    m = warp_max_nan<G>(m);
     const float mneg = -m * kLog2e;
     float S = 0.f, T = 0.f;
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
-        const int c = lane + 32 * j;
-        if (c < nchunks) {
-            acc_word(v[j].x, mneg, S, T);
-            acc_word(v[j].y, mneg, S, T);
-            acc_word(v[j].z, mneg, S, T);
-            acc_word(v[j].w, mneg, S, T);
-            if (has_next) v[j] = ld_stream_v4(next_row + c);
+        const int c = l + G * j;
+        if (c < row.nch) {
+            if (SAFE) {
+                acc_word_safe(v[j].x, mneg, S, T);
+                acc_word_safe(v[j].y, mneg, S, T);
+                acc_word_safe(v[j].z, mneg, S, T);
+                acc_word_safe(v[j].w, mneg, S, T);
+            } else {
+                acc_word(v[j].x, mneg, S, T);
+                acc_word(v[j].y, mneg, S, T);
+                acc_word(v[j].z, mneg, S, T);
+                acc_word(v[j].w, mneg, S, T);
+            }
+            if (!RAGGED && has_next) v[j] = ld_stream_v4(next.base + c);
         }
+        // neighbouring rows may differ by a chunk
+        if (RAGGED && has_next)
+            v[j] = c < next.nch ? load_chunk<true>(next, c, d, next_edge) : make_uint4(kFill, kFill, kFill, kFill);
     }
-    S = warp_sum(S);
-    T = warp_sum(T);
+    S = warp_sum<G>(S);
+    T = warp_sum<G>(T);
     float H = logf(S) - kLn2 * (T / S);
-    if (H != H) {
+    if (!SAFE && H != H) {
         // a -inf channel (t*e = -inf*0) lands here, as do genuinely undefined rows
-        H = row_entropy_careful(row, nchunks, lane, m);
+        H = row_entropy_careful(row.base, row.nch, l, m);
     }
     return H;
 }
 
-template <int NCH>
-__device__ __forceinline__ void load_resident_row(uint4 (&v)[NCH], const uint4* row, int32_t nchunks, int lane) {
+template <int NCH, int G, bool RAGGED>
+__device__ __forceinline__ void load_resident_row(uint4 (&v)[NCH], const RowSpan& row, int32_t d, bool edge, bool have, int l) {
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
-        const int c = lane + 32 * j;
-        v[j] = c < nchunks ? ld_stream_v4(row + c) : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
+        const int c = l + G * j;
+        v[j] = have && c < row.nch ? load_chunk<RAGGED>(row, c, d, edge) : make_uint4(kFill, kFill, kFill, kFill);
     }
 }
 
@@ -168,10 +260,10 @@ __device__ __forceinline__ void cta_merge_stats(const WarpStats& mine, int warp,
     }
 }
 
-// One warp per token, row resident in registers: NCH 16-byte chunks per lane.
-template <int NCH>
+// G lanes per token, row resident in registers: NCH 16-byte chunks per lane.
+template <int NCH, int G, bool RAGGED>
 __global__ void __launch_bounds__(kGateThreads)
-gate_rows_kernel(const uint4* __restrict__ feat, int64_t n, int32_t nchunks, float tau,
+gate_rows_kernel(const void* __restrict__ feat, int64_t n, int32_t d, float tau,
                  uint8_t* __restrict__ mask, float* __restrict__ entropy,
                  int32_t* __restrict__ block_counts, double* __restrict__ cta_stats, int64_t tokens_per_block) {
     const int lane = threadIdx.x & 31;
@@ -184,20 +276,36 @@ gate_rows_kernel(const uint4* __restrict__ feat, int64_t n, int32_t nchunks, flo
     int kept = 0;
     WarpStats st{0.0, 0.0, 0.0};
     uint4 v[NCH];
-    if (t_begin + warp < t_end) load_resident_row(v, feat + (t_begin + warp) * (int64_t)nchunks, nchunks, lane);
-    for (int64_t tok = t_begin + warp; tok < t_end; tok += kGateWarps) {
-        const uint4* row = feat + tok * (int64_t)nchunks;
-        const float H = resident_row_entropy(v, row, row + (int64_t)kGateWarps * nchunks, tok + kGateWarps < t_end,
-                                             nchunks, lane);
-        const bool keep = (H >= tau);  // false for NaN
-        if (lane == 0) {
+    auto edge = [&](int64_t i) { return edge_row<RAGGED>(i, n, d); };
+    constexpr int R = 32 / G;                // rows of a warp
+    const int l = lane % G, sub = lane / G;
+    RowSpan row = row_span<RAGGED>(feat, t_begin + warp * R + sub, d);
+    load_resident_row<NCH, G, RAGGED>(v, row, d, edge(t_begin + warp * R + sub), t_begin + warp * R + sub < t_end, l);
+    for (int64_t t0 = t_begin + warp * R; t0 < t_end; t0 += kGateWarps * R) {
+        const int64_t tok = t0 + sub, nx = tok + kGateWarps * R;
+        const RowSpan next = row_span<RAGGED>(feat, nx, d);
+        const float H = resident_row_entropy<NCH, G, RAGGED>(v, row, next, nx < t_end, edge(nx), d, l);
+        row = next;
+        if (l == 0 && tok < t_end) {
+            const bool keep = (H >= tau);  // false for NaN
             if (mask) mask[tok] = keep ? 1 : 0;
             if (entropy) entropy[tok] = H;
+            kept += keep ? 1 : 0;
+            if (cta_stats) { st.n += 1.0; st.s += (double)H; st.q += (double)H * (double)H; }
         }
-        kept += keep ? 1 : 0;
-        st.n += 1.0; st.s += (double)H; st.q += (double)H * (double)H;
     }
-    // block count (every lane of a warp holds the same `kept`)
+    if (G < 32) {                            // the warp's rows together, in a fixed order
+#pragma unroll
+        for (int o = 16; o >= G; o >>= 1) {
+            kept += __shfl_xor_sync(0xffffffffu, kept, o);
+            if (cta_stats) {
+                st.n += __shfl_xor_sync(0xffffffffu, st.n, o);
+                st.s += __shfl_xor_sync(0xffffffffu, st.s, o);
+                st.q += __shfl_xor_sync(0xffffffffu, st.q, o);
+            }
+        }
+    }
+    // block count (lane 0 holds the warp's)
     __shared__ int s_cnt[kGateWarps];
     if (lane == 0) s_cnt[warp] = kept;
     __syncthreads();
@@ -214,9 +322,9 @@ gate_rows_kernel(const uint4* __restrict__ feat, int64_t n, int32_t nchunks, flo
 // warps leave the row entropies in shared memory; then one thread per draft block forms the token indicators
 // (mean of the token's r row entropies, summed in row order), runs the prefix test, and writes mask, kept
 // length and, if asked, the indicators. No row entropy goes through global memory unless the caller wants it.
-template <int NCH>
+template <int NCH, int G, bool RAGGED>
 __global__ void __launch_bounds__(kGateThreads)
-gate_blocks_kernel(const uint4* __restrict__ feat, int64_t n_tokens, int32_t r, int32_t gamma, int32_t nchunks,
+gate_blocks_kernel(const void* __restrict__ feat, int64_t n_tokens, int32_t r, int32_t gamma, int32_t d,
                    float tau, float* __restrict__ row_entropy, float* __restrict__ token_entropy,
                    uint8_t* __restrict__ mask, int32_t* __restrict__ block_len, int32_t* __restrict__ cta_counts,
                    int64_t blocks_per_cta, int64_t n_blocks) {
@@ -230,12 +338,18 @@ gate_blocks_kernel(const uint4* __restrict__ feat, int64_t n_tokens, int32_t r, 
     const int64_t t_end = min(n_tokens, b_end * gamma);
     const int64_t r_begin = t_begin * r, r_end = t_end * r;
     uint4 v[NCH];
-    if (r_begin + warp < r_end) load_resident_row(v, feat + (r_begin + warp) * (int64_t)nchunks, nchunks, lane);
-    for (int64_t row_i = r_begin + warp; row_i < r_end; row_i += kGateWarps) {
-        const uint4* row = feat + row_i * (int64_t)nchunks;
-        const float H = resident_row_entropy(v, row, row + (int64_t)kGateWarps * nchunks, row_i + kGateWarps < r_end,
-                                             nchunks, lane);
-        if (lane == 0) {
+    const int64_t n_rows = n_tokens * r;
+    auto edge = [&](int64_t i) { return edge_row<RAGGED>(i, n_rows, d); };
+    constexpr int R = 32 / G;                // rows of a warp
+    const int l = lane % G, sub = lane / G;
+    RowSpan row = row_span<RAGGED>(feat, r_begin + warp * R + sub, d);
+    load_resident_row<NCH, G, RAGGED>(v, row, d, edge(r_begin + warp * R + sub), r_begin + warp * R + sub < r_end, l);
+    for (int64_t r0 = r_begin + warp * R; r0 < r_end; r0 += kGateWarps * R) {
+        const int64_t row_i = r0 + sub, nx = row_i + kGateWarps * R;
+        const RowSpan next = row_span<RAGGED>(feat, nx, d);
+        const float H = resident_row_entropy<NCH, G, RAGGED>(v, row, next, nx < r_end, edge(nx), d, l);
+        row = next;
+        if (l == 0 && row_i < r_end) {
             s_H[row_i - r_begin] = H;
             if (row_entropy) row_entropy[row_i] = H;
         }
@@ -273,12 +387,13 @@ gate_blocks_kernel(const uint4* __restrict__ feat, int64_t n_tokens, int32_t r, 
     }
 }
 
-// Rows longer than the registers hold (d > 8192, d % 8 == 0): still one pass with 128-bit loads. Every lane
-// keeps a running maximum of its own share of the row and rescales its partial sums when the maximum grows
+// Rows longer than the registers hold: still one pass with 128-bit loads. Every lane keeps a running maximum of its own
+// share of the row and rescales its partial sums when the maximum grows
 // (S <- S 2^D, T <- (T + D S) 2^D with D = (m_old - m_new) log2 e <= 0); the lanes' partials are merged the
-// same way at the end.
+// same way at the end. The next four chunks are asked for before the present four are worked on.
+template <bool RAGGED>
 __global__ void __launch_bounds__(kGateThreads)
-gate_rows_long_kernel(const uint4* __restrict__ feat, int64_t n, int32_t nchunks, float tau,
+gate_rows_long_kernel(const void* __restrict__ feat, int64_t n, int32_t d, float tau,
                       uint8_t* __restrict__ mask, float* __restrict__ entropy,
                       int32_t* __restrict__ block_counts, double* __restrict__ cta_stats, int64_t tokens_per_block) {
     const int lane = threadIdx.x & 31;
@@ -288,18 +403,27 @@ gate_rows_long_kernel(const uint4* __restrict__ feat, int64_t n, int32_t nchunks
     const int64_t t_end = min(n, t_begin + tokens_per_block);
     int kept = 0;
     WarpStats st{0.0, 0.0, 0.0};
+    constexpr int G = 4;
+    auto load_group = [&](uint4 (&v)[G], const RowSpan& row, bool edge, int c0) {
+#pragma unroll
+        for (int j = 0; j < G; ++j)
+            v[j] = c0 + 32 * j < row.nch ? load_chunk<RAGGED>(row, c0 + 32 * j, d, edge) : make_uint4(kFill, kFill, kFill, kFill);
+    };
     for (int64_t tok = t_begin + warp; tok < t_end; tok += kGateWarps) {
-        const uint4* row = feat + tok * (int64_t)nchunks;
+        const RowSpan row = row_span<RAGGED>(feat, tok, d);
+        const bool edge = edge_row<RAGGED>(tok, n, d);
         float ml = -CUDART_INF_F, S = 0.f, T = 0.f;
-        for (int c0 = lane; c0 < nchunks; c0 += 32 * 4) {
-            uint4 v[4];
+        uint4 v[G], nv[G];
+        load_group(v, row, edge, lane);
+        for (int c0 = lane; c0 < row.nch; c0 += 32 * G) {
+            load_group(nv, row, edge, c0 + 32 * G);
+            if (RAGGED) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                v[j] = c0 + 32 * j < nchunks ? ld_stream_v4(row + c0 + 32 * j)
-                                             : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
-            uint32_t mx = 0xff80ff80u;
+                for (int j = 0; j < G; ++j) v[j] = own_elements<true>(v[j], row, c0 + 32 * j, d);
+            }
+            uint32_t mx = kFill;
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
+            for (int j = 0; j < G; ++j)
                 mx = max_bf16x2_nan(mx, max_bf16x2_nan(max_bf16x2_nan(v[j].x, v[j].y), max_bf16x2_nan(v[j].z, v[j].w)));
             const float a = bf16_lo(mx), b = bf16_hi(mx);
             const float mc = (a != a || b != b) ? CUDART_NAN_F : fmaxf(a, b);
@@ -313,16 +437,28 @@ gate_rows_long_kernel(const uint4* __restrict__ feat, int64_t n, int32_t nchunks
                 }
                 ml = mc;
             }
-            const float mneg = -ml * kLog2e;
+            // a lane whose elements so far are all -inf has nothing to add (and no finite maximum to subtract)
+            if (!RAGGED || ml != -CUDART_INF_F) {
+                const float mneg = -ml * kLog2e;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                if (c0 + 32 * j < nchunks) {
-                    acc_word(v[j].x, mneg, S, T);
-                    acc_word(v[j].y, mneg, S, T);
-                    acc_word(v[j].z, mneg, S, T);
-                    acc_word(v[j].w, mneg, S, T);
+                for (int j = 0; j < G; ++j) {
+                    if (c0 + 32 * j < row.nch) {
+                        if (RAGGED) {
+                            acc_word_safe(v[j].x, mneg, S, T);
+                            acc_word_safe(v[j].y, mneg, S, T);
+                            acc_word_safe(v[j].z, mneg, S, T);
+                            acc_word_safe(v[j].w, mneg, S, T);
+                        } else {
+                            acc_word(v[j].x, mneg, S, T);
+                            acc_word(v[j].y, mneg, S, T);
+                            acc_word(v[j].z, mneg, S, T);
+                            acc_word(v[j].w, mneg, S, T);
+                        }
+                    }
                 }
             }
+#pragma unroll
+            for (int j = 0; j < G; ++j) v[j] = nv[j];
         }
         const float m = warp_max_nan(ml);
         if (S > 0.f && ml < m) {               // bring this lane's partials to the row maximum
@@ -334,61 +470,11 @@ gate_rows_long_kernel(const uint4* __restrict__ feat, int64_t n, int32_t nchunks
         S = warp_sum(S);
         T = warp_sum(T);
         float H = logf(S) - kLn2 * (T / S);
-        if (H != H) H = row_entropy_careful(row, nchunks, lane, m);
-        const bool keep = (H >= tau);
-        if (lane == 0) {
-            if (mask) mask[tok] = keep ? 1 : 0;
-            if (entropy) entropy[tok] = H;
+        if (RAGGED) {
+            if (!(fabsf(m) < CUDART_INF_F)) H = CUDART_NAN_F;       // NaN, +inf, or -inf alone
+        } else if (H != H) {
+            H = row_entropy_careful(row.base, row.nch, lane, m);
         }
-        kept += keep ? 1 : 0;
-        st.n += 1.0; st.s += (double)H; st.q += (double)H * (double)H;
-    }
-    __shared__ int s_cnt[kGateWarps];
-    if (lane == 0) s_cnt[warp] = kept;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int tot = 0;
-        for (int w = 0; w < kGateWarps; ++w) tot += s_cnt[w];
-        if (block_counts) block_counts[blockIdx.x] = tot;
-    }
-    if (cta_stats) cta_merge_stats(st, warp, lane, cta_stats + 3 * (size_t)blockIdx.x);
-}
-
-// Any d (no alignment assumption, any length): two passes over the row with scalar loads.
-__global__ void __launch_bounds__(kGateThreads)
-gate_rows_generic_kernel(const uint16_t* __restrict__ feat, int64_t n, int32_t d, float tau,
-                         uint8_t* __restrict__ mask, float* __restrict__ entropy,
-                         int32_t* __restrict__ block_counts, double* __restrict__ cta_stats,
-                         int64_t tokens_per_block) {
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int64_t t_begin = (int64_t)blockIdx.x * tokens_per_block;
-    const int64_t t_end = min(n, t_begin + tokens_per_block);
-    int kept = 0;
-    WarpStats st{0.0, 0.0, 0.0};
-    for (int64_t tok = t_begin + warp; tok < t_end; tok += kGateWarps) {
-        const uint16_t* row = feat + tok * (int64_t)d;
-        float m = -CUDART_INF_F;
-        bool nan = false;
-        for (int c = lane; c < d; c += 32) {
-            float x = __uint_as_float((uint32_t)row[c] << 16);
-            nan |= (x != x);
-            m = fmaxf(m, x);
-        }
-        if (nan) m = CUDART_NAN_F;
-        m = warp_max_nan(m);
-        const float mneg = -m * kLog2e;
-        float S = 0.f, T = 0.f;
-        for (int c = lane; c < d; c += 32) {
-            float x = __uint_as_float((uint32_t)row[c] << 16);
-            float t = fmaf(x, kLog2e, mneg);
-            float e = ex2_approx(t);
-            S += e;
-            if (e > 0.f || e != e) T = fmaf(t, e, T);
-        }
-        S = warp_sum(S);
-        T = warp_sum(T);
-        const float H = logf(S) - kLn2 * (T / S);
         const bool keep = (H >= tau);
         if (lane == 0) {
             if (mask) mask[tok] = keep ? 1 : 0;
@@ -548,54 +634,79 @@ cudaError_t launch_compact(int grid, cudaStream_t st, const uint8_t* mask, int64
     return cudaLaunchKernelEx(&cfg, compact_kernel, mask, n, block_counts, tpb, idx, count, cta_stats, out3);
 }
 
-// the row kernel that holds a row of `need` x 32 sixteen-byte chunks in registers: f(integral_constant<NCH>)
+// The row kernel for rows of up to `chunks` sixteen-byte pieces: f(integral_constant<NCH>, integral_constant<G>). Narrow rows
+// share a warp with 8 pieces per lane (fewer in the narrowest) and at least 4 lanes per row, so that a load still
+// covers whole 32-byte sectors; above 256 pieces a warp has one row and 9 to 32 pieces per lane.
 template <typename F>
-void dispatch_nch(int need, F&& f) {
-    if (need <= 1) f(std::integral_constant<int, 1>());
-    else if (need <= 2) f(std::integral_constant<int, 2>());
-    else if (need <= 4) f(std::integral_constant<int, 4>());
-    else if (need <= 8) f(std::integral_constant<int, 8>());
-    else if (need <= 12) f(std::integral_constant<int, 12>());
-    else if (need <= 16) f(std::integral_constant<int, 16>());
-    else if (need <= 20) f(std::integral_constant<int, 20>());
-    else if (need <= 24) f(std::integral_constant<int, 24>());
-    else f(std::integral_constant<int, 32>());
+void dispatch_row(int chunks, F&& f) {
+    auto call = [&](auto nch, auto g) { f(nch, g); };
+#define ROW(n, g) call(std::integral_constant<int, n>(), std::integral_constant<int, g>())
+    if (chunks <= 8) ROW(2, 4);
+    else if (chunks <= 16) ROW(4, 4);
+    else if (chunks <= 32) ROW(8, 4);
+    else if (chunks <= 64) ROW(8, 8);
+    else if (chunks <= 96) ROW(6, 16);
+    else if (chunks <= 128) ROW(8, 16);
+    else if (chunks <= 256) ROW(8, 32);
+    else if (chunks <= 384) ROW(12, 32);
+    else if (chunks <= 512) ROW(16, 32);
+    else if (chunks <= 640) ROW(20, 32);
+    else if (chunks <= 768) ROW(24, 32);
+    else ROW(32, 32);
+#undef ROW
+}
+constexpr int kRowClasses = 12;
+int row_class(int chunks) {
+    const int up_to[kRowClasses - 1] = {8, 16, 32, 64, 96, 128, 256, 384, 512, 640, 768};
+    int c = 0;
+    while (c < kRowClasses - 1 && chunks > up_to[c]) ++c;
+    return c;
 }
 
-// Launches the row kernel for any d (vector path when the row fits the registers, else the generic one).
+// 16-byte pieces that a row of d channels may cover: rows of a width that is no multiple of 8 start anywhere in a piece.
+// Up to kResidentChunks the row is held in registers, above it the long-row kernel runs.
+constexpr int kResidentChunks = 1024;
+int row_chunks(int32_t d) { return d % 8 == 0 ? d / 8 : (d + 14) / 8; }
+
+// Launches the row kernel for any d.
 void launch_rows(int grid, cudaStream_t st, const void* feat, int64_t n, int32_t d, float tau, uint8_t* mask,
                  float* entropy, int32_t* counts, double* cta_stats, int64_t tpb) {
-    const bool vec = (d % 8 == 0) && (d <= 8192);
-    if (vec) {
-        dispatch_nch((d / 8 + 31) / 32, [&](auto nch) {
-            gate_rows_kernel<decltype(nch)::value><<<grid, kGateThreads, 0, st>>>(
-                reinterpret_cast<const uint4*>(feat), n, d / 8, tau, mask, entropy, counts, cta_stats, tpb);
-        });
-    } else if (d % 8 == 0) {
-        gate_rows_long_kernel<<<grid, kGateThreads, 0, st>>>(reinterpret_cast<const uint4*>(feat), n, d / 8, tau, mask,
-                                                            entropy, counts, cta_stats, tpb);
-    } else {
-        gate_rows_generic_kernel<<<grid, kGateThreads, 0, st>>>(reinterpret_cast<const uint16_t*>(feat), n, d, tau,
-                                                               mask, entropy, counts, cta_stats, tpb);
+    const int chunks = row_chunks(d);
+    if (chunks > kResidentChunks) {
+        if (d % 8 == 0)
+            gate_rows_long_kernel<false><<<grid, kGateThreads, 0, st>>>(feat, n, d, tau, mask, entropy, counts, cta_stats, tpb);
+        else
+            gate_rows_long_kernel<true><<<grid, kGateThreads, 0, st>>>(feat, n, d, tau, mask, entropy, counts, cta_stats, tpb);
+        return;
     }
+    dispatch_row(chunks, [&](auto nch, auto g) {
+        constexpr int NCH = decltype(nch)::value, G = decltype(g)::value;
+        auto kern = d % 8 == 0 ? gate_rows_kernel<NCH, G, false> : gate_rows_kernel<NCH, G, true>;
+        kern<<<grid, kGateThreads, 0, st>>>(feat, n, d, tau, mask, entropy, counts, cta_stats, tpb);
+    });
 }
 
-// Resident blocks per SM of the row kernel that serves rows of `need` x 32 chunks (0: the generic kernel).
+// Resident blocks per SM of the row kernel that serves rows of d channels.
 // One block per resident slot, i.e. a grid of exactly one wave, measured best: with more blocks the later
 // waves start against a full memory system and the kernel grows a tail (32768 x 5120: 74.8 -> 68.6 us).
-int rows_blocks_per_sm(int need) {
-    static int cache[10] = {0};
-    int slot = need <= 0 ? 0 : need <= 1 ? 1 : need <= 2 ? 2 : need <= 4 ? 3 : need <= 8 ? 4 : need <= 12 ? 5
-               : need <= 16 ? 6 : need <= 20 ? 7 : need <= 24 ? 8 : 9;
-    if (cache[slot] > 0) return cache[slot];
+int rows_blocks_per_sm(int32_t d) {
+    static std::atomic<int> cache[2][kRowClasses + 1] = {};
+    const int chunks = row_chunks(d);
+    const bool ragged = d % 8 != 0;
+    const int slot = chunks > kResidentChunks ? kRowClasses : row_class(chunks);
+    const int known = cache[ragged][slot].load(std::memory_order_relaxed);
+    if (known > 0) return known;
     int occ = 0;
     cudaError_t e = cudaSuccess;
-    if (slot == 0) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, gate_rows_generic_kernel, kGateThreads, 0);
+    auto ask = [&](auto kern) { e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kGateThreads, 0); };
+    if (slot == kRowClasses) {
+        if (ragged) ask(gate_rows_long_kernel<true>);
+        else ask(gate_rows_long_kernel<false>);
     } else {
-        dispatch_nch(need, [&](auto nch) {
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, gate_rows_kernel<decltype(nch)::value>,
-                                                              kGateThreads, 0);
+        dispatch_row(chunks, [&](auto nch, auto g) {
+            constexpr int NCH = decltype(nch)::value, G = decltype(g)::value;
+            if (ragged) ask(gate_rows_kernel<NCH, G, true>);
+            else ask(gate_rows_kernel<NCH, G, false>);
         });
     }
     if (e != cudaSuccess || occ < 1) {
@@ -603,7 +714,7 @@ int rows_blocks_per_sm(int need) {
         occ = 2;
     }
     if (occ > 8) occ = 8;
-    cache[slot] = occ;
+    cache[ragged][slot].store(occ, std::memory_order_relaxed);
     return occ;
 }
 
@@ -643,10 +754,9 @@ int gate_launch(const void* feat, int64_t n, int32_t d, float tau, uint8_t* mask
     if (!feat || !mask || !idx || !block_counts) return ARDIFF_ERR_NULL;
     const int rc = check_feat(feat, d);
     if (rc != ARDIFF_OK) return rc;
-    const bool vec = (d % 8 == 0) && (d <= 8192);
 
     // contiguous token range per block; one block per resident slot of the GPU, each with >= 1 token per warp
-    int64_t want = (int64_t)n_sm * rows_blocks_per_sm(vec ? (d / 8 + 31) / 32 : 0);
+    int64_t want = (int64_t)n_sm * rows_blocks_per_sm(d);
     want *= grid_waves(n, d, want);
     if (want > max_blocks) want = max_blocks;
     int64_t tpb = (n + want - 1) / want;
@@ -667,8 +777,7 @@ int entropy_rows_launch(const void* feat, int64_t rows, int32_t d, float* entrop
     if (!feat || !entropy) return ARDIFF_ERR_NULL;
     const int rc = check_feat(feat, d);
     if (rc != ARDIFF_OK) return rc;
-    const bool vec = (d % 8 == 0) && (d <= 8192);
-    int64_t want = (int64_t)n_sm * rows_blocks_per_sm(vec ? (d / 8 + 31) / 32 : 0);
+    int64_t want = (int64_t)n_sm * rows_blocks_per_sm(d);
     want *= grid_waves(rows, d, want);
     int64_t tpb = (rows + want - 1) / want;
     if (tpb < kGateWarps) tpb = kGateWarps;
@@ -683,15 +792,13 @@ int entropy_rows_launch(const void* feat, int64_t rows, int32_t d, float* entrop
 int gate_blocks_fused_launch(const void* feat, int64_t n, int32_t r, int32_t d, int32_t gamma, float tau,
                              float* row_entropy, float* token_entropy, uint8_t* mask, int32_t* idx, int32_t* count,
                              int32_t* block_len, int32_t* cta_counts, int max_blocks, int n_sm, cudaStream_t st) {
-    const bool vec = (d % 8 == 0) && (d <= 8192);
     constexpr int64_t kMaxRowsPerCta = 24576;     // 96 KB of row entropies
-    if (!vec || (int64_t)gamma * r > kMaxRowsPerCta) return ARDIFF_ERR_UNSUPPORTED;
+    if (row_chunks(d) > kResidentChunks || (int64_t)gamma * r > kMaxRowsPerCta) return ARDIFF_ERR_UNSUPPORTED;
     const int rc = check_feat(feat, d);
     if (rc != ARDIFF_OK) return rc;
-    const int need = (d / 8 + 31) / 32;
     const int64_t n_blocks = (n + gamma - 1) / gamma;
     const int64_t rows = n * r;
-    int64_t want = (int64_t)n_sm * rows_blocks_per_sm(need);
+    int64_t want = (int64_t)n_sm * rows_blocks_per_sm(d);
     want *= grid_waves(rows, d, want);
     if (want > max_blocks) want = max_blocks;
     int64_t bpc = (n_blocks + want - 1) / want;                        // draft blocks per CTA
@@ -703,11 +810,12 @@ int gate_blocks_fused_launch(const void* feat, int64_t n, int32_t r, int32_t d, 
     const int grid = (int)grid64;
     const size_t smem = (size_t)(bpc * rows_per_block) * sizeof(float);
     cudaError_t e = cudaSuccess;
-    dispatch_nch(need, [&](auto nch) {
-        auto kern = gate_blocks_kernel<decltype(nch)::value>;
+    dispatch_row(row_chunks(d), [&](auto nch, auto g) {
+        constexpr int NCH = decltype(nch)::value, G = decltype(g)::value;
+        auto kern = d % 8 == 0 ? gate_blocks_kernel<NCH, G, false> : gate_blocks_kernel<NCH, G, true>;
         if (smem > 48 * 1024) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
         if (e == cudaSuccess)
-            kern<<<grid, kGateThreads, smem, st>>>(reinterpret_cast<const uint4*>(feat), n, r, gamma, d / 8, tau,
+            kern<<<grid, kGateThreads, smem, st>>>(feat, n, r, gamma, d, tau,
                                                   row_entropy, token_entropy, mask, block_len, cta_counts, bpc,
                                                   n_blocks);
     });

@@ -5,12 +5,16 @@
 //                               (the entropy-loss equation's mean over rows and heads);
 //   ardiff_tau_calibrate        the threshold equation tau = 0.3 mean(H) - 0.1 std(H);
 //   ardiff_accept_prefix        Algorithm 1, Step 4: accepted draft length per block.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "../../include/ardiff.h"
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -57,35 +61,63 @@ block_prefix_kernel(const float* __restrict__ row_entropy, int64_t n, int32_t r,
     }
 }
 
-// mean, standard deviation (divisor n) and tau of n entropies; one CTA, fp64, fixed summation order
-// (thread-strided partial sums, then a tree), two passes so that the deviations are taken from the mean.
-__global__ void __launch_bounds__(1024) tau_kernel(const float* __restrict__ H, int64_t n, double* __restrict__ out) {
-    __shared__ double s[1024];
-    __shared__ double s_mean;
-    double acc = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += 1024) acc += (double)H[i];
+// Mean, standard deviation (divisor n) and tau of n entropies: one cluster of CTAs, fp64, two passes so that the
+// deviations are taken from the mean, sums in a fixed order (thread-strided partial sums, a tree per CTA, the CTAs of the
+// cluster in rank order through distributed shared memory), no scratch. Bound by what a few SMs load: a million
+// entropies took one CTA 83 us, 8 take 20.
+constexpr int kTauThreads = 1024;
+__device__ __forceinline__ double cluster_sum(double acc, double* s, double* s_part, unsigned size) {
     s[threadIdx.x] = acc;
     __syncthreads();
-    for (int o = 512; o > 0; o >>= 1) {
-        if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
+    for (int o = kTauThreads / 2; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) s_mean = s[0] / (double)n;
-    __syncthreads();
-    const double mean = s_mean;
-    acc = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += 1024) {
-        const double dlt = (double)H[i] - mean;
-        acc += dlt * dlt;
-    }
-    s[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = 512; o > 0; o >>= 1) {
-        if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
+    if (size == 1) {
+        const double total = s[0];
         __syncthreads();
+        return total;
     }
-    if (threadIdx.x == 0) {
-        const double sd = sqrt(s[0] / (double)n);
+    if (threadIdx.x == 0) *s_part = s[0];
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    double total = 0.0;
+    for (unsigned r = 0; r < size; ++r) total += *cl.map_shared_rank(s_part, r);
+    cl.sync();                                           // the slot may be reused, or its CTA leave
+    return total;
+}
+template <typename F>
+__device__ __forceinline__ double tau_partial(const float* __restrict__ H, int64_t n, unsigned rank, unsigned size, F&& f) {
+    double a0 = 0.0, a1 = 0.0;
+    const int64_t t = (int64_t)rank * kTauThreads + threadIdx.x, stride = (int64_t)size * kTauThreads;
+    // the part before the first 16-byte boundary, whole float4s, the rest
+    const int64_t lead = min(n, (int64_t)((16 - (reinterpret_cast<uintptr_t>(H) & 15u)) & 15u) / 4);
+    const int64_t n4 = (n - lead) / 4;
+    const float4* H4 = reinterpret_cast<const float4*>(H + lead);
+    if (t < lead) a0 += f(H[t]);
+#pragma unroll 4
+    for (int64_t i = t; i < n4; i += stride) {
+        const float4 v = H4[i];
+        a0 += f(v.x) + f(v.y);
+        a1 += f(v.z) + f(v.w);
+    }
+    const int64_t rest = lead + 4 * n4 + t;
+    if (rest < n) a1 += f(H[rest]);
+    return a0 + a1;
+}
+__global__ void __launch_bounds__(kTauThreads) tau_kernel(const float* __restrict__ H, int64_t n, double* __restrict__ out) {
+    __shared__ double s[kTauThreads];
+    __shared__ double s_part;
+    cg::cluster_group cl = cg::this_cluster();
+    const unsigned rank = cl.block_rank(), size = cl.num_blocks();
+    const double mean =
+        cluster_sum(tau_partial(H, n, rank, size, [](float h) { return (double)h; }), s, &s_part, size) / (double)n;
+    const double q = cluster_sum(tau_partial(H, n, rank, size, [mean](float h) {
+        const double dlt = (double)h - mean;
+        return dlt * dlt;
+    }), s, &s_part, size);
+    if (rank == 0 && threadIdx.x == 0) {
+        const double sd = sqrt(q / (double)n);
         out[0] = mean;
         out[1] = sd;
         out[2] = 0.3 * mean - 0.1 * sd;
@@ -126,6 +158,7 @@ extern "C" int ardiff_entropy_gate_blocks(const void* feat, int64_t n, int32_t r
         return ardiff::write_zero_count(count, st);
     }
     if (!feat || !mask || !idx) return ARDIFF_ERR_NULL;
+    if (d % 8 != 0 && !row_entropy) return ARDIFF_ERR_NULL;      // the interface asks for it at such widths
     int32_t* counts = nullptr;
     int max_blocks = 0, sms = 0;
     int rc = ardiff::gate_scratch_get(st, &counts, &max_blocks, &sms);
@@ -155,7 +188,16 @@ extern "C" int ardiff_entropy_gate_blocks(const void* feat, int64_t n, int32_t r
 extern "C" int ardiff_tau_calibrate(const float* entropy, int64_t n, double* out3, void* stream) {
     if (!entropy || !out3) return ARDIFF_ERR_NULL;
     if (n < 1) return ARDIFF_ERR_SHAPE;
-    tau_kernel<<<1, 1024, 0, static_cast<cudaStream_t>(stream)>>>(entropy, n, out3);
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cudaLaunchAttribute at[1];
+    // one CTA while a thread has but a few entropies; 8 CTAs is the largest cluster every device takes
+    const unsigned ctas = n <= 8 * kTauThreads ? 1 : 8;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(ctas); cfg.blockDim = dim3(kTauThreads); cfg.stream = static_cast<cudaStream_t>(stream);
+    cfg.attrs = at; cfg.numAttrs = ctas > 1 ? 1 : 0;
+    (void)cudaLaunchKernelEx(&cfg, tau_kernel, entropy, n, out3);
     ardiff::set_launch_count(1);
     return cudaGetLastError() == cudaSuccess ? ARDIFF_OK : ARDIFF_ERR_CUDA;
 }

@@ -100,6 +100,40 @@ def test_shapes_generic_path(d):
         check(bits, quantile_tau(H, q))
 
 
+@pytest.mark.parametrize("d", [1, 3, 7, 9, 15, 241, 249, 250, 255, 257, 505, 777, 2041, 4099, 8177, 8178, 8179, 8191, 8193, 9001])
+@pytest.mark.parametrize("n,shift", [(1, 0), (2, 1), (3, 7), (9, 5), (67, 3)])
+def test_ragged_rows_at_any_even_address(n, shift, d):
+    """Widths that are no multiple of 8: rows covered by 16-byte pieces, matrices that start
+    `shift` elements after a 16-byte boundary, both sides of every register class and of the long-row path. The
+    elements around the matrix are NaN: none may be taken for the row's own."""
+    dev = require_cuda()
+    rng = np.random.default_rng(1000 * n + d)
+    x = rng.standard_normal((n, d)).astype(np.float32) * 2
+    x[::3] *= 4
+    if d > 4:
+        x[n // 2, [0, d // 2, d - 1]] = -np.inf
+    if n > 2:
+        x[1, d - 1] = np.nan
+        x[2, 0] = np.inf
+    if n > 8:
+        x[5] = -np.inf
+    bits = synth.f32_to_bf16(x)
+    around = torch.full((n * d + 16,), float("nan"), dtype=torch.bfloat16, device=dev)
+    feat = around[shift:shift + n * d].view(n, d)
+    feat.copy_(dev_bf16(bits))
+    H = oracle.entropy(bits)
+    tau = quantile_tau(H, 0.4)
+    mask, idx, count, ent = ardiff.ardiff_entropy_gate(feat, tau, want_entropy=True)
+    ent, mask, c = ent.cpu().numpy(), mask.cpu().numpy(), int(count.item())
+    nan = np.isnan(H)
+    assert np.array_equal(np.isnan(ent), nan)
+    # fp32 sums of up to 9001 terms: the file's bar is 1e-3, the worst rounding of such sums 9001 * 2^-24 of H <= 9.2
+    assert np.all(np.abs(ent[~nan] - H[~nan]) <= ENT_TOL)
+    sure = nan | (np.abs(H - float(np.float32(tau))) >= BAND)
+    assert np.array_equal(mask[sure], (H >= tau).astype(np.uint8)[sure])
+    assert np.array_equal(idx.cpu().numpy()[:c], np.flatnonzero(mask).astype(np.int32))
+
+
 def test_empty_input_writes_zero_count():
     dev = require_cuda()
     feat = torch.empty((0, 64), dtype=torch.bfloat16, device=dev)

@@ -57,7 +57,7 @@ def test_block_prefix_gate_single_row_tokens(n, gamma):
     check_blocks(bits, 1, gamma, tau)
 
 
-@pytest.mark.parametrize("r,d", [(4, 256), (16, 64), (3, 1001)])
+@pytest.mark.parametrize("r,d", [(4, 256), (16, 64), (3, 1001), (2, 777), (5, 9)])
 def test_block_prefix_gate_mean_over_rows(r, d):
     wl = synth.workload("cfg1", n=515 * r, d=d)
     bits = synth.features(wl)
@@ -88,6 +88,20 @@ def test_block_gate_with_gamma_one_equals_plain_gate_and_empty_input():
     empty = torch.empty((0, 64), dtype=torch.bfloat16, device=dev)
     _, _, count0, _, _, _ = ardiff.ardiff_entropy_gate_blocks(empty, 1, 8, 0.0)
     assert int(count0.item()) == 0
+
+
+@pytest.mark.parametrize("n,shift", [(1, 1), (3, 2), (8192, 0), (8193, 3), (1000003, 1)])
+def test_tau_calibration_at_any_address(n, shift):
+    """One CTA and a cluster of them, the pool starting anywhere: fp64 sums of fp32 values against numpy's (a million terms
+    of equal sign in another order differ by less than 1e6 * 2^-53 = 1e-10 of the mean, in practice 1e-13)."""
+    dev = require_cuda()
+    pool = torch.rand(n + shift, device=dev, generator=torch.Generator(device=dev).manual_seed(n)) * 9
+    h = pool[shift:]
+    a, b = ardiff.ardiff_tau_calibrate(h).cpu().numpy(), ardiff.ardiff_tau_calibrate(h).cpu().numpy()
+    x = h.cpu().numpy().astype(np.float64)
+    m, s = x.mean(), x.std()
+    assert np.all(np.abs(a - np.array([m, s, 0.3 * m - 0.1 * s])) <= 1e-9)
+    assert np.array_equal(a, b)
 
 
 @pytest.mark.parametrize("n", [1, 7, 1024, 100003])
