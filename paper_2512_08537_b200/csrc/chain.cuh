@@ -5,8 +5,6 @@
 // therefore only makes what does not depend on the residual stream (conditioning, s_k, all modulations of all steps,
 // read from the weights once); after a grid barrier this code runs the chain with as little as possible in each exchange:
 //   - CTA i owns 16 columns of every W-wide layer for the whole call; its piece of h never leaves registers.
-// It is a part of head_kernel, not a launch of its own: a cooperative kernel that only finds out that it has nothing to do
-// cost every larger call 13 us.
 //   - The 16 x W weight tiles of the coming layers stream into a shared-memory ring (they depend on nothing).
 //   - A value is its own flag: exchange buffers start as all ones (no bf16 pair or fp32 number that is stored can be
 //     that, NaN results are canonical) and are written once; readers check the words themselves, with relaxed loads, so
@@ -14,7 +12,15 @@
 //     spinning on the data itself made their reads queue before the writes they waited for.
 //   - Products are mma.sync m16n8k16: 16 weight rows x 8 tokens, the 8 warps split K, partials meet in shared memory.
 //     (tcgen05 would add a TMA and a tensor-memory round trip to every exchange; the arithmetic is not what bounds.)
-// What bounds it: L2 latency, then every CTA's read of all S x W activations (about 60 B per clock and SM).
+// It is a part of head_kernel, not a launch of its own: a cooperative kernel that only finds out that it has nothing to do
+// cost every larger call 13 us.
+// What bounds it: latency. An exchange takes 2 K cycles at W = 256 (16 CTAs) and 5 K at W = 1536 (96 CTAs), of which the
+// reads of all S x W activations by every CTA are 2 K at 32 tokens; a second pass of 32 tokens costs another 3 us there.
+// Whole calls with the tile schedule and with the chain, us, K = 4: W = 256, L = 2, 33 tokens 164 / 127; W = 1024, L = 3,
+// 32 tokens 345 / 179, 64 tokens 346 / 244, 128 tokens 346 / 419; W = 1536, L = 12, 8 / 29 / 64 tokens 1658 / 594, 1702 /
+// 681, 1702 / 958, 128 tokens about even: hence the limit of 64. Not kept: CTAs that start their reads at different
+// pieces (spills; 681 -> 800), two or one token tiles of 8 loaded at once instead of four (712, 803), LayerNorm partials
+// read by every CTA instead of one warp per token (10 K cycles an exchange instead of 5 K).
 #pragma once
 
 constexpr int CHAIN_MAX_TOKENS = 64;

@@ -1,9 +1,9 @@
 // Entropy gate + stream compaction for sm_100a.
 //
-// Kernel 1 (gate_rows_kernel): one warp per token. The whole bf16 row is fetched with
+// Kernel 1 (gate_rows_kernel): 4 to 32 lanes per token. The whole bf16 row is fetched with
 // 128-bit streaming loads into registers (one HBM pass), the row maximum is taken with packed
 // bf16x2 max, then S = sum 2^t and T = sum t 2^t with t = (x - m) log2(e) are accumulated in
-// fp32, and H = ln S - ln2 * T / S. The warp writes the mask byte (and the entropy, if asked)
+// fp32, and H = ln S - ln2 * T / S. One lane writes the mask byte (and the entropy, if asked)
 // and each block leaves its number of kept tokens in a small scratch array.
 // Kernel 2 (compact_kernel): every block sums the counts of the blocks before it and writes the
 // ascending token ids of its own contiguous token range (ballot + prefix), the last block

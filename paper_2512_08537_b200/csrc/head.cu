@@ -4,7 +4,8 @@
 // x = Diff_theta(x_t | t, z) of the AR+Diffusion hybrid, conditioned on the token's AR hidden
 // state z and on t, sampled with K Euler flow steps from caller-supplied noise.
 //
-// How: every matrix product of the head is cut into items of 128 tokens x 256 output columns. The two
+// How: every matrix product of the head is cut into items of 128 tokens x 256 output columns (128 or 64 when few
+// token tiles leave units idle: see width_limit; up to 64 tokens chain.cuh takes over after the modulations). The two
 // CTAs of a cluster form a unit: each owns one token tile, stages its own A tile (activations) and
 // half of the B tile (weights) per 64-wide K slice by TMA into a 6-stage shared-memory ring, and the
 // even CTA issues tcgen05.mma.cta_group::2 (256 x 256 x 16, bf16 -> fp32) into one of two TMEM
@@ -24,8 +25,9 @@
 // and they share their schedulers with two epilogue warps each (the TMEM lane quarter a warp may read is its
 // id modulo 4, so every scheduler hosts the epilogue of one quarter). Every slot an epilogue warp takes there
 // lengthens the chain, and the epilogue's own loads and stores compete with the copies; the ring drains and
-// the tensor pipe waits. Measured on copies of this kernel that skip work: without any epilogue work a slice
-// is consumed every 545 cycles and the launch takes 21 % fewer cycles (8 points of that are the epilogue's
+// the tensor pipe waits. (One elected lane walks the K loop: under `lane == 0` it took 540 cycles a slice even for 64
+// columns, see ptx::elect_one.) Measured on copies of this kernel that skip work, before that change: without any
+// epilogue work a slice is consumed every 545 cycles and the launch takes 21 % fewer cycles (8 points of that are the epilogue's
 // memory operations); with a sixteenth of the operand bytes it takes 4 % fewer. So the kernel keeps the two chains and the
 // epilogue short: biases travel in registers (one column per lane, handed round by shuffle), c never leaves
 // the accumulator, epilogue inputs are plain loads issued three units ahead, h and the gate values stay off
@@ -693,9 +695,11 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
                 const void* map_b = P.maps + it.map_b;
                 const uint32_t tx = 2u * (A_BYTES + (uint32_t)(it.umma_n / 2) * BK * 2);
                 const int b_row = it.b_row + rank * it.b_step;
-                // weights of slice kb into stage st: the even CTA arms its barrier for the bytes of both CTAs
-                auto load_weights = [&](int st, int kb) {
+                // the even CTA arms its barrier for the bytes of both CTAs
+                auto arm = [&](int st) {
                     if (rank == 0) ptx::mbar_arrive_expect_tx(full_bar(st), tx);
+                };
+                auto load_weights = [&](int st, int kb) {
                     ptx::tma_load_2d_pair(smem_base + st * STAGE_BYTES + A_BYTES, map_b, full_bar(st), kb * BK, b_row);
                 };
                 int pre = 0;        // slices whose weights were sent for before the item's inputs were complete
@@ -709,6 +713,7 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
                         if (BN == ACC_COLS || pre >= it.kblocks || pre >= STAGES ||
                             !ptx::mbar_test_wait(empty_bar(pst), pph ^ 1u))
                             return false;
+                        arm(pst);
                         load_weights(pst, pre);
                         issued |= 1u << pst;
                         issued_parity = (issued_parity & ~(1u << pst)) | (pph << pst);
@@ -728,14 +733,16 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
                     int st = src_stage;
                     uint32_t ph = src_phase;
                     for (int kb = 0; kb < it.kblocks; ++kb) {
-                        if (BN == ACC_COLS || kb >= pre) {
+                        const bool sent = BN < ACC_COLS && kb < pre;      // this slice's weights are on their way
+                        if (!sent) {
                             ok = wait_mbar(empty_bar(st), ph ^ 1u, P);
                             if (!ok) break;
-                            load_weights(st, kb);
                         }
                         if (kb == 0) TRACE(0, 1);
                         TRACE_STAGE(0, kb);
+                        if (!sent) arm(st);
                         ptx::tma_load_2d_pair(smem_base + st * STAGE_BYTES, map_a, full_bar(st), kb * BK, it.a_row0);
+                        if (!sent) load_weights(st, kb);
                         if (kb == peek_kb && have_nx) {
                             // issued here, looked at only after the last slice went out
                             const int* ctr = P.counters + (size_t)nx.abs_m * CTRS;
