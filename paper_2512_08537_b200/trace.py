@@ -25,7 +25,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(_HERE)
 PROFILE_LIB = os.path.join(_HERE, "libardiff_profile.so")
 TRACE_ITEMS = 4096
-TYPES = ["GATHER", "COND", "IN", "SS", "GATE", "G1", "G2", "FSS", "OUT", "NOP"]
+TYPES = ["GATHER", "COND", "IN", "SS", "GATE", "G1", "G2", "FSS", "OUT", "NOP", "MOD"]
 
 
 def build_profile_library() -> str:
