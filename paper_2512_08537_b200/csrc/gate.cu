@@ -103,8 +103,9 @@ __device__ __forceinline__ void acc_word_safe(uint32_t w, float mneg, float& S, 
 
 // Rows of a width that is no multiple of 8 start at any even address. They are read as the 16-byte chunks that cover
 // them: the first chunk starts with `head` elements of the row before, the last one ends with elements of the row
-// after; both are replaced by -inf once the chunk has arrived. Scalar loads in two passes, as before, took
-// 57 us for 65536 x 777 (1.8 TB/s).
+// after; both are replaced by -inf once the chunk has arrived. 65536 x 777: 57 us (1.8 TB/s) with scalar loads in two
+// passes, 39 us this way, 35 us with the tests for the matrix's edges and for the two partial chunks out of the loop over
+// the chunks (bound by instruction issue).
 constexpr uint32_t kFill = 0xff80ff80u;
 struct RowSpan {
     const uint4* base;       // first chunk
@@ -117,24 +118,24 @@ __device__ __forceinline__ RowSpan row_span(const void* feat, int64_t row, int32
     const int head = (int)(at & 15u) / 2;
     return RowSpan{reinterpret_cast<const uint4*>(at & ~(uintptr_t)15), (head + d + 7) / 8, head};
 }
-// Chunk c of a row. Rows at the edges of the matrix read their partial chunks element by element: nothing outside the
-// caller's array is touched.
+// A partial chunk of a row at an edge of the matrix, element by element: nothing outside the caller's array is touched.
+__device__ __noinline__ uint4 load_edge_chunk(const uint4* base, int head, int c, int32_t d) {
+    const uint16_t* e = reinterpret_cast<const uint16_t*>(base + c);
+    uint32_t w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        w[q] = kFill;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = 8 * c + 2 * q + h - head;
+            if (i >= 0 && i < d) w[q] = (w[q] & (h ? 0x0000ffffu : 0xffff0000u)) | ((uint32_t)e[2 * q + h] << (16 * h));
+        }
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
 template <bool RAGGED>
 __device__ __forceinline__ uint4 load_chunk(const RowSpan& r, int c, int32_t d, bool edge) {
-    if (RAGGED && edge && (c == 0 || c == r.nch - 1)) {
-        const uint16_t* e = reinterpret_cast<const uint16_t*>(r.base + c);
-        uint32_t w[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            w[q] = kFill;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int i = 8 * c + 2 * q + h - r.head;
-                if (i >= 0 && i < d) w[q] = (w[q] & (h ? 0x0000ffffu : 0xffff0000u)) | ((uint32_t)e[2 * q + h] << (16 * h));
-            }
-        }
-        return make_uint4(w[0], w[1], w[2], w[3]);
-    }
+    if (RAGGED && edge && (c == 0 || c == r.nch - 1)) return load_edge_chunk(r.base, r.head, c, d);
     return ld_stream_v4(r.base + c);
 }
 // elements lo .. hi - 1 of a chunk kept, the others -inf
@@ -193,8 +194,11 @@ __device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const Row
                                                       bool has_next, bool next_edge, int32_t d, int l) {
     constexpr bool SAFE = RAGGED || G < 32;
     if (RAGGED) {
+        if (l == 0) v[0] = keep_elements(v[0], row.head, 8);
+        const int last = row.nch - 1, keep = row.head + d - 8 * last;
 #pragma unroll
-        for (int j = 0; j < NCH; ++j) v[j] = own_elements<true>(v[j], row, l + G * j, d);
+        for (int j = 0; j < NCH; ++j)
+            if (l + G * j == last) v[j] = keep_elements(v[j], 0, keep);
     }
     // row maximum (packed, exact in bf16)
     uint32_t mx = kFill;
@@ -207,6 +211,8 @@ __device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const Row
     m = warp_max_nan<G>(m);
     const float mneg = -m * kLog2e;
     float S = 0.f, T = 0.f;
+    const int lo = RAGGED && next_edge ? 1 : 0, hi = !has_next ? 0 : RAGGED && next_edge ? next.nch - 1 : next.nch;
+    const uint4* np = next.base + l;
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
         const int c = l + G * j;
@@ -224,9 +230,16 @@ __device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const Row
             }
             if (!RAGGED && has_next) v[j] = ld_stream_v4(next.base + c);
         }
-        // neighbouring rows may differ by a chunk
-        if (RAGGED && has_next)
-            v[j] = c < next.nch ? load_chunk<true>(next, c, d, next_edge) : make_uint4(kFill, kFill, kFill, kFill);
+        // neighbouring rows may differ by a chunk; at an edge the partial chunks follow after the others
+        if (RAGGED) {
+            v[j] = make_uint4(kFill, kFill, kFill, kFill);
+            if (c < hi && (j > 0 || c >= lo)) v[j] = ld_stream_v4(np + G * j);
+        }
+    }
+    if (RAGGED && has_next && next_edge) {
+#pragma unroll
+        for (int j = 0; j < NCH; ++j)
+            if (l + G * j == 0 || l + G * j == next.nch - 1) v[j] = load_edge_chunk(next.base, next.head, l + G * j, d);
     }
     S = warp_sum<G>(S);
     T = warp_sum<G>(T);
@@ -801,7 +814,9 @@ int gate_blocks_fused_launch(const void* feat, int64_t n, int32_t r, int32_t d, 
     int64_t want = (int64_t)n_sm * rows_blocks_per_sm(d);
     want *= grid_waves(rows, d, want);
     if (want > max_blocks) want = max_blocks;
-    int64_t bpc = (n_blocks + want - 1) / want;                        // draft blocks per CTA
+    // draft blocks per CTA: one wave of CTAs, but where a CTA would have only two or three, one each: 512 draft blocks of
+    // 128 rows as 256 CTAs left half of the warps idle (21 % occupancy)
+    int64_t bpc = n_blocks <= 2 * want ? 1 : (n_blocks + want - 1) / want;
     const int64_t rows_per_block = (int64_t)gamma * r;
     if (bpc * rows_per_block > kMaxRowsPerCta) bpc = kMaxRowsPerCta / rows_per_block;
     if (bpc < 1) bpc = 1;
