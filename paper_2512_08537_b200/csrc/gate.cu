@@ -101,6 +101,25 @@ __device__ __forceinline__ void acc_word_safe(uint32_t w, float mneg, float& S, 
     T = fmaf(fmaxf(t1, -1e30f), e1, T);
 }
 
+// One 16-byte chunk of such words, summed by itself first: a lane that holds many chunks of one row (up to 64 elements where
+// rows share a warp) would else add them all in one chain. Error against 64 bits, 16384 rows of 256: 5.3e-8 of the norm in
+// one chain, 4.0e-8 this way (4.0e-8 with one row per warp, 8 elements per lane); one more operation per 8 elements.
+__device__ __forceinline__ void acc_chunk_safe(const uint4& v, float mneg, float& S, float& T) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    float s = 0.f, t = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float t0 = fmaf(bf16_lo(w[q]), kLog2e, mneg), t1 = fmaf(bf16_hi(w[q]), kLog2e, mneg);
+        const float e0 = ex2_approx(t0), e1 = ex2_approx(t1);
+        s = q == 0 ? e0 + e1 : (s + e0) + e1;
+        const float p0 = fmaxf(t0, -1e30f);
+        t = q == 0 ? p0 * e0 : fmaf(p0, e0, t);
+        t = fmaf(fmaxf(t1, -1e30f), e1, t);
+    }
+    S += s;
+    T += t;
+}
+
 // Rows of a width that is no multiple of 8 start at any even address. They are read as the 16-byte chunks that cover
 // them: the first chunk starts with `head` elements of the row before, the last one ends with elements of the row
 // after; both are replaced by -inf once the chunk has arrived. 65536 x 777: 57 us (1.8 TB/s) with scalar loads in two
@@ -218,10 +237,7 @@ __device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const Row
         const int c = l + G * j;
         if (c < row.nch) {
             if (SAFE) {
-                acc_word_safe(v[j].x, mneg, S, T);
-                acc_word_safe(v[j].y, mneg, S, T);
-                acc_word_safe(v[j].z, mneg, S, T);
-                acc_word_safe(v[j].w, mneg, S, T);
+                acc_chunk_safe(v[j], mneg, S, T);
             } else {
                 acc_word(v[j].x, mneg, S, T);
                 acc_word(v[j].y, mneg, S, T);
