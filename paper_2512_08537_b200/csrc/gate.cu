@@ -416,6 +416,15 @@ gate_blocks_kernel(const void* __restrict__ feat, int64_t n_tokens, int32_t r, i
     }
 }
 
+// Partial sums (S, T) of a lane whose maximum so far was `from`, brought to the larger maximum `to`. Where 2^D is 0 nothing
+// is left of them, also when they are not finite: from * log2 e overflows for the type's lowest values, which serve as masks.
+__device__ __forceinline__ void rescale_sums(float from, float to, float& S, float& T) {
+    const float D = (from - to) * kLog2e;
+    const float f = ex2_approx(D);
+    T = f > 0.f ? (T + D * S) * f : 0.f;
+    S = f > 0.f ? S * f : 0.f;
+}
+
 // Rows longer than the registers hold: still one pass with 128-bit loads. Every lane keeps a running maximum of its own
 // share of the row and rescales its partial sums when the maximum grows
 // (S <- S 2^D, T <- (T + D S) 2^D with D = (m_old - m_new) log2 e <= 0); the lanes' partials are merged the
@@ -458,12 +467,7 @@ gate_rows_long_kernel(const void* __restrict__ feat, int64_t n, int32_t d, float
             const float mc = (a != a || b != b) ? CUDART_NAN_F : fmaxf(a, b);
             if (mc != mc) ml = CUDART_NAN_F;
             else if (mc > ml) {
-                if (S > 0.f) {
-                    const float D = (ml - mc) * kLog2e;
-                    const float f = ex2_approx(D);
-                    T = (T + D * S) * f;
-                    S = S * f;
-                }
+                rescale_sums(ml, mc, S, T);
                 ml = mc;
             }
             // a lane whose elements so far are all -inf has nothing to add (and no finite maximum to subtract)
@@ -490,12 +494,7 @@ gate_rows_long_kernel(const void* __restrict__ feat, int64_t n, int32_t d, float
             for (int j = 0; j < G; ++j) v[j] = nv[j];
         }
         const float m = warp_max_nan(ml);
-        if (S > 0.f && ml < m) {               // bring this lane's partials to the row maximum
-            const float D = (ml - m) * kLog2e;
-            const float f = ex2_approx(D);
-            T = (T + D * S) * f;
-            S = S * f;
-        }
+        if (ml < m) rescale_sums(ml, m, S, T);      // bring this lane's partials to the row maximum
         S = warp_sum(S);
         T = warp_sum(T);
         float H = logf(S) - kLn2 * (T / S);

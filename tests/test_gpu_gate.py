@@ -138,13 +138,35 @@ def test_ragged_rows_at_any_even_address(n, shift, d):
 def test_rows_that_share_a_warp_lose_no_precision(d):
     """fp32 sums of a row against fp64, as a 2-norm over 8192 rows. One row per warp (8 to 32 terms per lane, then a tree)
     is off by 3.7e-8 to 4.3e-8 at these widths; one chain of 64 terms per lane by up to 5.3e-8. The bar lies between."""
-    dev = require_cuda()
     rng = np.random.default_rng(d)
     bits = synth.f32_to_bf16((rng.standard_normal((8192, d)) * 2).astype(np.float32))
     H = oracle.entropy(bits)
     _, _, _, ent = ardiff.ardiff_entropy_gate(dev_bf16(bits), 1.0, want_entropy=True)
     err = ent.cpu().numpy().astype(np.float64) - H
     assert np.linalg.norm(err) / np.linalg.norm(H) <= 4.6e-8
+
+
+@pytest.mark.parametrize("d", [64, 777, 1024, 4099, 8185, 8186, 8200, 9001, 16384, 16391])
+def test_rows_masked_with_the_lowest_value(d):
+    """Masks of the type's lowest value, at the start, in the middle, at the end of a row and over most of it: the masked
+    channels contribute nothing, as with -inf, in every row kernel."""
+    rng = np.random.default_rng(d)
+    x = (rng.standard_normal((40, d)) * 2).astype(np.float32)
+    low = float(torch.finfo(torch.bfloat16).min)
+    for i in range(40):
+        a, b = sorted(rng.integers(0, d, 2))
+        if i % 4 == 0:
+            x[i, :b] = low
+        elif i % 4 == 1:
+            x[i, a:] = low
+        elif i % 4 == 2:
+            x[i, a:b + 1] = low
+        else:
+            x[i, rng.permutation(d)[: d - 5]] = low
+    x[np.arange(40), rng.integers(0, d, 40)] = 1.0          # at least one channel of every row is not masked
+    bits = synth.f32_to_bf16(x)
+    _, _, _, ent = ardiff.ardiff_entropy_gate(dev_bf16(bits), 1.0, want_entropy=True)
+    assert np.all(np.abs(ent.cpu().numpy() - oracle.entropy(bits)) <= ENT_TOL)
 
 
 def test_empty_input_writes_zero_count():
