@@ -24,6 +24,7 @@
 
 #include "../../include/ardiff.h"
 #include "common.cuh"
+#include "gate_plan.h"
 
 namespace {
 
@@ -820,7 +821,6 @@ int entropy_rows_launch(const void* feat, int64_t rows, int32_t d, float* entrop
 int gate_blocks_fused_launch(const void* feat, int64_t n, int32_t r, int32_t d, int32_t gamma, float tau,
                              float* row_entropy, float* token_entropy, uint8_t* mask, int32_t* idx, int32_t* count,
                              int32_t* block_len, int32_t* cta_counts, int max_blocks, int n_sm, cudaStream_t st) {
-    constexpr int64_t kMaxRowsPerCta = 24576;     // 96 KB of row entropies
     if (row_chunks(d) > kResidentChunks || (int64_t)gamma * r > kMaxRowsPerCta) return ARDIFF_ERR_UNSUPPORTED;
     const int rc = check_feat(feat, d);
     if (rc != ARDIFF_OK) return rc;
@@ -828,16 +828,11 @@ int gate_blocks_fused_launch(const void* feat, int64_t n, int32_t r, int32_t d, 
     const int64_t rows = n * r;
     int64_t want = (int64_t)n_sm * rows_blocks_per_sm(d);
     want *= grid_waves(rows, d, want);
-    if (want > max_blocks) want = max_blocks;
-    // draft blocks per CTA: one wave of CTAs, but where a CTA would have only two or three, one each: 512 draft blocks of
-    // 128 rows as 256 CTAs left half of the warps idle (21 % occupancy)
-    int64_t bpc = n_blocks <= 2 * want ? 1 : (n_blocks + want - 1) / want;
     const int64_t rows_per_block = (int64_t)gamma * r;
-    if (bpc * rows_per_block > kMaxRowsPerCta) bpc = kMaxRowsPerCta / rows_per_block;
-    if (bpc < 1) bpc = 1;
-    const int64_t grid64 = (n_blocks + bpc - 1) / bpc;
-    if (grid64 > max_blocks) return ARDIFF_ERR_UNSUPPORTED;          // too many CTAs for the count scratch
-    const int grid = (int)grid64;
+    const DraftPlan plan = plan_draft_blocks(n_blocks, rows_per_block, want, max_blocks);
+    if (plan.grid == 0) return ARDIFF_ERR_UNSUPPORTED;               // too many CTAs for the count scratch
+    const int grid = (int)plan.grid;
+    const int64_t bpc = plan.blocks_per_cta;
     const size_t smem = (size_t)(bpc * rows_per_block) * sizeof(float);
     cudaError_t e = cudaSuccess;
     dispatch_row(row_chunks(d), [&](auto nch, auto g) {
