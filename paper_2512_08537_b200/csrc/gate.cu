@@ -829,7 +829,9 @@ int gate_blocks_fused_launch(const void* feat, int64_t n, int32_t r, int32_t d, 
     int64_t want = (int64_t)n_sm * rows_blocks_per_sm(d);
     want *= grid_waves(rows, d, want);
     const int64_t rows_per_block = (int64_t)gamma * r;
-    const DraftPlan plan = plan_draft_blocks(n_blocks, rows_per_block, want, max_blocks);
+    int64_t rows_per_round = 0;
+    dispatch_row(row_chunks(d), [&](auto, auto g) { rows_per_round = kGateThreads / decltype(g)::value; });
+    const DraftPlan plan = plan_draft_blocks(n_blocks, rows_per_block, rows_per_round, want, max_blocks);
     if (plan.grid == 0) return ARDIFF_ERR_UNSUPPORTED;               // too many CTAs for the count scratch
     const int grid = (int)plan.grid;
     const int64_t bpc = plan.blocks_per_cta;
