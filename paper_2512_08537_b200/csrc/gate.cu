@@ -102,22 +102,24 @@ __device__ __forceinline__ void acc_word_safe(uint32_t w, float mneg, float& S, 
     T = fmaf(fmaxf(t1, -1e30f), e1, T);
 }
 
-// One 16-byte chunk of such words, summed by itself first: a lane that holds many chunks of one row (up to 64 elements where
-// rows share a warp) would else add them all in one chain. Error against 64 bits, 16384 rows of 256: 5.3e-8 of the norm in
-// one chain, 4.0e-8 this way (4.0e-8 with one row per warp, 8 elements per lane); one more operation per 8 elements.
+// One 16-byte chunk of such words, summed by itself first: where rows share a warp a lane holds up to 64 elements of one
+// row, and would else add them all in one chain. Error against 64 bits, 16384 rows of 256: 5.3e-8 of the norm in one chain,
+// 4.0e-8 this way (4.0e-8 with one row per warp, 8 elements per lane), for one more operation per 8 elements (0 to 3 % of
+// the time). Two chains per lane instead cost as much and, with one ragged row per warp, an occupancy step (38 -> 48 us at
+// 16384 x 4099).
 __device__ __forceinline__ void acc_chunk_safe(const uint4& v, float mneg, float& S, float& T) {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    float s = 0.f, t = 0.f;
+    float s[4], t = 0.f;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const float t0 = fmaf(bf16_lo(w[q]), kLog2e, mneg), t1 = fmaf(bf16_hi(w[q]), kLog2e, mneg);
         const float e0 = ex2_approx(t0), e1 = ex2_approx(t1);
-        s = q == 0 ? e0 + e1 : (s + e0) + e1;
+        s[q] = e0 + e1;
         const float p0 = fmaxf(t0, -1e30f);
         t = q == 0 ? p0 * e0 : fmaf(p0, e0, t);
         t = fmaf(fmaxf(t1, -1e30f), e1, t);
     }
-    S += s;
+    S += (s[0] + s[1]) + (s[2] + s[3]);
     T += t;
 }
 
@@ -237,8 +239,13 @@ __device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const Row
     for (int j = 0; j < NCH; ++j) {
         const int c = l + G * j;
         if (c < row.nch) {
-            if (SAFE) {
+            if (G < 32) {
                 acc_chunk_safe(v[j], mneg, S, T);
+            } else if (SAFE) {
+                acc_word_safe(v[j].x, mneg, S, T);
+                acc_word_safe(v[j].y, mneg, S, T);
+                acc_word_safe(v[j].z, mneg, S, T);
+                acc_word_safe(v[j].w, mneg, S, T);
             } else {
                 acc_word(v[j].x, mneg, S, T);
                 acc_word(v[j].y, mneg, S, T);
