@@ -133,12 +133,13 @@ struct RowSpan {
     const uint4* base;       // first chunk
     int nch, head;
 };
+// (width: channels; of aligned rows chunks)
 template <bool RAGGED>
-__device__ __forceinline__ RowSpan row_span(const void* feat, int64_t row, int32_t d) {
-    if (!RAGGED) return RowSpan{static_cast<const uint4*>(feat) + row * (int64_t)(d / 8), d / 8, 0};
-    const uintptr_t at = reinterpret_cast<uintptr_t>(feat) + (uintptr_t)row * (uintptr_t)d * 2;
+__device__ __forceinline__ RowSpan row_span(const void* feat, int64_t row, int32_t width) {
+    if (!RAGGED) return RowSpan{static_cast<const uint4*>(feat) + row * (int64_t)width, width, 0};
+    const uintptr_t at = reinterpret_cast<uintptr_t>(feat) + (uintptr_t)row * (uintptr_t)width * 2;
     const int head = (int)(at & 15u) / 2;
-    return RowSpan{reinterpret_cast<const uint4*>(at & ~(uintptr_t)15), (head + d + 7) / 8, head};
+    return RowSpan{reinterpret_cast<const uint4*>(at & ~(uintptr_t)15), (head + width + 7) / 8, head};
 }
 // A partial chunk of a row at an edge of the matrix, element by element: nothing outside the caller's array is touched.
 __device__ __noinline__ uint4 load_edge_chunk(const uint4* base, int head, int c, int32_t d) {
@@ -205,24 +206,68 @@ __device__ __noinline__ float row_entropy_careful(const uint4* row, int nchunks,
     return logf(S) - kLn2 * (T / S);
 }
 
-// Entropy of the row held in v by G lanes (NCH 16-byte chunks per lane). Each chunk is refilled with the warp's NEXT row
-// as soon as the exponentials of the current row have consumed it, so a warp always has loads in flight while
+// Entropy of the aligned row that a warp holds in v (NCH 16-byte chunks per lane). Each chunk is refilled with the warp's
+// NEXT row as soon as the exponentials of the current row have consumed it, so a warp always has loads in flight while
 // it computes (with 128 registers per thread only 16 warps fit an SM: they cannot hide HBM latency by
-// switching alone). Up to 2048 channels a warp holds 32 / G rows: what a row costs beside its elements (three
-// reductions by shuffle, a logarithm, a division, the loop) is then paid once for all of them. One row per warp took
-// 243 us for 2^20 x 64 and 22 us for 65536 x 256.
+// switching alone). Plain pointers and the chunk count as an argument: the same through RowSpan and d / 8 took 77 us
+// instead of 55 at 16384 x 8192.
+template <int NCH>
+__device__ __forceinline__ float whole_row_entropy(uint4 (&v)[NCH], const uint4* row, const uint4* next_row,
+                                                   bool has_next, int32_t nchunks, int lane) {
+    // row maximum (packed, exact in bf16)
+    uint32_t mx = kFill;
+#pragma unroll
+    for (int j = 0; j < NCH; ++j) {
+        mx = max_bf16x2_nan(mx, max_bf16x2_nan(max_bf16x2_nan(v[j].x, v[j].y), max_bf16x2_nan(v[j].z, v[j].w)));
+    }
+    float ml = bf16_lo(mx), mh = bf16_hi(mx);
+    float m = (ml != ml || mh != mh) ? CUDART_NAN_F : fmaxf(ml, mh);
+    m = warp_max_nan(m);
+    const float mneg = -m * kLog2e;
+    float S = 0.f, T = 0.f;
+#pragma unroll
+    for (int j = 0; j < NCH; ++j) {
+        const int c = lane + 32 * j;
+        if (c < nchunks) {
+            acc_word(v[j].x, mneg, S, T);
+            acc_word(v[j].y, mneg, S, T);
+            acc_word(v[j].z, mneg, S, T);
+            acc_word(v[j].w, mneg, S, T);
+            if (has_next) v[j] = ld_stream_v4(next_row + c);
+        }
+    }
+    S = warp_sum(S);
+    T = warp_sum(T);
+    float H = logf(S) - kLn2 * (T / S);
+    if (H != H) {
+        // a -inf channel (t*e = -inf*0) lands here, as do genuinely undefined rows
+        H = row_entropy_careful(row, nchunks, lane, m);
+    }
+    return H;
+}
+template <int NCH>
+__device__ __forceinline__ void load_whole_row(uint4 (&v)[NCH], const uint4* row, int32_t nchunks, int lane) {
+#pragma unroll
+    for (int j = 0; j < NCH; ++j) {
+        const int c = lane + 32 * j;
+        v[j] = c < nchunks ? ld_stream_v4(row + c) : make_uint4(kFill, kFill, kFill, kFill);
+    }
+}
+
+// The same for rows at any even address (RAGGED) and for 32 / G rows to a warp, G lanes each. Where rows share a warp, what
+// a row costs beside its elements (three reductions by shuffle, a logarithm, a division, the loop) is paid once for all of
+// them: one row per warp takes 243 us for 2^20 x 64 and 22 us for 65536 x 256, this 45 and 12. `step` rows lie between a
+// lane's row and its next one.
 template <int NCH, int G, bool RAGGED>
-__device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const RowSpan& row, const RowSpan& next,
-                                                      bool has_next, bool next_edge, int32_t d, int l) {
-    constexpr bool SAFE = RAGGED || G < 32;
+__device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const RowSpan& row, const RowSpan& next, int step,
+                                                      bool has_next, bool next_edge, int32_t width, int l) {
     if (RAGGED) {
         if (l == 0) v[0] = keep_elements(v[0], row.head, 8);
-        const int last = row.nch - 1, keep = row.head + d - 8 * last;
+        const int last = row.nch - 1, keep = row.head + width - 8 * last;
 #pragma unroll
         for (int j = 0; j < NCH; ++j)
             if (l + G * j == last) v[j] = keep_elements(v[j], 0, keep);
     }
-    // row maximum (packed, exact in bf16)
     uint32_t mx = kFill;
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
@@ -241,18 +286,14 @@ __device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const Row
         if (c < row.nch) {
             if (G < 32) {
                 acc_chunk_safe(v[j], mneg, S, T);
-            } else if (SAFE) {
+            } else {
                 acc_word_safe(v[j].x, mneg, S, T);
                 acc_word_safe(v[j].y, mneg, S, T);
                 acc_word_safe(v[j].z, mneg, S, T);
                 acc_word_safe(v[j].w, mneg, S, T);
-            } else {
-                acc_word(v[j].x, mneg, S, T);
-                acc_word(v[j].y, mneg, S, T);
-                acc_word(v[j].z, mneg, S, T);
-                acc_word(v[j].w, mneg, S, T);
             }
-            if (!RAGGED && has_next) v[j] = ld_stream_v4(next.base + c);
+            // by the distance from this row: fewer registers than the next row's own pointer (16384 x 1024 11.3 us, not 12.3)
+            if (!RAGGED && has_next) v[j] = ld_stream_v4(row.base + (int64_t)step * row.nch + c);
         }
         // neighbouring rows may differ by a chunk; at an edge the partial chunks follow after the others
         if (RAGGED) {
@@ -263,24 +304,50 @@ __device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const Row
     if (RAGGED && has_next && next_edge) {
 #pragma unroll
         for (int j = 0; j < NCH; ++j)
-            if (l + G * j == 0 || l + G * j == next.nch - 1) v[j] = load_edge_chunk(next.base, next.head, l + G * j, d);
+            if (l + G * j == 0 || l + G * j == next.nch - 1) v[j] = load_edge_chunk(next.base, next.head, l + G * j, width);
     }
     S = warp_sum<G>(S);
     T = warp_sum<G>(T);
-    float H = logf(S) - kLn2 * (T / S);
-    if (!SAFE && H != H) {
-        // a -inf channel (t*e = -inf*0) lands here, as do genuinely undefined rows
-        H = row_entropy_careful(row.base, row.nch, l, m);
-    }
-    return H;
+    return logf(S) - kLn2 * (T / S);
 }
 
 template <int NCH, int G, bool RAGGED>
-__device__ __forceinline__ void load_resident_row(uint4 (&v)[NCH], const RowSpan& row, int32_t d, bool edge, bool have, int l) {
+__device__ __forceinline__ void load_resident_row(uint4 (&v)[NCH], const RowSpan& row, int32_t width, bool edge, bool have,
+                                                  int l) {
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
         const int c = l + G * j;
-        v[j] = have && c < row.nch ? load_chunk<RAGGED>(row, c, d, edge) : make_uint4(kFill, kFill, kFill, kFill);
+        v[j] = have && c < row.nch ? load_chunk<RAGGED>(row, c, width, edge) : make_uint4(kFill, kFill, kFill, kFill);
+    }
+}
+
+// f(row, its entropy, whether this lane answers for it) over rows begin + first row of the warp .. end - 1 of n, NCH chunks
+// per lane and G lanes per row, in registers. `width` is d of ragged rows, the chunk count of aligned ones.
+template <int NCH, int G, bool RAGGED, typename F>
+__device__ __forceinline__ void for_each_row(const void* __restrict__ feat, int64_t begin, int64_t end, int64_t n,
+                                             int32_t width, int warp, int lane, F&& f) {
+    uint4 v[NCH];
+    if constexpr (!RAGGED && G == 32) {
+        const uint4* base = static_cast<const uint4*>(feat);
+        if (begin + warp < end) load_whole_row(v, base + (begin + warp) * (int64_t)width, width, lane);
+        for (int64_t i = begin + warp; i < end; i += kGateWarps) {
+            const uint4* row = base + i * (int64_t)width;
+            f(i, whole_row_entropy(v, row, row + (int64_t)kGateWarps * width, i + kGateWarps < end, width, lane), lane == 0);
+        }
+    } else {
+        constexpr int R = 32 / G, STEP = kGateWarps * R;         // rows of a warp, of the CTA
+        const int l = lane % G, sub = lane / G;
+        auto edge = [&](int64_t i) { return edge_row<RAGGED>(i, n, width); };
+        const int64_t first = begin + warp * R + sub;
+        RowSpan row = row_span<RAGGED>(feat, first, width);
+        load_resident_row<NCH, G, RAGGED>(v, row, width, edge(first), first < end, l);
+        for (int64_t i0 = begin + warp * R; i0 < end; i0 += STEP) {
+            const int64_t i = i0 + sub, nx = i + STEP;
+            const RowSpan next = row_span<RAGGED>(feat, nx, width);
+            const float H = resident_row_entropy<NCH, G, RAGGED>(v, row, next, STEP, nx < end, edge(nx), width, l);
+            row = next;
+            f(i, H, l == 0 && i < end);
+        }
     }
 }
 
@@ -300,7 +367,7 @@ __device__ __forceinline__ void cta_merge_stats(const WarpStats& mine, int warp,
 // G lanes per token, row resident in registers: NCH 16-byte chunks per lane.
 template <int NCH, int G, bool RAGGED>
 __global__ void __launch_bounds__(kGateThreads)
-gate_rows_kernel(const void* __restrict__ feat, int64_t n, int32_t d, float tau,
+gate_rows_kernel(const void* __restrict__ feat, int64_t n, int32_t width, float tau,
                  uint8_t* __restrict__ mask, float* __restrict__ entropy,
                  int32_t* __restrict__ block_counts, double* __restrict__ cta_stats, int64_t tokens_per_block) {
     const int lane = threadIdx.x & 31;
@@ -312,25 +379,18 @@ gate_rows_kernel(const void* __restrict__ feat, int64_t n, int32_t d, float tau,
     const int64_t t_end = min(n, t_begin + tokens_per_block);
     int kept = 0;
     WarpStats st{0.0, 0.0, 0.0};
-    uint4 v[NCH];
-    auto edge = [&](int64_t i) { return edge_row<RAGGED>(i, n, d); };
-    constexpr int R = 32 / G;                // rows of a warp
-    const int l = lane % G, sub = lane / G;
-    RowSpan row = row_span<RAGGED>(feat, t_begin + warp * R + sub, d);
-    load_resident_row<NCH, G, RAGGED>(v, row, d, edge(t_begin + warp * R + sub), t_begin + warp * R + sub < t_end, l);
-    for (int64_t t0 = t_begin + warp * R; t0 < t_end; t0 += kGateWarps * R) {
-        const int64_t tok = t0 + sub, nx = tok + kGateWarps * R;
-        const RowSpan next = row_span<RAGGED>(feat, nx, d);
-        const float H = resident_row_entropy<NCH, G, RAGGED>(v, row, next, nx < t_end, edge(nx), d, l);
-        row = next;
-        if (l == 0 && tok < t_end) {
-            const bool keep = (H >= tau);  // false for NaN
+    for_each_row<NCH, G, RAGGED>(feat, t_begin, t_end, n, width, warp, lane, [&](int64_t tok, float H, bool mine) {
+        const bool keep = (H >= tau);  // false for NaN
+        if (mine) {
             if (mask) mask[tok] = keep ? 1 : 0;
             if (entropy) entropy[tok] = H;
-            kept += keep ? 1 : 0;
-            if (cta_stats) { st.n += 1.0; st.s += (double)H; st.q += (double)H * (double)H; }
         }
-    }
+        // (lane 0 speaks for the warp at the end: where a row has all lanes they all count it)
+        if (G == 32 || mine) {
+            kept += keep ? 1 : 0;
+            st.n += 1.0; st.s += (double)H; st.q += (double)H * (double)H;
+        }
+    });
     if (G < 32) {                            // the warp's rows together, in a fixed order
 #pragma unroll
         for (int o = 16; o >= G; o >>= 1) {
@@ -361,7 +421,7 @@ gate_rows_kernel(const void* __restrict__ feat, int64_t n, int32_t d, float tau,
 // length and, if asked, the indicators. No row entropy goes through global memory unless the caller wants it.
 template <int NCH, int G, bool RAGGED>
 __global__ void __launch_bounds__(kGateThreads)
-gate_blocks_kernel(const void* __restrict__ feat, int64_t n_tokens, int32_t r, int32_t gamma, int32_t d,
+gate_blocks_kernel(const void* __restrict__ feat, int64_t n_tokens, int32_t r, int32_t gamma, int32_t width,
                    float tau, float* __restrict__ row_entropy, float* __restrict__ token_entropy,
                    uint8_t* __restrict__ mask, int32_t* __restrict__ block_len, int32_t* __restrict__ cta_counts,
                    int64_t blocks_per_cta, int64_t n_blocks) {
@@ -374,23 +434,12 @@ gate_blocks_kernel(const void* __restrict__ feat, int64_t n_tokens, int32_t r, i
     const int64_t t_begin = b_begin * gamma;
     const int64_t t_end = min(n_tokens, b_end * gamma);
     const int64_t r_begin = t_begin * r, r_end = t_end * r;
-    uint4 v[NCH];
-    const int64_t n_rows = n_tokens * r;
-    auto edge = [&](int64_t i) { return edge_row<RAGGED>(i, n_rows, d); };
-    constexpr int R = 32 / G;                // rows of a warp
-    const int l = lane % G, sub = lane / G;
-    RowSpan row = row_span<RAGGED>(feat, r_begin + warp * R + sub, d);
-    load_resident_row<NCH, G, RAGGED>(v, row, d, edge(r_begin + warp * R + sub), r_begin + warp * R + sub < r_end, l);
-    for (int64_t r0 = r_begin + warp * R; r0 < r_end; r0 += kGateWarps * R) {
-        const int64_t row_i = r0 + sub, nx = row_i + kGateWarps * R;
-        const RowSpan next = row_span<RAGGED>(feat, nx, d);
-        const float H = resident_row_entropy<NCH, G, RAGGED>(v, row, next, nx < r_end, edge(nx), d, l);
-        row = next;
-        if (l == 0 && row_i < r_end) {
-            s_H[row_i - r_begin] = H;
-            if (row_entropy) row_entropy[row_i] = H;
+    for_each_row<NCH, G, RAGGED>(feat, r_begin, r_end, n_tokens * r, width, warp, lane, [&](int64_t i, float H, bool mine) {
+        if (mine) {
+            s_H[i - r_begin] = H;
+            if (row_entropy) row_entropy[i] = H;
         }
-    }
+    });
     __syncthreads();
     int kept_total = 0;
     const float inv = 1.0f / (float)r;
@@ -456,7 +505,7 @@ gate_rows_long_kernel(const void* __restrict__ feat, int64_t n, int32_t d, float
             v[j] = c0 + 32 * j < row.nch ? load_chunk<RAGGED>(row, c0 + 32 * j, d, edge) : make_uint4(kFill, kFill, kFill, kFill);
     };
     for (int64_t tok = t_begin + warp; tok < t_end; tok += kGateWarps) {
-        const RowSpan row = row_span<RAGGED>(feat, tok, d);
+        const RowSpan row = row_span<RAGGED>(feat, tok, RAGGED ? d : d / 8);
         const bool edge = edge_row<RAGGED>(tok, n, d);
         float ml = -CUDART_INF_F, S = 0.f, T = 0.f;
         uint4 v[G], nv[G];
@@ -703,6 +752,8 @@ int row_class(int chunks) {
 // Up to kResidentChunks the row is held in registers, above it the long-row kernel runs.
 constexpr int kResidentChunks = 1024;
 int row_chunks(int32_t d) { return d % 8 == 0 ? d / 8 : (d + 14) / 8; }
+// what the kernels of resident rows take as their width
+int32_t kernel_width(int32_t d) { return d % 8 == 0 ? d / 8 : d; }
 
 // Launches the row kernel for any d.
 void launch_rows(int grid, cudaStream_t st, const void* feat, int64_t n, int32_t d, float tau, uint8_t* mask,
@@ -718,7 +769,7 @@ void launch_rows(int grid, cudaStream_t st, const void* feat, int64_t n, int32_t
     dispatch_row(chunks, [&](auto nch, auto g) {
         constexpr int NCH = decltype(nch)::value, G = decltype(g)::value;
         auto kern = d % 8 == 0 ? gate_rows_kernel<NCH, G, false> : gate_rows_kernel<NCH, G, true>;
-        kern<<<grid, kGateThreads, 0, st>>>(feat, n, d, tau, mask, entropy, counts, cta_stats, tpb);
+        kern<<<grid, kGateThreads, 0, st>>>(feat, n, kernel_width(d), tau, mask, entropy, counts, cta_stats, tpb);
     });
 }
 
@@ -849,7 +900,7 @@ int gate_blocks_fused_launch(const void* feat, int64_t n, int32_t r, int32_t d, 
         auto kern = d % 8 == 0 ? gate_blocks_kernel<NCH, G, false> : gate_blocks_kernel<NCH, G, true>;
         if (smem > 48 * 1024) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
         if (e == cudaSuccess)
-            kern<<<grid, kGateThreads, smem, st>>>(feat, n, r, gamma, d, tau,
+            kern<<<grid, kGateThreads, smem, st>>>(feat, n, r, gamma, kernel_width(d), tau,
                                                   row_entropy, token_entropy, mask, block_len, cta_counts, bpc,
                                                   n_blocks);
     });
