@@ -102,12 +102,8 @@ __device__ __forceinline__ void acc_word_safe(uint32_t w, float mneg, float& S, 
     T = fmaf(fmaxf(t1, -1e30f), e1, T);
 }
 
-// One 16-byte chunk of such words, summed by itself first: where rows share a warp a lane holds up to 64 elements of one
-// row, and would else add them all in one chain. Error against 64 bits, 16384 rows of 256: 5.3e-8 of the norm in one chain,
-// 4.0e-8 this way (4.0e-8 with one row per warp, 8 elements per lane), for one more operation per 8 elements (0 to 3 % of
-// the time). Two chains per lane instead cost as much and, with one ragged row per warp, an occupancy step (38 -> 48 us at
-// 16384 x 4099).
-__device__ __forceinline__ void acc_chunk_safe(const uint4& v, float mneg, float& S, float& T) {
+// (S, T) of one 16-byte chunk of such words.
+__device__ __forceinline__ float2 chunk_sums(const uint4& v, float mneg) {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
     float s[4], t = 0.f;
 #pragma unroll
@@ -119,8 +115,25 @@ __device__ __forceinline__ void acc_chunk_safe(const uint4& v, float mneg, float
         t = q == 0 ? p0 * e0 : fmaf(p0, e0, t);
         t = fmaf(fmaxf(t1, -1e30f), e1, t);
     }
-    S += (s[0] + s[1]) + (s[2] + s[3]);
-    T += t;
+    return make_float2((s[0] + s[1]) + (s[2] + s[3]), t);
+}
+// Sum of f(0) .. f(NCH - 1) as a tree over the bits of the index, the highest first. Chunk l + G j of a row sits with lane l,
+// and the G lanes are added the same way (warp_sum), so a narrow row's sums are one tree over its chunks however many lanes
+// hold it: its entropy does not depend, to the bit, on how many rows the call has (see few_rows). It is also the more exact
+// order: one chain over a lane's 64 elements was off by 5.3e-8 of the norm at 16384 rows of 256, the tree is by 4.0e-8.
+template <int NCH, int J = 0, int STEP = 1, typename F>
+__device__ __forceinline__ float2 chunk_tree(F&& f) {
+    if constexpr (STEP >= NCH) {
+        return f(std::integral_constant<int, J>());
+    } else {
+        float2 a = chunk_tree<NCH, J, 2 * STEP>(f);
+        if constexpr (J + STEP < NCH) {
+            const float2 b = chunk_tree<NCH, J + STEP, 2 * STEP>(f);
+            a.x += b.x;
+            a.y += b.y;
+        }
+        return a;
+    }
 }
 
 // Rows of a width that is no multiple of 8 start at any even address. They are read as the 16-byte chunks that cover
@@ -279,26 +292,37 @@ __device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const Row
     const float mneg = -m * kLog2e;
     float S = 0.f, T = 0.f;
     const int lo = RAGGED && next_edge ? 1 : 0, hi = !has_next ? 0 : RAGGED && next_edge ? next.nch - 1 : next.nch;
-    const uint4* np = next.base + l;
+    auto refill = [&](uint4& w, int c, bool first_chunk) {
+        // by the distance from this row: fewer registers than the next row's own pointer (16384 x 1024 11.3 us, not 12.3)
+        if (!RAGGED && has_next && c < row.nch) w = ld_stream_v4(row.base + (int64_t)step * row.nch + c);
+        // neighbouring rows may differ by a chunk; at an edge the partial chunks follow after the others
+        if (RAGGED) {
+            w = make_uint4(kFill, kFill, kFill, kFill);
+            if (c < hi && (!first_chunk || c >= lo)) w = ld_stream_v4(next.base + c);
+        }
+    };
+    if constexpr (NCH * G <= 128) {
+        const float2 sums = chunk_tree<NCH>([&](auto J) {
+            constexpr int j = decltype(J)::value;
+            const int c = l + G * j;
+            float2 x = make_float2(0.f, 0.f);
+            if (c < row.nch) x = chunk_sums(v[j], mneg);
+            refill(v[j], c, j == 0);
+            return x;
+        });
+        S = sums.x;
+        T = sums.y;
+    } else {
 #pragma unroll
-    for (int j = 0; j < NCH; ++j) {
-        const int c = l + G * j;
-        if (c < row.nch) {
-            if (G < 32) {
-                acc_chunk_safe(v[j], mneg, S, T);
-            } else {
+        for (int j = 0; j < NCH; ++j) {
+            const int c = l + G * j;
+            if (c < row.nch) {
                 acc_word_safe(v[j].x, mneg, S, T);
                 acc_word_safe(v[j].y, mneg, S, T);
                 acc_word_safe(v[j].z, mneg, S, T);
                 acc_word_safe(v[j].w, mneg, S, T);
             }
-            // by the distance from this row: fewer registers than the next row's own pointer (16384 x 1024 11.3 us, not 12.3)
-            if (!RAGGED && has_next) v[j] = ld_stream_v4(row.base + (int64_t)step * row.nch + c);
-        }
-        // neighbouring rows may differ by a chunk; at an edge the partial chunks follow after the others
-        if (RAGGED) {
-            v[j] = make_uint4(kFill, kFill, kFill, kFill);
-            if (c < hi && (j > 0 || c >= lo)) v[j] = ld_stream_v4(np + G * j);
+            refill(v[j], c, j == 0);
         }
     }
     if (RAGGED && has_next && next_edge) {
@@ -327,7 +351,7 @@ template <int NCH, int G, bool RAGGED, typename F>
 __device__ __forceinline__ void for_each_row(const void* __restrict__ feat, int64_t begin, int64_t end, int64_t n,
                                              int32_t width, int warp, int lane, F&& f) {
     uint4 v[NCH];
-    if constexpr (!RAGGED && G == 32) {
+    if constexpr (!RAGGED && NCH * G > 128) {
         const uint4* base = static_cast<const uint4*>(feat);
         if (begin + warp < end) load_whole_row(v, base + (begin + warp) * (int64_t)width, width, lane);
         for (int64_t i = begin + warp; i < end; i += kGateWarps) {
@@ -719,14 +743,24 @@ cudaError_t launch_compact(int grid, cudaStream_t st, const uint8_t* mask, int64
     return cudaLaunchKernelEx(&cfg, compact_kernel, mask, n, block_counts, tpb, idx, count, cta_stats, out3);
 }
 
+// 16-byte pieces that a row of d channels may cover: rows of a width that is no multiple of 8 start anywhere in a piece.
+// Up to kResidentChunks the row is held in registers, above it the long-row kernel runs.
+constexpr int kResidentChunks = 1024;
+int row_chunks(int32_t d) { return d % 8 == 0 ? d / 8 : (d + 14) / 8; }
+// what the kernels of resident rows take as their width
+int32_t kernel_width(int32_t d) { return d % 8 == 0 ? d / 8 : d; }
+
 // The row kernel for rows of up to `chunks` sixteen-byte pieces: f(integral_constant<NCH>, integral_constant<G>). Narrow rows
 // share a warp with 8 pieces per lane (fewer in the narrowest) and at least 4 lanes per row, so that a load still
-// covers whole 32-byte sectors; above 256 pieces a warp has one row and 9 to 32 pieces per lane.
+// covers whole 32-byte sectors; above 128 pieces, and where there are few rows (`alone`), a row has a warp of its own.
 template <typename F>
-void dispatch_row(int chunks, F&& f) {
+void dispatch_row(int chunks, bool alone, F&& f) {
     auto call = [&](auto nch, auto g) { f(nch, g); };
 #define ROW(n, g) call(std::integral_constant<int, n>(), std::integral_constant<int, g>())
-    if (chunks <= 8) ROW(2, 4);
+    if (alone && chunks <= 32) ROW(1, 32);
+    else if (alone && chunks <= 64) ROW(2, 32);
+    else if (alone && chunks <= 128) ROW(4, 32);
+    else if (chunks <= 8) ROW(2, 4);
     else if (chunks <= 16) ROW(4, 4);
     else if (chunks <= 32) ROW(8, 4);
     else if (chunks <= 64) ROW(8, 8);
@@ -740,24 +774,30 @@ void dispatch_row(int chunks, F&& f) {
     else ROW(32, 32);
 #undef ROW
 }
-constexpr int kRowClasses = 12;
-int row_class(int chunks) {
-    const int up_to[kRowClasses - 1] = {8, 16, 32, 64, 96, 128, 256, 384, 512, 640, 768};
+constexpr int kRowClasses = 15;
+int row_class(int chunks, bool alone) {
+    const int up_to[kRowClasses - 4] = {8, 16, 32, 64, 96, 128, 256, 384, 512, 640, 768};
+    if (alone && chunks <= 128) return kRowClasses - 3 + (chunks > 32) + (chunks > 64);
     int c = 0;
-    while (c < kRowClasses - 1 && chunks > up_to[c]) ++c;
+    while (c < kRowClasses - 4 && chunks > up_to[c]) ++c;
     return c;
 }
 
-// 16-byte pieces that a row of d channels may cover: rows of a width that is no multiple of 8 start anywhere in a piece.
-// Up to kResidentChunks the row is held in registers, above it the long-row kernel runs.
-constexpr int kResidentChunks = 1024;
-int row_chunks(int32_t d) { return d % 8 == 0 ? d / 8 : (d + 14) / 8; }
-// what the kernels of resident rows take as their width
-int32_t kernel_width(int32_t d) { return d % 8 == 0 ? d / 8 : d; }
+// Whether n rows of d channels, narrow enough to share warps, get one each: a call of few rows lasts as long as the chain of
+// one row's instructions, which is shorter with 32 lanes on it. Measured, alone / shared, us: 1000 x 256 4.1 / 4.8, 3000 x
+// 256 5.0 / 5.4, 5000 x 256 6.0 / 6.3, 6000 x 256 6.6 / 6.4, 4000 x 1024 6.4 / 6.6, 5000 x 1024 7.4 / 7.5; 2000 x 128
+// 4.3 / 4.5, 3000 x 128 5.0 / 4.8, 2000 x 65 5.0 / 5.4, 4000 x 65 6.4 / 6.1; 1500 x 64 4.3 / 4.4, 4000 x 64 5.3 / 4.8.
+// Up to 64 aligned channels the two are even at the few rows and sharing wins from there on.
+bool few_rows(int32_t d, int64_t n, int n_sm) {
+    const int chunks = row_chunks(d);
+    if (chunks > 128 || (chunks <= 8 && d % 8 == 0)) return false;
+    const bool long_lanes = (chunks > 16 && chunks <= 64) || chunks > 96;      // 8 chunks per lane where warps are shared
+    return n <= (int64_t)n_sm * (long_lanes ? 36 : 14);
+}
 
 // Launches the row kernel for any d.
 void launch_rows(int grid, cudaStream_t st, const void* feat, int64_t n, int32_t d, float tau, uint8_t* mask,
-                 float* entropy, int32_t* counts, double* cta_stats, int64_t tpb) {
+                 float* entropy, int32_t* counts, double* cta_stats, int64_t tpb, bool alone) {
     const int chunks = row_chunks(d);
     if (chunks > kResidentChunks) {
         if (d % 8 == 0)
@@ -766,7 +806,7 @@ void launch_rows(int grid, cudaStream_t st, const void* feat, int64_t n, int32_t
             gate_rows_long_kernel<true><<<grid, kGateThreads, 0, st>>>(feat, n, d, tau, mask, entropy, counts, cta_stats, tpb);
         return;
     }
-    dispatch_row(chunks, [&](auto nch, auto g) {
+    dispatch_row(chunks, alone, [&](auto nch, auto g) {
         constexpr int NCH = decltype(nch)::value, G = decltype(g)::value;
         auto kern = d % 8 == 0 ? gate_rows_kernel<NCH, G, false> : gate_rows_kernel<NCH, G, true>;
         kern<<<grid, kGateThreads, 0, st>>>(feat, n, kernel_width(d), tau, mask, entropy, counts, cta_stats, tpb);
@@ -776,11 +816,11 @@ void launch_rows(int grid, cudaStream_t st, const void* feat, int64_t n, int32_t
 // Resident blocks per SM of the row kernel that serves rows of d channels.
 // One block per resident slot, i.e. a grid of exactly one wave, measured best: with more blocks the later
 // waves start against a full memory system and the kernel grows a tail (32768 x 5120: 74.8 -> 68.6 us).
-int rows_blocks_per_sm(int32_t d) {
+int rows_blocks_per_sm(int32_t d, bool alone) {
     static std::atomic<int> cache[2][kRowClasses + 1] = {};
     const int chunks = row_chunks(d);
     const bool ragged = d % 8 != 0;
-    const int slot = chunks > kResidentChunks ? kRowClasses : row_class(chunks);
+    const int slot = chunks > kResidentChunks ? kRowClasses : row_class(chunks, alone);
     const int known = cache[ragged][slot].load(std::memory_order_relaxed);
     if (known > 0) return known;
     int occ = 0;
@@ -790,7 +830,7 @@ int rows_blocks_per_sm(int32_t d) {
         if (ragged) ask(gate_rows_long_kernel<true>);
         else ask(gate_rows_long_kernel<false>);
     } else {
-        dispatch_row(chunks, [&](auto nch, auto g) {
+        dispatch_row(chunks, alone, [&](auto nch, auto g) {
             constexpr int NCH = decltype(nch)::value, G = decltype(g)::value;
             if (ragged) ask(gate_rows_kernel<NCH, G, true>);
             else ask(gate_rows_kernel<NCH, G, false>);
@@ -842,15 +882,17 @@ int gate_launch(const void* feat, int64_t n, int32_t d, float tau, uint8_t* mask
     const int rc = check_feat(feat, d);
     if (rc != ARDIFF_OK) return rc;
 
-    // contiguous token range per block; one block per resident slot of the GPU, each with >= 1 token per warp
-    int64_t want = (int64_t)n_sm * rows_blocks_per_sm(d);
+    // contiguous token range per block; one block per resident slot of the GPU, each with at least 8 tokens (one per warp;
+    // where warps are shared, one warp's worth: spread thin, few rows start their loads on as many SMs as there are)
+    const bool alone = few_rows(d, n, n_sm);
+    int64_t want = (int64_t)n_sm * rows_blocks_per_sm(d, alone);
     want *= grid_waves(n, d, want);
     if (want > max_blocks) want = max_blocks;
     int64_t tpb = (n + want - 1) / want;
     if (tpb < kGateWarps) tpb = kGateWarps;
     const int grid = (int)((n + tpb - 1) / tpb);
 
-    launch_rows(grid, st, feat, n, d, tau, mask, entropy, block_counts, stats_out3 ? cta_stats : nullptr, tpb);
+    launch_rows(grid, st, feat, n, d, tau, mask, entropy, block_counts, stats_out3 ? cta_stats : nullptr, tpb, alone);
     (void)launch_compact(grid, st, mask, n, block_counts, tpb, idx, count, stats_out3 ? cta_stats : nullptr,
                          stats_out3);
     set_launch_count(2);
@@ -864,12 +906,13 @@ int entropy_rows_launch(const void* feat, int64_t rows, int32_t d, float* entrop
     if (!feat || !entropy) return ARDIFF_ERR_NULL;
     const int rc = check_feat(feat, d);
     if (rc != ARDIFF_OK) return rc;
-    int64_t want = (int64_t)n_sm * rows_blocks_per_sm(d);
+    const bool alone = few_rows(d, rows, n_sm);
+    int64_t want = (int64_t)n_sm * rows_blocks_per_sm(d, alone);
     want *= grid_waves(rows, d, want);
     int64_t tpb = (rows + want - 1) / want;
     if (tpb < kGateWarps) tpb = kGateWarps;
     const int grid = (int)((rows + tpb - 1) / tpb);
-    launch_rows(grid, st, feat, rows, d, 0.f, nullptr, entropy, nullptr, nullptr, tpb);
+    launch_rows(grid, st, feat, rows, d, 0.f, nullptr, entropy, nullptr, nullptr, tpb, alone);
     return cudaGetLastError() == cudaSuccess ? ARDIFF_OK : ARDIFF_ERR_CUDA;
 }
 
@@ -884,18 +927,21 @@ int gate_blocks_fused_launch(const void* feat, int64_t n, int32_t r, int32_t d, 
     if (rc != ARDIFF_OK) return rc;
     const int64_t n_blocks = (n + gamma - 1) / gamma;
     const int64_t rows = n * r;
-    int64_t want = (int64_t)n_sm * rows_blocks_per_sm(d);
-    want *= grid_waves(rows, d, want);
     const int64_t rows_per_block = (int64_t)gamma * r;
+    // with more rows in a draft block than the CTA has warps, shared warps take fewer rounds (8 blocks of 128 rows of 1024
+    // channels: 15.1 us, 16.7 with one row per warp; 64 blocks of 8 rows: 6.2 and 5.8)
+    const bool alone = rows_per_block <= kGateWarps && few_rows(d, rows, n_sm);
+    int64_t want = (int64_t)n_sm * rows_blocks_per_sm(d, alone);
+    want *= grid_waves(rows, d, want);
     int64_t rows_per_round = 0;
-    dispatch_row(row_chunks(d), [&](auto, auto g) { rows_per_round = kGateThreads / decltype(g)::value; });
+    dispatch_row(row_chunks(d), alone, [&](auto, auto g) { rows_per_round = kGateThreads / decltype(g)::value; });
     const DraftPlan plan = plan_draft_blocks(n_blocks, rows_per_block, rows_per_round, want, max_blocks);
     if (plan.grid == 0) return ARDIFF_ERR_UNSUPPORTED;               // too many CTAs for the count scratch
     const int grid = (int)plan.grid;
     const int64_t bpc = plan.blocks_per_cta;
     const size_t smem = (size_t)(bpc * rows_per_block) * sizeof(float);
     cudaError_t e = cudaSuccess;
-    dispatch_row(row_chunks(d), [&](auto nch, auto g) {
+    dispatch_row(row_chunks(d), alone, [&](auto nch, auto g) {
         constexpr int NCH = decltype(nch)::value, G = decltype(g)::value;
         auto kern = d % 8 == 0 ? gate_blocks_kernel<NCH, G, false> : gate_blocks_kernel<NCH, G, true>;
         if (smem > 48 * 1024) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);

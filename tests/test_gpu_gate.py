@@ -146,6 +146,16 @@ def test_rows_that_share_a_warp_lose_no_precision(d):
     assert np.linalg.norm(err) / np.linalg.norm(H) <= 4.6e-8
 
 
+@pytest.mark.parametrize("d", [48, 64, 72, 104, 128, 200, 256, 264, 400, 512, 520, 640, 768, 776, 1000, 1024])
+def test_a_rows_entropy_does_not_depend_on_how_many_rows_there_are(d):
+    """Narrow rows share a warp unless there are few of them; the sums are the same tree either way: the same bits."""
+    rng = np.random.default_rng(d)
+    feat = dev_bf16(synth.f32_to_bf16((rng.standard_normal((9000, d)) * 2).astype(np.float32)))
+    ent = [ardiff.ardiff_entropy_gate(feat[:n], 1.0, want_entropy=True)[3] for n in (7, 1500, 2072, 2073, 5328, 5329, 9000)]
+    for e in ent[:-1]:
+        assert torch.equal(e, ent[-1][: len(e)])
+
+
 @pytest.mark.parametrize("d", [64, 777, 1024, 4099, 8185, 8186, 8200, 9001, 16384, 16391])
 def test_rows_masked_with_the_lowest_value(d):
     """Masks of the type's lowest value, at the start, in the middle, at the end of a row and over most of it: the masked
