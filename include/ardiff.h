@@ -116,7 +116,7 @@ int ardiff_entropy_gate_blocks(const void* feat, int64_t n, int32_t rows_per_tok
 /* Threshold from entropy statistics (the tau equation of "Entropy-Based Early Stopping in Inference
  * Phase"): out3 = { mean(H), std(H), 0.3 * mean - 0.1 * std }, std with divisor n, all in fp64
  * with a fixed summation order (results are reproducible run to run).
- *   entropy dev float [n], n >= 1;  out3 dev double [3]. One cluster of CTAs: meant for calibration, not the hot path. */
+ *   entropy dev float [n], n >= 1;  out3 dev double [3]. One CTA, or one cluster of 8 above 57344 entropies: meant for calibration, not the hot path. */
 int ardiff_tau_calibrate(const float* entropy, int64_t n, double* out3, void* stream);
 
 /* Accepted draft length per block (Algorithm 1, Step 4):

@@ -61,11 +61,13 @@ block_prefix_kernel(const float* __restrict__ row_entropy, int64_t n, int32_t r,
     }
 }
 
-// Mean, standard deviation (divisor n) and tau of n entropies: one cluster of CTAs, fp64, two passes so that the
+// Mean, standard deviation (divisor n) and tau of n entropies: one CTA or a cluster of them, fp64, two passes so that the
 // deviations are taken from the mean, sums in a fixed order (thread-strided partial sums, a tree per CTA, the CTAs of the
 // cluster in rank order through distributed shared memory), no scratch. Bound by what a few SMs load: a million
-// entropies took one CTA 83 us, 8 take 20.
+// entropies take one CTA 87 us, 8 take 18. A cluster costs 3 us to start and to meet in, so few entropies have one CTA, in a
+// kernel without the cluster's barriers: us, one CTA / 8: 8192 4.7 / 7.6, 16384 5.1 / 7.6, 49152 7.6 / 8.3, 65536 9.1 / 8.2.
 constexpr int kTauThreads = 1024;
+constexpr int64_t kTauOneCta = 56 * kTauThreads;
 __device__ __forceinline__ double cluster_sum(double acc, double* s, double* s_part, unsigned size) {
     s[threadIdx.x] = acc;
     __syncthreads();
@@ -105,11 +107,16 @@ __device__ __forceinline__ double tau_partial(const float* __restrict__ H, int64
     if (rest < n) a1 += f(H[rest]);
     return a0 + a1;
 }
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kTauThreads) tau_kernel(const float* __restrict__ H, int64_t n, double* __restrict__ out) {
     __shared__ double s[kTauThreads];
     __shared__ double s_part;
-    cg::cluster_group cl = cg::this_cluster();
-    const unsigned rank = cl.block_rank(), size = cl.num_blocks();
+    unsigned rank = 0, size = 1;
+    if constexpr (CLUSTER) {
+        cg::cluster_group cl = cg::this_cluster();
+        rank = cl.block_rank();
+        size = cl.num_blocks();
+    }
     const double mean =
         cluster_sum(tau_partial(H, n, rank, size, [](float h) { return (double)h; }), s, &s_part, size) / (double)n;
     const double q = cluster_sum(tau_partial(H, n, rank, size, [mean](float h) {
@@ -188,16 +195,19 @@ extern "C" int ardiff_entropy_gate_blocks(const void* feat, int64_t n, int32_t r
 extern "C" int ardiff_tau_calibrate(const float* entropy, int64_t n, double* out3, void* stream) {
     if (!entropy || !out3) return ARDIFF_ERR_NULL;
     if (n < 1) return ARDIFF_ERR_SHAPE;
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cudaLaunchAttribute at[1];
-    // one CTA while a thread has but a few entropies; 8 CTAs is the largest cluster every device takes
-    const unsigned ctas = n <= 8 * kTauThreads ? 1 : 8;
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(ctas); cfg.blockDim = dim3(kTauThreads); cfg.stream = static_cast<cudaStream_t>(stream);
-    cfg.attrs = at; cfg.numAttrs = ctas > 1 ? 1 : 0;
-    (void)cudaLaunchKernelEx(&cfg, tau_kernel, entropy, n, out3);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (n <= kTauOneCta) {
+        tau_kernel<false><<<1, kTauThreads, 0, st>>>(entropy, n, out3);
+    } else {
+        cudaLaunchConfig_t cfg;
+        memset(&cfg, 0, sizeof(cfg));
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;      // 8 CTAs: the largest cluster that every device takes
+        at[0].val.clusterDim.x = 8; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(8); cfg.blockDim = dim3(kTauThreads); cfg.stream = st;
+        cfg.attrs = at; cfg.numAttrs = 1;
+        (void)cudaLaunchKernelEx(&cfg, tau_kernel<true>, entropy, n, out3);
+    }
     ardiff::set_launch_count(1);
     return cudaGetLastError() == cudaSuccess ? ARDIFF_OK : ARDIFF_ERR_CUDA;
 }
