@@ -61,8 +61,9 @@ int ardiff_version(void);
  * aligned 16-byte pieces that cover them. n == 0 is valid (writes *count = 0).
  *
  * Scratch and concurrency. The two kernels of a call hand per-block counts to each other
- * through a small per-device scratch (512 KB) that the library allocates on the first call on
- * each device: make that first call outside any stream capture. Every stream gets a slice of
+ * through a small per-device scratch (3.5 MB) that the library allocates on the first call on
+ * each device, where it also loads the kernels of every feature width and row count: make that
+ * first call, with any shape, outside any stream capture. Every stream gets a slice of
  * its own, so calls on different streams may overlap on the GPU and calls on one stream are
  * ordered anyway. The table holds 31 streams per device; calls on any further stream share one
  * slice and must not overlap each other on the GPU. A call captured into a graph keeps the slice
@@ -147,9 +148,8 @@ int ardiff_accept_prefix(const float* r, const float* ratio, int64_t n, int32_t 
  * one more limit: n <= ARDIFF_GATE_NOALLOC_MAX_TOKENS, else ARDIFF_ERR_SHAPE and nothing is
  * launched (the fixed number of blocks would otherwise each walk an ever longer token range).
  * The first call on each device looks up the array's device address (cudaGetSymbolAddress,
- * with that device current), and the first call for each feature-width class (d / 256 rounded up
- * to 1, 2, 4, 8, 12, 16, 20, 24, 32, or longer rows; multiples of 8 and other widths apart) loads
- * that kernel and queries its occupancy: make those first calls before any stream capture starts.
+ * with that device current) and loads the kernels of every feature width and row count: make that
+ * call, with any shape, before any stream capture starts.
  * All calls on one device share the one array. Every call overwrites the entries it uses
  * before it reads them, so nothing needs clearing between calls and back-to-back calls on one
  * stream are safe; two calls that can run on the GPU at the same time (different streams

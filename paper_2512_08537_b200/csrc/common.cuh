@@ -26,6 +26,9 @@ int compact_launch(const uint8_t* mask, int64_t n, const int32_t* block_counts, 
 // per-block count scratch of the allocating gate calls: a slice private to `st` on the current device
 int gate_scratch_get(cudaStream_t st, int32_t** counts, int* max_blocks, int* sms);
 int write_zero_count(int32_t* count, cudaStream_t st);
+// load the gate's kernels on the current device, ahead of their first use
+void gate_load_kernels();
+void load_prefix_kernel();
 
 // shape of a head (for callers that must match their buffers to it)
 const ardiff_head_desc* head_desc(const ardiff_head* head);

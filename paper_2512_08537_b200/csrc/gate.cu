@@ -694,6 +694,8 @@ struct GateScratch {
 GateScratch g_scratch[kMaxDevices];
 std::mutex g_scratch_mutex;
 
+void load_gate_kernels();
+
 int gate_scratch(cudaStream_t st, int32_t** counts, double** stats, int* sms) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return ARDIFF_ERR_CUDA;
@@ -709,6 +711,7 @@ int gate_scratch(cudaStream_t st, int32_t** counts, double** stats, int* sms) {
             (void)cudaGetLastError();
             return ARDIFF_ERR_NOMEM;
         }
+        load_gate_kernels();
         g.n_sm = n_sm;
         g.base = static_cast<char*>(p);
     }
@@ -845,6 +848,31 @@ int rows_blocks_per_sm(int32_t d, bool alone) {
     return occ;
 }
 
+// Loads every kernel that a gate call may launch on the current device (the runtime loads a kernel when it is first used,
+// and takes device memory for it: 2 MB for all of these). So a device's first gate call is the only one that does so, and
+// any other shape may follow inside a stream capture. (That first call takes 11 to 12 ms with and without this.)
+void load_gate_kernels() {
+    auto load = [](auto kern) {
+        cudaFuncAttributes a;
+        if (cudaFuncGetAttributes(&a, kern) != cudaSuccess) (void)cudaGetLastError();
+    };
+    for (int chunks : {8, 16, 32, 64, 96, 128, 256, 384, 512, 640, 768, kResidentChunks})
+        for (bool alone : {false, true})
+            if (!alone || chunks <= 128)
+                dispatch_row(chunks, alone, [&](auto nch, auto g) {
+                    constexpr int NCH = decltype(nch)::value, G = decltype(g)::value;
+                    load(gate_rows_kernel<NCH, G, false>);
+                    load(gate_rows_kernel<NCH, G, true>);
+                    load(gate_blocks_kernel<NCH, G, false>);
+                    load(gate_blocks_kernel<NCH, G, true>);
+                });
+    load(gate_rows_long_kernel<false>);
+    load(gate_rows_long_kernel<true>);
+    load(compact_kernel);
+    load(write_zero_count_kernel);
+    ardiff::load_prefix_kernel();
+}
+
 // Waves of blocks: one while a block's share of the input stays small (then ramp and tail dominate and a
 // single wave is fastest), up to four once a block would stream more than 4 MB (then finer blocks even out
 // the finish: 2^19 x 5120 is 1 % faster with four waves than with one).
@@ -968,6 +996,8 @@ int gate_scratch_get(cudaStream_t st, int32_t** counts, int* max_blocks, int* sm
     double* stats = nullptr;
     return gate_scratch(st, counts, &stats, sms);
 }
+
+void gate_load_kernels() { load_gate_kernels(); }
 
 int write_zero_count(int32_t* count, cudaStream_t st) {
     write_zero_count_kernel<<<1, 1, 0, st>>>(count);

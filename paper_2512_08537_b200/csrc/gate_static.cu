@@ -48,6 +48,7 @@ int static_scratch(int32_t** ptr, int* sms) {
         int n_sm = 0;
         if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sm < 1)
             return ARDIFF_ERR_CUDA;
+        ardiff::gate_load_kernels();
         g_static_sms[dev] = n_sm;
         g_static_ptr[dev] = static_cast<int32_t*>(p);
     }

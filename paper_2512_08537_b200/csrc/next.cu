@@ -152,6 +152,13 @@ accept_prefix_kernel(const float* __restrict__ r, const float* __restrict__ rati
 
 }  // namespace
 
+namespace ardiff {
+void load_prefix_kernel() {
+    cudaFuncAttributes a;
+    if (cudaFuncGetAttributes(&a, block_prefix_kernel) != cudaSuccess) (void)cudaGetLastError();
+}
+}  // namespace ardiff
+
 extern "C" int ardiff_entropy_gate_blocks(const void* feat, int64_t n, int32_t rows_per_token, int32_t d,
                                           int32_t gamma, float tau, float* row_entropy, float* token_entropy,
                                           uint8_t* mask, int32_t* idx, int32_t* count, int32_t* block_len,
