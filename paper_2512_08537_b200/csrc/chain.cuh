@@ -23,9 +23,6 @@
 // read by every CTA instead of one warp per token (10 K cycles an exchange instead of 5 K).
 #pragma once
 
-constexpr int CHAIN_MAX_TOKENS = 64;
-constexpr int CHAIN_COLS = 16;                 // columns of a layer that one CTA owns
-constexpr int CHAIN_WARPS = 8;                 // consumer warps; one more feeds the weight ring
 constexpr int CHAIN_MAX_NC = 8;                // W / 256
 constexpr int CHAIN_GROUPS = CHAIN_MAX_TOKENS / 32;
 __host__ __device__ constexpr int chain_token_tiles(int nc) { return nc <= 2 ? 8 : 4; }   // of 8, in a pass
@@ -34,8 +31,6 @@ __host__ __device__ constexpr int chain_red_bytes(int nc) {
 }
 constexpr int CHAIN_MAX_SLOTS = 8;
 constexpr uint32_t CHAIN_EMPTY = 0xffffffffu;
-constexpr int CHAIN_HINT_LINE = 128;           // one hint per line and K eighth
-constexpr int CHAIN_HINT_BYTES = CHAIN_WARPS * CHAIN_HINT_LINE;
 
 struct ChainParams {
     int C, W, L, K, n_slots;
@@ -51,32 +46,6 @@ struct ChainParams {
     float ax[KMAX], av[KMAX], an[KMAX];
 };
 
-// Where things are in the exchange buffer of a call with S tokens: u, LayerNorm partials and (mean, 1 / std) per (step,
-// block or final layer), a per (step, block), x per step.
-// u and a are stored as the B fragments their readers load: [K chunk of 32][token tile of 8][lane][16 bytes].
-// The hints come first, zeroed; everything else starts as CHAIN_EMPTY.
-struct ChainLayout {
-    size_t act;                                // bytes of one u or a
-    size_t hints, u, a, st, fin, xb, total;    // byte offsets
-    __host__ __device__ ChainLayout(int S, int K, int L, int W, int C) {
-        const size_t S8 = (size_t)(S + 7) / 8 * 8, layers = (size_t)K * (L + 1);
-        act = S8 * W * 2;
-        hints = 0;
-        u = 2 * layers * CHAIN_HINT_BYTES;
-        a = u + layers * act;
-        st = a + (size_t)K * L * act;
-        fin = st + layers * S8 * (W / 2);
-        xb = fin + layers * S8 * 16;
-        total = xb + (size_t)K * S8 * C * 2;
-    }
-};
-// exchange buffer for calls of S tokens and K steps with S K <= token_steps
-inline size_t chain_xch_bytes(size_t token_steps, int K_max, int L, int W, int C) {
-    const ChainLayout one(8, 1, L, W, C);
-    // tokens are rounded up to 8 in every step
-    return (token_steps / 8 + 1 + (size_t)K_max) * (one.total - one.u) + (size_t)K_max * one.u;
-}
-inline size_t mods_floats_per_token_step(int L, int W) { return (size_t)(3 * L + 2) * W; }
 // modulation values of step k: [block][shift, scale, gate][token][W], then the final layer's [shift, scale][token][W]
 __host__ __device__ __forceinline__ size_t mods_index(int S, int L, int W, int k, int block, int which) {
     return ((size_t)k * (3 * L + 2) + 3 * block + which) * (size_t)S * W;
@@ -405,7 +374,7 @@ struct Chain {
                 shv[g] = *reinterpret_cast<const float2*>(sh + at);
                 scv[g] = *reinterpret_cast<const float2*>(sc + at);
             }
-            // token t is served by warp t / CTAs of CTA t % CTAs: at most 8 tokens a CTA (16 CTAs, 128 tokens)
+            // token t is served by warp t / CTAs of CTA t % CTAs: at most 4 tokens a CTA (16 CTAs, 64 tokens)
             {
                 const int tok = warp * (W / CHAIN_COLS) + cta;
                 if (tok < S)

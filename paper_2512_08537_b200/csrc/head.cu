@@ -44,6 +44,7 @@
 #include <vector>
 
 #include "../../include/ardiff.h"
+#include "chain_plan.h"
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -1390,7 +1391,7 @@ struct ardiff_head {
     int device, n_sm, grid, coop;
     int TGu, slots;
     Program prog[N_PROGRAMS];
-    size_t chain_token_steps;   // survivors x steps that mods and xch hold; 0: no chain for this shape
+    size_t mods_bytes, xch_bytes;   // 0: no chain for this shape
     size_t out_row0;
     int chain_slots;
     float* mods;
@@ -1685,21 +1686,17 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     TRY(dev_alloc(H, &H->x, R * C, true));
     TRY(dev_alloc(H, &H->h, R * W, true));
     TRY(dev_alloc(H, &H->stats, R * 2 * (W / item_cols(N_WIDTHS - 1)), true));
-    // the chain: its buffers hold token_steps survivors x steps (as many as K_max and max_tokens can ask for, up
-    // to 128 MB of modulations)
+    // the chain's buffers
     H->out_row0 = out_row0;
     if (W / 256 <= CHAIN_MAX_NC && W / CHAIN_COLS <= H->grid && d.K_max > 0 && d.max_tokens > 0) {
-        const size_t per = mods_floats_per_token_step(L, W);
-        const size_t most = (size_t)d.K_max * (size_t)(d.max_tokens < CHAIN_MAX_TOKENS ? d.max_tokens : CHAIN_MAX_TOKENS);
-        const size_t fit = ((size_t)128 << 20) / (per * sizeof(float));
-        H->chain_token_steps = most < fit ? most : fit;
         const int tile = CHAIN_COLS * (W * 2 + 64);
         H->chain_slots = (RING_BYTES + EPI_BYTES - chain_smem(0, W)) / tile;
         if (H->chain_slots > CHAIN_MAX_SLOTS) H->chain_slots = CHAIN_MAX_SLOTS;
-        if (H->chain_token_steps > 0) {
-            TRY(dev_alloc(H, &H->mods, H->chain_token_steps * per, false));
-            TRY(dev_alloc(H, &H->xch, chain_xch_bytes(H->chain_token_steps, d.K_max, L, W, C), false));
-        }
+        const size_t mb = chain_mods_bytes(d.K_max, d.max_tokens, L, W), xb = chain_xch_bytes(d.K_max, d.max_tokens, L, W, C);
+        TRY(dev_alloc(H, &H->mods, mb / sizeof(float), false));
+        TRY(dev_alloc(H, &H->xch, xb, false));
+        H->mods_bytes = mb;
+        H->xch_bytes = xb;
     }
     TRY(dev_alloc(H, &H->counters, ((size_t)H->max_tiles + 2) * CTRS, true));
     TRY(dev_alloc(H, &H->status, 2, true));
@@ -1846,8 +1843,7 @@ int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise,
 
     TimeArgs ta;
     for (int k = 0; k < K; ++k) ta.t[k] = t_sched[k];
-    const size_t chain_fit = H->chain_token_steps / (size_t)K;
-    const int chain_count = chain_limit((int)(chain_fit < CHAIN_MAX_TOKENS ? chain_fit : CHAIN_MAX_TOKENS));
+    const int chain_count = chain_limit(chain_survivors(H->mods_bytes, H->xch_bytes, K, H->d.L, W, C));
     PrepArgs A;
     A.Wt1 = H->Wt1; A.bt1 = H->bt1; A.hidden = H->temb_hidden; A.W = W; A.F = H->d.F; A.K = K;
     A.counters = H->counters; A.n_counters = (int)((H->max_tiles + 2) * CTRS); A.abort_flag = H->status + 1;

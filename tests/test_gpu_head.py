@@ -117,7 +117,7 @@ def test_item_width_boundaries(count):
 
 @pytest.mark.parametrize("W", [256, 512, 768, 1024, 1280, 1536, 1792, 2048, 2304])
 def test_few_tokens_at_every_width(W):
-    """Up to 64 survivors the chain of layers runs in its own kernel (one instance per W / 256 up to 8): one token, a
+    """Up to 64 survivors the chain of layers leaves the tile schedule (one instance per W / 256 up to 8): one token, a
     ragged token tile, a second pass, the last count it takes and the first that it does not; the same call twice gives
     the same bits. Tolerance: the agreement bar of this file."""
     wl = synth.workload("cfg1", n=80, W=W, L=2, K=3, C=32 if W % 512 else 64, Dc=192)
@@ -131,6 +131,22 @@ def test_few_tokens_at_every_width(W):
         assert_parity(got, want, idx, f"{count} tokens")
         assert np.all(got[np.setdiff1d(np.arange(wl.n), idx)] == SENTINEL)
         assert np.array_equal(run_head(head, cond_bits, noise, t, idx), got)
+    head.close()
+
+
+def test_few_token_limit_set_by_the_buffers():
+    """64 steps of 12 blocks: the few-token buffers (128 MB of modulations) hold 26 survivors. The last count that they serve
+    and the first that they do not. Tolerance: the agreement bar of this file."""
+    wl = synth.workload("cfg1", n=40, W=512, L=12, K=64)
+    w, cond_bits, noise, t = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
+    order = np.random.default_rng(26).permutation(wl.n).astype(np.int32)
+    rows = order[[0, 7, 25, 26]]
+    want = oracle.head_sample(w, cond_bits, noise, t, rows)
+    head = make_head(wl, w)
+    for count in (26, 27):
+        got = run_head(head, cond_bits, noise, t, order[:count])
+        assert_parity(got, want, rows[:3] if count == 26 else rows, f"{count} tokens")
+        assert np.all(got[np.setdiff1d(np.arange(wl.n), order[:count])] == SENTINEL)
     head.close()
 
 
