@@ -1686,17 +1686,23 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     TRY(dev_alloc(H, &H->x, R * C, true));
     TRY(dev_alloc(H, &H->h, R * W, true));
     TRY(dev_alloc(H, &H->stats, R * 2 * (W / item_cols(N_WIDTHS - 1)), true));
-    // the chain's buffers
+    // the chain's buffers; a device without room for them runs the tile schedule at every count
     H->out_row0 = out_row0;
     if (W / 256 <= CHAIN_MAX_NC && W / CHAIN_COLS <= H->grid && d.K_max > 0 && d.max_tokens > 0) {
         const int tile = CHAIN_COLS * (W * 2 + 64);
         H->chain_slots = (RING_BYTES + EPI_BYTES - chain_smem(0, W)) / tile;
         if (H->chain_slots > CHAIN_MAX_SLOTS) H->chain_slots = CHAIN_MAX_SLOTS;
         const size_t mb = chain_mods_bytes(d.K_max, d.max_tokens, L, W), xb = chain_xch_bytes(d.K_max, d.max_tokens, L, W, C);
-        TRY(dev_alloc(H, &H->mods, mb / sizeof(float), false));
-        TRY(dev_alloc(H, &H->xch, xb, false));
-        H->mods_bytes = mb;
-        H->xch_bytes = xb;
+        if (dev_alloc(H, &H->mods, mb / sizeof(float), false) == ARDIFF_OK) {
+            if (dev_alloc(H, &H->xch, xb, false) == ARDIFF_OK) {
+                H->mods_bytes = mb;
+                H->xch_bytes = xb;
+            } else {
+                H->allocs.pop_back();
+                cudaFree(H->mods);
+                H->mods = nullptr;
+            }
+        }
     }
     TRY(dev_alloc(H, &H->counters, ((size_t)H->max_tiles + 2) * CTRS, true));
     TRY(dev_alloc(H, &H->status, 2, true));

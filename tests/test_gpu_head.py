@@ -150,6 +150,36 @@ def test_few_token_limit_set_by_the_buffers():
     head.close()
 
 
+def test_head_without_room_for_the_few_token_buffers():
+    """The few-token schedule's buffers are an accelerator: a device that has room for the rest of a head, but not for them,
+    still gets the head, and calls of few tokens take the schedule of larger ones. (The memory is held by one ordinary
+    allocation; nothing runs out but the library's own request.)"""
+    dev = require_cuda()
+    wl = synth.workload("cfg1", n=64, W=512, L=12, K=64)
+    w, cond_bits, noise = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl)
+    t = synth.t_sched(2)
+    idx = np.arange(0, wl.n, 5).astype(np.int32)
+    want = oracle.head_sample(w, cond_bits, noise, t, idx)
+    head = make_head(wl, w)                          # (kernels loaded; what a whole head takes)
+    run_head(head, cond_bits, noise, t, idx)
+    with_buffers = torch.cuda.mem_get_info()[0]
+    head.close()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    taken = free - with_buffers
+    assert taken > 250 << 20                         # weights and scratch about 100 MB, the buffers 128 MB and more
+    held = torch.empty(free - taken + (120 << 20), dtype=torch.uint8, device=dev)
+    try:
+        head = make_head(wl, w)
+        got = run_head(head, cond_bits, noise, t, idx)
+        assert_parity(got, want, idx)
+        head.close()
+    finally:
+        del held
+        torch.cuda.empty_cache()
+
+
 def test_few_tokens_with_fresh_noise_and_after_a_stall():
     """The sampler form with step noise on few tokens, before and after a call whose conditioning never completes."""
     dev = require_cuda()
