@@ -856,6 +856,7 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
                     ok = wait_counters(P.counters + (size_t)(it.abs_m - P.slots) * CTRS, EPI_WARPS * (V.C_pro + X.steps * V.C_step),
                                        nullptr, 0, P);
                 ok = __all_sync(0xffffffffu, ok);
+                __syncwarp();            // orders lane 0's acquire before the other lanes' accesses (a vote does not)
                 if (!ok) break;
                 gather_rows(P, it, ew, lane, X.count);
             } else {
@@ -891,6 +892,7 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
                     if (BN < ACC_COLS) {
                         if (lane == 0) ok = wait_counters(P.counters + (size_t)it.abs_m * CTRS, it.needE, nullptr, 0, P);
                         ok = __all_sync(0xffffffffu, ok);
+                        __syncwarp();    // lane 0 alone acquired: a vote orders no memory, the warp barrier does
                         if (!ok) break;
                     }
                     if (!mod_idle) {
