@@ -285,7 +285,7 @@ struct Chain {
     __device__ static __forceinline__ void feed(const ChainParams& P, int cta, uint32_t ring, uint32_t bars, ChainWait& wait) {
         // one thread: the weight tiles in the order they are used
         int slot = 0;
-        uint32_t ph = 0;
+        uint32_t ph = 0, issued = 0, parity = 0;     // slots ever filled, phase of each one's last filling
         auto tile = [&](size_t row0) {
             wait.mbar(bars + 8u * (CHAIN_MAX_SLOTS + slot), ph ^ 1u);
             if (*wait.s_abort) return;
@@ -293,6 +293,8 @@ struct Chain {
             ptx::mbar_arrive_expect_tx(full, CHAIN_COLS * W * 2);
             const bf16* src = P.Wcat + row0 * W;
             for (int r = 0; r < CHAIN_COLS; ++r) ptx::bulk_load(dst + r * ROW_BYTES, src + (size_t)r * W, W * 2, full);
+            issued |= 1u << slot;
+            parity = (parity & ~(1u << slot)) | (ph << slot);
             if (++slot == P.n_slots) { slot = 0; ph ^= 1u; }
         };
         for (int k = 0; k < P.K && !*wait.s_abort; ++k) {
@@ -302,11 +304,10 @@ struct Chain {
             }
             if (cta < P.C / CHAIN_COLS) tile(P.out_row0 + cta * CHAIN_COLS);
         }
-        // copies in flight land before the CTA may leave (bounded; after a normal run all were consumed)
-        if (*wait.s_abort) {
-            const uint64_t t0 = ptx::globaltimer_ns();
-            while (ptx::globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
-        }
+        // Copies in flight land before the CTA may leave, also where the call is aborted after the last tile was sent for
+        // (the consumers then return without waiting for it). Bounded by time; after a normal run all have landed.
+        for (int s = 0; s < P.n_slots; ++s)
+            if (issued & (1u << s)) drain_mbar(bars + 8u * s, (parity >> s) & 1u);
     }
 
     __device__ static __forceinline__ void run(const ChainParams& P, int S, int cta, uint32_t ring, uint32_t bars, float* red,
