@@ -1145,10 +1145,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
     if (count < 0) count = 0;
     const int MT = (count + BM - 1) / BM;
     const int MTu = (MT + 1) / 2;                  // an odd last tile gets an all-padding partner
-    // A lone group may be a tenth larger than the others: 12188 tokens at W = 1024 (48 pairs, groups of 47) take 1796 us as
-    // one group and 1848 us as two of 24, whose phases are too short for the latency of the chain. Much larger ones lose
-    // (56 pairs as one group 2161 us, as two 2090 us): their residual stream no longer fits the set-aside part of L2.
-    const int n_groups = MTu <= P.TGu + P.TGu / 10 ? 1 : (MTu + P.TGu - 1) / P.TGu;
+    // No group is larger than TGu, not even a lone one by a tenth: that takes 2 to 17 % fewer cycles (phases as long as the
+    // latency of the chain needs), but its residual stream no longer fits the set-aside part of L2, and launches back to
+    // back at the power cap take longer: us, two groups / one: W = 1536, 6 blocks, 7950 / 8700 tokens 4511 / 4683, 4791 /
+    // 5006; 12 blocks, 8300 tokens 9056 / 9418; W = 2560, 5110 tokens 3990 / 4161; W = 256, 51900 tokens 852 / 881. Only
+    // W = 1024 (12500 tokens 1946 / 1889) and W = 512 (23900 tokens 1334 / 1297) gain.
+    const int n_groups = (MTu + P.TGu - 1) / P.TGu;
     const int tgu = n_groups > 0 ? (MTu + n_groups - 1) / n_groups : 1;   // balanced group size
     // the narrowest items that the number of token tiles allows (see width_limit)
     const bool chained = count > 0 && count <= P.chain_count;
