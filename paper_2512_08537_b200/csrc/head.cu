@@ -388,16 +388,28 @@ __device__ __forceinline__ void unpack_item(const HeadParams& P, const Packed& p
     }
 }
 
+// What the roles of a CTA share: its place in the grid and the item list of the call. It lies in shared memory and is read
+// where it is needed (volatile), as the clock's start stamps are: held in registers through the launch these two made the
+// full-width epilogues spill (92 bytes stored and 116 loaded instead of 60 and 68; 1 to 3 % of the time at W = 1024).
+struct Place {
+    uint32_t smem_base, bars, tmem_base;
+    int rank, unit_id, n_units;             // token tile of the unit this CTA owns, its unit, all units
+    int count, MTu, tgu;                    // survivors; pairs of token tiles (modulations only: of steps): of the call,
+                                            // of one group
+    int steps;                              // repetitions of the program's step
+    long long total;                        // items of the call
+};
+
 // The items of one CTA, decoded 32 at a time (lane l decodes the l-th of the next 32) and handed
 // out by shuffle. Every lane of the warp calls next() together.
 template <int WI, int PI>
 struct ItemStream {
     Packed mine;
     int n = 0;
-    __device__ __forceinline__ bool next(const HeadParams& P, int MTu, int tgu, int steps, int rank, int unit_id, int n_units,
-                                         long long total, int lane, Item& it) {
+    __device__ __forceinline__ bool next(const HeadParams& P, const volatile Place& X, int rank, int lane, Item& it) {
         if ((n & 31) == 0)
-            mine = decode_packed<WI, PI>(P, MTu, tgu, steps, rank, (long long)unit_id + (long long)(n + lane) * n_units, total);
+            mine = decode_packed<WI, PI>(P, X.MTu, X.tgu, X.steps, rank, (long long)X.unit_id + (long long)(n + lane) * X.n_units,
+                                         X.total);
         Packed cur;
         const int src = n & 31;
         cur.w0 = __shfl_sync(0xffffffffu, mine.w0, src);
@@ -637,19 +649,9 @@ __device__ __forceinline__ void gather_rows(const HeadParams& P, const Item& it,
     }
 }
 
-// What the roles of a CTA share: its place in the grid and the item list of the call.
-struct Place {
-    uint32_t smem_base, bars, tmem_base;
-    int rank, unit_id, n_units;             // token tile of the unit this CTA owns, its unit, all units
-    int count, MTu, tgu;                    // survivors; pairs of token tiles (modulations only: of steps): of the call,
-                                            // of one group
-    int steps;                              // repetitions of the program's step
-    long long total;                        // items of the call
-};
-
 // The three roles of a CTA over the call's items, which are item_cols(WI) columns wide.
 template <int WI, int PI = WI>
-__device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, int warp, int lane) {
+__device__ __forceinline__ void run_roles(const HeadParams& P, const volatile Place& X, int warp, int lane) {
     constexpr int BN = item_cols(WI);
     constexpr int STAGES = Ring<BN>::STAGES, STAGE_BYTES = Ring<BN>::STAGE_BYTES;
     constexpr int SPAN = BN / 2;                                 // accumulator columns of one epilogue warp
@@ -679,7 +681,7 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
         // next item with operands to load (gather items have none)
         auto next_item = [&](Item& dst) {
             bool have;
-            do have = ist.next(P, X.MTu, X.tgu, X.steps, rank, X.unit_id, X.n_units, X.total, lane, dst);
+            do have = ist.next(P, X, rank, lane, dst);
             while (have && (dst.type == OP_GATHER || dst.type == OP_NOP));
             return have;
         };
@@ -790,7 +792,7 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
             ItemStream<WI, PI> ist;
             Item it;
             TRACE_DECL
-            while (ist.next(P, X.MTu, X.tgu, X.steps, rank, X.unit_id, X.n_units, X.total, lane, it)) {
+            while (ist.next(P, X, rank, lane, it)) {
                 if (it.type == OP_GATHER || it.type == OP_NOP) continue;
                 const uint32_t buf = acc_iter & 1u;
                 const uint32_t acc_phase = (acc_iter >> 1) & 1u;
@@ -846,7 +848,7 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
         ItemStream<WI, PI> ist;
         Item it;
         TRACE_DECL
-        while (ist.next(P, X.MTu, X.tgu, X.steps, rank, X.unit_id, X.n_units, X.total, lane, it)) {
+        while (ist.next(P, X, rank, lane, it)) {
             bool fail = false;
             if (it.type == OP_NOP) continue;
             if (it.type == OP_GATHER) {
@@ -1108,7 +1110,7 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const Place& X, i
 
 // The modulations-only list, and the exchange buffer cleared, as a call: inlined beside the other three they made those
 // spill (730 tokens, W = 1024: 443 -> 454 us).
-__device__ __noinline__ void run_modulations(const HeadParams& P, const Place X, int warp, int lane) {
+__device__ __noinline__ void run_modulations(const HeadParams& P, const volatile Place& X, int warp, int lane) {
     const ChainLayout lay(X.count, P.K, P.L, P.W, P.C);
     for (size_t i = (size_t)blockIdx.x * NUM_THREADS + threadIdx.x; i < lay.total / 16; i += (size_t)gridDim.x * NUM_THREADS) {
         const uint32_t v = i * 16 < lay.u ? 0u : CHAIN_EMPTY;
@@ -1127,6 +1129,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t s_chain_bars[2 * CHAIN_MAX_SLOTS];
     __shared__ int s_chain_abort;
+    __shared__ Place s_place;
+    __shared__ volatile long long s_probe[2];       // SM cycles and nanoseconds at the start (CTA 0)
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t smem_base = ptx::smem_u32(smem);
     const uint32_t bars = smem_base + RING_BYTES + EPI_BYTES;
@@ -1172,13 +1176,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
     ptx::tc_fence_before();
     ptx::cluster_sync_all();
     ptx::tc_fence_after();
-    const Place X{smem_base, bars, *tmem_slot, rank, unit_id, n_units, count, pairs, chained ? pairs : tgu, steps,
-                  (long long)MTu * P.prog[program].T_pro + (long long)pairs * steps * P.prog[program].T_step};
-    long long probe_c0 = 0;
-    unsigned long long probe_g0 = 0;
+    if (threadIdx.x == 0)
+        s_place = Place{smem_base, bars, *tmem_slot, rank, unit_id, n_units, count, pairs, chained ? pairs : tgu, steps,
+                        (long long)MTu * P.prog[program].T_pro + (long long)pairs * steps * P.prog[program].T_step};
+    __syncthreads();
+    const volatile Place& X = s_place;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        probe_c0 = clock64();
-        probe_g0 = ptx::globaltimer_ns();
+        s_probe[0] = clock64();
+        s_probe[1] = (long long)ptx::globaltimer_ns();
     }
 
     if (program == 0) run_roles<0>(P, X, warp, lane);
@@ -1226,8 +1231,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
     }
     if (blockIdx.x == 0 && threadIdx.x == 0 && P.clock_probe) {
         // SM cycles and wall time of this launch as seen by CTA 0: their ratio is the clock the SM really ran at
-        P.clock_probe[0] = clock64() - probe_c0;
-        P.clock_probe[1] = (long long)(ptx::globaltimer_ns() - probe_g0);
+        P.clock_probe[0] = clock64() - s_probe[0];
+        P.clock_probe[1] = (long long)ptx::globaltimer_ns() - s_probe[1];
     }
 }
 
