@@ -1149,12 +1149,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
     if (count < 0) count = 0;
     const int MT = (count + BM - 1) / BM;
     const int MTu = (MT + 1) / 2;                  // an odd last tile gets an all-padding partner
-    // No group is larger than TGu, not even a lone one by a tenth: that takes 2 to 17 % fewer cycles (phases as long as the
-    // latency of the chain needs), but its residual stream no longer fits the set-aside part of L2, and launches back to
-    // back at the power cap take longer: us, two groups / one: W = 1536, 6 blocks, 7950 / 8700 tokens 4511 / 4683, 4791 /
-    // 5006; 12 blocks, 8300 tokens 9056 / 9418; W = 2560, 5110 tokens 3990 / 4161; W = 256, 51900 tokens 852 / 881. Only
-    // W = 1024 (12500 tokens 1946 / 1889) and W = 512 (23900 tokens 1334 / 1297) gain.
-    const int n_groups = (MTu + P.TGu - 1) / P.TGu;
+    // At W = 512 to 1024 a lone group may be a tenth larger than the others. One group in place of two takes 2 to 17 % fewer
+    // cycles at every width (phases as long as the latency of the chain needs), but its residual stream no longer fits the
+    // set-aside part of L2, and launches back to back at the power cap gain or lose, us, two groups / one: W = 1024, 12050 /
+    // 12500 / 13000 tokens 1907 / 1875, 1946 / 1889, 2007 / 1979; W = 512, 23900 / 26000 tokens 1334 / 1297, 1433 / 1435;
+    // but W = 256, 50000 / 51900 tokens 829 / 846, 852 / 881; W = 1536, 6 blocks, 7950 / 8700 tokens 4511 / 4683, 4791 /
+    // 5006, 12 blocks, 8300 tokens 9056 / 9418; W = 2048, 6200 tokens 3264 / 3369; W = 2560, 5110 tokens 3990 / 4161.
+    // Much larger ones lose at 1024 too (56 pairs 2090 / 2161).
+    const int lone = P.W >= 512 && P.W <= 1024 ? P.TGu + P.TGu / 10 : P.TGu;
+    const int n_groups = MTu <= lone ? 1 : (MTu + P.TGu - 1) / P.TGu;
     const int tgu = n_groups > 0 ? (MTu + n_groups - 1) / n_groups : 1;   // balanced group size
     // the narrowest items that the number of token tiles allows (see width_limit)
     const bool chained = count > 0 && count <= P.chain_count;

@@ -99,10 +99,11 @@ def test_small_head_ragged_counts(std, count):
     head.close()
 
 
-@pytest.mark.parametrize("count", [512, 513, 3072, 3073])
+@pytest.mark.parametrize("count", [512, 513, 3072, 3073, 23808, 23809, 26112, 26113])
 def test_item_width_boundaries(count):
     """The last token count of each item width and the first of the next one (W = 512 on 148 SMs: 64 output columns
-    per item up to 2 pairs of token tiles, 128 up to 12, then 256). Tolerance: the agreement bar of this file."""
+    per item up to 2 pairs of token tiles, 128 up to 12, then 256), of a group of the usual size (93 pairs), and of a lone
+    group (102). Tolerance: the agreement bar of this file."""
     wl = synth.workload("cfg1", n=count + 5, W=512, L=2, K=2)
     w, cond_bits, noise, t = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
     idx = np.random.default_rng(count).permutation(wl.n)[:count].astype(np.int32)
