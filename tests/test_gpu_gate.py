@@ -104,8 +104,8 @@ def test_shapes_generic_path(d):
 @pytest.mark.parametrize("n,shift", [(1, 0), (2, 1), (3, 7), (9, 5), (67, 3)])
 def test_ragged_rows_at_any_even_address(n, shift, d):
     """Widths that are no multiple of 8: rows covered by 16-byte pieces, matrices that start
-    `shift` elements after a 16-byte boundary, both sides of every register class and of the long-row path. The
-    elements around the matrix are NaN: none may be taken for the row's own."""
+    `shift` elements after a 16-byte boundary, from one channel to the long-row path. The elements around the
+    matrix are NaN: none may be taken for the row's own. (Every row kernel: the test after this one.)"""
     dev = require_cuda()
     rng = np.random.default_rng(1000 * n + d)
     x = rng.standard_normal((n, d)).astype(np.float32) * 2
@@ -132,6 +132,36 @@ def test_ragged_rows_at_any_even_address(n, shift, d):
     sure = nan | (np.abs(H - float(np.float32(tau))) >= BAND)
     assert np.array_equal(mask[sure], (H >= tau).astype(np.uint8)[sure])
     assert np.array_equal(idx.cpu().numpy()[:c], np.flatnonzero(mask).astype(np.int32))
+
+
+# the last width of every row kernel and the first of the next: pieces of 16 bytes up to 8, 16, 32, 64, 96, 128, 256, 384, 512,
+# 640, 768, 1024, then the long-row kernel; a width d that is no multiple of 8 covers up to (d + 14) / 8 of them
+ALIGNED_EDGES = [64, 72, 128, 136, 256, 264, 512, 520, 768, 776, 1024, 1032, 2048, 2056, 3072, 3080, 4096, 4104, 5120, 5128,
+                 6144, 6152, 8192, 8200]
+RAGGED_EDGES = [57, 58, 121, 122, 249, 250, 505, 506, 761, 762, 1017, 1018, 2041, 2042, 3065, 3066, 4089, 4090, 5113, 5114, 6137,
+                6138, 8185, 8186]
+
+
+@pytest.mark.parametrize("n", [300, 5500])
+@pytest.mark.parametrize("d", ALIGNED_EDGES + RAGGED_EDGES)
+def test_every_row_kernel(d, n):
+    """Both sides of every limit between row kernels, few rows (one per warp) and many (narrow ones share a warp). Against
+    fp64: fp32 sums, off by up to 2.5e-6 in one value of thousands; the bar is four times that. The block form runs its own
+    kernel over the same rows."""
+    rng = np.random.default_rng(d)
+    x = (rng.standard_normal((n, d)) * 2).astype(np.float32)
+    x[::5, : d // 3] = -np.inf
+    bits = synth.f32_to_bf16(x)
+    H = oracle.entropy(bits)
+    feat = dev_bf16(bits)
+    tau = quantile_tau(H, 0.4)
+    mask, idx, count, ent = ardiff.ardiff_entropy_gate(feat, tau, want_entropy=True)
+    ent, c = ent.cpu().numpy(), int(count.item())
+    assert np.all(np.abs(ent - H) <= 1e-5)
+    assert np.array_equal(idx.cpu().numpy()[:c], np.flatnonzero(mask.cpu().numpy()).astype(np.int32))
+    for rows, gamma in ((1, 5), (4, 25)):
+        row_ent = ardiff.ardiff_entropy_gate_blocks(feat, rows, gamma, tau)[4]
+        assert np.all(np.abs(row_ent.cpu().numpy() - H) <= 1e-5)
 
 
 @pytest.mark.parametrize("d", [64, 104, 128, 250, 256, 400, 500, 512, 768, 777, 1000, 1024])
