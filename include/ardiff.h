@@ -98,7 +98,7 @@ int ardiff_entropy_gate_stats(const void* feat, int64_t n, int32_t d, float tau,
  *
  *   feat           dev bf16 [n * rows_per_token][d], alignment as for ardiff_entropy_gate
  *   row_entropy    dev float [n * rows_per_token]  out, or NULL. One pass over the features does all of it
- *                  (row entropies stay in shared memory) when d <= 8192 (8178 at widths that are no
+ *                  (row entropies stay in shared memory) when d <= 8192 (8185 at widths that are no
  *                  multiple of 8) and gamma * rows_per_token <= 24576; other shapes go through
  *                  row_entropy as scratch. Those, and widths that are no multiple of 8, return
  *                  ARDIFF_ERR_NULL without it
@@ -245,6 +245,12 @@ int ardiff_head_destroy(ardiff_head* head);
  * runs out the kernel finishes early, the results are invalid and ardiff_head_status reports
  * ARDIFF_ERR_TIMEOUT. Calls on one head must not overlap on the device (they share its
  * scratch): enqueue them on one stream or order them with events.
+ *
+ * The schedule follows *count (1 .. 64 survivors; two ranges of narrow tiles; full-width tiles), and with
+ * it the order in which sums over a row's W channels are formed: the same token may come out different in
+ * the last bf16 roundings in a call with another number of survivors (as a shard of a batch, for
+ * instance). Equal calls give equal bits. (The gate's results do not depend on the other rows, but those
+ * of widths that are no multiple of 8 depend, in the last bits, on the row's address modulo 16.)
  */
 int ardiff_head_sample(const ardiff_head* head, const void* cond, const float* noise,
                        const float* t_sched, int32_t K, const int32_t* idx, const int32_t* count,
