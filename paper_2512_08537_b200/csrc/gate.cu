@@ -139,8 +139,8 @@ __device__ __forceinline__ float2 chunk_tree(F&& f) {
 // Rows of a width that is no multiple of 8 start at any even address. They are read as the 16-byte chunks that cover
 // them: the first chunk starts with `head` elements of the row before, the last one ends with elements of the row
 // after; both are replaced by -inf once the chunk has arrived. 65536 x 777: 57 us (1.8 TB/s) with scalar loads in two
-// passes, 39 us this way, 35 us with the tests for the matrix's edges and for the two partial chunks out of the loop over
-// the chunks (bound by instruction issue).
+// passes, 39 us this way, 34 to 37 us with the tests for the matrix's edges and for the two partial chunks out of the loop
+// over the chunks (bound by instruction issue).
 constexpr uint32_t kFill = 0xff80ff80u;
 struct RowSpan {
     const uint4* base;       // first chunk
@@ -269,7 +269,7 @@ __device__ __forceinline__ void load_whole_row(uint4 (&v)[NCH], const uint4* row
 
 // The same for rows at any even address (RAGGED) and for 32 / G rows to a warp, G lanes each. Where rows share a warp, what
 // a row costs beside its elements (three reductions by shuffle, a logarithm, a division, the loop) is paid once for all of
-// them: one row per warp takes 243 us for 2^20 x 64 and 22 us for 65536 x 256, this 45 and 12. `step` rows lie between a
+// them: one row per warp takes 242 us for 2^20 x 64 and 20 us for 65536 x 256, this 43 and 12. `step` rows lie between a
 // lane's row and its next one.
 template <int NCH, int G, bool RAGGED>
 __device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const RowSpan& row, const RowSpan& next, int step,

@@ -277,8 +277,8 @@ __device__ __forceinline__ Packed decode_packed(const HeadParams& P, int MTu, in
     int r = (int)(item - (long long)grp * per_group);
     const int m0 = grp * tgu;
     const int mtg = min(tgu, MTu - m0);
-    // The modulations-only list has one pair of token tiles; its "token units" are pairs of steps, so that the items of
-    // one weight tile lie side by side in the list and the weights come from HBM once.
+    // The modulations-only list has one pair of token tiles; its "token units" are pairs of steps: the items of one weight
+    // tile lie within a phase (a block's 2 or 3 NT column tiles apart), and the weights come from HBM once.
     const int mtp = PI == MOD_PROGRAM ? 1 : mtg;
     const int pro = mtp * V.T_pro;
     int m, type, nt = 0, k = 0, block = 0, gsel = 0;
