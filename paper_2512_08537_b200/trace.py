@@ -31,7 +31,8 @@ TYPES = ["GATHER", "COND", "IN", "SS", "GATE", "G1", "G2", "FSS", "OUT", "NOP", 
 def build_profile_library() -> str:
     from . import build as lib_build
     srcs = sorted(glob.glob(os.path.join(_HERE, "csrc", "*.cu")))
-    deps = srcs + glob.glob(os.path.join(_HERE, "csrc", "*.cuh")) + [os.path.join(ROOT, "include", "ardiff.h")]
+    deps = srcs + glob.glob(os.path.join(_HERE, "csrc", "*.cuh")) + glob.glob(os.path.join(_HERE, "csrc", "*.h"))
+    deps.append(os.path.join(ROOT, "include", "ardiff.h"))
     if os.path.exists(PROFILE_LIB) and all(os.path.getmtime(p) <= os.path.getmtime(PROFILE_LIB) for p in deps):
         return PROFILE_LIB
     bdir = os.path.join(_HERE, "_build", "profile")
