@@ -20,16 +20,14 @@
 // are placed between the dependent phases of block b, where they cover the latency of the chain.
 // Dependencies between items are tracked per token tile by three counters (chain, gates of even
 // blocks, gates of odd blocks) with release/acquire at gpu scope; every wait is bounded.
-// What binds it: the producer and the MMA issuer each walk a chain of dependent instructions per K slice
-// (poll, vote, descriptors, two copies or four MMAs, commit) that takes most of the 512 cycles a slice lasts,
-// and they share their schedulers with two epilogue warps each (the TMEM lane quarter a warp may read is its
-// id modulo 4, so every scheduler hosts the epilogue of one quarter). Every slot an epilogue warp takes there
-// lengthens the chain, and the epilogue's own loads and stores compete with the copies; the ring drains and
-// the tensor pipe waits. (One elected lane walks the K loop: under `lane == 0` it took 540 cycles a slice even for 64
-// columns, see ptx::elect_one.) Measured on copies of this kernel that skip work, before that change: without any
-// epilogue work a slice is consumed every 545 cycles and the launch takes 21 % fewer cycles (8 points of that are the epilogue's
-// memory operations); with a sixteenth of the operand bytes it takes 4 % fewer. So the kernel keeps the two chains and the
-// epilogue short: biases travel in registers (one column per lane, handed round by shuffle), c never leaves
+// What binds it: at full width the K loop runs at the tensor pipe's own pace (one elected lane walks it, see ptx::elect_one:
+// a 64-wide slice every 493 to 567 cycles in a traced build, 670 to 720 under `lane == 0`), and what is lost is lost between
+// items: the MMA issuer waits for a free accumulator (2.0 K cycles an item at W = 1024, 1.3 K at 1536), because the epilogue
+// of a gated-residual item takes 10.8 K cycles and the MMAs that hide it 8.1 K at W = 1024, and for the first slice of an item
+// whose input is still being published (0.9 K and 1.7 K). The producer and the MMA issuer share their schedulers with two
+// epilogue warps each (the TMEM lane quarter a warp may read is its id modulo 4, so every scheduler hosts the epilogue of one
+// quarter): slots that the epilogue takes there cost most. Operand bytes are not it (a sixteenth of them: 4 % fewer cycles).
+// So the epilogue is kept short: biases travel in registers (one column per lane, handed round by shuffle), c never leaves
 // the accumulator, epilogue inputs are plain loads issued three units ahead, h and the gate values stay off
 // shared memory, and proxy fences sit only where a proxy is really crossed.
 #include <cuda.h>
