@@ -277,8 +277,9 @@ __device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const Row
     if (RAGGED) {
         if (l == 0) v[0] = keep_elements(v[0], row.head, 8);
         const int last = row.nch - 1, keep = row.head + width - 8 * last;
+        // every instance serves rows of more than half of its capacity (dispatch_row): the last chunk is not in the first half
 #pragma unroll
-        for (int j = 0; j < NCH; ++j)
+        for (int j = NCH > 2 ? NCH / 2 - 1 : 0; j < NCH; ++j)
             if (l + G * j == last) v[j] = keep_elements(v[j], 0, keep);
     }
     uint32_t mx = kFill;
