@@ -121,16 +121,19 @@ __device__ __forceinline__ float2 chunk_sums(const uint4& v, float mneg) {
 // and the G lanes are added the same way (warp_sum), so a narrow row's sums are one tree over its chunks however many lanes
 // hold it: its entropy does not depend, to the bit, on how many rows the call has (see few_rows). It is also the more exact
 // order: one chain over a lane's 64 elements was off by 5.3e-8 of the norm at 16384 rows of 256, the tree is by 4.0e-8.
-template <int NCH, int J = 0, int STEP = 1, typename F>
-__device__ __forceinline__ float2 chunk_tree(F&& f) {
+// A part of the tree whose first index is not wanted(j) holds nothing and is left out (272 channels use 34 of 64 chunks).
+template <int NCH, int J = 0, int STEP = 1, typename F, typename W>
+__device__ __forceinline__ float2 chunk_tree(F&& f, W&& wanted) {
     if constexpr (STEP >= NCH) {
         return f(std::integral_constant<int, J>());
     } else {
-        float2 a = chunk_tree<NCH, J, 2 * STEP>(f);
+        float2 a = chunk_tree<NCH, J, 2 * STEP>(f, wanted);
         if constexpr (J + STEP < NCH) {
-            const float2 b = chunk_tree<NCH, J + STEP, 2 * STEP>(f);
-            a.x += b.x;
-            a.y += b.y;
+            if (wanted(J + STEP)) {
+                const float2 b = chunk_tree<NCH, J + STEP, 2 * STEP>(f, wanted);
+                a.x += b.x;
+                a.y += b.y;
+            }
         }
         return a;
     }
@@ -310,7 +313,7 @@ __device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const Row
             if (c < row.nch) x = chunk_sums(v[j], mneg);
             refill(v[j], c, j == 0);
             return x;
-        });
+        }, [&](int j) { return RAGGED || l + G * j < row.nch; });      // (a ragged row's next one may need the chunk)
         S = sums.x;
         T = sums.y;
     } else {
