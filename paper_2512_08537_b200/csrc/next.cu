@@ -11,6 +11,8 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <atomic>
+
 #include "../../include/ardiff.h"
 #include "common.cuh"
 
@@ -61,74 +63,112 @@ block_prefix_kernel(const float* __restrict__ row_entropy, int64_t n, int32_t r,
     }
 }
 
-// Mean, standard deviation (divisor n) and tau of n entropies: one CTA or a cluster of them, fp64, two passes so that the
-// deviations are taken from the mean, sums in a fixed order (thread-strided partial sums, a tree per CTA, the CTAs of the
-// cluster in rank order through distributed shared memory), no scratch. Bound by what a few SMs load: a million
-// entropies take one CTA 87 us, 8 take 18. A cluster costs 3 us to start and to meet in, so few entropies have one CTA, in a
-// kernel without the cluster's barriers: us, one CTA / 8: 8192 4.7 / 7.6, 16384 5.1 / 7.6, 49152 7.6 / 8.3, 65536 9.1 / 8.2.
+// Mean, standard deviation (divisor n) and tau of n entropies: one CTA or a cluster of them, fp64, no scratch. Every CTA
+// takes a contiguous part in two passes (the deviations are taken from the part's own mean), sums in a fixed order
+// (thread-strided partial sums, a tree per CTA); a cluster's parts are merged once, in rank order, through distributed
+// shared memory. Bound by what a few SMs load: a million entropies take one CTA 87 us, 8 18.4 (with
+// two exchanges, one for the mean and one for the deviations), 16 12.0; 65536 8.4 with 8 and 6.9 with 16. A cluster costs
+// 3 us to start and to meet in, so few entropies have one CTA, in a kernel without the cluster's barriers: us, one CTA / 8:
+// 8192 4.7 / 7.6, 16384 5.1 / 7.6, 49152 7.6 / 8.3, 65536 9.1 / 8.2.
 constexpr int kTauThreads = 1024;
 constexpr int64_t kTauOneCta = 56 * kTauThreads;
-__device__ __forceinline__ double cluster_sum(double acc, double* s, double* s_part, unsigned size) {
+__device__ __forceinline__ double cta_sum(double acc, double* s) {
     s[threadIdx.x] = acc;
     __syncthreads();
     for (int o = kTauThreads / 2; o > 0; o >>= 1) {
         if ((int)threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
         __syncthreads();
     }
-    if (size == 1) {
-        const double total = s[0];
-        __syncthreads();
-        return total;
-    }
-    if (threadIdx.x == 0) *s_part = s[0];
-    cg::cluster_group cl = cg::this_cluster();
-    cl.sync();
-    double total = 0.0;
-    for (unsigned r = 0; r < size; ++r) total += *cl.map_shared_rank(s_part, r);
-    cl.sync();                                           // the slot may be reused, or its CTA leave
+    const double total = s[0];
+    __syncthreads();
     return total;
 }
 template <typename F>
-__device__ __forceinline__ double tau_partial(const float* __restrict__ H, int64_t n, unsigned rank, unsigned size, F&& f) {
+__device__ __forceinline__ double tau_partial(const float* __restrict__ H, int64_t n, F&& f) {
     double a0 = 0.0, a1 = 0.0;
-    const int64_t t = (int64_t)rank * kTauThreads + threadIdx.x, stride = (int64_t)size * kTauThreads;
     // the part before the first 16-byte boundary, whole float4s, the rest
     const int64_t lead = min(n, (int64_t)((16 - (reinterpret_cast<uintptr_t>(H) & 15u)) & 15u) / 4);
     const int64_t n4 = (n - lead) / 4;
     const float4* H4 = reinterpret_cast<const float4*>(H + lead);
-    if (t < lead) a0 += f(H[t]);
+    if ((int64_t)threadIdx.x < lead) a0 += f(H[threadIdx.x]);
 #pragma unroll 4
-    for (int64_t i = t; i < n4; i += stride) {
+    for (int64_t i = threadIdx.x; i < n4; i += kTauThreads) {
         const float4 v = H4[i];
         a0 += f(v.x) + f(v.y);
         a1 += f(v.z) + f(v.w);
     }
-    const int64_t rest = lead + 4 * n4 + t;
+    const int64_t rest = lead + 4 * n4 + threadIdx.x;
     if (rest < n) a1 += f(H[rest]);
     return a0 + a1;
 }
+struct TauPart { double n, mean, m2; };
 template <bool CLUSTER>
 __global__ void __launch_bounds__(kTauThreads) tau_kernel(const float* __restrict__ H, int64_t n, double* __restrict__ out) {
     __shared__ double s[kTauThreads];
-    __shared__ double s_part;
+    __shared__ TauPart s_part;
     unsigned rank = 0, size = 1;
+    int64_t begin = 0, own = n;
     if constexpr (CLUSTER) {
         cg::cluster_group cl = cg::this_cluster();
         rank = cl.block_rank();
         size = cl.num_blocks();
+        const int64_t per = (n + size - 1) / size;
+        begin = (int64_t)rank * per;
+        own = min(n, begin + per) - begin;                   // (more entropies than CTAs squared: every part has some)
     }
-    const double mean =
-        cluster_sum(tau_partial(H, n, rank, size, [](float h) { return (double)h; }), s, &s_part, size) / (double)n;
-    const double q = cluster_sum(tau_partial(H, n, rank, size, [mean](float h) {
+    double mean = cta_sum(tau_partial(H + begin, own, [](float h) { return (double)h; }), s) / (double)own;
+    double q = cta_sum(tau_partial(H + begin, own, [mean](float h) {
         const double dlt = (double)h - mean;
         return dlt * dlt;
-    }), s, &s_part, size);
+    }), s);
+    if constexpr (CLUSTER) {
+        cg::cluster_group cl = cg::this_cluster();
+        if (threadIdx.x == 0) s_part = TauPart{(double)own, mean, q};
+        cl.sync();
+        if (rank == 0 && threadIdx.x == 0) {
+            double sum = 0.0;
+            for (unsigned r = 0; r < size; ++r) {
+                const TauPart* p = cl.map_shared_rank(&s_part, r);
+                sum += p->n * p->mean;
+            }
+            mean = sum / (double)n;
+            q = 0.0;
+            for (unsigned r = 0; r < size; ++r) {
+                const TauPart* p = cl.map_shared_rank(&s_part, r);
+                const double d = p->mean - mean;
+                q += p->m2 + p->n * d * d;
+            }
+        }
+        cl.sync();                                           // a CTA leaves when its part has been read
+    }
     if (rank == 0 && threadIdx.x == 0) {
         const double sd = sqrt(q / (double)n);
         out[0] = mean;
         out[1] = sd;
         out[2] = 0.3 * mean - 0.1 * sd;
     }
+}
+
+// CTAs of the cluster on the current device: 16 where it takes such a cluster, else 8, which every device takes.
+int tau_cluster() {
+    static std::atomic<int> known[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 8;
+    int c = known[dev].load(std::memory_order_relaxed);
+    if (c) return c;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 16; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(16); cfg.blockDim = dim3(kTauThreads); cfg.attrs = at; cfg.numAttrs = 1;
+    int fit = 0;
+    c = cudaFuncSetAttribute(tau_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                cudaOccupancyMaxActiveClusters(&fit, tau_kernel<true>, &cfg) == cudaSuccess && fit >= 1
+            ? 16 : 8;
+    if (c == 8) (void)cudaGetLastError();
+    known[dev].store(c, std::memory_order_relaxed);
+    return c;
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -209,9 +249,10 @@ extern "C" int ardiff_tau_calibrate(const float* entropy, int64_t n, double* out
         cudaLaunchConfig_t cfg;
         memset(&cfg, 0, sizeof(cfg));
         cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;      // 8 CTAs: the largest cluster that every device takes
-        at[0].val.clusterDim.x = 8; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3(8); cfg.blockDim = dim3(kTauThreads); cfg.stream = st;
+        const int ctas = tau_cluster();
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(ctas); cfg.blockDim = dim3(kTauThreads); cfg.stream = st;
         cfg.attrs = at; cfg.numAttrs = 1;
         (void)cudaLaunchKernelEx(&cfg, tau_kernel<true>, entropy, n, out3);
     }
