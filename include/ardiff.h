@@ -208,8 +208,8 @@ typedef struct {
 /*
  * Packs the weights into the kernels' tile layout on the current device and allocates
  * the head's scratch (a fixed-size activation workspace for two groups of token tiles,
- * max_tokens/128 progress counters and, for calls of few tokens, up to 128 MB of modulation values
- * and up to 128 MB of exchange buffer: without room for these two such calls take the schedule of
+ * max_tokens/128 progress counters and, for calls of few tokens, up to 256 MB of modulation values
+ * and up to 140 MB of exchange buffers: without room for these such calls take the schedule of
  * larger ones). Synchronous; the only head call that allocates.
  * Side effect on the CUDA context: while at least one head exists on a device, the context's
  * cudaLimitPersistingL2CacheSize is at least the size of one token group's fp32 residual
@@ -239,14 +239,17 @@ int ardiff_head_destroy(ardiff_head* head);
  *                 status word as ARDIFF_ERR_SHAPE)
  *   out      dev  float [n][C]: rows idx[j] are written, all other rows are left untouched
  * One persistent cooperative kernel walks a static schedule of GEMM tiles; tiles wait for
- * their producers on device-side counters with bounded spins. Up to 64 survivors (as many as
- * *count says, for widths up to 2048) the layers that depend on x leave that schedule and run with
- * one exchange of values between SMs per layer; those waits are bounded the same way. If a wait
+ * their producers on device-side counters with bounded spins. For few survivors (as many as
+ * *count says, for widths up to 2048: up to about 200 at the largest, 700 at W = 1024, 4000 at
+ * W = 256) the layers that depend on x leave that schedule: clusters of CTAs take groups of up to
+ * 64 tokens through all steps in a second kernel (up to 32 survivors of widths from 1280 on run
+ * with one exchange of values between SMs per layer); those waits are bounded the same way. If a wait
  * runs out the kernel finishes early, the results are invalid and ardiff_head_status reports
  * ARDIFF_ERR_TIMEOUT. Calls on one head must not overlap on the device (they share its
  * scratch): enqueue them on one stream or order them with events.
  *
- * The schedule follows *count (1 .. 64 survivors; two ranges of narrow tiles; full-width tiles), and with
+ * The schedule follows *count (few survivors; two ranges of narrow tiles; full-width tiles) and, for few
+ * survivors, the number of tokens in a group (and max_tokens up to 64 or above), and with
  * it the order in which sums over a row's W channels are formed: the same token may come out different in
  * the last bf16 roundings in a call with another number of survivors (as a shard of a batch, for
  * instance). Equal calls give equal bits. (The gate's results do not depend on the other rows, but those

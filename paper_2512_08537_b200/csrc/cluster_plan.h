@@ -1,0 +1,88 @@
+// How the cluster schedule (cluster.cuh) lays a head out: arithmetic alone, also for the host.
+#pragma once
+#include <stddef.h>
+#include <stdint.h>
+
+#ifndef ARDIFF_HD
+#ifdef __CUDACC__
+#define ARDIFF_HD __host__ __device__
+#else
+#define ARDIFF_HD
+#endif
+#endif
+
+constexpr int CL_MAX_CTAS = 16;                // CTAs of a cluster
+constexpr int CL_UNIT = 16;                    // tokens: the fewest that one product takes
+constexpr int CL_MAX_UNITS = 4;                // units of 16 tokens in a cluster's group
+constexpr int CL_MAX_STAGES = 6;               // of weights in the ring
+constexpr int CL_MIN_STAGES = 2;
+constexpr int CL_SMEM = 226 * 1024;            // dynamic shared memory, 1 KB of it to align the ring
+constexpr int CL_THREADS = 32 * 11;            // weights, products, eight epilogue warps, activations
+constexpr int CL_KS = 64;                      // K slice: one swizzle row of weights
+// K slices of a stage: 32 KB of weights or a little more (36 at 96 rows), the columns of 4, 2 or 1 CTAs.
+ARDIFF_HD constexpr int cl_slices(int rows) { return rows == 64 ? 4 : rows == 96 ? 3 : 2; }
+
+// Shared memory of one CTA: the weight ring, activations (u and a share a buffer where two do not fit), x as bf16 (operand of
+// the in-projection) and as fp32, LayerNorm partials of all CTAs, those of this CTA's warps.
+struct ClusterLayout {
+    int bufs, stages;
+    uint32_t stage, act, u, a, xb, x, stats, part, total;
+    ARDIFF_HD ClusterLayout(int W, int C, int rows, int units) {
+        const uint32_t N = (uint32_t)units * CL_UNIT, ctas = (uint32_t)(W / rows);
+        stage = (uint32_t)rows * CL_KS * 2 * cl_slices(rows);
+        act = N * (uint32_t)W * 2;
+        const uint32_t rest = N * 128 + N * (uint32_t)C * 4 + N * ctas * 8 + N * 32, room = CL_SMEM - 1024;
+        bufs = 2 * act + rest + 3 * stage <= room ? 2 : 1;
+        const uint32_t used = (uint32_t)bufs * act + rest;
+        int fit = used < room ? (int)((room - used) / stage) : 0;
+        stages = fit < CL_MAX_STAGES ? fit : CL_MAX_STAGES;
+        u = (uint32_t)stages * stage;
+        a = u + (uint32_t)(bufs - 1) * act;
+        xb = a + act;
+        x = xb + N * 128;
+        stats = x + N * (uint32_t)C * 4;
+        part = stats + N * ctas * 8;
+        total = part + N * 32;
+    }
+};
+
+// Heads created for at most so many tokens split a layer over as many CTAs as a cluster may have. us, 64 or 96 columns a CTA /
+// 128: W = 256, 32 tokens 74 / 76, 1024 101 / 95; W = 1024, 64 tokens 168 / 174, 128 207 / 177; W = 1536, 64 745 / 776.
+constexpr int CL_FEW_TOKENS = 64;
+// u (or a) of a cluster's tokens, bytes up to which the CTAs copy it to one another. us, copied / through L2: 8 KB (W = 256, 16
+// tokens) 74 / 97, 32 KB (1024, 16) 168 / 190, 48 KB (1536, 16) 745 / 773, 64 KB (2048, 16) 332 / 330, 96 KB (1024, 48) 359 / 318.
+constexpr uint32_t CL_DIRECT_BYTES = 48 * 1024;
+// Bytes of u and of a on their way between the CTAs of the clusters, through L2.
+inline size_t cluster_xch_bytes(int W, int units, int clusters) {
+    return (size_t)clusters * 2 * units * CL_UNIT * W * 2;
+}
+
+// Output columns that one CTA of a cluster owns of every W-wide layer; 0: no cluster schedule for this width. Heads for few
+// tokens take as many CTAs as there may be in a cluster (each streams fewer weights), others have room for more clusters.
+inline int cluster_rows(int W, int64_t max_tokens) {
+    const int choices[] = {64, 96, 128};
+    for (int rows : choices)
+        if (W % rows == 0 && W / rows <= CL_MAX_CTAS && (rows == 128 || max_tokens <= CL_FEW_TOKENS)) return rows;
+    return 0;
+}
+// Most units of 16 tokens that a cluster takes at once.
+inline int cluster_units(int W, int C, int rows) {
+    int units = CL_MAX_UNITS;
+    while (units > 0 && ClusterLayout(W, C, rows, units).stages < CL_MIN_STAGES) --units;
+    return units;
+}
+
+constexpr size_t CL_MODS_LIMIT = (size_t)256 << 20;      // bytes of the modulation buffer
+// Survivors up to which a modulation buffer of this size serves a call of K steps.
+inline int64_t mods_survivors(size_t bytes, int K, int L, int W) {
+    return (int64_t)(bytes / ((size_t)K * (3 * L + 2) * W * sizeof(float))) / 8 * 8;
+}
+inline size_t mods_bytes(int K_max, int64_t max_tokens, int L, int W) {
+    const size_t per_token = (size_t)K_max * (3 * L + 2) * W * sizeof(float);
+    const size_t tokens = (size_t)(max_tokens + 7) / 8 * 8;
+    return tokens < CL_MODS_LIMIT / per_token ? tokens * per_token : CL_MODS_LIMIT;
+}
+
+// Modulation values of one layer and step: tiles of 32 channels x 8 tokens as the epilogue's lanes hold them (cluster.cuh),
+// 1 KB each, the tokens of 32 channels side by side. Tokens rounded up to whole tiles:
+ARDIFF_HD inline int mods_stride(int S) { return (S + 7) / 8 * 8; }

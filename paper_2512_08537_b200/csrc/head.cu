@@ -5,7 +5,8 @@
 // state z and on t, sampled with K Euler flow steps from caller-supplied noise.
 //
 // How: every matrix product of the head is cut into items of 128 tokens x 256 output columns (128 or 64 when few
-// token tiles leave units idle: see width_limit; up to 64 tokens chain.cuh takes over after the modulations). The two
+// token tiles leave units idle: see width_limit; for few tokens this kernel only makes the modulations of all steps and
+// cluster.cuh, up to 32 tokens of wide heads chain.cuh, takes over: see few_count in head_sample_impl). The two
 // CTAs of a cluster form a unit: each owns one token tile, stages its own A tile (activations) and
 // half of the B tile (weights) per 64-wide K slice by TMA into a 6-stage shared-memory ring, and the
 // even CTA issues tcgen05.mma.cta_group::2 (256 x 256 x 16, bf16 -> fp32) into one of two TMEM
@@ -38,11 +39,13 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 #include <vector>
 
 #include "../../include/ardiff.h"
 #include "chain_plan.h"
+#include "cluster_plan.h"
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -53,7 +56,7 @@ using bf16 = __nv_bfloat16;
 constexpr int BM = 128;           // tokens per tile (one CTA)
 constexpr int BK = 64;            // K slice per pipeline stage (128 bytes of bf16: one swizzle row)
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int N_PROGRAMS = 4;     // item lists: one per item width, and what the chain (chain.cuh) leaves
+constexpr int N_PROGRAMS = 4;     // item lists: one per item width, and what the schedules for few tokens leave
 constexpr int MOD_PROGRAM = 3, MOD_WIDTH = 1;
 constexpr int N_WIDTHS = 3;       // item widths: width w has item_cols(w) output columns per item (UMMA N)
 __host__ __device__ constexpr int item_cols(int w) { return 256 >> w; }
@@ -109,7 +112,8 @@ enum MapId : int {
     MAP_Z = 0, MAP_XB, MAP_S, MAP_U, MAP_A, MAP_WOUT,   // GEMM operands
     EMAP_S, EMAP_U, EMAP_A,                             // epilogue output slabs
     MAP_B,                                              // weights, one set of boxes per item width: + 3 w + W_C ..
-    MAP_COUNT = MAP_B + 3 * N_WIDTHS
+    MAP_CL = MAP_B + 3 * N_WIDTHS,                      // weights for the cluster schedule: packed layers, Win, Wout
+    MAP_COUNT = MAP_CL + 3
 };
 
 // One phase of the per-step program: `ntiles` column tiles (tile0 ..) of one layer for every token
@@ -160,10 +164,11 @@ struct HeadParams {
     long long step_stride;                  // n * C
     float ax[KMAX], av[KMAX], an[KMAX];     // sampler step k: x <- ax x + av v + an z_k
     unsigned long long wait_limit_ns;       // bound of every dependency wait
-    int chain_count;                        // up to this many survivors chain.cuh does what depends on x and h:
+    int few_count, chain_count;             // up to so many survivors cluster.cuh (in a launch of its own), up to so many
+                                            // chain.cuh does what depends on x and h: here only s_k and all modulations
     int grid_counter;                       // index of the grid barrier's counter
-    float* mods;                            // here only s_k and all modulations (into mods), and its exchange buffer
-    uint8_t* xch;                           // is set to "nothing there yet"
+    float* mods;                            // the modulations, and the chain's exchange buffer, set to "nothing there
+    uint8_t* xch;                           // yet"
     int stall_tile;                         // self-test: conditioning items of this token tile wait for one
                                             // predecessor more than exists (-1: none)
     long long* clock_probe;                 // [4]: clock64 and globaltimer of CTA 0 at start and end
@@ -270,14 +275,15 @@ __device__ __forceinline__ Packed decode_packed(const HeadParams& P, int MTu, in
     const Program& V = P.prog[PI];
     Packed pk{(uint32_t)OP_END << 24, 0u, 0u, 0u, 0u};
     if (item >= total) return pk;
+    // The modulations-only list: conditioning items of all token tiles, then the modulations of MTu pairs of (step, token
+    // tile): the items of one weight tile lie within a phase (a block's 2 or 3 NT column tiles apart), and the weights come
+    // from HBM once. (tgu: pairs of token tiles; steps: token tiles)
     const long long per_group = (long long)tgu * (V.T_pro + steps * V.T_step);
-    const int grp = (int)(item / per_group);
+    const int grp = PI == MOD_PROGRAM ? 0 : (int)(item / per_group);
     int r = (int)(item - (long long)grp * per_group);
     const int m0 = grp * tgu;
-    const int mtg = min(tgu, MTu - m0);
-    // The modulations-only list has one pair of token tiles; its "token units" are pairs of steps: the items of one weight
-    // tile lie within a phase (a block's 2 or 3 NT column tiles apart), and the weights come from HBM once.
-    const int mtp = PI == MOD_PROGRAM ? 1 : mtg;
+    const int mtg = PI == MOD_PROGRAM ? MTu : min(tgu, MTu - m0);
+    const int mtp = PI == MOD_PROGRAM ? tgu : mtg;
     const int pro = mtp * V.T_pro;
     int m, type, nt = 0, k = 0, block = 0, gsel = 0;
     int needA = 0, needB = 0, b_row = 0;
@@ -337,11 +343,11 @@ __device__ __forceinline__ Packed decode_packed(const HeadParams& P, int MTu, in
             b_row = p.b_row0 + (nt * (BN / 2) / 128) * 256 + nt * (BN / 2) % 128;
         }
     }
-    if (PI == MOD_PROGRAM) {
-        k = m;
-        m = 0;
+    int abs_m = (m0 + m) * 2 + rank;
+    if (PI == MOD_PROGRAM && type == OP_MOD) {
+        k = abs_m / steps;                      // (an odd number of them: the last pair's second step does not exist)
+        abs_m = k < P.K ? abs_m - k * steps : 0;
     }
-    const int abs_m = (m0 + m) * 2 + rank;
     if (type == OP_COND && abs_m == P.stall_tile) needA += 1;   // self-test: never satisfied
     pk.w0 = (uint32_t)abs_m | ((uint32_t)type << 24);
     pk.w1 = (uint32_t)nt | ((uint32_t)k << 8) | ((uint32_t)(block & 0xff) << 16) | ((uint32_t)gsel << 24);
@@ -376,10 +382,7 @@ __device__ __forceinline__ void unpack_item(const HeadParams& P, const Packed& p
         case OP_G1: it.map_a = MAP_U; break;
         case OP_G2: it.map_a = MAP_A; break;
         case OP_MOD:
-            // the pair takes two steps of the one token tile: rank r of it step 2 k + r
-            it.k = 2 * it.k + it.abs_m;
-            it.abs_m = 0; it.slot_row0 = 0;
-            it.a_row0 = min(it.k, P.K - 1) * P.R;
+            it.a_row0 = min(it.k, P.K - 1) * P.R + it.slot_row0;
             break;
         case OP_OUT: it.map_a = MAP_U; it.map_b = MAP_WOUT; it.umma_n = P.C; it.b_step = P.C / 2; break;
         default: break;
@@ -423,6 +426,7 @@ struct ItemStream {
 };
 
 #include "chain.cuh"
+#include "cluster.cuh"
 
 // ------------------------------------------------------------------------------------------
 // epilogues. Two epilogue warps share each 32-row quarter of the tile (TMEM lane quarter*32 + lane);
@@ -1001,21 +1005,38 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const volatile Pl
                         store_unit_g(gdst, chunk0, u, lane, v);
                     }
                 } else if (PI == MOD_PROGRAM && it.type == OP_MOD) {
-                    // acc + bias of step it.k in fp32, for the chain: tiles of 128 rows, shift and scale in turn,
-                    // then the gates
+                    // acc + bias of step it.k in fp32: items of 128 channels, shift and scale in turn, then the gates
                     const int which = it.nt < 2 * V.NT ? it.nt & 1 : 2;
                     const int ch = (which == 2 ? it.nt - 2 * V.NT : it.nt >> 1) * BN + half * SPAN;
-                    float* dst = P.mods + mods_index(X.count, P.L, P.W, it.k, it.block, which) + (size_t)row * P.W + ch;
-                    const bool live = it.k < P.K && row < X.count;
+                    // (tiles in the layout of cluster.cuh: of two neighbouring tokens one lane stores the channels l .. l + 3
+                    // and l + 8 .. l + 11 of both, the other the rest)
+                    const int tok = it.abs_m * BM + row, ld = mods_stride(X.count);
+                    const bool odd = lane & 1;
+                    float* dst = P.mods + mods_at(P.L, P.W, ld, it.k, it.block, which, ch / 32, tok / 8) + (tok % 8 / 2) * 4 + (odd ? 64 : 0);
+                    // (the chain wants a token's channels side by side)
+                    const bool chained = X.count <= P.chain_count;
+                    float* flat = P.mods + mods_index(X.count, P.L, P.W, it.k, it.block, which) + (size_t)tok * P.W + ch;
+                    const bool live = it.k < P.K && (chained ? tok : tok & ~1) < X.count;
 #pragma unroll
                     for (int u = 0; u < UNITS; ++u) {
                         float v[16];
                         load_acc16(tacc + acc0 + 16 * u, v);
                         add_bias16(v, (u >> 1) == 0 ? bq[0] : (u >> 1) == 1 ? bq[1] : (u >> 1) == 2 ? bq[2] : bq[3], 16 * (u & 1));
-                        if (live) {
+                        if (chained) {
+                            if (live) {
 #pragma unroll
-                            for (int i = 0; i < 16; i += 4)
-                                ptx::st_f4(dst + 16 * u + i, make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]));
+                                for (int i = 0; i < 16; i += 4)
+                                    ptx::st_f4(flat + 16 * u + i, make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]));
+                            }
+                            continue;
+                        }
+                        float* to = dst + (size_t)(u >> 1) * (ld / 8) * 256 + (u & 1) * 128;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float lo = __shfl_xor_sync(0xffffffffu, odd ? v[i] : v[4 + i], 1);
+                            const float hi = __shfl_xor_sync(0xffffffffu, odd ? v[8 + i] : v[12 + i], 1);
+                            const float4 w = odd ? make_float4(lo, v[4 + i], hi, v[12 + i]) : make_float4(v[i], lo, v[8 + i], hi);
+                            if (live) ptx::st_f4(to + i * 16, w);
                         }
                     }
                 } else if (it.type == OP_G1) {
@@ -1110,7 +1131,8 @@ __device__ __forceinline__ void run_roles(const HeadParams& P, const volatile Pl
 // spill (730 tokens, W = 1024: 443 -> 454 us).
 __device__ __noinline__ void run_modulations(const HeadParams& P, const volatile Place& X, int warp, int lane) {
     const ChainLayout lay(X.count, P.K, P.L, P.W, P.C);
-    for (size_t i = (size_t)blockIdx.x * NUM_THREADS + threadIdx.x; i < lay.total / 16; i += (size_t)gridDim.x * NUM_THREADS) {
+    const size_t pieces = X.count <= P.chain_count ? lay.total / 16 : 0;
+    for (size_t i = (size_t)blockIdx.x * NUM_THREADS + threadIdx.x; i < pieces; i += (size_t)gridDim.x * NUM_THREADS) {
         const uint32_t v = i * 16 < lay.u ? 0u : CHAIN_EMPTY;
         ptx::st_u4(P.xch + i * 16, make_uint4(v, v, v, v));
     }
@@ -1129,6 +1151,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
     __shared__ int s_chain_abort;
     __shared__ Place s_place;
     __shared__ volatile long long s_probe[2];       // SM cycles and nanoseconds at the start (CTA 0)
+    ptx::allow_next_kernel();                       // (the clusters', where the call is theirs)
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t smem_base = ptx::smem_u32(smem);
     const uint32_t bars = smem_base + RING_BYTES + EPI_BYTES;
@@ -1158,10 +1181,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
     const int n_groups = MTu <= lone ? 1 : (MTu + P.TGu - 1) / P.TGu;
     const int tgu = n_groups > 0 ? (MTu + n_groups - 1) / n_groups : 1;   // balanced group size
     // the narrowest items that the number of token tiles allows (see width_limit)
-    const bool chained = count > 0 && count <= P.chain_count;
-    const int program = chained ? MOD_PROGRAM : MTu <= P.prog[2].max_units ? 2 : MTu <= P.prog[1].max_units ? 1 : 0;
-    const int pairs = chained ? (P.K + 1) / 2 : MTu;             // of steps, or of token tiles
-    const int steps = chained ? 1 : P.K;
+    const bool few = count > 0 && count <= P.few_count;
+    const int program = few ? MOD_PROGRAM : MTu <= P.prog[2].max_units ? 2 : MTu <= P.prog[1].max_units ? 1 : 0;
+    const int pairs = few ? (P.K * MT + 1) / 2 : MTu;            // of (step, token tile), or of token tiles
 
     if (threadIdx.x == 0) {
         // full[MAX_STAGES], empty[MAX_STAGES], accumulator full[2], accumulator free[2], drain, inputs complete[DEP_BARS]
@@ -1178,8 +1200,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
     ptx::cluster_sync_all();
     ptx::tc_fence_after();
     if (threadIdx.x == 0)
-        s_place = Place{smem_base, bars, *tmem_slot, rank, unit_id, n_units, count, pairs, chained ? pairs : tgu, steps,
-                        (long long)MTu * P.prog[program].T_pro + (long long)pairs * steps * P.prog[program].T_step};
+        s_place = Place{smem_base, bars, *tmem_slot, rank, unit_id, n_units, count, pairs, few ? MTu : tgu, few ? MT : P.K,
+                        (long long)MTu * P.prog[program].T_pro +
+                            (long long)pairs * (few ? 1 : P.K) * P.prog[program].T_step};
     __syncthreads();
     const volatile Place& X = s_place;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1198,29 +1221,31 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) head_kernel(const __grid_const
             ptx::fence_mbar_init();
         }
         run_modulations(P, X, warp, lane);
-        // grid barrier: every CTA's modulations and its share of the cleared exchange buffer are there
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int* arrived = P.counters + P.grid_counter;
-            ptx::red_release_gpu_add(arrived, 1);
-            if (!wait_counters(arrived, (int)gridDim.x, nullptr, 0, P)) s_chain_abort = 1;
-        }
-        __syncthreads();
-        if ((int)blockIdx.x < P.W / CHAIN_COLS && !s_chain_abort) {
-            const uint32_t cb = ptx::smem_u32(s_chain_bars);
-            switch (P.W / 256) {
-                case 1: chain_cta<1>(Q, count, smem, cb, &s_chain_abort); break;
-                case 2: chain_cta<2>(Q, count, smem, cb, &s_chain_abort); break;
-                case 3: chain_cta<3>(Q, count, smem, cb, &s_chain_abort); break;
-                case 4: chain_cta<4>(Q, count, smem, cb, &s_chain_abort); break;
-                case 5: chain_cta<5>(Q, count, smem, cb, &s_chain_abort); break;
-                case 6: chain_cta<6>(Q, count, smem, cb, &s_chain_abort); break;
-                case 7: chain_cta<7>(Q, count, smem, cb, &s_chain_abort); break;
-                case 8: chain_cta<8>(Q, count, smem, cb, &s_chain_abort); break;
-                default: break;
+        if (count <= P.chain_count) {
+            // grid barrier: every CTA's modulations and its share of the cleared exchange buffer are there
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                int* arrived = P.counters + P.grid_counter;
+                ptx::red_release_gpu_add(arrived, 1);
+                if (!wait_counters(arrived, (int)gridDim.x, nullptr, 0, P)) s_chain_abort = 1;
             }
+            __syncthreads();
+            if ((int)blockIdx.x < P.W / CHAIN_COLS && !s_chain_abort) {
+                const uint32_t cb = ptx::smem_u32(s_chain_bars);
+                switch (P.W / 256) {
+                    case 1: chain_cta<1>(Q, count, smem, cb, &s_chain_abort); break;
+                    case 2: chain_cta<2>(Q, count, smem, cb, &s_chain_abort); break;
+                    case 3: chain_cta<3>(Q, count, smem, cb, &s_chain_abort); break;
+                    case 4: chain_cta<4>(Q, count, smem, cb, &s_chain_abort); break;
+                    case 5: chain_cta<5>(Q, count, smem, cb, &s_chain_abort); break;
+                    case 6: chain_cta<6>(Q, count, smem, cb, &s_chain_abort); break;
+                    case 7: chain_cta<7>(Q, count, smem, cb, &s_chain_abort); break;
+                    case 8: chain_cta<8>(Q, count, smem, cb, &s_chain_abort); break;
+                    default: break;
+                }
+            }
+            __syncthreads();
         }
-        __syncthreads();
     }
 
     ptx::tc_fence_before();
@@ -1252,10 +1277,10 @@ struct PrepArgs {
     int* counters;              // zeroed
     int n_counters;
     int* abort_flag;            // zeroed
-    const bf16* cond;           // calls that the chain serves: z = cond[idx[j]]
+    const bf16* cond;           // calls of few tokens: z = cond[idx[j]]
     bf16* z;
     const int *idx, *count;
-    int Dc, max_tokens, chain_count;
+    int Dc, max_tokens, few_count;
 };
 constexpr int PREP_BLOCKS = 148;        // beside the time embedding's
 
@@ -1265,6 +1290,7 @@ constexpr int PREP_BLOCKS = 148;        // beside the time embedding's
 // thousands of tokens there are enough items and the rows are gathered where they are used).
 __global__ void __launch_bounds__(256) prep_kernel(const __grid_constant__ PrepArgs A, TimeArgs ta) {
     extern __shared__ float e_s[];
+    ptx::allow_next_kernel();
     const int W = A.W, F = A.F;
     const int per_step = (W + 7) / 8;
     if ((int)blockIdx.x >= per_step * A.K) {
@@ -1272,7 +1298,7 @@ __global__ void __launch_bounds__(256) prep_kernel(const __grid_constant__ PrepA
         for (int i = t0; i < A.n_counters; i += stride) A.counters[i] = 0;
         if (t0 == 0) *A.abort_flag = 0;
         const int S = min(*A.count, A.max_tokens);
-        if (S > A.chain_count) return;
+        if (S > A.few_count) return;
         const int chunks = A.Dc / 8;
         for (int i = t0; i < S * chunks; i += stride) {
             const int j = i / chunks, c = i - j * chunks;
@@ -1313,6 +1339,7 @@ __global__ void __launch_bounds__(256) temb_out_kernel(const bf16* __restrict__ 
     const int k = blockIdx.y;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int o = blockIdx.x * 8 + warp;
+    ptx::wait_for_prior_kernel();
     if (o >= W) return;
     const bf16* wr = Wt2 + (size_t)o * W;
     const float* hk = hidden + (size_t)k * W;
@@ -1401,11 +1428,13 @@ struct ardiff_head {
     int device, n_sm, grid, coop;
     int TGu, slots;
     Program prog[N_PROGRAMS];
-    size_t mods_bytes, xch_bytes;   // 0: no chain for this shape
+    size_t mods_bytes;              // 0: neither chain nor clusters for this shape
+    size_t chain_bytes;             // of the chain's exchange buffer; 0: no chain
+    int chain_slots, chain_tokens;  // (survivors that it may serve)
     size_t out_row0;
-    int chain_slots;
+    int cl_rows, cl_units, cl_clusters;          // (0 clusters: none)
     float* mods;
-    uint8_t* xch;
+    uint8_t *chain_xch, *cl_xch;
     int64_t max_tiles;
     std::vector<void*> allocs;
     // device
@@ -1468,14 +1497,6 @@ int env_int(const char* name, int dflt) {
 }  // namespace
 
 namespace {
-// survivors up to which the chain is used, of `fit` that its buffers hold
-int chain_limit(int fit) {
-#ifdef ARDIFF_TUNING
-    const int lim = env_int("ARDIFF_HEAD_CHAIN", CHAIN_MAX_TOKENS);
-    if (lim < fit) fit = lim;
-#endif
-    return fit;
-}
 // shared memory of the chain with `slots` weight tiles
 int chain_smem(int slots, int W) {
     return 2 * chain_red_bytes(W / 256) + CHAIN_COLS * XB_COLS * 2 + slots * CHAIN_COLS * (W * 2 + 64);
@@ -1496,6 +1517,58 @@ int width_limit(int wi, int W, int units, int TGu) {
     lim = lim < TGu ? lim : TGu;
     const int run = 3 * units * item_cols(wi) / W;
     return lim < run ? lim : run;
+}
+}  // namespace
+
+namespace {
+// Widths from which the chain stays the schedule of up to 32 survivors beside the clusters: there it spreads the weights of
+// a layer over 80 to 128 SMs, a cluster over 16. us, chain / clusters: W = 1280, 3 blocks, 16 tokens 207 / 210; W = 1536, 12
+// blocks, 8 tokens 640 / 749, 28 726 / 749; W = 2048, 3 blocks, 8 tokens 254 / 333, 28 301 / 332; but 33 and more are two
+// passes of the chain (64 tokens 440 / 333), and at W = 1024 28 tokens take 197 / 168.
+constexpr int CHAIN_BESIDE_CLUSTERS = 1280, CHAIN_BESIDE_TOKENS = 32;
+// The kernel of the cluster schedule for `rows` columns of a layer per CTA.
+typedef void (*ClusterKernel)(const ClusterParams);
+ClusterKernel cluster_kernel_of(int rows) {
+    return rows == 64 ? cluster_kernel<64> : rows == 96 ? cluster_kernel<96> : cluster_kernel<128>;
+}
+void cluster_config(const ardiff_head* H, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at) {
+    const int ctas = H->d.W / H->cl_rows;
+    memset(&cfg, 0, sizeof(cfg));
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    const int64_t groups = (H->d.max_tokens + CL_UNIT - 1) / CL_UNIT;
+    cfg.gridDim = dim3(ctas * (int)std::max((int64_t)1, std::min(groups, (int64_t)H->cl_clusters))); cfg.blockDim = dim3(CL_THREADS);
+    cfg.dynamicSmemBytes = CL_SMEM; cfg.attrs = at; cfg.numAttrs = 1;
+}
+// Chooses the split of a layer over a cluster; false: this width has none, or the device does not take such clusters.
+bool cluster_setup(ardiff_head* H) {
+    H->cl_rows = cluster_rows(H->d.W, H->d.max_tokens);
+#ifdef ARDIFF_TUNING
+    if (H->cl_rows) H->cl_rows = env_int("ARDIFF_HEAD_ROWS", H->cl_rows);
+#endif
+    if (H->cl_rows == 0) return false;
+    H->cl_units = cluster_units(H->d.W, H->d.C, H->cl_rows);
+#ifdef ARDIFF_TUNING
+    H->cl_units = env_int("ARDIFF_HEAD_UNITS", H->cl_units);
+#endif
+    if (H->cl_units < 1) return false;
+    const void* fn = reinterpret_cast<const void*>(cluster_kernel_of(H->cl_rows));
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[1];
+    H->cl_clusters = 0;
+    cluster_config(H, cfg, at);
+    int n = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, CL_SMEM) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess || n < 1) {
+        (void)cudaGetLastError();
+        return false;
+    }
+#ifdef ARDIFF_TUNING
+    n = env_int("ARDIFF_HEAD_CLUSTERS", n);
+#endif
+    H->cl_clusters = n;
+    return true;
 }
 }  // namespace
 
@@ -1663,7 +1736,9 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     }
     {
         std::vector<uint16_t> win((size_t)W * XB_COLS, 0);
-        for (int o = 0; o < W; ++o) memcpy(&win[(size_t)o * XB_COLS], w->Win + (size_t)o * C, (size_t)C * 2);
+        for (int o = 0; o < W; ++o)      // (twice where it fits: see store_x in cluster.cuh; elsewhere x is zero there)
+            for (int c = 0; c < XB_COLS / (int)C && c < 2; ++c)
+                memcpy(&win[(size_t)o * XB_COLS + c * C], w->Win + (size_t)o * C, (size_t)C * 2);
         TRY(dev_alloc(H, &H->Win, win.size(), false));
         TRY(upload(H->Win, win.data(), win.size() * 2));
     }
@@ -1696,22 +1771,26 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     TRY(dev_alloc(H, &H->x, R * C, true));
     TRY(dev_alloc(H, &H->h, R * W, true));
     TRY(dev_alloc(H, &H->stats, R * 2 * (W / item_cols(N_WIDTHS - 1)), true));
-    // the chain's buffers; a device without room for them runs the tile schedule at every count
+    // Buffers of the schedules for few tokens; a device without room for them, or for such clusters, does without.
     H->out_row0 = out_row0;
-    if (W / 256 <= CHAIN_MAX_NC && W / CHAIN_COLS <= H->grid && d.K_max > 0 && d.max_tokens > 0) {
-        const int tile = CHAIN_COLS * (W * 2 + 64);
-        H->chain_slots = (RING_BYTES + EPI_BYTES - chain_smem(0, W)) / tile;
-        if (H->chain_slots > CHAIN_MAX_SLOTS) H->chain_slots = CHAIN_MAX_SLOTS;
-        const size_t mb = chain_mods_bytes(d.K_max, d.max_tokens, L, W), xb = chain_xch_bytes(d.K_max, d.max_tokens, L, W, C);
-        if (dev_alloc(H, &H->mods, mb / sizeof(float), false) == ARDIFF_OK) {
-            if (dev_alloc(H, &H->xch, xb, false) == ARDIFF_OK) {
-                H->mods_bytes = mb;
-                H->xch_bytes = xb;
-            } else {
-                H->allocs.pop_back();
-                cudaFree(H->mods);
-                H->mods = nullptr;
-            }
+    if (d.K_max > 0 && d.max_tokens > 0) {
+        const bool clusters = cluster_setup(H);
+        const int chained = !(W / 256 <= CHAIN_MAX_NC && W / CHAIN_COLS <= H->grid) ? 0
+                            : !clusters ? CHAIN_MAX_TOKENS : W >= CHAIN_BESIDE_CLUSTERS ? CHAIN_BESIDE_TOKENS : 0;
+        const int64_t chain_tokens = d.max_tokens < chained ? d.max_tokens : chained;
+        const size_t mb = clusters ? mods_bytes(d.K_max, d.max_tokens, L, W) : chain_mods_bytes(d.K_max, chain_tokens, L, W);
+        if ((clusters || chained) && dev_alloc(H, &H->mods, mb / sizeof(float), false) == ARDIFF_OK) {
+            H->mods_bytes = mb;
+            if (clusters && dev_alloc(H, &H->cl_xch, cluster_xch_bytes(W, H->cl_units, H->cl_clusters), false) != ARDIFF_OK)
+                H->cl_clusters = 0;
+            const size_t xb = chained ? chain_xch_bytes(d.K_max, chain_tokens, L, W, C) : 0;
+            if (chained && dev_alloc(H, &H->chain_xch, xb, false) == ARDIFF_OK) H->chain_bytes = xb;
+            const int tile = CHAIN_COLS * (W * 2 + 64);
+            H->chain_slots = (RING_BYTES + EPI_BYTES - chain_smem(0, W)) / tile;
+            if (H->chain_slots > CHAIN_MAX_SLOTS) H->chain_slots = CHAIN_MAX_SLOTS;
+            H->chain_tokens = (int)chain_tokens;
+        } else {
+            H->cl_clusters = 0;
         }
     }
     TRY(dev_alloc(H, &H->counters, ((size_t)H->max_tiles + 2) * CTRS, true));
@@ -1799,6 +1878,12 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
             ok &= make_map(&maps[MAP_B + 3 * wi + W_CAT], H->Wcat, cat_rows, W, b_rows);
         }
         ok &= make_map(&maps[MAP_WOUT], H->Wcat, cat_rows, W, (uint32_t)C / 2);
+        memset(&maps[MAP_CL], 0, 3 * sizeof(CUtensorMap));
+        if (H->cl_clusters) {
+            ok &= make_map(&maps[MAP_CL], H->Wcat, cat_rows, W, (uint32_t)H->cl_rows);
+            ok &= make_map(&maps[MAP_CL + 1], H->Win, W, XB_COLS, (uint32_t)H->cl_rows);
+            ok &= make_map(&maps[MAP_CL + 2], H->Wcat, cat_rows, W, (uint32_t)C);
+        }
         ok &= make_slab_map(&maps[EMAP_S], H->s, (uint64_t)kmax * R, W);
         ok &= make_slab_map(&maps[EMAP_U], H->u, R, W);
         ok &= make_slab_map(&maps[EMAP_A], H->a, R, W);
@@ -1859,21 +1944,46 @@ int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise,
 
     TimeArgs ta;
     for (int k = 0; k < K; ++k) ta.t[k] = t_sched[k];
-    const int chain_count = chain_limit(chain_survivors(H->mods_bytes, H->xch_bytes, K, H->d.L, W, C));
+    int chain_count = 0, few_count = 0;
+    if (H->chain_bytes)
+        chain_count = std::min(H->chain_tokens, chain_survivors(H->mods_bytes, H->chain_bytes, K, H->d.L, W, C));
+    // one round of groups: a second one takes as long again, and the tile schedule hardly longer for twice the tokens (W =
+    // 1024, 700 / 1434 tokens: clusters 321 / 565 us, tiles 426 / 475)
+    if (H->cl_clusters) {
+        const int64_t lim = std::min(mods_survivors(H->mods_bytes, K, H->d.L, W), (int64_t)H->slots * BM);
+        few_count = (int)std::min(lim, (int64_t)H->cl_clusters * H->cl_units * CL_UNIT);
+    }
+#ifdef ARDIFF_TUNING
+    few_count = std::min(few_count, env_int("ARDIFF_HEAD_FEW", few_count));
+    chain_count = std::min(chain_count, env_int("ARDIFF_HEAD_CHAIN", chain_count));
+#endif
+    few_count = std::max(few_count, chain_count);
     PrepArgs A;
     A.Wt1 = H->Wt1; A.bt1 = H->bt1; A.hidden = H->temb_hidden; A.W = W; A.F = H->d.F; A.K = K;
     A.counters = H->counters; A.n_counters = (int)((H->max_tiles + 2) * CTRS); A.abort_flag = H->status + 1;
     A.cond = reinterpret_cast<const bf16*>(cond); A.z = H->z; A.idx = idx; A.count = count;
-    A.Dc = H->d.Dc; A.max_tokens = (int)H->d.max_tokens; A.chain_count = chain_count;
+    A.Dc = H->d.Dc; A.max_tokens = (int)H->d.max_tokens; A.few_count = few_count;
     prep_kernel<<<(W + 7) / 8 * K + PREP_BLOCKS, 256, H->d.F * sizeof(float), st>>>(A, ta);
-    temb_out_kernel<<<dim3((W + 7) / 8, K), 256, 0, st>>>(H->Wt2, H->bt2, W, H->temb_hidden, H->temb);
+    cudaLaunchAttribute early[1];
+    early[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early[0].val.programmaticStreamSerializationAllowed = 1;
+    {
+        cudaLaunchConfig_t cfg;
+        memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3((W + 7) / 8, K); cfg.blockDim = dim3(256); cfg.stream = st; cfg.attrs = early; cfg.numAttrs = 1;
+        if (cudaLaunchKernelEx(&cfg, temb_out_kernel, (const bf16*)H->Wt2, (const float*)H->bt2, W, (const float*)H->temb_hidden,
+                               H->temb) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return ARDIFF_ERR_CUDA;
+        }
+    }
     launches += 2;
     HeadParams P;
     memset(&P, 0, sizeof(P));
     P.C = C; P.Dc = H->d.Dc; P.W = W; P.L = H->d.L; P.K = K; P.TGu = H->TGu; P.slots = H->slots;
     for (int pi = 0; pi < N_PROGRAMS; ++pi) P.prog[pi] = H->prog[pi];
-    P.chain_count = chain_count;
-    P.mods = H->mods; P.xch = H->xch;
+    P.few_count = few_count; P.chain_count = chain_count;
+    P.mods = H->mods; P.xch = H->chain_xch;
     P.grid_counter = (int)((H->max_tiles + 1) * CTRS);
     P.R = H->slots * BM;
     P.max_tokens = (int)H->d.max_tokens;
@@ -1903,7 +2013,7 @@ int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise,
     Q.C = C; Q.W = W; Q.L = H->d.L; Q.K = K; Q.n_slots = H->chain_slots; Q.out_row0 = H->out_row0;
     Q.idx = idx; Q.Wcat = H->Wcat; Q.Win = H->Win; Q.bias_cat = H->bias_cat; Q.bin = H->bin;
     Q.noise = noise; Q.step_noise = step_noise; Q.step_stride = P.step_stride; Q.mods = H->mods; Q.out = out;
-    Q.xch = H->xch; Q.status = H->status; Q.abort_flag = P.abort_flag; Q.wait_limit_ns = P.wait_limit_ns;
+    Q.xch = H->chain_xch; Q.status = H->status; Q.abort_flag = P.abort_flag; Q.wait_limit_ns = P.wait_limit_ns;
     memcpy(Q.ax, P.ax, sizeof(Q.ax)); memcpy(Q.av, P.av, sizeof(Q.av)); memcpy(Q.an, P.an, sizeof(Q.an));
 
     if (H->timing) cudaEventRecord(H->ev0, st);
@@ -1929,6 +2039,32 @@ int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise,
         }
     }
     launches += 1;
+    if (few_count > chain_count && H->d.max_tokens > chain_count) {
+        ClusterParams R;
+        memset(&R, 0, sizeof(R));
+        R.C = C; R.W = W; R.L = H->d.L; R.K = K; R.n_ctas = W / H->cl_rows; R.max_units = H->cl_units;
+        R.above = chain_count; R.limit = few_count;
+        R.max_tokens = P.max_tokens; R.map_cat = MAP_CL; R.map_in = MAP_CL + 1; R.map_out = MAP_CL + 2;
+        R.out_row0 = H->out_row0; R.maps = H->maps; R.idx = idx; R.count = count; R.bias_cat = H->bias_cat; R.bin = H->bin;
+        R.noise = noise; R.step_noise = step_noise; R.mods = H->mods; R.step_stride = P.step_stride; R.out = out;
+        R.xch = H->cl_xch; R.direct_bytes = CL_DIRECT_BYTES;
+#ifdef ARDIFF_TUNING
+        R.direct_bytes = (uint32_t)env_int("ARDIFF_HEAD_DIRECT", CL_DIRECT_BYTES);
+#endif
+        R.status = H->status; R.abort_flag = P.abort_flag; R.wait_limit_ns = P.wait_limit_ns;
+        memcpy(R.ax, P.ax, sizeof(R.ax)); memcpy(R.av, P.av, sizeof(R.av)); memcpy(R.an, P.an, sizeof(R.an));
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at[2];
+        cluster_config(H, cfg, at);
+        at[1] = early[0];
+        cfg.numAttrs = 2;
+        cfg.stream = st;
+        if (cudaLaunchKernelEx(&cfg, cluster_kernel_of(H->cl_rows), R) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return ARDIFF_ERR_CUDA;
+        }
+        launches += 1;
+    }
     if (H->timing) {
         cudaEventRecord(H->ev1, st);
         H->timed = 1;

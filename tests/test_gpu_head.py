@@ -135,6 +135,41 @@ def test_few_tokens_at_every_width(W):
     head.close()
 
 
+@pytest.mark.parametrize("W,counts", [(256, (80, 81, 2112, 4224, 4225, 4737)), (512, (129, 1600, 2112, 2113)),
+                                      (768, (100, 337, 1300)), (1024, (240, 241, 481, 720, 721)),
+                                      (1280, (32, 33, 177, 353, 529)), (1536, (32, 33, 112, 113, 224, 225)),
+                                      (1792, (33, 112, 225)), (2048, (32, 33, 112, 113, 224, 225))])
+def test_token_groups_of_the_clusters(W, counts):
+    """Clusters of W / 128 CTAs take groups of 16, 32, 48 or 64 tokens: counts on both sides of where the group grows, where the
+    values go through L2 instead of directly, and of the last that fits (on 148 SMs); a ragged last group; fresh noise; the
+    same call twice gives the same bits. Tolerance: the agreement bar of this file."""
+    dev = require_cuda()
+    wl = synth.workload("cfg1", n=max(counts) + 3, W=W, L=2, K=2, C=48 if W % 512 else 16, Dc=128)
+    w, cond_bits, noise = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl)
+    t_in = np.array([0.9, 0.4], np.float32)
+    coef = np.array([[0.4, 0.7, 0.5], [0.2, 1.0, 0.1]], np.float32)
+    z = np.random.default_rng(9).standard_normal((2, wl.n, wl.C)).astype(np.float32)
+    order = np.random.default_rng(W).permutation(wl.n).astype(np.int32)
+    pos = np.unique(np.concatenate([[0, 15, 16, 31, 47, 63], np.array(counts) - 1, np.random.default_rng(1).integers(0, max(counts), 24)]))
+    want = np.zeros((wl.n, wl.C))
+    want[order[pos]] = oracle.head_sample_coef(w, cond_bits, noise, t_in, coef, order[pos], step_noise=z)[order[pos]]
+    head = make_head(wl, w)
+    cond, noise_d, z_d = dev_bf16(cond_bits), dev_f32(noise), torch.from_numpy(z).to(dev)
+    for count in counts:
+        outs = []
+        for _ in range(2):
+            out = torch.full(noise.shape, SENTINEL, dtype=torch.float32, device=dev)
+            head.ardiff_head_sample_coef(cond, noise_d, t_in, coef, torch.from_numpy(order[:count].copy()).to(dev),
+                                         torch.tensor([count], dtype=torch.int32, device=dev), out, step_noise=z_d)
+            assert head.status() == 0
+            outs.append(out.cpu().numpy())
+        rows = order[pos[pos < count]]
+        assert_parity(outs[0], want, rows, f"{count} tokens")
+        assert np.array_equal(outs[0], outs[1])
+        assert np.all(outs[0][order[count:]] == SENTINEL) and not np.any(outs[0][order[:count]] == SENTINEL)
+    head.close()
+
+
 def test_few_token_limit_set_by_the_buffers():
     """64 steps of 12 blocks: the few-token buffers (128 MB of modulations) hold 26 survivors. The last count that they serve
     and the first that they do not. Tolerance: the agreement bar of this file."""
