@@ -242,7 +242,7 @@ int ardiff_head_destroy(ardiff_head* head);
  * their producers on device-side counters with bounded spins. For few survivors (as many as
  * *count says, for widths up to 2048: up to about 200 at the largest, 700 at W = 1024, 4000 at
  * W = 256) the layers that depend on x leave that schedule: clusters of CTAs take groups of up to
- * 64 tokens through all steps in a second kernel (up to 32 survivors of widths from 1280 on run
+ * 64 tokens through all steps in a second kernel (up to 32 survivors of widths from 1024 on run
  * with one exchange of values between SMs per layer); those waits are bounded the same way. If a wait
  * runs out the kernel finishes early, the results are invalid and ardiff_head_status reports
  * ARDIFF_ERR_TIMEOUT. Calls on one head must not overlap on the device (they share its

@@ -1,5 +1,5 @@
 // The head's chain of dependent layers for calls of few tokens (at most CHAIN_MAX_TOKENS survivors; beside the clusters of
-// cluster.cuh at most 32, and at the widths where it is the faster one: CHAIN_BESIDE_CLUSTERS).
+// cluster.cuh at most 32, and where it is the faster one: chain_beside_clusters).
 //
 // With few tokens the head is K * (3 L + 3) exchanges between SMs in a row, and a call takes as long as they do: the tile
 // schedule spends 5 to 12 us on each (TMA round trip, K loop, epilogue, store completion, release, poll). There it

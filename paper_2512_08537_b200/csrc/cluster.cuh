@@ -17,7 +17,7 @@
 // tokens 125 / 72, 256 177 / 76, 4096 212 / 180; W = 512, 3 blocks, 64 232 / 115, 2048 346 / 289; W = 1024, 3 blocks, 28
 // 197 / 168, 128 358 / 178, 700 426 / 321, but two rounds of groups, 1434 475 / 565: hence one round at most. W = 1280 16
 // 201 / 210, 64 336 / 216; W = 1536, 12 blocks, 28 728 / 749, 64 1094 / 745, 220 1675 / 972; W = 2048, 28 303 / 330, 64 434 /
-// 331, 200 604 / 460: hence chain.cuh up to 32 tokens from W = 1280 on.
+// 331, 200 604 / 460: hence chain.cuh for the fewest tokens of wide heads.
 #pragma once
 
 struct ClusterParams {
@@ -78,9 +78,6 @@ struct ClusterWait {
         }
     }
 };
-
-// SiLU with an exponential and a division: here these are few, and silu_f's tanh is a quarter of the error of the bf16 result.
-__device__ __forceinline__ float cluster_silu(float a) { return __fdividef(a, 1.0f + __expf(-a)); }
 
 template <int ROWS, int G>
 struct ClusterEpilogue {
@@ -389,7 +386,7 @@ struct ClusterEpilogue {
 #pragma unroll
                             for (int i = 0; i < 2; ++i)
 #pragma unroll
-                                for (int e = 0; e < 4; ++e) a[g][i][e] = cluster_silu(a[g][i][e] + b1[i][e >> 1]);
+                                for (int e = 0; e < 4; ++e) a[g][i][e] = silu_f(a[g][i][e] + b1[i][e >> 1]);
                         publish(lay.a, B.src_a, &B.sig[1], xch + lay.act, a);
                     }
                     {   // h += gate * (W2 a + b2)

@@ -1521,11 +1521,14 @@ int width_limit(int wi, int W, int units, int TGu) {
 }  // namespace
 
 namespace {
-// Widths from which the chain stays the schedule of up to 32 survivors beside the clusters: there it spreads the weights of
-// a layer over 80 to 128 SMs, a cluster over 16. us, chain / clusters: W = 1280, 3 blocks, 16 tokens 207 / 210; W = 1536, 12
-// blocks, 8 tokens 640 / 749, 28 726 / 749; W = 2048, 3 blocks, 8 tokens 254 / 333, 28 301 / 332; but 33 and more are two
-// passes of the chain (64 tokens 440 / 333), and at W = 1024 28 tokens take 197 / 168.
-constexpr int CHAIN_BESIDE_CLUSTERS = 1280, CHAIN_BESIDE_TOKENS = 32;
+// Survivors up to which the chain stays the schedule beside the clusters: it spreads the weights of a layer over 64 to 128
+// SMs, a cluster over 16, and is one launch, but takes longer for each step and a second pass above 32 tokens. us, chain /
+// clusters: W = 1024, 3 blocks, K = 1, 1 token 69 / 78, 24 73 / 78, 32 82 / 78, K = 4, 4 167 / 168, 8 181 / 168; W = 1280, K = 1, 32
+// 87 / 88, K = 4, 16 210 / 217, 24 225 / 217; W = 1536, 12 blocks, K = 4, 8 640 / 749, 28 726 / 749; W = 2048, K = 4, 4 238 / 337,
+// 32 313 / 338. Below, one token at W = 768 and K = 1 takes 62 / 65, all else less with clusters.
+int chain_beside_clusters(int W, int K) {
+    return W >= 1536 ? 32 : W >= 1280 ? (K == 1 ? 32 : 16) : W >= 1024 ? (K == 1 ? 24 : 4) : 0;
+}
 // The kernel of the cluster schedule for `rows` columns of a layer per CTA.
 typedef void (*ClusterKernel)(const ClusterParams);
 ClusterKernel cluster_kernel_of(int rows) {
@@ -1776,9 +1779,10 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     if (d.K_max > 0 && d.max_tokens > 0) {
         const bool clusters = cluster_setup(H);
         const int chained = !(W / 256 <= CHAIN_MAX_NC && W / CHAIN_COLS <= H->grid) ? 0
-                            : !clusters ? CHAIN_MAX_TOKENS : W >= CHAIN_BESIDE_CLUSTERS ? CHAIN_BESIDE_TOKENS : 0;
+                            : !clusters ? CHAIN_MAX_TOKENS : chain_beside_clusters(W, 1);
         const int64_t chain_tokens = d.max_tokens < chained ? d.max_tokens : chained;
-        const size_t mb = clusters ? mods_bytes(d.K_max, d.max_tokens, L, W) : chain_mods_bytes(d.K_max, chain_tokens, L, W);
+        const int64_t round = std::min((int64_t)d.max_tokens, (int64_t)H->cl_clusters * H->cl_units * CL_UNIT);
+        const size_t mb = clusters ? mods_bytes(d.K_max, round, L, W) : chain_mods_bytes(d.K_max, chain_tokens, L, W);
         if ((clusters || chained) && dev_alloc(H, &H->mods, mb / sizeof(float), false) == ARDIFF_OK) {
             H->mods_bytes = mb;
             if (clusters && dev_alloc(H, &H->cl_xch, cluster_xch_bytes(W, H->cl_units, H->cl_clusters), false) != ARDIFF_OK)
@@ -1946,8 +1950,9 @@ int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise,
     for (int k = 0; k < K; ++k) ta.t[k] = t_sched[k];
     int chain_count = 0, few_count = 0;
     if (H->chain_bytes)
-        chain_count = std::min(H->chain_tokens, chain_survivors(H->mods_bytes, H->chain_bytes, K, H->d.L, W, C));
-    // one round of groups: a second one takes as long again, and the tile schedule hardly longer for twice the tokens (W =
+        chain_count = std::min(H->cl_clusters ? std::min(H->chain_tokens, chain_beside_clusters(W, K)) : H->chain_tokens,
+                               chain_survivors(H->mods_bytes, H->chain_bytes, K, H->d.L, W, C));
+    // one round of groups (of which the buffer has the size): a second one takes as long again, and the tile schedule hardly longer for twice the tokens (W =
     // 1024, 700 / 1434 tokens: clusters 321 / 565 us, tiles 426 / 475)
     if (H->cl_clusters) {
         const int64_t lim = std::min(mods_survivors(H->mods_bytes, K, H->d.L, W), (int64_t)H->slots * BM);
