@@ -6,6 +6,7 @@ cannot be loaded, or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 from typing import Dict, Optional
@@ -13,6 +14,7 @@ from typing import Dict, Optional
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libardiff.so")
 _lib = None
+_STAY = contextlib.nullcontext()
 
 ARDIFF_OK = 0
 ARDIFF_ERR_NULL, ARDIFF_ERR_SHAPE, ARDIFF_ERR_ALIGN, ARDIFF_ERR_UNSUPPORTED = -1, -2, -3, -4
@@ -74,6 +76,32 @@ def lib() -> ctypes.CDLL:
         L.ardiff_pipeline_destroy.argtypes = [vp]
         L.ardiff_pipeline_run_host.restype = ctypes.c_int
         L.ardiff_pipeline_run_host.argtypes = [vp, vp, vp, vp, i64, f32, vp, i32, vp, vp, vp, vp]
+        L.ardiff_entropy_gate_noalloc.restype = ctypes.c_int
+        L.ardiff_entropy_gate_noalloc.argtypes = [vp, i64, i32, f32, vp, vp, vp, vp]
+        L.ardiff_entropy_gate_stats.restype = ctypes.c_int
+        L.ardiff_entropy_gate_stats.argtypes = [vp, i64, i32, f32, vp, vp, vp, vp, vp, vp]
+        L.ardiff_entropy_gate_blocks.restype = ctypes.c_int
+        L.ardiff_entropy_gate_blocks.argtypes = [vp, i64, i32, i32, i32, f32, vp, vp, vp, vp, vp, vp, vp]
+        L.ardiff_tau_calibrate.restype = ctypes.c_int
+        L.ardiff_tau_calibrate.argtypes = [vp, i64, vp, vp]
+        L.ardiff_accept_prefix.restype = ctypes.c_int
+        L.ardiff_accept_prefix.argtypes = [vp, vp, i64, i32, vp, vp, vp]
+        L.ardiff_head_sample_coef.restype = ctypes.c_int
+        L.ardiff_head_sample_coef.argtypes = [vp, vp, vp, vp, i32, vp, vp, i64, vp, vp, vp, vp]
+        L.ardiff_head_last_kernel_clock.restype = ctypes.c_int
+        L.ardiff_head_last_kernel_clock.argtypes = [vp, vp, ctypes.POINTER(ctypes.c_double)]
+        L.ardiff_head_set_cooperative.restype = ctypes.c_int
+        L.ardiff_head_set_cooperative.argtypes = [vp, ctypes.c_int]
+        L.ardiff_head_inject_stall.restype = ctypes.c_int
+        L.ardiff_head_inject_stall.argtypes = [vp, i32, ctypes.c_uint32]
+        L.ardiff_pipeline_create_slots.restype = ctypes.c_int
+        L.ardiff_pipeline_create_slots.argtypes = [vp, i64, i32, i32, i32, i32, ctypes.POINTER(vp)]
+        L.ardiff_pipeline_submit.restype = ctypes.c_int
+        L.ardiff_pipeline_submit.argtypes = [vp, i32, vp, vp, vp, i64, f32, vp, i32, vp, vp, vp, vp]
+        L.ardiff_pipeline_wait.restype = ctypes.c_int
+        L.ardiff_pipeline_wait.argtypes = [vp, i32]
+        L.ardiff_pipeline_join.restype = ctypes.c_int
+        L.ardiff_pipeline_join.argtypes = [vp, vp]
         _lib = L
     return _lib
 
@@ -96,10 +124,17 @@ def _check(rc: int, where: str):
 
 
 def _stream_ptr(stream) -> int:
+    """The stream's handle; without one that of the current stream (asked for as a number: a Stream object takes 2 us)."""
     import torch
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return int(stream.cuda_stream)
+
+
+def _on(device):
+    """with _on(device): calls go to `device`. Nothing to enter and leave where it is current already, as it mostly is."""
+    import torch
+    return _STAY if torch.cuda.current_device() == device.index else torch.cuda.device(device)
 
 
 def ardiff_entropy_gate(feat, tau: float, mask=None, idx=None, count=None, entropy=None,
@@ -121,7 +156,7 @@ def ardiff_entropy_gate(feat, tau: float, mask=None, idx=None, count=None, entro
         count = torch.empty((1,), dtype=torch.int32, device=dev)
     if entropy is None and want_entropy:
         entropy = torch.empty((n,), dtype=torch.float32, device=dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         rc = lib().ardiff_entropy_gate_ex(
             feat.data_ptr(), n, d, float(tau), mask.data_ptr(), idx.data_ptr(), count.data_ptr(),
             entropy.data_ptr() if entropy is not None else None, _stream_ptr(stream))
@@ -141,22 +176,12 @@ def ardiff_entropy_gate_stats(feat, tau: float = -1.0, want_entropy: bool = Fals
     count = torch.empty((1,), dtype=torch.int32, device=dev)
     entropy = torch.empty((n,), dtype=torch.float32, device=dev) if want_entropy else None
     out3 = torch.empty((3,), dtype=torch.float64, device=dev)
-    vp = ctypes.c_void_p
-    fn = _fn("ardiff_entropy_gate_stats", [vp, ctypes.c_int64, ctypes.c_int32, ctypes.c_float, vp, vp, vp, vp, vp, vp])
-    with torch.cuda.device(dev):
+    fn = lib().ardiff_entropy_gate_stats
+    with _on(dev):
         rc = fn(feat.data_ptr(), n, d, float(tau), mask.data_ptr(), idx.data_ptr(), count.data_ptr(),
                 entropy.data_ptr() if entropy is not None else None, out3.data_ptr(), _stream_ptr(stream))
     _check(rc, "ardiff_entropy_gate_stats")
     return mask, idx, count, entropy, out3
-
-
-def _fn(name, argtypes):
-    """A library function with its ctypes signature set (lazily, once)."""
-    fn = getattr(lib(), name)
-    if fn.argtypes is None:
-        fn.restype = ctypes.c_int
-        fn.argtypes = argtypes
-    return fn
 
 
 def ardiff_entropy_gate_blocks(feat, rows_per_token: int, gamma: int, tau: float, want_token_entropy: bool = False,
@@ -170,16 +195,14 @@ def ardiff_entropy_gate_blocks(feat, rows_per_token: int, gamma: int, tau: float
     assert rows % rows_per_token == 0
     n = rows // rows_per_token
     dev = feat.device
-    vp = ctypes.c_void_p
-    fn = _fn("ardiff_entropy_gate_blocks", [vp, ctypes.c_int64, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32,
-                                            ctypes.c_float, vp, vp, vp, vp, vp, vp, vp])
+    fn = lib().ardiff_entropy_gate_blocks
     mask = torch.empty((n,), dtype=torch.uint8, device=dev)
     idx = torch.empty((max(n, 1),), dtype=torch.int32, device=dev)
     count = torch.empty((1,), dtype=torch.int32, device=dev)
     block_len = torch.empty((max((n + gamma - 1) // gamma, 1),), dtype=torch.int32, device=dev)
     row_ent = torch.empty((max(rows, 1),), dtype=torch.float32, device=dev) if want_row_entropy else None
     tok_ent = torch.empty((max(n, 1),), dtype=torch.float32, device=dev) if want_token_entropy else None
-    with torch.cuda.device(dev):
+    with _on(dev):
         rc = fn(feat.data_ptr(), n, rows_per_token, d, gamma, float(tau),
                 row_ent.data_ptr() if row_ent is not None else None,
                 tok_ent.data_ptr() if tok_ent is not None else None, mask.data_ptr(), idx.data_ptr(),
@@ -193,9 +216,8 @@ def ardiff_tau_calibrate(entropy, stream=None):
     import torch
     assert entropy.is_cuda and entropy.dtype == torch.float32 and entropy.is_contiguous()
     out = torch.empty((3,), dtype=torch.float64, device=entropy.device)
-    vp = ctypes.c_void_p
-    fn = _fn("ardiff_tau_calibrate", [vp, ctypes.c_int64, vp, vp])
-    with torch.cuda.device(entropy.device):
+    fn = lib().ardiff_tau_calibrate
+    with _on(entropy.device):
         rc = fn(entropy.data_ptr(), entropy.numel(), out.data_ptr(), _stream_ptr(stream))
     _check(rc, "ardiff_tau_calibrate")
     return out
@@ -211,9 +233,8 @@ def ardiff_accept_prefix(r, ratio, gamma: int, block_len=None, stream=None):
     out = torch.empty((max(nb, 1),), dtype=torch.int32, device=r.device)
     if block_len is not None:
         assert block_len.is_cuda and block_len.dtype == torch.int32 and block_len.numel() >= nb
-    vp = ctypes.c_void_p
-    fn = _fn("ardiff_accept_prefix", [vp, vp, ctypes.c_int64, ctypes.c_int32, vp, vp, vp])
-    with torch.cuda.device(r.device):
+    fn = lib().ardiff_accept_prefix
+    with _on(r.device):
         rc = fn(r.data_ptr(), ratio.data_ptr(), n, gamma, block_len.data_ptr() if block_len is not None else None,
                 out.data_ptr(), _stream_ptr(stream))
     _check(rc, "ardiff_accept_prefix")
@@ -234,12 +255,8 @@ def ardiff_entropy_gate_noalloc(feat, tau: float, mask, idx, count, stream=None)
     import torch
     assert feat.is_cuda and feat.dtype == torch.bfloat16 and feat.dim() == 2 and feat.is_contiguous()
     fn = lib().ardiff_entropy_gate_noalloc
-    if fn.argtypes is None:
-        vp = ctypes.c_void_p
-        fn.restype = ctypes.c_int
-        fn.argtypes = [vp, ctypes.c_int64, ctypes.c_int32, ctypes.c_float, vp, vp, vp, vp]
     n, d = feat.shape
-    with torch.cuda.device(feat.device):
+    with _on(feat.device):
         rc = fn(feat.data_ptr(), n, d, float(tau), mask.data_ptr(), idx.data_ptr(), count.data_ptr(),
                 _stream_ptr(stream))
     _check(rc, "ardiff_entropy_gate_noalloc")
@@ -273,7 +290,7 @@ class Head:
         assert idx.dtype == torch.int32 and count.dtype == torch.int32
         ts = np.ascontiguousarray(t_sched, dtype=np.float32)
         K = ts.shape[0] - 1
-        with torch.cuda.device(cond.device):
+        with _on(cond.device):
             rc = lib().ardiff_head_sample(self._h, cond.data_ptr(), noise.data_ptr(), ts.ctypes.data, K,
                                           idx.data_ptr(), count.data_ptr(), out.data_ptr(),
                                           _stream_ptr(stream))
@@ -296,9 +313,8 @@ class Head:
         if step_noise is not None:
             assert step_noise.is_cuda and step_noise.dtype == torch.float32 and step_noise.is_contiguous()
             assert tuple(step_noise.shape) == (K, n, noise.shape[1])
-        vp = ctypes.c_void_p
-        fn = _fn("ardiff_head_sample_coef", [vp, vp, vp, vp, ctypes.c_int32, vp, vp, ctypes.c_int64, vp, vp, vp, vp])
-        with torch.cuda.device(cond.device):
+        fn = lib().ardiff_head_sample_coef
+        with _on(cond.device):
             rc = fn(self._h, cond.data_ptr(), noise.data_ptr(), ts.ctypes.data, K, cf.ctypes.data,
                     step_noise.data_ptr() if step_noise is not None else None, n, idx.data_ptr(), count.data_ptr(),
                     out.data_ptr(), _stream_ptr(stream))
@@ -319,17 +335,17 @@ class Head:
     def last_kernel_clock_mhz(self, stream=None) -> float:
         """SM clock the last head kernel ran at (cycles / wall time, stamped on the device)."""
         mhz = ctypes.c_double(0.0)
-        fn = _fn("ardiff_head_last_kernel_clock", [ctypes.c_void_p, ctypes.c_void_p, ctypes.POINTER(ctypes.c_double)])
+        fn = lib().ardiff_head_last_kernel_clock
         _check(fn(self._h, _stream_ptr(stream), ctypes.byref(mhz)), "ardiff_head_last_kernel_clock")
         return float(mhz.value)
 
     def set_cooperative(self, on: bool):
-        fn = _fn("ardiff_head_set_cooperative", [ctypes.c_void_p, ctypes.c_int])
+        fn = lib().ardiff_head_set_cooperative
         _check(fn(self._h, 1 if on else 0), "ardiff_head_set_cooperative")
 
     def inject_stall(self, token_tile: int, wait_limit_us: int):
         """Arms the bounded-wait self-test for the next sample call (see ardiff_head_inject_stall)."""
-        fn = _fn("ardiff_head_inject_stall", [ctypes.c_void_p, ctypes.c_int32, ctypes.c_uint32])
+        fn = lib().ardiff_head_inject_stall
         _check(fn(self._h, token_tile, wait_limit_us), "ardiff_head_inject_stall")
 
     def close(self):
@@ -355,8 +371,7 @@ class Pipeline:
         self.slots = slots
         self._counts = [ctypes.c_int32(0) for _ in range(slots)]
         p = ctypes.c_void_p()
-        vp, i64, i32 = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32
-        fn = _fn("ardiff_pipeline_create_slots", [vp, i64, i32, i32, i32, i32, ctypes.POINTER(vp)])
+        fn = lib().ardiff_pipeline_create_slots
         _check(fn(head._h, max_n, d, self.Dc, self.C, slots, ctypes.byref(p)), "ardiff_pipeline_create_slots")
         self._p = p
 
@@ -378,8 +393,7 @@ class Pipeline:
         be pinned) until ardiff_pipeline_wait(slot)."""
         import numpy as np
         ts = np.ascontiguousarray(t_sched, dtype=np.float32)
-        vp, i64, i32, f32 = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32, ctypes.c_float
-        fn = _fn("ardiff_pipeline_submit", [vp, i32, vp, vp, vp, i64, f32, vp, i32, vp, vp, vp, vp])
+        fn = lib().ardiff_pipeline_submit
         if not 0 <= slot < self.slots:
             raise ValueError("slot out of range")
         rc = fn(self._p, slot, feat.data_ptr(), cond.data_ptr(), noise.data_ptr(), feat.shape[0], float(tau),
@@ -389,13 +403,13 @@ class Pipeline:
 
     def ardiff_pipeline_wait(self, slot: int) -> int:
         """Block until the batch on `slot` has been copied out; returns its number of kept tokens."""
-        fn = _fn("ardiff_pipeline_wait", [ctypes.c_void_p, ctypes.c_int32])
+        fn = lib().ardiff_pipeline_wait
         _check(fn(self._p, slot), "ardiff_pipeline_wait")
         return int(self._counts[slot].value)
 
     def ardiff_pipeline_join(self, stream=None) -> None:
         """Make `stream` wait on the device for every batch submitted so far."""
-        fn = _fn("ardiff_pipeline_join", [ctypes.c_void_p, ctypes.c_void_p])
+        fn = lib().ardiff_pipeline_join
         _check(fn(self._p, _stream_ptr(stream)), "ardiff_pipeline_join")
 
     def close(self):
