@@ -270,6 +270,20 @@ __device__ __forceinline__ void load_whole_row(uint4 (&v)[NCH], const uint4* row
     }
 }
 
+// The least chunk counts that the instances of dispatch_row serve, and the first of a lane's chunks that a row's last one may
+// be (a row of a width that is no multiple of 8 may have one less than others of it). Instances of 5 and 7 chunks a lane, and
+// the last chunk looked for in two of them instead of in the upper half: 65536 x 777 33.2 -> 32.3 us, 500000 x 777 210 -> 203,
+// 65536 x 800 27.5 -> 26.8. (At 8 a lane the upper half: two take 36.2 us at 65536 x 900, five 35.4.)
+__host__ __device__ constexpr int least_chunks(int nch, int g) {
+    return g == 4 ? (nch == 2 ? 1 : nch == 4 ? 9 : 17)
+         : g == 8 ? 33
+         : g == 16 ? 16 * (nch - 1) + 1
+         : nch <= 2 ? 32 * (nch - 1) + 1 : nch == 4 ? 65 : nch == 8 ? 129 : nch == 32 ? 769 : 32 * (nch - 4) + 1;
+}
+__host__ __device__ constexpr int last_chunk_from(int nch, int g) {
+    return nch == 8 && g == 16 ? 3 : least_chunks(nch, g) < 2 ? 0 : (least_chunks(nch, g) - 2) / g;
+}
+
 // The same for rows at any even address (RAGGED) and for 32 / G rows to a warp, G lanes each. Where rows share a warp, what
 // a row costs beside its elements (three reductions by shuffle, a logarithm, a division, the loop) is paid once for all of
 // them: one row per warp takes 242 us for 2^20 x 64 and 20 us for 65536 x 256, this 43 and 12. `step` rows lie between a
@@ -280,9 +294,8 @@ __device__ __forceinline__ float resident_row_entropy(uint4 (&v)[NCH], const Row
     if (RAGGED) {
         if (l == 0) v[0] = keep_elements(v[0], row.head, 8);
         const int last = row.nch - 1, keep = row.head + width - 8 * last;
-        // every instance serves rows of more than half of its capacity (dispatch_row): the last chunk is not in the first half
 #pragma unroll
-        for (int j = NCH > 2 ? NCH / 2 - 1 : 0; j < NCH; ++j)
+        for (int j = last_chunk_from(NCH, G); j < NCH; ++j)
             if (l + G * j == last) v[j] = keep_elements(v[j], 0, keep);
     }
     uint32_t mx = kFill;
@@ -758,7 +771,7 @@ int row_chunks(int32_t d) { return d % 8 == 0 ? d / 8 : (d + 14) / 8; }
 int32_t kernel_width(int32_t d) { return d % 8 == 0 ? d / 8 : d; }
 
 // The row kernel for rows of up to `chunks` sixteen-byte pieces: f(integral_constant<NCH>, integral_constant<G>). Narrow rows
-// share a warp with 8 pieces per lane (fewer in the narrowest) and at least 4 lanes per row, so that a load still
+// share a warp with 5 to 8 pieces per lane (fewer in the narrowest) and at least 4 lanes per row, so that a load still
 // covers whole 32-byte sectors; above 128 pieces, and where there are few rows (`alone`), a row has a warp of its own.
 template <typename F>
 void dispatch_row(int chunks, bool alone, F&& f) {
@@ -771,7 +784,9 @@ void dispatch_row(int chunks, bool alone, F&& f) {
     else if (chunks <= 16) ROW(4, 4);
     else if (chunks <= 32) ROW(8, 4);
     else if (chunks <= 64) ROW(8, 8);
+    else if (chunks <= 80) ROW(5, 16);
     else if (chunks <= 96) ROW(6, 16);
+    else if (chunks <= 112) ROW(7, 16);
     else if (chunks <= 128) ROW(8, 16);
     else if (chunks <= 256) ROW(8, 32);
     else if (chunks <= 384) ROW(12, 32);
@@ -781,9 +796,9 @@ void dispatch_row(int chunks, bool alone, F&& f) {
     else ROW(32, 32);
 #undef ROW
 }
-constexpr int kRowClasses = 15;
+constexpr int kRowClasses = 17;
 int row_class(int chunks, bool alone) {
-    const int up_to[kRowClasses - 4] = {8, 16, 32, 64, 96, 128, 256, 384, 512, 640, 768};
+    const int up_to[kRowClasses - 4] = {8, 16, 32, 64, 80, 96, 112, 128, 256, 384, 512, 640, 768};
     if (alone && chunks <= 128) return kRowClasses - 3 + (chunks > 32) + (chunks > 64);
     int c = 0;
     while (c < kRowClasses - 4 && chunks > up_to[c]) ++c;
@@ -860,7 +875,7 @@ void load_gate_kernels() {
         cudaFuncAttributes a;
         if (cudaFuncGetAttributes(&a, kern) != cudaSuccess) (void)cudaGetLastError();
     };
-    for (int chunks : {8, 16, 32, 64, 96, 128, 256, 384, 512, 640, 768, kResidentChunks})
+    for (int chunks : {8, 16, 32, 64, 80, 96, 112, 128, 256, 384, 512, 640, 768, kResidentChunks})
         for (bool alone : {false, true})
             if (!alone || chunks <= 128)
                 dispatch_row(chunks, alone, [&](auto nch, auto g) {

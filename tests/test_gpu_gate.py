@@ -164,6 +164,14 @@ def test_every_row_kernel(d, n):
         assert np.all(np.abs(row_ent.cpu().numpy() - H) <= 1e-5)
 
 
+@pytest.mark.parametrize("n", [300, 5500])
+@pytest.mark.parametrize("d", [640, 648, 896, 904, 633, 634, 761, 762, 889, 890])
+def test_limits_between_five_and_eight_pieces_a_lane(d, n):
+    """Both sides of the limits at 80, 96 and 112 pieces (aligned rows, and rows of widths that are no multiple of 8, whose
+    last piece lies in either of two places). Bounds and oracle as in the test above."""
+    test_every_row_kernel(d, n)
+
+
 @pytest.mark.parametrize("d", [64, 104, 128, 250, 256, 400, 500, 512, 768, 777, 1000, 1024])
 def test_rows_that_share_a_warp_lose_no_precision(d):
     """fp32 sums of a row against fp64, as a 2-norm over 8192 rows. One row per warp (8 to 32 terms per lane, then a tree)
