@@ -285,8 +285,8 @@ int ardiff_head_sample_coef(const ardiff_head* head, const void* cond, const flo
 int ardiff_head_status(ardiff_head* head, void* stream);
 
 /* Profiling aids. With on != 0, every later ardiff_head_sample on this head records CUDA events
- * on its stream directly around the persistent head kernel. ardiff_head_last_kernel_ms waits
- * for that kernel and writes its device time in milliseconds (ERR_SHAPE if nothing was timed).
+ * on its stream directly around the head kernel (and that of the clusters behind it).
+ * ardiff_head_last_kernel_ms waits for them and writes their device time in milliseconds (ERR_SHAPE if nothing was timed).
  * ardiff_head_last_kernel_clock waits for `stream` and writes the SM clock the last head kernel
  * really ran at, in MHz: SM cycles divided by wall time, both stamped by one CTA at the start and
  * the end of the launch (ERR_SHAPE before the first launch).
