@@ -16,7 +16,7 @@
 // Kernel times of a call (K = 4, modulations included), us, tile schedule or chain.cuh / clusters: W = 256, 2 blocks, 32
 // tokens 125 / 72, 256 177 / 76, 4096 212 / 180; W = 512, 3 blocks, 64 232 / 115, 2048 346 / 289; W = 1024, 3 blocks, 28
 // 197 / 168, 128 358 / 178, 700 426 / 321, but two rounds of groups, 1434 475 / 565: hence one round at most. W = 1280 16
-// 201 / 210, 64 336 / 216; W = 1536, 12 blocks, 28 728 / 749, 64 1094 / 745, 220 1675 / 972; W = 2048, 28 303 / 330, 64 434 /
+// 201 / 210, 64 336 / 216; W = 1536, 12 blocks, 28 728 / 749, 64 1094 / 745, 224 1675 / 912; W = 2048, 28 303 / 330, 64 434 /
 // 331, 200 604 / 460: hence chain.cuh for the fewest tokens of wide heads.
 #pragma once
 

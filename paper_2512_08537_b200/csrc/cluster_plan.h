@@ -47,7 +47,7 @@ struct ClusterLayout {
 };
 
 // Heads created for at most so many tokens split a layer over as many CTAs as a cluster may have. us, 64 or 96 columns a CTA /
-// 128: W = 256, 32 tokens 74 / 76, 1024 101 / 95; W = 1024, 64 tokens 168 / 174, 128 207 / 177; W = 1536, 64 745 / 776.
+// 128: W = 256, 32 tokens 74 / 76, 1024 101 / 95; W = 1024, 64 tokens 168 / 174, 128 207 / 177.
 constexpr int CL_FEW_TOKENS = 64;
 // u (or a) of a cluster's tokens, bytes up to which the CTAs copy it to one another. us, copied / through L2: 8 KB (W = 256, 16
 // tokens) 74 / 97, 32 KB (1024, 16) 168 / 190, 48 KB (1536, 16) 745 / 773, 64 KB (2048, 16) 332 / 330, 96 KB (1024, 48) 359 / 318.
@@ -62,7 +62,8 @@ inline size_t cluster_xch_bytes(int W, int units, int clusters) {
 inline int cluster_rows(int W, int64_t max_tokens) {
     const int choices[] = {64, 96, 128};
     for (int rows : choices)
-        if (W % rows == 0 && W / rows <= CL_MAX_CTAS && (rows == 128 || max_tokens <= CL_FEW_TOKENS)) return rows;
+        if (W % rows == 0 && W / rows <= CL_MAX_CTAS && (rows == 128 || max_tokens <= CL_FEW_TOKENS || W > 8 * 128))
+            return rows;
     return 0;
 }
 // Most units of 16 tokens that a cluster takes at once.
