@@ -176,7 +176,8 @@ struct ClusterEpilogue {
 
         for (int grp = cluster; grp < n_groups; grp += n_clusters) {
             const int tok0 = grp * N + half * 8 * G + 2 * c4;
-            // modulations of this thread's channels and tokens
+            // modulations of this thread's channels and tokens (no read-only loads: the kernel before, which writes them, may
+            // still run when this one starts)
             auto mods = [&](int k, int block, int which, Tile& v) {
                 const float* m = P.mods + mods_at(L, W, ld, k, block, which, rank * NQ + quarter, 0) + lane * 4;
 #pragma unroll
@@ -184,7 +185,7 @@ struct ClusterEpilogue {
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
                         const int tok8 = min(grp * (N / 8) + half * G + g, ld / 8 - 1);
-                        const float4 w = __ldg(reinterpret_cast<const float4*>(m + (size_t)tok8 * 256 + i * 128));
+                        const float4 w = ptx::ldcg_f4(m + (size_t)tok8 * 256 + i * 128);
                         v[g][i][0] = w.x; v[g][i][1] = w.y; v[g][i][2] = w.z; v[g][i][3] = w.w;
                     }
             };

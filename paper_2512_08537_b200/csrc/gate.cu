@@ -623,15 +623,15 @@ gate_rows_long_kernel(const void* __restrict__ feat, int64_t n, int32_t d, float
 // Stable compaction: block b writes the ids of kept tokens of its own range at the offset given
 // by the counts of blocks 0..b-1.
 __global__ void __launch_bounds__(kGateThreads)
-compact_kernel(const uint8_t* __restrict__ mask, int64_t n, const int32_t* __restrict__ block_counts,
-               int64_t tokens_per_block, int32_t* __restrict__ idx, int32_t* __restrict__ count,
-               const double* __restrict__ cta_stats, double* __restrict__ stats_out3) {
+compact_kernel(const uint8_t* mask, int64_t n, const int32_t* block_counts, int64_t tokens_per_block, int32_t* idx,
+               int32_t* count, const double* cta_stats, double* stats_out3) {
     __shared__ int s_warp[kGateWarps];
     __shared__ int s_base;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     // launched with programmatic stream serialization: its blocks may be resident before the kernel that
-    // writes mask and block_counts has finished; nothing of that kernel's output is read before this wait
+    // writes mask and block_counts has finished; nothing of that kernel's output is read before this wait, and none of it
+    // through the read-only path (no __restrict__), which wants data that does not change while this kernel runs
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // Threshold statistics of the entropies (the tau equation): the per-CTA partial sums of the row kernel,
     // merged in a fixed order (lane-strided, then a fixed tree) so that the result is reproducible run to run.

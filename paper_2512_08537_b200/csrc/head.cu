@@ -1331,11 +1331,11 @@ __global__ void __launch_bounds__(256) prep_kernel(const __grid_constant__ PrepA
     }
 }
 
-// temb[k][o] = Wt2[o] . hidden[k] + bt2[o]
+// temb[k][o] = Wt2[o] . hidden[k] + bt2[o]. (Launched while the kernel that writes `hidden` runs: not __restrict__, so that no
+// read-only load is made of it.)
 __global__ void __launch_bounds__(256) temb_out_kernel(const bf16* __restrict__ Wt2,
                                                       const float* __restrict__ bt2, int W,
-                                                      const float* __restrict__ hidden,
-                                                      float* __restrict__ temb) {
+                                                      const float* hidden, float* temb) {
     const int k = blockIdx.y;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int o = blockIdx.x * 8 + warp;
