@@ -208,9 +208,9 @@ typedef struct {
 /*
  * Packs the weights into the kernels' tile layout on the current device and allocates
  * the head's scratch (a fixed-size activation workspace for two groups of token tiles,
- * max_tokens/128 progress counters and, for calls of few tokens, up to 256 MB of modulation values
- * and up to 140 MB of exchange buffers: without room for these such calls take the schedule of
- * larger ones). Synchronous; the only head call that allocates.
+ * max_tokens/128 progress counters and, for calls of few tokens, up to 256 MB of modulation values,
+ * in the workspace as far as it reaches, and up to 140 MB of exchange buffers: without room for these
+ * such calls take the schedule of larger ones). Synchronous; the only head call that allocates.
  * Side effect on the CUDA context: while at least one head exists on a device, the context's
  * cudaLimitPersistingL2CacheSize is at least the size of one token group's fp32 residual
  * stream (about 49 MB, capped at the device's maximum); the kernel keeps that array in the

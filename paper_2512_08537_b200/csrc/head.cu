@@ -1767,35 +1767,46 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     TRY(dev_alloc(H, &H->z, R * Dc, true));
     TRY(dev_alloc(H, &H->xb, R * XB_COLS, true));  // columns >= C stay zero for ever
     TRY(dev_alloc(H, &H->s, (size_t)kmax * R * W, true));   // s_k for every step, [k][row][W]
-    TRY(dev_alloc(H, &H->u, R * W, true));
-    TRY(dev_alloc(H, &H->a, R * W, true));
-    TRY(dev_alloc(H, &H->g0, R * W, true));
-    TRY(dev_alloc(H, &H->g1, R * W, true));
-    TRY(dev_alloc(H, &H->x, R * C, true));
-    TRY(dev_alloc(H, &H->h, R * W, true));
-    TRY(dev_alloc(H, &H->stats, R * 2 * (W / item_cols(N_WIDTHS - 1)), true));
-    // Buffers of the schedules for few tokens; a device without room for them, or for such clusters, does without.
+    // Schedules for few tokens; a device without room for their buffers, or for such clusters, does without.
     H->out_row0 = out_row0;
-    if (d.K_max > 0 && d.max_tokens > 0) {
-        const bool clusters = cluster_setup(H);
-        const int chained = !(W / 256 <= CHAIN_MAX_NC && W / CHAIN_COLS <= H->grid) ? 0
-                            : !clusters ? CHAIN_MAX_TOKENS : chain_beside_clusters(W, 1);
-        const int64_t chain_tokens = d.max_tokens < chained ? d.max_tokens : chained;
-        const int64_t round = std::min((int64_t)d.max_tokens, (int64_t)H->cl_clusters * H->cl_units * CL_UNIT);
-        const size_t mb = clusters ? mods_bytes(d.K_max, round, L, W) : chain_mods_bytes(d.K_max, chain_tokens, L, W);
-        if ((clusters || chained) && dev_alloc(H, &H->mods, mb / sizeof(float), false) == ARDIFF_OK) {
+    const bool may_be_few = d.K_max > 0 && d.max_tokens > 0;
+    const bool clusters = may_be_few && cluster_setup(H);
+    const int chained = !may_be_few || !(W / 256 <= CHAIN_MAX_NC && W / CHAIN_COLS <= H->grid) ? 0
+                        : !clusters ? CHAIN_MAX_TOKENS : chain_beside_clusters(W, 1);
+    const int64_t chain_tokens = d.max_tokens < chained ? d.max_tokens : chained;
+    const int64_t round = std::min((int64_t)d.max_tokens, (int64_t)H->cl_clusters * H->cl_units * CL_UNIT);
+    const size_t mb = clusters  ? mods_bytes(d.K_max, round, L, W)
+                      : chained ? chain_mods_bytes(d.K_max, chain_tokens, L, W) : 0;
+    {
+        // What the tile schedule alone uses, u, a, the gates and h, is one piece of memory, and the modulations of the calls
+        // that do not take that schedule lie in it too: every call writes there all that it reads. A head for a large batch
+        // (291 MB here) thus holds nothing more for its small calls (class-sized with K = 4: 173 MB in a buffer of their own).
+        const size_t tile_bytes = R * W * (4 * sizeof(bf16) + sizeof(float));
+        uint8_t* pool = nullptr;
+        bool fits = mb <= tile_bytes;
+        if (!fits) fits = dev_alloc(H, &pool, mb, true) == ARDIFF_OK;
+        if (!pool) TRY(dev_alloc(H, &pool, tile_bytes, true));
+        if (fits) {
+            H->mods = reinterpret_cast<float*>(pool);
             H->mods_bytes = mb;
-            if (clusters && dev_alloc(H, &H->cl_xch, cluster_xch_bytes(W, H->cl_units, H->cl_clusters), false) != ARDIFF_OK)
-                H->cl_clusters = 0;
-            const size_t xb = chained ? chain_xch_bytes(d.K_max, chain_tokens, L, W, C) : 0;
-            if (chained && dev_alloc(H, &H->chain_xch, xb, false) == ARDIFF_OK) H->chain_bytes = xb;
-            const int tile = CHAIN_COLS * (W * 2 + 64);
-            H->chain_slots = (RING_BYTES + EPI_BYTES - chain_smem(0, W)) / tile;
-            if (H->chain_slots > CHAIN_MAX_SLOTS) H->chain_slots = CHAIN_MAX_SLOTS;
-            H->chain_tokens = (int)chain_tokens;
-        } else {
-            H->cl_clusters = 0;
         }
+        bf16* const half = reinterpret_cast<bf16*>(pool);
+        H->u = half; H->a = half + R * W; H->g0 = half + 2 * R * W; H->g1 = half + 3 * R * W;
+        H->h = reinterpret_cast<float*>(half + 4 * R * W);     // (last: its lines stay in L2 for long)
+    }
+    TRY(dev_alloc(H, &H->x, R * C, true));
+    TRY(dev_alloc(H, &H->stats, R * 2 * (W / item_cols(N_WIDTHS - 1)), true));
+    if (H->mods_bytes > 0) {
+        if (clusters && dev_alloc(H, &H->cl_xch, cluster_xch_bytes(W, H->cl_units, H->cl_clusters), false) != ARDIFF_OK)
+            H->cl_clusters = 0;
+        const size_t xb = chained ? chain_xch_bytes(d.K_max, chain_tokens, L, W, C) : 0;
+        if (chained && dev_alloc(H, &H->chain_xch, xb, false) == ARDIFF_OK) H->chain_bytes = xb;
+        const int tile = CHAIN_COLS * (W * 2 + 64);
+        H->chain_slots = (RING_BYTES + EPI_BYTES - chain_smem(0, W)) / tile;
+        if (H->chain_slots > CHAIN_MAX_SLOTS) H->chain_slots = CHAIN_MAX_SLOTS;
+        H->chain_tokens = (int)chain_tokens;
+    } else {
+        H->cl_clusters = 0;
     }
     TRY(dev_alloc(H, &H->counters, ((size_t)H->max_tiles + 2) * CTRS, true));
     TRY(dev_alloc(H, &H->status, 2, true));

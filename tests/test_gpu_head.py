@@ -216,6 +216,44 @@ def test_head_without_room_for_the_few_token_buffers():
         torch.cuda.empty_cache()
 
 
+def test_a_head_for_large_batches_holds_no_modulation_buffer_beside_its_workspace():
+    """W = 1024, 3 blocks, 4 steps, 16384 tokens: weights, two groups of 47 pairs of token tiles of every activation, and 64 MB
+    for the rest (exchange buffers, tables, allocation granularity); the modulations of one round of clusters are 173 MB."""
+    wl = synth.workload("cfg2")
+    w = synth.head_weights(wl)
+    make_head(wl, w).close()                         # (kernels loaded)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    head = make_head(wl, w)
+    taken = free - torch.cuda.mem_get_info()[0]
+    head.close()
+    R = 4 * 47 * 128
+    weights = 2 * wl.W * (wl.W * (5 * wl.L + 3) + wl.Dc + wl.C + 64 + wl.F)
+    scratch = R * (2 * wl.Dc + 2 * 64 + 4 * wl.C + wl.W * (2 * wl.K + 4 * 2 + 4) + 2 * 8 * wl.W // 64)
+    assert taken <= weights + scratch + (64 << 20), (taken >> 20, weights >> 20, scratch >> 20)
+
+
+@pytest.mark.parametrize("W,few", [(512, 300), (1536, 20)])
+def test_schedules_that_share_memory_leave_nothing_to_one_another(W, few):
+    """Modulations of few tokens and the activations of the tile schedule lie in the same memory: calls of either kind between
+    calls of the other give the bits of a head that has only ever run theirs. (W = 512: clusters, 1536: the chain.)"""
+    wl = synth.workload("cfg1", n=2600, W=W, L=2, K=2)
+    w, cond_bits, noise, t = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
+    order = np.random.default_rng(5).permutation(wl.n).astype(np.int32)
+    head = make_head(wl, w)
+    got = {}
+    for count in (few, 2590, few, 2470, few + 7, 2590, few):
+        out = run_head(head, cond_bits, noise, t, order[:count])
+        assert count not in got or np.array_equal(got[count], out)
+        got[count] = out
+    for count, out in got.items():
+        fresh = make_head(wl, w)
+        assert np.array_equal(run_head(fresh, cond_bits, noise, t, order[:count]), out)
+        fresh.close()
+    head.close()
+
+
 def test_few_tokens_with_fresh_noise_and_after_a_stall():
     """The sampler form with step noise on few tokens, before and after a call whose conditioning never completes."""
     dev = require_cuda()
