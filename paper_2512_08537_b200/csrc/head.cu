@@ -1521,14 +1521,6 @@ int width_limit(int wi, int W, int units, int TGu) {
 }  // namespace
 
 namespace {
-// Survivors up to which the chain stays the schedule beside the clusters: it spreads the weights of a layer over 64 to 128
-// SMs, a cluster over 16, and is one launch, but takes longer for each step and a second pass above 32 tokens. us, chain /
-// clusters: W = 1024, 3 blocks, K = 1, 1 token 69 / 78, 24 73 / 78, 32 82 / 78, K = 4, 4 167 / 168, 8 181 / 168; W = 1280, K = 1, 32
-// 87 / 88, K = 4, 16 210 / 217, 24 225 / 217; W = 1536, 12 blocks, K = 4, 8 640 / 749, 28 726 / 749; W = 2048, K = 4, 4 238 / 337,
-// 32 313 / 338. Below, one token at W = 768 and K = 1 takes 62 / 65, all else less with clusters.
-int chain_beside_clusters(int W, int K) {
-    return W >= 1536 ? 32 : W >= 1280 ? (K == 1 ? 32 : 16) : W >= 1024 ? (K == 1 ? 24 : 4) : 0;
-}
 // The kernel of the cluster schedule for `rows` columns of a layer per CTA.
 typedef void (*ClusterKernel)(const ClusterParams);
 ClusterKernel cluster_kernel_of(int rows) {
@@ -1772,7 +1764,7 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     const bool may_be_few = d.K_max > 0 && d.max_tokens > 0;
     const bool clusters = may_be_few && cluster_setup(H);
     const int chained = !may_be_few || !(W / 256 <= CHAIN_MAX_NC && W / CHAIN_COLS <= H->grid) ? 0
-                        : !clusters ? CHAIN_MAX_TOKENS : chain_beside_clusters(W, 1);
+                        : !clusters ? CHAIN_MAX_TOKENS : chain_beside_clusters(W, H->cl_rows, 1, L);
     const int64_t chain_tokens = d.max_tokens < chained ? d.max_tokens : chained;
     const int64_t round = std::min((int64_t)d.max_tokens, (int64_t)H->cl_clusters * H->cl_units * CL_UNIT);
     const size_t mb = clusters  ? mods_bytes(d.K_max, round, L, W)
@@ -1799,7 +1791,9 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     if (H->mods_bytes > 0) {
         if (clusters && dev_alloc(H, &H->cl_xch, cluster_xch_bytes(W, H->cl_units, H->cl_clusters), false) != ARDIFF_OK)
             H->cl_clusters = 0;
-        const size_t xb = chained ? chain_xch_bytes(d.K_max, chain_tokens, L, W, C) : 0;
+        int steps = d.K_max;                         // the most that the chain serves
+        while (H->cl_clusters && steps > 1 && chain_beside_clusters(W, H->cl_rows, steps, L) == 0) --steps;
+        const size_t xb = chained ? chain_xch_bytes(steps, chain_tokens, L, W, C) : 0;
         if (chained && dev_alloc(H, &H->chain_xch, xb, false) == ARDIFF_OK) H->chain_bytes = xb;
         const int tile = CHAIN_COLS * (W * 2 + 64);
         H->chain_slots = (RING_BYTES + EPI_BYTES - chain_smem(0, W)) / tile;
@@ -1934,6 +1928,26 @@ extern "C" int ardiff_head_destroy(ardiff_head* H) {
 }
 
 namespace {
+// Survivors up to which a call of K steps is served by the chain, and by the clusters above those: what the rules say, as far as
+// the buffers reach.
+void few_limits(const ardiff_head* H, int K, int* chain_count, int* few_count) {
+    const int W = H->d.W, L = H->d.L;
+    int chain = 0, few = 0;
+    if (H->chain_bytes)
+        chain = std::min(H->cl_clusters ? std::min(H->chain_tokens, chain_beside_clusters(W, H->cl_rows, K, L)) : H->chain_tokens,
+                         chain_survivors(H->mods_bytes, H->chain_bytes, K, L, W, H->d.C));
+    if (H->cl_clusters) {
+        const int64_t fit = std::min(mods_survivors(H->mods_bytes, K, L, W), (int64_t)H->slots * BM);
+        few = (int)std::min(fit, cluster_survivors(W, H->cl_clusters, H->cl_units, K, L));
+    }
+#ifdef ARDIFF_TUNING
+    few = std::min(few, env_int("ARDIFF_HEAD_FEW", few));
+    chain = std::min(chain, env_int("ARDIFF_HEAD_CHAIN", chain));
+#endif
+    *chain_count = chain;
+    *few_count = std::max(few, chain);
+}
+
 // t_in [K]: the times fed to the head; coef [3K]: (ax, av, an) of every step
 int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise, const float* t_sched, int32_t K,
                      const float* coef, const float* step_noise, int64_t n_rows, const int32_t* idx,
@@ -1960,20 +1974,7 @@ int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise,
     TimeArgs ta;
     for (int k = 0; k < K; ++k) ta.t[k] = t_sched[k];
     int chain_count = 0, few_count = 0;
-    if (H->chain_bytes)
-        chain_count = std::min(H->cl_clusters ? std::min(H->chain_tokens, chain_beside_clusters(W, K)) : H->chain_tokens,
-                               chain_survivors(H->mods_bytes, H->chain_bytes, K, H->d.L, W, C));
-    // one round of groups (of which the buffer has the size): a second one takes as long again, and the tile schedule hardly longer for twice the tokens (W =
-    // 1024, 700 / 1434 tokens: clusters 321 / 565 us, tiles 426 / 475)
-    if (H->cl_clusters) {
-        const int64_t lim = std::min(mods_survivors(H->mods_bytes, K, H->d.L, W), (int64_t)H->slots * BM);
-        few_count = (int)std::min(lim, (int64_t)H->cl_clusters * H->cl_units * CL_UNIT);
-    }
-#ifdef ARDIFF_TUNING
-    few_count = std::min(few_count, env_int("ARDIFF_HEAD_FEW", few_count));
-    chain_count = std::min(chain_count, env_int("ARDIFF_HEAD_CHAIN", chain_count));
-#endif
-    few_count = std::max(few_count, chain_count);
+    few_limits(H, K, &chain_count, &few_count);
     PrepArgs A;
     A.Wt1 = H->Wt1; A.bt1 = H->bt1; A.hidden = H->temb_hidden; A.W = W; A.F = H->d.F; A.K = K;
     A.counters = H->counters; A.n_counters = (int)((H->max_tiles + 2) * CTRS); A.abort_flag = H->status + 1;
