@@ -21,7 +21,7 @@
 #pragma once
 
 struct ClusterParams {
-    int C, W, L, K, n_ctas, max_units, max_tokens;
+    int C, W, L, K, n_ctas, max_tokens;
     int above, limit;                          // calls of more than `above` and up to `limit` survivors
     uint32_t direct_bytes;                     // up to this size u and a go from CTA to CTA directly (see cluster_kernel)
     int map_cat, map_in, map_out;              // weight boxes: ROWS x 64 of the packed weights and of Win, C x 64 of Wout
@@ -106,9 +106,8 @@ struct ClusterEpilogue {
         return v;
     }
 
-    __device__ static __forceinline__ void run(const ClusterParams& P, int S, int n_groups, int cluster, int n_clusters,
-                                               int rank, uint32_t smem, uint32_t tmem, ClusterBars& B, int warp, int lane,
-                                               ClusterWait& wait) {
+    __device__ static __forceinline__ void run(const ClusterParams& P, int S, int cluster, int rank, uint32_t smem, uint32_t tmem,
+                                               ClusterBars& B, int warp, int lane, ClusterWait& wait) {
         const int quarter = (warp + 2) & 3, half = warp >> 2;    // (warp: 0 .. 7 of the epilogue; quarter = hardware warp % 4)
         if (quarter >= NQ) return;
         const int W = P.W, C = P.C, L = P.L, K = P.K, n_ctas = P.n_ctas;
@@ -174,247 +173,226 @@ struct ClusterEpilogue {
             }
         };
 
-        for (int grp = cluster; grp < n_groups; grp += n_clusters) {
-            const int tok0 = grp * N + half * 8 * G + 2 * c4;
-            // modulations of this thread's channels and tokens (no read-only loads: the kernel before, which writes them, may
-            // still run when this one starts)
-            auto mods = [&](int k, int block, int which, Tile& v) {
-                const float* m = P.mods + mods_at(L, W, ld, k, block, which, rank * NQ + quarter, 0) + lane * 4;
+        const int tok0 = cluster * N + half * 8 * G + 2 * c4;
+        // modulations of this thread's channels and tokens (no read-only loads: the kernel before, which writes them, may
+        // still run when this one starts)
+        auto mods = [&](int k, int block, int which, Tile& v) {
+            const float* m = P.mods + mods_at(L, W, ld, k, block, which, rank * NQ + quarter, 0) + lane * 4;
 #pragma unroll
-                for (int g = 0; g < G; ++g)
+            for (int g = 0; g < G; ++g)
 #pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-                        const int tok8 = min(grp * (N / 8) + half * G + g, ld / 8 - 1);
-                        const float4 w = ptx::ldcg_f4(m + (size_t)tok8 * 256 + i * 128);
-                        v[g][i][0] = w.x; v[g][i][1] = w.y; v[g][i][2] = w.z; v[g][i][3] = w.w;
-                    }
-            };
-            // those of the CTA into L2, for later: many tokens' lie in HBM
-            auto fetch = [&](int k, int block, int which) {
+                for (int i = 0; i < 2; ++i) {
+                    const int tok8 = min(cluster * (N / 8) + half * G + g, ld / 8 - 1);
+                    const float4 w = ptx::ldcg_f4(m + (size_t)tok8 * 256 + i * 128);
+                    v[g][i][0] = w.x; v[g][i][1] = w.y; v[g][i][2] = w.z; v[g][i][3] = w.w;
+                }
+        };
+        // those of the CTA into L2, for later: many tokens' lie in HBM
+        auto fetch = [&](int k, int block, int which) {
 #pragma unroll
-                for (int q = 0; q < NQ; ++q)
-                    ptx::bulk_prefetch_l2(P.mods + mods_at(L, W, ld, k, block, which, rank * NQ + q, grp * (N / 8)),
-                                          (uint32_t)min(N / 8, ld / 8 - grp * (N / 8)) * 1024);
-            };
-            auto bias = [&](const float* b, float (&v)[2][2]) {
+            for (int q = 0; q < NQ; ++q)
+                ptx::bulk_prefetch_l2(P.mods + mods_at(L, W, ld, k, block, which, rank * NQ + q, cluster * (N / 8)),
+                                      (uint32_t)min(N / 8, ld / 8 - cluster * (N / 8)) * 1024);
+        };
+        auto bias = [&](const float* b, float (&v)[2][2]) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) v[i][j] = __ldg(b + 16 * i + 8 * j);
+        };
+        Tile h;
+        // x of this thread's output channels (the warps of the first 64 channels; the same in every CTA): few steps
+        // change it, so it lies in shared memory
+        const bool has_x = quarter < 2;
+        const int cx = quarter * 32 + r8;
+        auto row_of = [&](int g, int e) {                  // token id, or -1
+            const int tok = tok0 + 8 * g + e;
+            return tok < S ? __ldg(P.idx + tok) : -1;
+        };
+        auto rows_of = [&](const float* base, Tile& v) {
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int rw = row_of(g, e);
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            const int c = cx + 16 * i + 8 * j;
+                            v[g][i][2 * j + e] = c < C && rw >= 0 ? __ldg(base + (size_t)rw * C + c) : 0.f;
+                        }
+                }
+        };
+        const uint32_t x_at = smem + lay.x + (uint32_t)(cx * N + half * 8 * G + 2 * c4) * 4;
+        auto store_x = [&](const Tile& x) {
+#pragma unroll
+            for (int g = 0; g < G; ++g)
 #pragma unroll
                 for (int i = 0; i < 2; ++i)
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) v[i][j] = __ldg(b + 16 * i + 8 * j);
-            };
-            Tile h;
-            // x of this thread's output channels (the warps of the first 64 channels; the same in every CTA): few steps
-            // change it, so it lies in shared memory
-            const bool has_x = quarter < 2;
-            const int cx = quarter * 32 + r8;
-            auto row_of = [&](int g, int e) {                  // token id, or -1
-                const int tok = tok0 + 8 * g + e;
-                return tok < S ? __ldg(P.idx + tok) : -1;
-            };
-            auto rows_of = [&](const float* base, Tile& v) {
-#pragma unroll
-                for (int g = 0; g < G; ++g)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int rw = row_of(g, e);
-#pragma unroll
-                        for (int i = 0; i < 2; ++i)
-#pragma unroll
-                            for (int j = 0; j < 2; ++j) {
-                                const int c = cx + 16 * i + 8 * j;
-                                v[g][i][2 * j + e] = c < C && rw >= 0 ? __ldg(base + (size_t)rw * C + c) : 0.f;
-                            }
-                    }
-            };
-            const uint32_t x_at = smem + lay.x + (uint32_t)(cx * N + half * 8 * G + 2 * c4) * 4;
-            auto store_x = [&](const Tile& x) {
+                    for (int j = 0; j < 2; ++j)
+                        if (cx + 16 * i + 8 * j < C)
+                            ptx::sts_f2(x_at + (uint32_t)((16 * i + 8 * j) * N + 8 * g) * 4, x[g][i][2 * j], x[g][i][2 * j + 1]);
+            // as bf16, and where the slice of 64 has room for it what the rounding took off in the C columns behind (Win
+            // is there twice): the in-projection then sees x to 16 bits, for nothing
+            if (C <= 32) {
+                Tile lo;
 #pragma unroll
                 for (int g = 0; g < G; ++g)
 #pragma unroll
                     for (int i = 0; i < 2; ++i)
 #pragma unroll
-                        for (int j = 0; j < 2; ++j)
-                            if (cx + 16 * i + 8 * j < C)
-                                ptx::sts_f2(x_at + (uint32_t)((16 * i + 8 * j) * N + 8 * g) * 4, x[g][i][2 * j], x[g][i][2 * j + 1]);
-                // as bf16, and where the slice of 64 has room for it what the rounding took off in the C columns behind (Win
-                // is there twice): the in-projection then sees x to 16 bits, for nothing
-                if (C <= 32) {
-                    Tile lo;
+                        for (int e = 0; e < 4; ++e) lo[g][i][e] = x[g][i][e] - __bfloat162float(__float2bfloat16_rn(x[g][i][e]));
+                if (C == 16) {
 #pragma unroll
                     for (int g = 0; g < G; ++g)
 #pragma unroll
-                        for (int i = 0; i < 2; ++i)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) lo[g][i][e] = x[g][i][e] - __bfloat162float(__float2bfloat16_rn(x[g][i][e]));
-                    if (C == 16) {
-#pragma unroll
-                        for (int g = 0; g < G; ++g)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float v = lo[g][0][e];
-                                lo[g][0][e] = x[g][0][e];
-                                lo[g][1][e] = quarter == 0 ? v : 0.f;
-                            }
-                        store_blocks(smem + lay.xb + put, lo);
-                    } else if (quarter == 0) {
-                        store_blocks(smem + lay.xb + put, x);
-                        store_blocks(smem + lay.xb + put + 4 * N * 16, lo);
-                    }
-                } else {
+                        for (int e = 0; e < 4; ++e) {
+                            const float v = lo[g][0][e];
+                            lo[g][0][e] = x[g][0][e];
+                            lo[g][1][e] = quarter == 0 ? v : 0.f;
+                        }
+                    store_blocks(smem + lay.xb + put, lo);
+                } else if (quarter == 0) {
                     store_blocks(smem + lay.xb + put, x);
+                    store_blocks(smem + lay.xb + put + 4 * N * 16, lo);
                 }
-                ptx::fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar_x);
-            };
-            if (has_x) {
-                Tile x;
-                rows_of(P.noise, x);
-                store_x(x);
+            } else {
+                store_blocks(smem + lay.xb + put, x);
             }
-            for (int k = 0; k < K; ++k) {
-                {   // h = Win x + bin
-                    float b[2][2];
-                    bias(P.bin + ch0, b);
-                    next_acc(h);
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(bar_x);
+        };
+        if (has_x) {
+            Tile x;
+            rows_of(P.noise, x);
+            store_x(x);
+        }
+        for (int k = 0; k < K; ++k) {
+            {   // h = Win x + bin
+                float b[2][2];
+                bias(P.bin + ch0, b);
+                next_acc(h);
+#pragma unroll
+                for (int g = 0; g < G; ++g)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) h[g][i][e] += b[i][e >> 1];
+            }
+            for (int b = 0;; ++b) {
+                // u = LN(h) (1 + scale) + shift
+                {
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        float mean[2], m2[2];
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const float s = add8((h[g][0][e] + h[g][0][2 + e]) + (h[g][1][e] + h[g][1][2 + e]));
+                            mean[e] = s * (1.0f / 32.0f);
+                            float q = 0.f;
+#pragma unroll
+                            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                                for (int j = 0; j < 2; ++j) {
+                                    const float d = h[g][i][2 * j + e] - mean[e];
+                                    q = fmaf(d, d, q);
+                                }
+                            m2[e] = add8(q);
+                        }
+                        if (r8 == 0) ptx::sts_f4(part + (uint32_t)((4 * g + c4) * NQ + quarter) * 16, mean[0], m2[0], mean[1], m2[1]);
+                    }
+                    ptx::bar_sync(2 + half, 32 * NQ);
+                    // the CTA's partials of 4 G pairs of tokens, to every CTA of the cluster
+                    for (int t = quarter * 32 + lane; t < 4 * G * n_ctas; t += 32 * NQ) {
+                        const int pair = t % (4 * G), peer = t / (4 * G);
+                        float4 v[NQ];
+#pragma unroll
+                        for (int q = 0; q < NQ; ++q) v[q] = ptx::lds_f4(part + (uint32_t)(pair * NQ + q) * 16);
+                        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                        for (int q = 0; q < NQ; ++q) { o.x += v[q].x; o.z += v[q].z; o.y += v[q].y; o.w += v[q].w; }
+                        o.x *= 1.0f / NQ;
+                        o.z *= 1.0f / NQ;
+#pragma unroll
+                        for (int q = 0; q < NQ; ++q) {
+                            const float d0 = v[q].x - o.x, d1 = v[q].z - o.z;
+                            o.y = fmaf(32.0f * d0, d0, o.y);
+                            o.w = fmaf(32.0f * d1, d1, o.w);
+                        }
+                        if (!wait.aborted())
+                            ptx::st_async_f4(ptx::map_peer(stats + (uint32_t)(pair * n_ctas + rank) * 16, peer), o,
+                                             ptx::map_peer(bar_stat, peer));
+                    }
+                    Tile sh, u;                          // (u: the scale, then the result)
+                    mods(k, b, 0, sh);
+                    mods(k, b, 1, u);
+                    const bool there = wait.mbar(bar_stat, ph_stat);
+                    ph_stat ^= 1;
+                    __syncwarp();
+                    // (never twice in a phase: not after a wait that gave up, nor after one that came too early because
+                    // of it)
+                    if (quarter == 0 && lane == 0 && there && !wait.aborted())
+                        ptx::mbar_arrive_expect_tx(bar_stat, 4 * G * n_ctas * 16);
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        float4 v[2];
+#pragma unroll
+                        for (int s = 0; s < 2; ++s) {
+                            v[s] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (r8 + 8 * s < n_ctas) v[s] = ptx::lds_f4(stats + (uint32_t)((4 * g + c4) * n_ctas + r8 + 8 * s) * 16);
+                        }
+                        const float mean[2] = {add8(v[0].x + v[1].x) * inv_ctas, add8(v[0].z + v[1].z) * inv_ctas};
+                        float q0 = v[0].y + v[1].y, q1 = v[0].w + v[1].w;
+#pragma unroll
+                        for (int s = 0; s < 2; ++s)
+                            if (r8 + 8 * s < n_ctas) {
+                                const float d0 = v[s].x - mean[0], d1 = v[s].z - mean[1];
+                                q0 = fmaf((float)ROWS * d0, d0, q0);
+                                q1 = fmaf((float)ROWS * d1, d1, q1);
+                            }
+                        const float rstd[2] = {rsqrtf(add8(q0) * inv_w + 1e-6f), rsqrtf(add8(q1) * inv_w + 1e-6f)};
+#pragma unroll
+                        for (int i = 0; i < 2; ++i)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                u[g][i][e] = fmaf((h[g][i][e] - mean[e & 1]) * rstd[e & 1], 1.0f + u[g][i][e], sh[g][i][e]);
+                    }
+                    publish(lay.u, B.src_u, &B.sig[0], xch, u);
+                }
+                if (me == 0 && ptx::elect_one()) {
+                    if (b < L) {
+                        fetch(k, b, 2);
+                        fetch(k, b + 1, 0);
+                        fetch(k, b + 1, 1);
+                    } else if (k + 1 < K) {
+                        fetch(k + 1, 0, 0);
+                        fetch(k + 1, 0, 1);
+                    }
+                }
+                __syncwarp();
+                if (b == L) break;
+                const float* b_blk = P.bias_cat + (size_t)b * 5 * W + ch0;
+                {   // a = SiLU(W1 u + b1)
+                    float b1[2][2];
+                    bias(b_blk + 3 * (size_t)W, b1);
+                    Tile a;
+                    next_acc(a);
 #pragma unroll
                     for (int g = 0; g < G; ++g)
 #pragma unroll
                         for (int i = 0; i < 2; ++i)
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) h[g][i][e] += b[i][e >> 1];
+                            for (int e = 0; e < 4; ++e) a[g][i][e] = silu_f(a[g][i][e] + b1[i][e >> 1]);
+                    publish(lay.a, B.src_a, &B.sig[1], xch + lay.act, a);
                 }
-                for (int b = 0;; ++b) {
-                    // u = LN(h) (1 + scale) + shift
-                    {
-#pragma unroll
-                        for (int g = 0; g < G; ++g) {
-                            float mean[2], m2[2];
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                const float s = add8((h[g][0][e] + h[g][0][2 + e]) + (h[g][1][e] + h[g][1][2 + e]));
-                                mean[e] = s * (1.0f / 32.0f);
-                                float q = 0.f;
-#pragma unroll
-                                for (int i = 0; i < 2; ++i)
-#pragma unroll
-                                    for (int j = 0; j < 2; ++j) {
-                                        const float d = h[g][i][2 * j + e] - mean[e];
-                                        q = fmaf(d, d, q);
-                                    }
-                                m2[e] = add8(q);
-                            }
-                            if (r8 == 0) ptx::sts_f4(part + (uint32_t)((4 * g + c4) * NQ + quarter) * 16, mean[0], m2[0], mean[1], m2[1]);
-                        }
-                        ptx::bar_sync(2 + half, 32 * NQ);
-                        // the CTA's partials of 4 G pairs of tokens, to every CTA of the cluster
-                        for (int t = quarter * 32 + lane; t < 4 * G * n_ctas; t += 32 * NQ) {
-                            const int pair = t % (4 * G), peer = t / (4 * G);
-                            float4 v[NQ];
-#pragma unroll
-                            for (int q = 0; q < NQ; ++q) v[q] = ptx::lds_f4(part + (uint32_t)(pair * NQ + q) * 16);
-                            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                            for (int q = 0; q < NQ; ++q) { o.x += v[q].x; o.z += v[q].z; o.y += v[q].y; o.w += v[q].w; }
-                            o.x *= 1.0f / NQ;
-                            o.z *= 1.0f / NQ;
-#pragma unroll
-                            for (int q = 0; q < NQ; ++q) {
-                                const float d0 = v[q].x - o.x, d1 = v[q].z - o.z;
-                                o.y = fmaf(32.0f * d0, d0, o.y);
-                                o.w = fmaf(32.0f * d1, d1, o.w);
-                            }
-                            if (!wait.aborted())
-                                ptx::st_async_f4(ptx::map_peer(stats + (uint32_t)(pair * n_ctas + rank) * 16, peer), o,
-                                                 ptx::map_peer(bar_stat, peer));
-                        }
-                        Tile sh, u;                          // (u: the scale, then the result)
-                        mods(k, b, 0, sh);
-                        mods(k, b, 1, u);
-                        const bool there = wait.mbar(bar_stat, ph_stat);
-                        ph_stat ^= 1;
-                        __syncwarp();
-                        // (never twice in a phase: not after a wait that gave up, nor after one that came too early because
-                        // of it)
-                        if (quarter == 0 && lane == 0 && there && !wait.aborted())
-                            ptx::mbar_arrive_expect_tx(bar_stat, 4 * G * n_ctas * 16);
-#pragma unroll
-                        for (int g = 0; g < G; ++g) {
-                            float4 v[2];
-#pragma unroll
-                            for (int s = 0; s < 2; ++s) {
-                                v[s] = make_float4(0.f, 0.f, 0.f, 0.f);
-                                if (r8 + 8 * s < n_ctas) v[s] = ptx::lds_f4(stats + (uint32_t)((4 * g + c4) * n_ctas + r8 + 8 * s) * 16);
-                            }
-                            const float mean[2] = {add8(v[0].x + v[1].x) * inv_ctas, add8(v[0].z + v[1].z) * inv_ctas};
-                            float q0 = v[0].y + v[1].y, q1 = v[0].w + v[1].w;
-#pragma unroll
-                            for (int s = 0; s < 2; ++s)
-                                if (r8 + 8 * s < n_ctas) {
-                                    const float d0 = v[s].x - mean[0], d1 = v[s].z - mean[1];
-                                    q0 = fmaf((float)ROWS * d0, d0, q0);
-                                    q1 = fmaf((float)ROWS * d1, d1, q1);
-                                }
-                            const float rstd[2] = {rsqrtf(add8(q0) * inv_w + 1e-6f), rsqrtf(add8(q1) * inv_w + 1e-6f)};
-#pragma unroll
-                            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                                for (int e = 0; e < 4; ++e)
-                                    u[g][i][e] = fmaf((h[g][i][e] - mean[e & 1]) * rstd[e & 1], 1.0f + u[g][i][e], sh[g][i][e]);
-                        }
-                        publish(lay.u, B.src_u, &B.sig[0], xch, u);
-                    }
-                    if (me == 0 && ptx::elect_one()) {
-                        if (b < L) {
-                            fetch(k, b, 2);
-                            fetch(k, b + 1, 0);
-                            fetch(k, b + 1, 1);
-                        } else if (k + 1 < K) {
-                            fetch(k + 1, 0, 0);
-                            fetch(k + 1, 0, 1);
-                        }
-                    }
-                    __syncwarp();
-                    if (b == L) break;
-                    const float* b_blk = P.bias_cat + (size_t)b * 5 * W + ch0;
-                    {   // a = SiLU(W1 u + b1)
-                        float b1[2][2];
-                        bias(b_blk + 3 * (size_t)W, b1);
-                        Tile a;
-                        next_acc(a);
-#pragma unroll
-                        for (int g = 0; g < G; ++g)
-#pragma unroll
-                            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) a[g][i][e] = silu_f(a[g][i][e] + b1[i][e >> 1]);
-                        publish(lay.a, B.src_a, &B.sig[1], xch + lay.act, a);
-                    }
-                    {   // h += gate * (W2 a + b2)
-                        Tile gate;
-                        mods(k, b, 2, gate);
-                        float b2[2][2];
-                        bias(b_blk + 4 * (size_t)W, b2);
-                        Tile v;
-                        next_acc(v);
-#pragma unroll
-                        for (int g = 0; g < G; ++g)
-#pragma unroll
-                            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) h[g][i][e] = fmaf(gate[g][i][e], v[g][i][e] + b2[i][e >> 1], h[g][i][e]);
-                    }
-                }
-                if (!has_x) { ++n_acc; continue; }
-                {   // x <- ax x + av (Wout u + bout) + an z
-                    Tile z;
-                    if (P.step_noise) rows_of(P.step_noise + (size_t)k * (size_t)P.step_stride, z);
-                    float bo[2][2];
-#pragma unroll
-                    for (int i = 0; i < 2; ++i)
-#pragma unroll
-                        for (int j = 0; j < 2; ++j) bo[i][j] = cx + 16 * i + 8 * j < C ? __ldg(P.bias_cat + P.out_row0 + cx + 16 * i + 8 * j) : 0.f;
-                    const float ax = P.ax[k], av = P.av[k], an = P.an[k];
+                {   // h += gate * (W2 a + b2)
+                    Tile gate;
+                    mods(k, b, 2, gate);
+                    float b2[2][2];
+                    bias(b_blk + 4 * (size_t)W, b2);
                     Tile v;
                     next_acc(v);
 #pragma unroll
@@ -422,34 +400,53 @@ struct ClusterEpilogue {
 #pragma unroll
                         for (int i = 0; i < 2; ++i)
 #pragma unroll
-                            for (int j = 0; j < 2; ++j) {
-                                const bool have = cx + 16 * i + 8 * j < C;
-                                float2 x = make_float2(0.f, 0.f);
-                                if (have) x = ptx::lds_f2(x_at + (uint32_t)((16 * i + 8 * j) * N + 8 * g) * 4);
-                                x.x *= ax;                                    // ax = 1: exactly x
-                                x.y *= ax;
-                                if (P.step_noise) {
-                                    x.x = fmaf(an, z[g][i][2 * j], x.x);
-                                    x.y = fmaf(an, z[g][i][2 * j + 1], x.y);
-                                }
-                                v[g][i][2 * j] = have ? fmaf(av, v[g][i][2 * j] + bo[i][j], x.x) : 0.f;
-                                v[g][i][2 * j + 1] = have ? fmaf(av, v[g][i][2 * j + 1] + bo[i][j], x.y) : 0.f;
+                            for (int e = 0; e < 4; ++e) h[g][i][e] = fmaf(gate[g][i][e], v[g][i][e] + b2[i][e >> 1], h[g][i][e]);
+                }
+            }
+            if (!has_x) { ++n_acc; continue; }
+            {   // x <- ax x + av (Wout u + bout) + an z
+                Tile z;
+                if (P.step_noise) rows_of(P.step_noise + (size_t)k * (size_t)P.step_stride, z);
+                float bo[2][2];
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) bo[i][j] = cx + 16 * i + 8 * j < C ? __ldg(P.bias_cat + P.out_row0 + cx + 16 * i + 8 * j) : 0.f;
+                const float ax = P.ax[k], av = P.av[k], an = P.an[k];
+                Tile v;
+                next_acc(v);
+#pragma unroll
+                for (int g = 0; g < G; ++g)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            const bool have = cx + 16 * i + 8 * j < C;
+                            float2 x = make_float2(0.f, 0.f);
+                            if (have) x = ptx::lds_f2(x_at + (uint32_t)((16 * i + 8 * j) * N + 8 * g) * 4);
+                            x.x *= ax;                                    // ax = 1: exactly x
+                            x.y *= ax;
+                            if (P.step_noise) {
+                                x.x = fmaf(an, z[g][i][2 * j], x.x);
+                                x.y = fmaf(an, z[g][i][2 * j + 1], x.y);
                             }
-                    if (k + 1 < K) store_x(v);
-                    else if (rank == 0) {
+                            v[g][i][2 * j] = have ? fmaf(av, v[g][i][2 * j] + bo[i][j], x.x) : 0.f;
+                            v[g][i][2 * j + 1] = have ? fmaf(av, v[g][i][2 * j + 1] + bo[i][j], x.y) : 0.f;
+                        }
+                if (k + 1 < K) store_x(v);
+                else if (rank == 0) {
 #pragma unroll
-                        for (int g = 0; g < G; ++g)
+                    for (int g = 0; g < G; ++g)
 #pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                const int rw = row_of(g, e);
+                        for (int e = 0; e < 2; ++e) {
+                            const int rw = row_of(g, e);
 #pragma unroll
-                                for (int i = 0; i < 2; ++i)
+                            for (int i = 0; i < 2; ++i)
 #pragma unroll
-                                    for (int j = 0; j < 2; ++j)
-                                        if (cx + 16 * i + 8 * j < C && rw >= 0)
-                                            P.out[(size_t)rw * C + cx + 16 * i + 8 * j] = v[g][i][2 * j + e];
-                            }
-                    }
+                                for (int j = 0; j < 2; ++j)
+                                    if (cx + 16 * i + 8 * j < C && rw >= 0)
+                                        P.out[(size_t)rw * C + cx + 16 * i + 8 * j] = v[g][i][2 * j + e];
+                        }
                 }
             }
         }
@@ -459,8 +456,8 @@ struct ClusterEpilogue {
 // One thread: the weight slices in the order they are used. A layer's K slices start with the CTA's own channels, whose
 // activations are there first.
 template <int ROWS>
-__device__ __forceinline__ void cluster_feed(const ClusterParams& P, int n_groups, int cluster, int n_clusters, int rank,
-                                             const ClusterLayout& lay, uint32_t ring, ClusterBars& B, ClusterWait& wait) {
+__device__ __forceinline__ void cluster_feed(const ClusterParams& P, int rank, const ClusterLayout& lay, uint32_t ring,
+                                             ClusterBars& B, ClusterWait& wait) {
     const uint32_t full = ptx::smem_u32(B.full), empty = ptx::smem_u32(B.empty);
     constexpr int SL = cl_slices(ROWS), SRCS = SL * CL_KS / ROWS;
     const int W = P.W, stages = W / (CL_KS * SL), layers = 2 * P.L + 2;
@@ -468,28 +465,27 @@ __device__ __forceinline__ void cluster_feed(const ClusterParams& P, int n_group
     uint32_t ph = 0, issued = 0, parity = 0;
     bool ok = true;
     // (one loop over the layers of a step with one copy in it: see cluster_mma)
-    for (int grp = cluster; ok && grp < n_groups; grp += n_clusters)
-        for (int k = 0; ok && k < P.K; ++k)
-            for (int l = 0; ok && l < layers; ++l) {
-                const bool in = l == 0, out = l == layers - 1;
-                const int n = in ? 1 : stages, sl = in ? 1 : SL;
-                const void* map = P.maps + (in ? P.map_in : out ? P.map_out : P.map_cat);
-                const int row = in ? rank * ROWS : out ? (int)P.out_row0 : (5 * ((l - 1) >> 1) + 3 + ((l - 1) & 1)) * W + rank * ROWS;
-                const uint32_t bytes = (uint32_t)(out ? P.C : ROWS) * CL_KS * 2 * sl;
-                int kp = in ? 0 : rank / SRCS;
-                for (int i = 0; i < n; ++i) {
-                    ok = wait.mbar(empty + 8 * st, ph ^ 1u);
-                    if (!ok) break;
-                    ptx::mbar_arrive_expect_tx(full + 8 * st, bytes);
-                    const uint32_t dst = ring + (uint32_t)st * lay.stage;
-                    for (int j = 0; j < sl; ++j)
-                        ptx::tma_load_2d(dst + (uint32_t)j * (ROWS * CL_KS * 2), map, full + 8 * st, (kp * SL + j) * CL_KS, row);
-                    issued |= 1u << st;
-                    parity = (parity & ~(1u << st)) | (ph << st);
-                    if (++st == lay.stages) { st = 0; ph ^= 1u; }
-                    if (++kp == n) kp = 0;
-                }
+    for (int k = 0; ok && k < P.K; ++k)
+        for (int l = 0; ok && l < layers; ++l) {
+            const bool in = l == 0, out = l == layers - 1;
+            const int n = in ? 1 : stages, sl = in ? 1 : SL;
+            const void* map = P.maps + (in ? P.map_in : out ? P.map_out : P.map_cat);
+            const int row = in ? rank * ROWS : out ? (int)P.out_row0 : (5 * ((l - 1) >> 1) + 3 + ((l - 1) & 1)) * W + rank * ROWS;
+            const uint32_t bytes = (uint32_t)(out ? P.C : ROWS) * CL_KS * 2 * sl;
+            int kp = in ? 0 : rank / SRCS;
+            for (int i = 0; i < n; ++i) {
+                ok = wait.mbar(empty + 8 * st, ph ^ 1u);
+                if (!ok) break;
+                ptx::mbar_arrive_expect_tx(full + 8 * st, bytes);
+                const uint32_t dst = ring + (uint32_t)st * lay.stage;
+                for (int j = 0; j < sl; ++j)
+                    ptx::tma_load_2d(dst + (uint32_t)j * (ROWS * CL_KS * 2), map, full + 8 * st, (kp * SL + j) * CL_KS, row);
+                issued |= 1u << st;
+                parity = (parity & ~(1u << st)) | (ph << st);
+                if (++st == lay.stages) { st = 0; ph ^= 1u; }
+                if (++kp == n) kp = 0;
             }
+        }
     // copies in flight land before the CTA may leave (bounded by time: an aborted call has slices nobody waits for)
     for (int s = 0; s < lay.stages; ++s)
         if (issued & (1u << s)) drain_mbar(full + 8 * s, (parity >> s) & 1u);
@@ -498,9 +494,8 @@ __device__ __forceinline__ void cluster_feed(const ClusterParams& P, int n_group
 // One thread: the products. Weights are the A operand (128 rows of it, ROWS of them this CTA's), the activations of all
 // CTAs the B operand, which lies in shared memory as [8 channels][token][16 bytes].
 template <int ROWS>
-__device__ __forceinline__ void cluster_mma(const ClusterParams& P, int units, int n_groups, int cluster, int n_clusters,
-                                            int rank, const ClusterLayout& lay, uint32_t smem, uint32_t tmem, ClusterBars& B,
-                                            ClusterWait& wait) {
+__device__ __forceinline__ void cluster_mma(const ClusterParams& P, int units, int rank, const ClusterLayout& lay, uint32_t smem,
+                                            uint32_t tmem, ClusterBars& B, ClusterWait& wait) {
     const uint32_t full = ptx::smem_u32(B.full), empty = ptx::smem_u32(B.empty), acc = ptx::smem_u32(B.acc);
     constexpr int SL = cl_slices(ROWS), SRCS = SL * CL_KS / ROWS;
     const int stages = P.W / (CL_KS * SL);
@@ -519,49 +514,48 @@ __device__ __forceinline__ void cluster_mma(const ClusterParams& P, int units, i
     bool ok = true;
     // One loop with one set of asynchronous instructions in it: called from several places the body becomes a function, in
     // which the compiler no longer knows that one thread is active (see ptx::elect_one).
-    for (int grp = cluster; ok && grp < n_groups; grp += n_clusters)
-        for (int k = 0; ok && k < P.K; ++k)
-            for (int l = 0; ok && l < layers; ++l) {
-                const bool in = l == 0, odd = l & 1;         // odd: operand u, even: operand a
-                const int n = in ? 1 : stages;
-                const uint32_t act = smem + (in ? lay.xb : odd ? lay.u : lay.a), src = odd ? bar_u : bar_a;
-                const uint32_t phase = odd ? ph_u : ph_a, d = tmem + (n_acc & 1) * 64;
-                // a layer's stages start with the one that holds this CTA's own channels: they are there first
-                int kp = in ? 0 : rank / SRCS;
-                if (in) ok = wait.mbar(ptx::smem_u32(&B.x), ph_x);
-                for (int i = 0; ok && i < n; ++i) {
-                    ok = wait.mbar(full + 8 * st, ph);
-                    const uint32_t a0 = smem + (uint32_t)st * lay.stage, b0 = act + (uint32_t)(kp * SL) * (8 * N * 16);
+    for (int k = 0; ok && k < P.K; ++k)
+        for (int l = 0; ok && l < layers; ++l) {
+            const bool in = l == 0, odd = l & 1;         // odd: operand u, even: operand a
+            const int n = in ? 1 : stages;
+            const uint32_t act = smem + (in ? lay.xb : odd ? lay.u : lay.a), src = odd ? bar_u : bar_a;
+            const uint32_t phase = odd ? ph_u : ph_a, d = tmem + (n_acc & 1) * 64;
+            // a layer's stages start with the one that holds this CTA's own channels: they are there first
+            int kp = in ? 0 : rank / SRCS;
+            if (in) ok = wait.mbar(ptx::smem_u32(&B.x), ph_x);
+            for (int i = 0; ok && i < n; ++i) {
+                ok = wait.mbar(full + 8 * st, ph);
+                const uint32_t a0 = smem + (uint32_t)st * lay.stage, b0 = act + (uint32_t)(kp * SL) * (8 * N * 16);
 #pragma unroll
-                    for (int j = 0; j < SL; ++j) {
-                        if (in && j > 0) break;
-                        // the CTAs whose channels the slice holds
-                        if (!in && SRCS == SL) ok = ok && wait.mbar(src + 8 * (kp * SRCS + j), phase);
-                        else if (!in && j == 0)
-                            for (int q = 0; q < SRCS; ++q) ok = ok && wait.mbar(src + 8 * (kp * SRCS + q), phase);
-                        if (!ok) break;
-                        ptx::tc_fence_after();
-                        const uint64_t da = ptx::smem_desc_sw128(a0 + (uint32_t)j * (ROWS * CL_KS * 2));
-                        const uint64_t db = ptx::smem_desc_plain(b0 + (uint32_t)j * (8 * N * 16), N * 16, 128);
-#pragma unroll
-                        for (int q = 0; q < CL_KS / 16; ++q)
-                            ptx::mma_f16_ss(d, da + (uint64_t)(2 * q), db + (uint64_t)(q * 2) * N, idesc, (i | j | q) != 0 ? 1u : 0u);
-                    }
+                for (int j = 0; j < SL; ++j) {
+                    if (in && j > 0) break;
+                    // the CTAs whose channels the slice holds
+                    if (!in && SRCS == SL) ok = ok && wait.mbar(src + 8 * (kp * SRCS + j), phase);
+                    else if (!in && j == 0)
+                        for (int q = 0; q < SRCS; ++q) ok = ok && wait.mbar(src + 8 * (kp * SRCS + q), phase);
                     if (!ok) break;
-                    ptx::mma_commit(empty + 8 * st);
-                    if (++st == lay.stages) { st = 0; ph ^= 1u; }
-                    if (++kp == n) kp = 0;
+                    ptx::tc_fence_after();
+                    const uint64_t da = ptx::smem_desc_sw128(a0 + (uint32_t)j * (ROWS * CL_KS * 2));
+                    const uint64_t db = ptx::smem_desc_plain(b0 + (uint32_t)j * (8 * N * 16), N * 16, 128);
+#pragma unroll
+                    for (int q = 0; q < CL_KS / 16; ++q)
+                        ptx::mma_f16_ss(d, da + (uint64_t)(2 * q), db + (uint64_t)(q * 2) * N, idesc, (i | j | q) != 0 ? 1u : 0u);
                 }
-                if (ok) ptx::mma_commit(acc + 8 * (n_acc & 1));
-                ++n_acc;
-                // what the next exchange of this operand brings (its first bytes may come before this, but not its last:
-                // the barrier waits for this arrival)
-                for (int p = 0; direct && ok && !in && p < P.n_ctas; ++p)
-                    if (p != rank) ptx::mbar_arrive_expect_tx(src + 8 * p, part);
-                if (in) ph_x ^= 1;
-                else if (odd) ph_u ^= 1;
-                else ph_a ^= 1;
+                if (!ok) break;
+                ptx::mma_commit(empty + 8 * st);
+                if (++st == lay.stages) { st = 0; ph ^= 1u; }
+                if (++kp == n) kp = 0;
             }
+            if (ok) ptx::mma_commit(acc + 8 * (n_acc & 1));
+            ++n_acc;
+            // what the next exchange of this operand brings (its first bytes may come before this, but not its last:
+            // the barrier waits for this arrival)
+            for (int p = 0; direct && ok && !in && p < P.n_ctas; ++p)
+                if (p != rank) ptx::mbar_arrive_expect_tx(src + 8 * p, part);
+            if (in) ph_x ^= 1;
+            else if (odd) ph_u ^= 1;
+            else ph_a ^= 1;
+        }
     // all products are done before tensor memory is freed
     ptx::mma_commit(ptx::smem_u32(&B.drain));
     drain_mbar(ptx::smem_u32(&B.drain), 0);
@@ -570,36 +564,35 @@ __device__ __forceinline__ void cluster_mma(const ClusterParams& P, int units, i
 // One thread: u and a of the other CTAs from L2, when all have said that their parts are there (a wait for each, with the
 // fences it needs, took 1000 cycles a CTA).
 template <int ROWS>
-__device__ __forceinline__ void cluster_fetch(const ClusterParams& P, int units, int n_groups, int cluster, int n_clusters,
-                                              int rank, const ClusterLayout& lay, uint32_t smem, ClusterBars& B, ClusterWait& wait) {
+__device__ __forceinline__ void cluster_fetch(const ClusterParams& P, int units, int cluster, int rank, const ClusterLayout& lay,
+                                              uint32_t smem, ClusterBars& B, ClusterWait& wait) {
     if (lay.act <= P.direct_bytes) return;
     const uint32_t part = ROWS * 2 * (uint32_t)units * CL_UNIT, acc = ptx::smem_u32(B.acc);
     const uint8_t* xch = P.xch + (size_t)cluster * 2 * lay.act;
     uint32_t ph_u = 0, ph_a = 0, n_acc = 0;
     bool ok = true;
-    for (int grp = cluster; ok && grp < n_groups; grp += n_clusters)
-        for (int k = 0; ok && k < P.K; ++k) {
-            ++n_acc;                                          // the in-projection
-            for (int l = 1; ok && l < 2 * P.L + 2; ++l, ++n_acc) {
-                const bool odd = l & 1;                       // u, else a
-                const uint32_t act = smem + (odd ? lay.u : lay.a), src = ptx::smem_u32(odd ? B.src_u : B.src_a);
-                const uint32_t sig = ptx::smem_u32(&B.sig[odd ? 0 : 1]), phase = odd ? ph_u : ph_a;
-                const uint8_t* from = odd ? xch : xch + lay.act;
-                // where they share a buffer a takes u's place when the products of u are done (u takes a's when all CTAs
-                // have sent their partials of the LayerNorm that it comes from, this one among them: after its products)
-                if (!odd && lay.bufs == 1) ok = wait.mbar(acc + 8 * ((n_acc - 1) & 1), ((n_acc - 1) >> 1) & 1);
-                ok = ok && wait.template mbar<true>(sig, phase);
-                if (ok) ptx::fence_proxy_async();
-                int s = rank;
-                for (int i = 1; ok && i < P.n_ctas; ++i) {
-                    if (++s == P.n_ctas) s = 0;
-                    ptx::mbar_arrive_expect_tx(src + 8 * s, part);
-                    ptx::bulk_load(act + (uint32_t)s * part, from + (size_t)s * part, part, src + 8 * s);
-                }
-                if (odd) ph_u ^= 1;
-                else ph_a ^= 1;
+    for (int k = 0; ok && k < P.K; ++k) {
+        ++n_acc;                                          // the in-projection
+        for (int l = 1; ok && l < 2 * P.L + 2; ++l, ++n_acc) {
+            const bool odd = l & 1;                       // u, else a
+            const uint32_t act = smem + (odd ? lay.u : lay.a), src = ptx::smem_u32(odd ? B.src_u : B.src_a);
+            const uint32_t sig = ptx::smem_u32(&B.sig[odd ? 0 : 1]), phase = odd ? ph_u : ph_a;
+            const uint8_t* from = odd ? xch : xch + lay.act;
+            // where they share a buffer a takes u's place when the products of u are done (u takes a's when all CTAs
+            // have sent their partials of the LayerNorm that it comes from, this one among them: after its products)
+            if (!odd && lay.bufs == 1) ok = wait.mbar(acc + 8 * ((n_acc - 1) & 1), ((n_acc - 1) >> 1) & 1);
+            ok = ok && wait.template mbar<true>(sig, phase);
+            if (ok) ptx::fence_proxy_async();
+            int s = rank;
+            for (int i = 1; ok && i < P.n_ctas; ++i) {
+                if (++s == P.n_ctas) s = 0;
+                ptx::mbar_arrive_expect_tx(src + 8 * s, part);
+                ptx::bulk_load(act + (uint32_t)s * part, from + (size_t)s * part, part, src + 8 * s);
             }
+            if (odd) ph_u ^= 1;
+            else ph_a ^= 1;
         }
+    }
     // (after a normal run all of them have landed: the products waited for them; after an abort the kernel waits)
 }
 
@@ -621,13 +614,10 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cluster_kernel(const __grid_con
     }
     ptx::wait_for_prior_kernel();
     const int n_ctas = P.n_ctas, rank = (int)blockIdx.x % n_ctas, cluster = (int)blockIdx.x / n_ctas;
-    const int n_clusters = (int)gridDim.x / n_ctas;
-    // units of 16 tokens dealt evenly to the clusters, in as many rounds as they need
-    const int all_units = (S + CL_UNIT - 1) / CL_UNIT;
-    const int rounds = max(1, (all_units + n_clusters * P.max_units - 1) / (n_clusters * P.max_units));
-    const int units = max(1, (all_units + n_clusters * rounds - 1) / (n_clusters * rounds));
-    const int n_groups = (all_units + units - 1) / units;
-    if (cluster >= n_groups) return;            // (all CTAs of the cluster)
+    // units of 16 tokens dealt evenly to the clusters (one round of groups: the host's limit, cluster_survivors)
+    const int n_clusters = (int)gridDim.x / n_ctas, all_units = (S + CL_UNIT - 1) / CL_UNIT;
+    const int units = (all_units + n_clusters - 1) / n_clusters;
+    if (cluster * units >= all_units) return;   // (all CTAs of the cluster)
     const ClusterLayout lay(P.W, P.C, ROWS, units);
     const uint32_t smem = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -661,20 +651,24 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cluster_kernel(const __grid_con
     if (gave_up) {
         // nothing to work on
     } else if (warp == 0) {
-        if (ptx::elect_one()) cluster_feed<ROWS>(P, n_groups, cluster, n_clusters, rank, lay, smem, B, wait);
+        if (ptx::elect_one()) cluster_feed<ROWS>(P, rank, lay, smem, B, wait);
         __syncwarp();
     } else if (warp == 1) {
-        if (ptx::elect_one()) cluster_mma<ROWS>(P, units, n_groups, cluster, n_clusters, rank, lay, smem, tmem, B, wait);
+        if (ptx::elect_one()) cluster_mma<ROWS>(P, units, rank, lay, smem, tmem, B, wait);
         __syncwarp();
     } else if (warp == 10) {
-        if (ptx::elect_one()) cluster_fetch<ROWS>(P, units, n_groups, cluster, n_clusters, rank, lay, smem, B, wait);
+        if (ptx::elect_one()) cluster_fetch<ROWS>(P, units, cluster, rank, lay, smem, B, wait);
         __syncwarp();
     } else {
+        auto run = [&](auto g) {
+            if constexpr (decltype(g)::value <= cl_most_units(ROWS))
+                ClusterEpilogue<ROWS, decltype(g)::value>::run(P, S, cluster, rank, smem, tmem, B, warp - 2, lane, wait);
+        };
         switch (units) {
-            case 1: ClusterEpilogue<ROWS, 1>::run(P, S, n_groups, cluster, n_clusters, rank, smem, tmem, B, warp - 2, lane, wait); break;
-            case 2: ClusterEpilogue<ROWS, 2>::run(P, S, n_groups, cluster, n_clusters, rank, smem, tmem, B, warp - 2, lane, wait); break;
-            case 3: ClusterEpilogue<ROWS, 3>::run(P, S, n_groups, cluster, n_clusters, rank, smem, tmem, B, warp - 2, lane, wait); break;
-            case 4: ClusterEpilogue<ROWS, 4>::run(P, S, n_groups, cluster, n_clusters, rank, smem, tmem, B, warp - 2, lane, wait); break;
+            case 1: run(std::integral_constant<int, 1>{}); break;
+            case 2: run(std::integral_constant<int, 2>{}); break;
+            case 3: run(std::integral_constant<int, 3>{}); break;
+            case 4: run(std::integral_constant<int, 4>{}); break;
             default: break;
         }
         __syncwarp();

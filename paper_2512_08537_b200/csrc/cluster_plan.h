@@ -67,9 +67,11 @@ inline int cluster_rows(int W, int64_t max_tokens) {
             return rows;
     return 0;
 }
-// Most units of 16 tokens that a cluster takes at once.
+// Most units of 16 tokens that a cluster takes at once: as many as fit, where a split can need them (64 columns a CTA are for heads
+// of at most CL_FEW_TOKENS = 64 tokens, and on any device with 4 such clusters one unit each is all of them; 96 are for W = 1536).
+ARDIFF_HD constexpr int cl_most_units(int rows) { return rows == 64 ? 1 : rows == 96 ? 2 : CL_MAX_UNITS; }
 inline int cluster_units(int W, int C, int rows) {
-    int units = CL_MAX_UNITS;
+    int units = cl_most_units(rows);
     while (units > 0 && ClusterLayout(W, C, rows, units).stages < CL_MIN_STAGES) --units;
     return units;
 }

@@ -41,6 +41,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/ardiff.h"
@@ -2059,7 +2060,7 @@ int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise,
     if (few_count > chain_count && H->d.max_tokens > chain_count) {
         ClusterParams R;
         memset(&R, 0, sizeof(R));
-        R.C = C; R.W = W; R.L = H->d.L; R.K = K; R.n_ctas = W / H->cl_rows; R.max_units = H->cl_units;
+        R.C = C; R.W = W; R.L = H->d.L; R.K = K; R.n_ctas = W / H->cl_rows;
         R.above = chain_count; R.limit = few_count;
         R.max_tokens = P.max_tokens; R.map_cat = MAP_CL; R.map_in = MAP_CL + 1; R.map_out = MAP_CL + 2;
         R.out_row0 = H->out_row0; R.maps = H->maps; R.idx = idx; R.count = count; R.bias_cat = H->bias_cat; R.bin = H->bin;
