@@ -1,5 +1,7 @@
-// The head's chain of dependent layers for calls of few tokens (at most CHAIN_MAX_TOKENS survivors; beside the clusters of
-// cluster.cuh at most 32, and where it is the faster one: chain_beside_clusters).
+// The head's chain of dependent layers for calls of few tokens: at most 32 beside the clusters of cluster.cuh, of heads 768 and
+// more wide, where it is the faster one (chain_beside_clusters); up to CHAIN_MAX_TOKENS at any width, in two passes, on a device
+// that takes no clusters of this size. (Without the second pass, which a whole B200 never runs, the compiler's code for the
+// first is slower: W = 1536, 12 blocks, 28 tokens 728 -> 773 us, W = 1024, one token 153 -> 165.)
 //
 // With few tokens the head is K * (3 L + 3) exchanges between SMs in a row, and a call takes as long as they do: the tile
 // schedule spends 5 to 12 us on each (TMA round trip, K loop, epilogue, store completion, release, poll). There it
