@@ -293,11 +293,15 @@ int ardiff_head_status(ardiff_head* head, void* stream);
  * ardiff_head_set_cooperative(head, 0) launches the head kernel without the cooperative attribute,
  * for profilers that cannot replay cooperative launches; the kernel and its grid are unchanged, but
  * the launch no longer fails when the GPU cannot hold the whole grid at once (then waits run into
- * their bound and ARDIFF_ERR_TIMEOUT is reported). Default: on. */
+ * their bound and ARDIFF_ERR_TIMEOUT is reported). Default: on.
+ * ardiff_head_few_limits tells which schedule serves a call of K steps (1 .. K_max): up to *chain survivors
+ * the one with an exchange per layer, above those and up to *clusters the clusters (equal where there are
+ * none), above both the tiles. */
 int ardiff_head_set_timing(ardiff_head* head, int on);
 int ardiff_head_last_kernel_ms(ardiff_head* head, float* ms);
 int ardiff_head_last_kernel_clock(ardiff_head* head, void* stream, double* sm_mhz);
 int ardiff_head_set_cooperative(ardiff_head* head, int on);
+int ardiff_head_few_limits(const ardiff_head* head, int32_t K, int32_t* chain, int32_t* clusters);
 
 /* Self-test of the bounded device-side waits. Arms the NEXT ardiff_head_sample call on this head:
  * its dependency waits give up after wait_limit_us microseconds (100 .. 4 000 000) instead of the

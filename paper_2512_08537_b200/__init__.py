@@ -92,6 +92,8 @@ def lib() -> ctypes.CDLL:
         L.ardiff_head_last_kernel_clock.argtypes = [vp, vp, ctypes.POINTER(ctypes.c_double)]
         L.ardiff_head_set_cooperative.restype = ctypes.c_int
         L.ardiff_head_set_cooperative.argtypes = [vp, ctypes.c_int]
+        L.ardiff_head_few_limits.restype = ctypes.c_int
+        L.ardiff_head_few_limits.argtypes = [vp, i32, ctypes.POINTER(i32), ctypes.POINTER(i32)]
         L.ardiff_head_inject_stall.restype = ctypes.c_int
         L.ardiff_head_inject_stall.argtypes = [vp, i32, ctypes.c_uint32]
         L.ardiff_pipeline_create_slots.restype = ctypes.c_int
@@ -342,6 +344,12 @@ class Head:
     def set_cooperative(self, on: bool):
         fn = lib().ardiff_head_set_cooperative
         _check(fn(self._h, 1 if on else 0), "ardiff_head_set_cooperative")
+
+    def few_limits(self, K: int):
+        """(chain, clusters): the survivors up to which a call of K steps takes either schedule; above both it takes the tiles."""
+        chain, clusters = ctypes.c_int32(0), ctypes.c_int32(0)
+        _check(lib().ardiff_head_few_limits(self._h, K, ctypes.byref(chain), ctypes.byref(clusters)), "ardiff_head_few_limits")
+        return int(chain.value), int(clusters.value)
 
     def inject_stall(self, token_tile: int, wait_limit_us: int):
         """Arms the bounded-wait self-test for the next sample call (see ardiff_head_inject_stall)."""

@@ -2156,6 +2156,13 @@ extern "C" int ardiff_head_set_cooperative(ardiff_head* H, int on) {
     return ARDIFF_OK;
 }
 
+extern "C" int ardiff_head_few_limits(const ardiff_head* H, int32_t K, int32_t* chain, int32_t* clusters) {
+    if (!H || !chain || !clusters) return ARDIFF_ERR_NULL;
+    if (K < 1 || K > H->d.K_max) return ARDIFF_ERR_SHAPE;
+    few_limits(H, K, chain, clusters);
+    return ARDIFF_OK;
+}
+
 extern "C" int ardiff_head_inject_stall(ardiff_head* H, int32_t token_tile, uint32_t wait_limit_us) {
     if (!H) return ARDIFF_ERR_NULL;
     if (token_tile < 0 || wait_limit_us < 100 || wait_limit_us > 4000000u) return ARDIFF_ERR_SHAPE;

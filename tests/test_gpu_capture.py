@@ -1,4 +1,4 @@
-"""Gate calls inside a stream capture after one call outside it.
+"""Gate and head calls inside a stream capture after one call outside it.
 
 One call of an entry point on a device loads all its row kernels (which takes device memory): calls of any other width and
 number of rows take none and may be captured. Each case runs in a fresh process, where no kernel has been loaded before that call.
@@ -65,3 +65,44 @@ def test_any_width_can_be_captured_after_one_call(kind, first):
                        capture_output=True, text=True)
     print(r.stdout[-500:])
     assert r.returncode == 0, r.stdout[-1000:] + r.stderr[-1500:]
+
+
+@pytest.mark.parametrize("W,counts", [(256, (300, 33, 4900)), (1536, (20, 200, 1000)), (2304, (60, 700))])
+def test_a_captured_head_call_follows_the_count(W, counts):
+    """One captured head call, its launches over the one before included, replayed with the count of every schedule in turn
+    (clusters, chain at W = 1536, tiles): the bits of eager calls, and again after them."""
+    import numpy as np
+    import torch
+    import synth
+    import paper_2512_08537_b200 as ardiff
+    dev = require_cuda()
+    wl = synth.workload("cfg1", n=max(counts), W=W, L=2, K=2, Dc=128)
+    head = ardiff.Head(wl.C, wl.Dc, wl.W, wl.L, wl.F, wl.K, wl.n, synth.head_weights(wl))
+    chain, clusters = head.few_limits(wl.K)
+    assert clusters < max(counts) and (W > 2048 or sorted(counts)[-2] > chain) and (W != 1536 or min(counts) <= chain)
+    gen = torch.Generator(device=dev).manual_seed(2)
+    cond = torch.randn((wl.n, wl.Dc), device=dev, generator=gen).to(torch.bfloat16)
+    noise = torch.randn((wl.n, wl.C), device=dev, generator=gen)
+    idx = torch.randperm(wl.n, device=dev, generator=gen).to(torch.int32)
+    count, out, t = torch.zeros(1, dtype=torch.int32, device=dev), torch.zeros_like(noise), synth.t_sched(wl.K)
+
+    def run(call, c):
+        count.fill_(c)
+        out.fill_(-5.0)
+        call()
+        assert head.status() == 0
+        return out.cpu().numpy()
+
+    def eager():
+        head.ardiff_head_sample(cond, noise, t, idx, count, out)
+
+    want = {c: run(eager, c) for c in counts}
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=side):
+        eager()
+    for c in counts + counts[::-1]:
+        assert np.array_equal(run(graph.replay, c), want[c]), c
+    assert np.array_equal(run(eager, counts[0]), want[counts[0]])
+    del graph
+    head.close()

@@ -101,9 +101,9 @@ def test_small_head_ragged_counts(std, count):
 
 @pytest.mark.parametrize("count", [512, 513, 3072, 3073, 23808, 23809, 26112, 26113])
 def test_item_width_boundaries(count):
-    """The last token count of each item width and the first of the next one (W = 512 on 148 SMs: 64 output columns
-    per item up to 2 pairs of token tiles, 128 up to 12, then 256), of a group of the usual size (93 pairs), and of a lone
-    group (102). Tolerance: the agreement bar of this file."""
+    """The last token count of 128-column items and the first of 256 (W = 512 on 148 SMs: 12 pairs of token tiles), of a group of
+    the usual size (93 pairs), and of a lone group (102). (512 and 513 are the clusters'; items of 64 columns: the test below.)
+    Tolerance: the agreement bar of this file."""
     wl = synth.workload("cfg1", n=count + 5, W=512, L=2, K=2)
     w, cond_bits, noise, t = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
     idx = np.random.default_rng(count).permutation(wl.n)[:count].astype(np.int32)
@@ -116,17 +116,37 @@ def test_item_width_boundaries(count):
     head.close()
 
 
+@pytest.mark.parametrize("count", [104, 105, 1024, 1025, 6144, 6145])
+def test_item_widths_where_the_modulations_hold_few_tokens(count):
+    """64 steps of 12 blocks, W = 256: 256 MB of modulations are those of 104 survivors, so that the tiles begin there, with items
+    of 64 columns up to 4 pairs of token tiles, then 128 up to 24, then 256. Tolerance: the agreement bar of this file."""
+    wl = synth.workload("cfg1", n=6150, W=256, L=12, K=64)
+    w, cond_bits, noise, t = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
+    idx = np.random.default_rng(count).permutation(wl.n)[:count].astype(np.int32)
+    rows = idx[np.unique(np.concatenate([[0, 63, 64, count // 2, count - 1], np.random.default_rng(2).integers(0, count, 16)]))]
+    want = oracle.head_sample(w, cond_bits, noise, t, rows)
+    head = make_head(wl, w)
+    assert head.few_limits(wl.K) == (0, 104)
+    got = run_head(head, cond_bits, noise, t, idx)
+    assert_parity(got, want, rows)
+    assert np.all(got[np.setdiff1d(np.arange(wl.n), idx)] == SENTINEL)
+    head.close()
+
+
+@pytest.mark.parametrize("n", [64, 80])
 @pytest.mark.parametrize("W", [256, 512, 768, 1024, 1280, 1536, 1792, 2048, 2304])
-def test_few_tokens_at_every_width(W):
-    """Up to 64 survivors the chain of layers leaves the tile schedule (one instance per W / 256 up to 8): one token, a
-    ragged token tile, a second pass, the last count it takes and the first that it does not; the same call twice gives
-    the same bits. Tolerance: the agreement bar of this file."""
-    wl = synth.workload("cfg1", n=80, W=W, L=2, K=3, C=32 if W % 512 else 64, Dc=192)
+def test_few_tokens_at_every_width(W, n):
+    """One token, the chain where it serves some (its last count and the first of the clusters), ragged token tiles, and up to
+    the 64 tokens of heads that split a layer over as many CTAs as a cluster may have (n = 64: 64 columns each up to W = 1024);
+    no such schedule above W = 2048. The same call twice gives the same bits. Tolerance: the agreement bar of this file."""
+    wl = synth.workload("cfg1", n=n, W=W, L=2, K=3, C=32 if W % 512 else 64, Dc=192)
     w, cond_bits, noise, t = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
     order = np.random.default_rng(W).permutation(wl.n).astype(np.int32)
     want = oracle.head_sample(w, cond_bits, noise, t, order[:65])
     head = make_head(wl, w)
-    for count in (1, 9, 33, 64, 65):
+    chain, clusters = head.few_limits(wl.K)
+    assert (chain > 0) == (1024 <= W <= 2048) and (clusters >= 64) == (W <= 2048)
+    for count in sorted({1, 9, 33, 64, min(n, 65), chain or 2, chain + 1}):
         idx = order[:count]
         got = run_head(head, cond_bits, noise, t, idx)
         assert_parity(got, want, idx, f"{count} tokens")
@@ -135,25 +155,28 @@ def test_few_tokens_at_every_width(W):
     head.close()
 
 
-@pytest.mark.parametrize("W,counts", [(256, (80, 81, 2112, 4224, 4225, 4737)), (512, (129, 1600, 2112, 2113)),
-                                      (768, (100, 337, 1300)), (1024, (240, 241, 481, 720, 721)),
-                                      (1280, (32, 33, 177, 353, 529)), (1536, (32, 33, 112, 113, 224, 225)),
-                                      (1792, (33, 112, 225)), (2048, (32, 33, 112, 113, 224, 225))])
-def test_token_groups_of_the_clusters(W, counts):
-    """Clusters of W / 128 CTAs take groups of 16, 32, 48 or 64 tokens: counts on both sides of where the group grows, where the
-    values go through L2 instead of directly, and of the last that fits (on 148 SMs); a ragged last group; fresh noise; the
-    same call twice gives the same bits. Tolerance: the agreement bar of this file."""
+@pytest.mark.parametrize("W,n,counts", [(256, 4740, (80, 81, 1184, 2112, 3552, 3553)), (512, 2116, (129, 528, 529, 1600)),
+                                        (768, 1412, (100, 337, 1300)), (1024, 964, (240, 241, 481, 720, 721)),
+                                        (1280, 532, (32, 33, 177, 353)), (1536, 228, (32, 33, 112, 113)),
+                                        (1792, 228, (33, 112, 113)), (2048, 228, (32, 33, 112, 113))])
+def test_token_groups_of_the_clusters(W, n, counts):
+    """Clusters of W / 128 CTAs (W / 96 at 1536) take groups of 16, 32, 48 or 64 tokens: counts on both sides of where the group
+    grows, where the values go through L2 instead of directly, the last that they serve and the first that they do not; a
+    ragged last group; fresh noise; the same call twice gives the same bits. Tolerance: the agreement bar of this file."""
     dev = require_cuda()
-    wl = synth.workload("cfg1", n=max(counts) + 3, W=W, L=2, K=2, C=48 if W % 512 else 16, Dc=128)
+    wl = synth.workload("cfg1", n=n, W=W, L=2, K=2, C=48 if W % 512 else 16, Dc=128)
     w, cond_bits, noise = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl)
     t_in = np.array([0.9, 0.4], np.float32)
     coef = np.array([[0.4, 0.7, 0.5], [0.2, 1.0, 0.1]], np.float32)
     z = np.random.default_rng(9).standard_normal((2, wl.n, wl.C)).astype(np.float32)
     order = np.random.default_rng(W).permutation(wl.n).astype(np.int32)
+    head = make_head(wl, w)
+    chain, last = head.few_limits(wl.K)
+    assert chain <= 32 and max(counts) <= last < n
+    counts = counts + (last, last + 1)
     pos = np.unique(np.concatenate([[0, 15, 16, 31, 47, 63], np.array(counts) - 1, np.random.default_rng(1).integers(0, max(counts), 24)]))
     want = np.zeros((wl.n, wl.C))
     want[order[pos]] = oracle.head_sample_coef(w, cond_bits, noise, t_in, coef, order[pos], step_noise=z)[order[pos]]
-    head = make_head(wl, w)
     cond, noise_d, z_d = dev_bf16(cond_bits), dev_f32(noise), torch.from_numpy(z).to(dev)
     for count in counts:
         outs = []
@@ -171,17 +194,18 @@ def test_token_groups_of_the_clusters(W, counts):
 
 
 def test_few_token_limit_set_by_the_buffers():
-    """64 steps of 12 blocks: the few-token buffers (128 MB of modulations) hold 26 survivors. The last count that they serve
+    """64 steps of 12 blocks: the modulations (at most 256 MB) are those of 48 survivors. The last count that the clusters serve
     and the first that they do not. Tolerance: the agreement bar of this file."""
-    wl = synth.workload("cfg1", n=40, W=512, L=12, K=64)
+    wl = synth.workload("cfg1", n=64, W=512, L=12, K=64)
     w, cond_bits, noise, t = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
     order = np.random.default_rng(26).permutation(wl.n).astype(np.int32)
-    rows = order[[0, 7, 25, 26]]
+    rows = order[[0, 7, 47, 48]]
     want = oracle.head_sample(w, cond_bits, noise, t, rows)
     head = make_head(wl, w)
-    for count in (26, 27):
+    assert head.few_limits(64) == (0, 48) and head.few_limits(32)[1] >= 64
+    for count in (48, 49):
         got = run_head(head, cond_bits, noise, t, order[:count])
-        assert_parity(got, want, rows[:3] if count == 26 else rows, f"{count} tokens")
+        assert_parity(got, want, rows[:3] if count == 48 else rows, f"{count} tokens")
         assert np.all(got[np.setdiff1d(np.arange(wl.n), order[:count])] == SENTINEL)
     head.close()
 
@@ -208,6 +232,7 @@ def test_head_without_room_for_the_few_token_buffers():
     held = torch.empty(free - taken + (120 << 20), dtype=torch.uint8, device=dev)
     try:
         head = make_head(wl, w)
+        assert head.few_limits(2) == (0, 0)
         got = run_head(head, cond_bits, noise, t, idx)
         assert_parity(got, want, idx)
         head.close()
@@ -369,6 +394,43 @@ def test_full_size_runs_are_bit_identical(name, runs, K):
     head.close()
 
 
+@pytest.mark.parametrize("W,n,few", [(1536, 300, (17, 23)), (256, 2000, (300, 1100)), (1024, 900, (200, 470)),
+                                     (1024, 960, (700, 941)), (2048, 300, (100, 220))])
+def test_few_token_runs_are_bit_identical(W, n, few):
+    """The same for the chain (first) and the clusters (values copied between shared memories, and through L2): a flush, another
+    call of the head and a busy second stream between and beside the runs."""
+    dev = require_cuda()
+    wl = synth.workload("cfg1", n=n, W=W, L=3, K=4, Dc=256)
+    w, t = synth.head_weights(wl, std=None), synth.t_sched(wl.K)
+    cond, noise = dev_bf16(synth.cond(wl)), dev_f32(synth.noise(wl))
+    head = make_head(wl, w)
+    chain, clusters = head.few_limits(wl.K)
+    assert max(few) <= (chain if W == 1536 else clusters) and (W == 1536 or min(few) > chain)
+    idx = torch.randperm(n, device=dev, generator=torch.Generator(device=dev).manual_seed(3)).to(torch.int32)
+    counts = [torch.tensor([c], dtype=torch.int32, device=dev) for c in few]
+    flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
+    busy = torch.randn(1 << 22, device=dev)
+    side = torch.cuda.Stream(device=dev)
+    ref = [None, None]
+    for r in range(24):
+        if r % 3 == 0:
+            flush.fill_(r)
+        if r % 4 == 1:
+            side.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(side):
+                for _ in range(r):
+                    busy = busy * 1.0001
+        k = int(r % 5 in (1, 3))
+        out = torch.full((n, wl.C), SENTINEL, dtype=torch.float32, device=dev)
+        head.ardiff_head_sample(cond, noise, t, idx, counts[k], out)
+        assert head.status() == 0
+        if ref[k] is None:
+            ref[k] = out
+        assert torch.equal(out, ref[k]), f"run {r} with {few[k]} tokens differs"
+    torch.cuda.synchronize()
+    head.close()
+
+
 @pytest.mark.parametrize("name,extra,K", [("cfg2", 160, None), ("cfg3", 48, None), ("cfg4", 32, None),
                                           ("cfg3", 24, 1), ("cfg3", 12, 8)])
 def test_workload_configs_sampled_tokens(name, extra, K):
@@ -418,12 +480,13 @@ def test_workload_configs_sampled_tokens(name, extra, K):
     head.close()
 
 
-def test_two_heads_on_two_streams():
-    """Two heads of different shapes, driven from two streams without any ordering between them: every
-    launch needs the whole GPU (cooperative launch), so the launches take turns; both results must
-    match what each head gives alone."""
+@pytest.mark.parametrize("na,nb", [(700, 900), (4900, 2300), (4900, 900)])
+def test_two_heads_on_two_streams(na, nb):
+    """Two heads of different shapes, driven from two streams without any ordering between them, with the clusters, with tiles and
+    one with each: every launch of the head kernel needs the whole GPU (cooperative launch), so the launches take turns; both
+    results must match what each head gives alone."""
     dev = require_cuda()
-    wa, wb = synth.workload("cfg1", n=700), synth.workload("cfg1", n=900, W=512, L=3, seed=77)
+    wa, wb = synth.workload("cfg1", n=na), synth.workload("cfg1", n=nb, W=512, L=3, seed=77)
     outs = {}
     heads = {}
     for key, wl in (("a", wa), ("b", wb)):
@@ -435,6 +498,7 @@ def test_two_heads_on_two_streams():
         alone = torch.empty((wl.n, wl.C), dtype=torch.float32, device=dev)
         head.ardiff_head_sample(cond, noise, t, idx, count, alone)
         heads[key] = (head, cond, noise, t, idx, count, alone, wl)
+        assert (head.few_limits(wl.K)[1] < wl.n) == (wl.n > 1000)
     torch.cuda.synchronize()
     streams = {k: torch.cuda.Stream(device=dev) for k in heads}
     for rep in range(4):
@@ -541,16 +605,36 @@ def test_extreme_shapes(shape):
     head.close()
 
 
-def test_bounded_wait_runs_out_reports_timeout_and_the_head_recovers():
-    """The self-test hook makes one tile's dependency wait unsatisfiable and shortens the wait limit to 3 ms:
+@pytest.mark.parametrize("shape", [dict(W=256, L=5, K=3, C=48, Dc=1024, n=4800), dict(W=512, L=1, K=64, C=16, Dc=64, n=420),
+                                   dict(W=256, L=64, K=1, C=16, Dc=64, n=1500), dict(W=512, L=2, K=2, C=16, Dc=128, F=1024, n=2200)])
+def test_extreme_shapes_beyond_the_clusters(shape):
+    """The same with more tokens than the clusters serve: an odd number of blocks, the largest step count, the deepest head, the
+    largest time embedding with the tiles. The oracle takes some tokens of the first, a middle and the last token tile."""
+    shape = dict(shape)
+    n = shape.pop("n")
+    wl = synth.workload("cfg1", n=n, **shape)
+    w, cond_bits, noise, t = synth.head_weights(wl), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
+    idx = np.arange(n, dtype=np.int32)
+    rows = sample_tokens(idx, extra=16)[::5]
+    want = oracle.head_sample(w, cond_bits, noise, t, rows)
+    head = make_head(wl, w)
+    assert head.few_limits(wl.K)[1] < n
+    assert_parity(run_head(head, cond_bits, noise, t, idx), want, rows, str(shape))
+    head.close()
+
+
+@pytest.mark.parametrize("n,tiles", [(900, (0, 3, 7)), (5000, (0, 3, 39))])
+def test_bounded_wait_runs_out_reports_timeout_and_the_head_recovers(n, tiles):
+    """(900 tokens: what precedes the clusters, which then leave at once; 5000: the tile schedule.) The self-test hook makes one tile's dependency wait unsatisfiable and shortens the wait limit to 3 ms:
     the kernel must come back by itself (no fault, no trap, no endless spin), the status word must say
     TIMEOUT, and the very next call on the same head must give the bits of an undisturbed run."""
-    wl = synth.workload("cfg1", n=900)
+    wl = synth.workload("cfg1", n=n)
     w, cond_bits, noise, t = synth.head_weights(wl), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
     idx = np.arange(wl.n, dtype=np.int32)
     head = make_head(wl, w)
+    assert (head.few_limits(wl.K)[1] < n) == (n == 5000)
     clean = run_head(head, cond_bits, noise, t, idx)
-    for tile in (0, 3, 7):                                # first, an odd (partner CTA) and the last, ragged tile
+    for tile in tiles:                                    # first, an odd (partner CTA) and the last, ragged tile
         head.inject_stall(tile, 3000)
         dev = require_cuda()
         out = torch.zeros(noise.shape, dtype=torch.float32, device=dev)
