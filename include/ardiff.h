@@ -310,8 +310,12 @@ int ardiff_head_few_limits(const ardiff_head* head, int32_t K, int32_t* chain, i
  * abort flag, every CTA leaves its loops, waits for its own copies in flight, frees its tensor
  * memory and returns; ardiff_head_status reports ARDIFF_ERR_TIMEOUT and the call's results are
  * invalid. Nothing faults or traps, and the call after it runs normally. A token_tile beyond the
- * tiles of that call has no effect. */
+ * tiles of that call has no effect.
+ * ardiff_head_inject_cluster_stall does the same for a wait inside the clusters: the last CTA of cluster
+ * `cluster` (of those that the call's tokens need) gets no weights from the second layer of the first
+ * block on, so that all others of the cluster wait for it. */
 int ardiff_head_inject_stall(ardiff_head* head, int32_t token_tile, uint32_t wait_limit_us);
+int ardiff_head_inject_cluster_stall(ardiff_head* head, int32_t cluster, uint32_t wait_limit_us);
 
 /* ---------------------------------------------------------------------------------------
  * Host-buffer front end: one call takes a batch that lives in HOST memory through the whole

@@ -96,6 +96,8 @@ def lib() -> ctypes.CDLL:
         L.ardiff_head_few_limits.argtypes = [vp, i32, ctypes.POINTER(i32), ctypes.POINTER(i32)]
         L.ardiff_head_inject_stall.restype = ctypes.c_int
         L.ardiff_head_inject_stall.argtypes = [vp, i32, ctypes.c_uint32]
+        L.ardiff_head_inject_cluster_stall.restype = ctypes.c_int
+        L.ardiff_head_inject_cluster_stall.argtypes = [vp, i32, ctypes.c_uint32]
         L.ardiff_pipeline_create_slots.restype = ctypes.c_int
         L.ardiff_pipeline_create_slots.argtypes = [vp, i64, i32, i32, i32, i32, ctypes.POINTER(vp)]
         L.ardiff_pipeline_submit.restype = ctypes.c_int
@@ -355,6 +357,10 @@ class Head:
         """Arms the bounded-wait self-test for the next sample call (see ardiff_head_inject_stall)."""
         fn = lib().ardiff_head_inject_stall
         _check(fn(self._h, token_tile, wait_limit_us), "ardiff_head_inject_stall")
+
+    def inject_cluster_stall(self, cluster: int, wait_limit_us: int):
+        """The same for a wait inside a cluster (see ardiff_head_inject_cluster_stall)."""
+        _check(lib().ardiff_head_inject_cluster_stall(self._h, cluster, wait_limit_us), "ardiff_head_inject_cluster_stall")
 
     def close(self):
         if getattr(self, "_h", None) is not None and self._h:

@@ -34,6 +34,7 @@ struct ClusterParams {
     uint8_t* xch;                              // u and a of every cluster
     int *status, *abort_flag;
     unsigned long long wait_limit_ns;
+    int stall_cluster;                         // self-test: this cluster's last CTA gets no weights after the first block's W1 (-1: none)
     float ax[KMAX], av[KMAX], an[KMAX];
 };
 
@@ -456,7 +457,7 @@ struct ClusterEpilogue {
 // One thread: the weight slices in the order they are used. A layer's K slices start with the CTA's own channels, whose
 // activations are there first.
 template <int ROWS>
-__device__ __forceinline__ void cluster_feed(const ClusterParams& P, int rank, const ClusterLayout& lay, uint32_t ring,
+__device__ __forceinline__ void cluster_feed(const ClusterParams& P, int cluster, int rank, const ClusterLayout& lay, uint32_t ring,
                                              ClusterBars& B, ClusterWait& wait) {
     const uint32_t full = ptx::smem_u32(B.full), empty = ptx::smem_u32(B.empty);
     constexpr int SL = cl_slices(ROWS), SRCS = SL * CL_KS / ROWS;
@@ -473,6 +474,10 @@ __device__ __forceinline__ void cluster_feed(const ClusterParams& P, int rank, c
             const int row = in ? rank * ROWS : out ? (int)P.out_row0 : (5 * ((l - 1) >> 1) + 3 + ((l - 1) & 1)) * W + rank * ROWS;
             const uint32_t bytes = (uint32_t)(out ? P.C : ROWS) * CL_KS * 2 * sl;
             int kp = in ? 0 : rank / SRCS;
+            if (l == 2 && cluster == P.stall_cluster && rank == P.n_ctas - 1) {      // self-test (nothing ends this wait)
+                ok = wait.mbar(ptx::smem_u32(&B.drain), 0);
+                break;
+            }
             for (int i = 0; i < n; ++i) {
                 ok = wait.mbar(empty + 8 * st, ph ^ 1u);
                 if (!ok) break;
@@ -651,7 +656,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cluster_kernel(const __grid_con
     if (gave_up) {
         // nothing to work on
     } else if (warp == 0) {
-        if (ptx::elect_one()) cluster_feed<ROWS>(P, rank, lay, smem, B, wait);
+        if (ptx::elect_one()) cluster_feed<ROWS>(P, cluster, rank, lay, smem, B, wait);
         __syncwarp();
     } else if (warp == 1) {
         if (ptx::elect_one()) cluster_mma<ROWS>(P, units, rank, lay, smem, tmem, B, wait);
@@ -660,15 +665,12 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cluster_kernel(const __grid_con
         if (ptx::elect_one()) cluster_fetch<ROWS>(P, units, cluster, rank, lay, smem, B, wait);
         __syncwarp();
     } else {
-        auto run = [&](auto g) {
-            if constexpr (decltype(g)::value <= cl_most_units(ROWS))
-                ClusterEpilogue<ROWS, decltype(g)::value>::run(P, S, cluster, rank, smem, tmem, B, warp - 2, lane, wait);
-        };
+        constexpr int M = cl_most_units(ROWS);
         switch (units) {
-            case 1: run(std::integral_constant<int, 1>{}); break;
-            case 2: run(std::integral_constant<int, 2>{}); break;
-            case 3: run(std::integral_constant<int, 3>{}); break;
-            case 4: run(std::integral_constant<int, 4>{}); break;
+            case 1: ClusterEpilogue<ROWS, 1>::run(P, S, cluster, rank, smem, tmem, B, warp - 2, lane, wait); break;
+            case 2: if constexpr (M >= 2) ClusterEpilogue<ROWS, 2>::run(P, S, cluster, rank, smem, tmem, B, warp - 2, lane, wait); break;
+            case 3: if constexpr (M >= 3) ClusterEpilogue<ROWS, 3>::run(P, S, cluster, rank, smem, tmem, B, warp - 2, lane, wait); break;
+            case 4: if constexpr (M >= 4) ClusterEpilogue<ROWS, 4>::run(P, S, cluster, rank, smem, tmem, B, warp - 2, lane, wait); break;
             default: break;
         }
         __syncwarp();

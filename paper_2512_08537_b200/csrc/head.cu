@@ -41,7 +41,6 @@
 
 #include <algorithm>
 #include <mutex>
-#include <type_traits>
 #include <vector>
 
 #include "../../include/ardiff.h"
@@ -1453,7 +1452,7 @@ struct ardiff_head {
     mutable int timed;
     cudaEvent_t ev0, ev1;
     // self-test of the bounded waits, armed for the next sample call only
-    mutable int stall_tile;
+    mutable int stall_tile, stall_cluster;
     mutable unsigned int stall_limit_us;
 };
 
@@ -1647,7 +1646,7 @@ extern "C" int ardiff_head_create(const ardiff_head_desc* desc, const ardiff_hea
     // launch fail instead of start when the grid cannot be co-resident (ardiff_head_set_cooperative
     // drops it for profilers that cannot replay such launches).
     H->coop = 1;
-    H->stall_tile = -1;
+    H->stall_tile = H->stall_cluster = -1;
     H->grid = H->n_sm;
 #ifdef ARDIFF_TUNING
     H->grid = env_int("ARDIFF_HEAD_GRID", H->n_sm);
@@ -2020,10 +2019,11 @@ int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise,
     P.clock_probe = H->clock_probe;
     P.wait_limit_ns = kWaitLimitNs;
     P.stall_tile = -1;
-    if (H->stall_tile >= 0) {             // armed self-test: this call only
+    const int stall_cluster = H->stall_cluster;
+    if (H->stall_tile >= 0 || stall_cluster >= 0) {             // armed self-test: this call only
         P.stall_tile = H->stall_tile;
         P.wait_limit_ns = (unsigned long long)H->stall_limit_us * 1000ull;
-        H->stall_tile = -1;
+        H->stall_tile = H->stall_cluster = -1;
     }
 
     ChainParams Q;
@@ -2069,7 +2069,7 @@ int head_sample_impl(const ardiff_head* H, const void* cond, const float* noise,
 #ifdef ARDIFF_TUNING
         R.direct_bytes = (uint32_t)env_int("ARDIFF_HEAD_DIRECT", CL_DIRECT_BYTES);
 #endif
-        R.status = H->status; R.abort_flag = P.abort_flag; R.wait_limit_ns = P.wait_limit_ns;
+        R.status = H->status; R.abort_flag = P.abort_flag; R.wait_limit_ns = P.wait_limit_ns; R.stall_cluster = stall_cluster;
         memcpy(R.ax, P.ax, sizeof(R.ax)); memcpy(R.av, P.av, sizeof(R.av)); memcpy(R.an, P.an, sizeof(R.an));
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute at[2];
@@ -2167,6 +2167,14 @@ extern "C" int ardiff_head_inject_stall(ardiff_head* H, int32_t token_tile, uint
     if (!H) return ARDIFF_ERR_NULL;
     if (token_tile < 0 || wait_limit_us < 100 || wait_limit_us > 4000000u) return ARDIFF_ERR_SHAPE;
     H->stall_tile = token_tile;
+    H->stall_limit_us = wait_limit_us;
+    return ARDIFF_OK;
+}
+
+extern "C" int ardiff_head_inject_cluster_stall(ardiff_head* H, int32_t cluster, uint32_t wait_limit_us) {
+    if (!H) return ARDIFF_ERR_NULL;
+    if (cluster < 0 || wait_limit_us < 100 || wait_limit_us > 4000000u) return ARDIFF_ERR_SHAPE;
+    H->stall_cluster = cluster;
     H->stall_limit_us = wait_limit_us;
     return ARDIFF_OK;
 }

@@ -653,6 +653,31 @@ def test_bounded_wait_runs_out_reports_timeout_and_the_head_recovers(n, tiles):
     head.close()
 
 
+@pytest.mark.parametrize("W,n", [(256, 500), (1024, 64), (1024, 500), (1536, 200), (2048, 200)])
+def test_a_wait_inside_the_clusters_runs_out(W, n):
+    """One CTA of the first, or of a later, cluster stops between two layers (values copied between shared memories at the first two
+    sizes, through L2 at the others): its peers' waits end at the limit, the status says TIMEOUT, and the next call gives the
+    bits of an undisturbed run. A cluster that the call does not need: no effect."""
+    dev = require_cuda()
+    wl = synth.workload("cfg1", n=n, W=W, L=2, K=2, Dc=128)
+    w, cond_bits, noise, t = synth.head_weights(wl), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
+    idx = np.arange(n, dtype=np.int32)
+    head = make_head(wl, w)
+    chain, clusters = head.few_limits(wl.K)
+    assert chain < n <= clusters
+    clean = run_head(head, cond_bits, noise, t, idx)
+    for cluster in (0, 3):
+        head.inject_cluster_stall(cluster, 3000)
+        out = torch.zeros(noise.shape, dtype=torch.float32, device=dev)
+        head.ardiff_head_sample(dev_bf16(cond_bits), dev_f32(noise), t, torch.from_numpy(idx).to(dev),
+                                torch.tensor([n], dtype=torch.int32, device=dev), out)
+        assert head.status() == ardiff.ARDIFF_ERR_TIMEOUT
+        assert np.array_equal(run_head(head, cond_bits, noise, t, idx), clean)
+    head.inject_cluster_stall(400, 3000)
+    assert np.array_equal(run_head(head, cond_bits, noise, t, idx), clean)
+    head.close()
+
+
 def test_more_survivors_than_the_head_was_created_for():
     """*count above max_tokens: the head runs the first max_tokens survivors, leaves every other row
     untouched and flags the call with ARDIFF_ERR_SHAPE in its status word; the next call is clean."""
