@@ -128,10 +128,14 @@ def _check(rc: int, where: str):
 
 
 def _stream_ptr(stream) -> int:
-    """The stream's handle; without one that of the current stream (asked for as a number: a Stream object takes 2 us)."""
+    """The stream's handle; without one that of the current stream (asked for as a number where torch has that: a Stream object
+    takes 2 us)."""
     import torch
     if stream is None:
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None:
+            return raw(torch.cuda.current_device())
+        stream = torch.cuda.current_stream()
     return int(stream.cuda_stream)
 
 
