@@ -474,8 +474,9 @@ __device__ __forceinline__ void cluster_feed(const ClusterParams& P, int cluster
             const int row = in ? rank * ROWS : out ? (int)P.out_row0 : (5 * ((l - 1) >> 1) + 3 + ((l - 1) & 1)) * W + rank * ROWS;
             const uint32_t bytes = (uint32_t)(out ? P.C : ROWS) * CL_KS * 2 * sl;
             int kp = in ? 0 : rank / SRCS;
-            if (l == 2 && cluster == P.stall_cluster && rank == P.n_ctas - 1) {      // self-test (nothing ends this wait)
-                ok = wait.mbar(ptx::smem_u32(&B.drain), 0);
+            if (l == 2 && cluster == P.stall_cluster && rank == P.n_ctas - 1) {      // self-test (nothing ends this wait in time)
+                wait.mbar(ptx::smem_u32(&B.drain), 0);
+                ok = false;
                 break;
             }
             for (int i = 0; i < n; ++i) {

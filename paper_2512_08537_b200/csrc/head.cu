@@ -395,9 +395,9 @@ __device__ __forceinline__ void unpack_item(const HeadParams& P, const Packed& p
 struct Place {
     uint32_t smem_base, bars, tmem_base;
     int rank, unit_id, n_units;             // token tile of the unit this CTA owns, its unit, all units
-    int count, MTu, tgu;                    // survivors; pairs of token tiles (modulations only: of steps): of the call,
-                                            // of one group
-    int steps;                              // repetitions of the program's step
+    int count, MTu, tgu;                    // survivors; pairs of token tiles of the call, of one group (modulations only:
+                                            // pairs of (step, token tile), and pairs of token tiles of the call)
+    int steps;                              // repetitions of the program's step (modulations only: token tiles)
     long long total;                        // items of the call
 };
 
