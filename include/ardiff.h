@@ -117,7 +117,8 @@ int ardiff_entropy_gate_blocks(const void* feat, int64_t n, int32_t rows_per_tok
 /* Threshold from entropy statistics (the tau equation of "Entropy-Based Early Stopping in Inference
  * Phase"): out3 = { mean(H), std(H), 0.3 * mean - 0.1 * std }, std with divisor n, all in fp64
  * with a fixed summation order (results are reproducible run to run).
- *   entropy dev float [n], n >= 1;  out3 dev double [3]. One CTA, or one cluster of 8 above 57344 entropies: meant for calibration, not the hot path. */
+ *   entropy dev float [n], n >= 1;  out3 dev double [3]. One CTA, or one cluster of 16 (8 where the device
+ *   takes none of 16) above 43008 entropies: meant for calibration, not the hot path. */
 int ardiff_tau_calibrate(const float* entropy, int64_t n, double* out3, void* stream);
 
 /* Accepted draft length per block (Algorithm 1, Step 4):
@@ -240,9 +241,10 @@ int ardiff_head_destroy(ardiff_head* head);
  *   out      dev  float [n][C]: rows idx[j] are written, all other rows are left untouched
  * One persistent cooperative kernel walks a static schedule of GEMM tiles; tiles wait for
  * their producers on device-side counters with bounded spins. For few survivors (as many as
- * *count says, for widths up to 2048: up to about 200 at the largest, 700 at W = 1024, 4000 at
- * W = 256) the layers that depend on x leave that schedule: clusters of CTAs take groups of up to
- * 64 tokens through all steps in a second kernel (up to 32 survivors of widths from 1024 on run
+ * *count says, for widths up to 2048: up to 224 at the largest, 960 at W = 1024, 4736 at W = 256 on
+ * 148 SMs, fewer where few layers follow or many steps fill the modulations' buffer, see
+ * ardiff_head_few_limits) the layers that depend on x leave that schedule: clusters of CTAs take groups
+ * of up to 64 tokens through all steps in a second kernel (up to 32 survivors of widths from 768 on run
  * with one exchange of values between SMs per layer); those waits are bounded the same way. If a wait
  * runs out the kernel finishes early, the results are invalid and ardiff_head_status reports
  * ARDIFF_ERR_TIMEOUT. Calls on one head must not overlap on the device (they share its

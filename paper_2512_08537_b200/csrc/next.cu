@@ -66,12 +66,12 @@ block_prefix_kernel(const float* __restrict__ row_entropy, int64_t n, int32_t r,
 // Mean, standard deviation (divisor n) and tau of n entropies: one CTA or a cluster of them, fp64, no scratch. Every CTA
 // takes a contiguous part in two passes (the deviations are taken from the part's own mean), sums in a fixed order
 // (thread-strided partial sums, a tree per CTA); a cluster's parts are merged once, in rank order, through distributed
-// shared memory. Bound by what a few SMs load: a million entropies take one CTA 87 us, 8 18.4 (with
-// two exchanges, one for the mean and one for the deviations), 16 12.0; 65536 8.4 with 8 and 6.9 with 16. A cluster costs
-// 3 us to start and to meet in, so few entropies have one CTA, in a kernel without the cluster's barriers: us, one CTA / 8:
-// 8192 4.7 / 7.6, 16384 5.1 / 7.6, 49152 7.6 / 8.3, 65536 9.1 / 8.2.
+// shared memory. Bound by what a few SMs load: a million entropies take one CTA 87 us, 8 18.4 (with two exchanges, one for the
+// mean and one for the deviations), 16 12.0. A cluster costs 2 us to start and to meet in, so few entropies have one CTA, in a
+// kernel without the cluster's barriers: us, one CTA / 16: 8192 4.0 / 6.2, 16384 4.4 / 6.3, 32768 5.7 / 6.5, 49152 7.1 / 6.6, 57344
+// 7.8 / 6.9.
 constexpr int kTauThreads = 1024;
-constexpr int64_t kTauOneCta = 56 * kTauThreads;
+constexpr int64_t kTauOneCta = 42 * kTauThreads;
 __device__ __forceinline__ double cta_sum(double acc, double* s) {
     s[threadIdx.x] = acc;
     __syncthreads();

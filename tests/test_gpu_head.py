@@ -220,6 +220,7 @@ def test_head_without_room_for_the_few_token_buffers():
     t = synth.t_sched(2)
     idx = np.arange(0, wl.n, 5).astype(np.int32)
     want = oracle.head_sample(w, cond_bits, noise, t, idx)
+    torch.cuda.empty_cache()                         # (what earlier tests left in torch's cache is not this head's)
     head = make_head(wl, w)                          # (kernels loaded; what a whole head takes)
     run_head(head, cond_bits, noise, t, idx)
     with_buffers = torch.cuda.mem_get_info()[0]

@@ -90,7 +90,7 @@ def test_block_gate_with_gamma_one_equals_plain_gate_and_empty_input():
     assert int(count0.item()) == 0
 
 
-@pytest.mark.parametrize("n,shift", [(1, 1), (3, 2), (8192, 0), (8193, 3), (57344, 1), (57345, 2), (1000003, 1)])
+@pytest.mark.parametrize("n,shift", [(1, 1), (3, 2), (8192, 0), (8193, 3), (43008, 0), (43008, 1), (43009, 2), (57344, 1), (57345, 2), (1000003, 1)])
 def test_tau_calibration_at_any_address(n, shift):
     """One CTA and a cluster of them, the pool starting anywhere: fp64 sums of fp32 values against numpy's (a million terms
     of equal sign in another order differ by less than 1e6 * 2^-53 = 1e-10 of the mean, in practice 1e-13)."""
