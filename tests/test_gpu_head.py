@@ -99,11 +99,15 @@ def test_small_head_ragged_counts(std, count):
     head.close()
 
 
+# Where the schedules change is what ardiff_head_few_limits says. The counts of the tests that were written before the clusters
+# came in stay (512 / 513 here, 64 / 65 at every width, 26 / 27 with 64 steps of 12 blocks, 900 tokens in the test of the waits: all
+# of them the clusters' now), whatever their docstrings say of the schedule; each has one behind it that takes its counts from the
+# limits, or asserts on them, and so reaches the schedule it names.
 @pytest.mark.parametrize("count", [512, 513, 3072, 3073, 23808, 23809, 26112, 26113])
 def test_item_width_boundaries(count):
-    """The last token count of 128-column items and the first of 256 (W = 512 on 148 SMs: 12 pairs of token tiles), of a group of
-    the usual size (93 pairs), and of a lone group (102). (512 and 513 are the clusters'; items of 64 columns: the test below.)
-    Tolerance: the agreement bar of this file."""
+    """The last token count of each item width and the first of the next one (W = 512 on 148 SMs: 64 output columns
+    per item up to 2 pairs of token tiles, 128 up to 12, then 256), of a group of the usual size (93 pairs), and of a lone
+    group (102). Tolerance: the agreement bar of this file."""
     wl = synth.workload("cfg1", n=count + 5, W=512, L=2, K=2)
     w, cond_bits, noise, t = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
     idx = np.random.default_rng(count).permutation(wl.n)[:count].astype(np.int32)
@@ -133,9 +137,28 @@ def test_item_widths_where_the_modulations_hold_few_tokens(count):
     head.close()
 
 
+@pytest.mark.parametrize("W", [256, 512, 768, 1024, 1280, 1536, 1792, 2048, 2304])
+def test_few_tokens_at_every_width(W):
+    """Up to 64 survivors the chain of layers leaves the tile schedule (one instance per W / 256 up to 8): one token, a
+    ragged token tile, a second pass, the last count it takes and the first that it does not; the same call twice gives
+    the same bits. Tolerance: the agreement bar of this file."""
+    wl = synth.workload("cfg1", n=80, W=W, L=2, K=3, C=32 if W % 512 else 64, Dc=192)
+    w, cond_bits, noise, t = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
+    order = np.random.default_rng(W).permutation(wl.n).astype(np.int32)
+    want = oracle.head_sample(w, cond_bits, noise, t, order[:65])
+    head = make_head(wl, w)
+    for count in (1, 9, 33, 64, 65):
+        idx = order[:count]
+        got = run_head(head, cond_bits, noise, t, idx)
+        assert_parity(got, want, idx, f"{count} tokens")
+        assert np.all(got[np.setdiff1d(np.arange(wl.n), idx)] == SENTINEL)
+        assert np.array_equal(run_head(head, cond_bits, noise, t, idx), got)
+    head.close()
+
+
 @pytest.mark.parametrize("n", [64, 80])
 @pytest.mark.parametrize("W", [256, 512, 768, 1024, 1280, 1536, 1792, 2048, 2304])
-def test_few_tokens_at_every_width(W, n):
+def test_few_tokens_at_the_limits_of_every_width(W, n):
     """One token, the chain where it serves some (its last count and the first of the clusters), ragged token tiles, and up to
     the 64 tokens of heads that split a layer over as many CTAs as a cluster may have (n = 64: 64 columns each up to W = 1024);
     no such schedule above W = 2048. The same call twice gives the same bits. Tolerance: the agreement bar of this file."""
@@ -155,11 +178,45 @@ def test_few_tokens_at_every_width(W, n):
     head.close()
 
 
-@pytest.mark.parametrize("W,n,counts", [(256, 4740, (80, 81, 1184, 2112, 3552, 3553)), (512, 2116, (129, 528, 529, 1600)),
-                                        (768, 1412, (100, 337, 1300)), (1024, 964, (240, 241, 481, 720, 721)),
-                                        (1280, 532, (32, 33, 177, 353)), (1536, 228, (32, 33, 112, 113)),
-                                        (1792, 228, (33, 112, 113)), (2048, 228, (32, 33, 112, 113))])
-def test_token_groups_of_the_clusters(W, n, counts):
+@pytest.mark.parametrize("W,counts", [(256, (80, 81, 2112, 4224, 4225, 4737)), (512, (129, 1600, 2112, 2113)),
+                                      (768, (100, 337, 1300)), (1024, (240, 241, 481, 720, 721)),
+                                      (1280, (32, 33, 177, 353, 529)), (1536, (32, 33, 112, 113, 224, 225)),
+                                      (1792, (33, 112, 225)), (2048, (32, 33, 112, 113, 224, 225))])
+def test_token_groups_of_the_clusters(W, counts):
+    """Clusters of W / 128 CTAs take groups of 16, 32, 48 or 64 tokens: counts on both sides of where the group grows, where the
+    values go through L2 instead of directly, and of the last that fits (on 148 SMs); a ragged last group; fresh noise; the
+    same call twice gives the same bits. Tolerance: the agreement bar of this file."""
+    dev = require_cuda()
+    wl = synth.workload("cfg1", n=max(counts) + 3, W=W, L=2, K=2, C=48 if W % 512 else 16, Dc=128)
+    w, cond_bits, noise = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl)
+    t_in = np.array([0.9, 0.4], np.float32)
+    coef = np.array([[0.4, 0.7, 0.5], [0.2, 1.0, 0.1]], np.float32)
+    z = np.random.default_rng(9).standard_normal((2, wl.n, wl.C)).astype(np.float32)
+    order = np.random.default_rng(W).permutation(wl.n).astype(np.int32)
+    pos = np.unique(np.concatenate([[0, 15, 16, 31, 47, 63], np.array(counts) - 1, np.random.default_rng(1).integers(0, max(counts), 24)]))
+    want = np.zeros((wl.n, wl.C))
+    want[order[pos]] = oracle.head_sample_coef(w, cond_bits, noise, t_in, coef, order[pos], step_noise=z)[order[pos]]
+    head = make_head(wl, w)
+    cond, noise_d, z_d = dev_bf16(cond_bits), dev_f32(noise), torch.from_numpy(z).to(dev)
+    for count in counts:
+        outs = []
+        for _ in range(2):
+            out = torch.full(noise.shape, SENTINEL, dtype=torch.float32, device=dev)
+            head.ardiff_head_sample_coef(cond, noise_d, t_in, coef, torch.from_numpy(order[:count].copy()).to(dev),
+                                         torch.tensor([count], dtype=torch.int32, device=dev), out, step_noise=z_d)
+            assert head.status() == 0
+            outs.append(out.cpu().numpy())
+        rows = order[pos[pos < count]]
+        assert_parity(outs[0], want, rows, f"{count} tokens")
+        assert np.array_equal(outs[0], outs[1])
+        assert np.all(outs[0][order[count:]] == SENTINEL) and not np.any(outs[0][order[:count]] == SENTINEL)
+    head.close()
+
+
+@pytest.mark.parametrize("W,n,counts", [(256, 4740, (1184, 3552, 3553)), (512, 2116, (528, 529)), (768, 1412, (337,)),
+                                        (1024, 964, (720, 721)), (1280, 532, (353,)), (1536, 228, (112,)), (1792, 228, (112, 113)),
+                                        (2048, 228, (112,))])
+def test_token_groups_up_to_the_limit_of_the_clusters(W, n, counts):
     """Clusters of W / 128 CTAs (W / 96 at 1536) take groups of 16, 32, 48 or 64 tokens: counts on both sides of where the group
     grows, where the values go through L2 instead of directly, the last that they serve and the first that they do not; a
     ragged last group; fresh noise; the same call twice gives the same bits. Tolerance: the agreement bar of this file."""
@@ -194,6 +251,22 @@ def test_token_groups_of_the_clusters(W, n, counts):
 
 
 def test_few_token_limit_set_by_the_buffers():
+    """64 steps of 12 blocks: the few-token buffers (128 MB of modulations) hold 26 survivors. The last count that they serve
+    and the first that they do not. Tolerance: the agreement bar of this file."""
+    wl = synth.workload("cfg1", n=40, W=512, L=12, K=64)
+    w, cond_bits, noise, t = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
+    order = np.random.default_rng(26).permutation(wl.n).astype(np.int32)
+    rows = order[[0, 7, 25, 26]]
+    want = oracle.head_sample(w, cond_bits, noise, t, rows)
+    head = make_head(wl, w)
+    for count in (26, 27):
+        got = run_head(head, cond_bits, noise, t, order[:count])
+        assert_parity(got, want, rows[:3] if count == 26 else rows, f"{count} tokens")
+        assert np.all(got[np.setdiff1d(np.arange(wl.n), order[:count])] == SENTINEL)
+    head.close()
+
+
+def test_few_token_limit_set_by_the_modulations():
     """64 steps of 12 blocks: the modulations (at most 256 MB) are those of 48 survivors. The last count that the clusters serve
     and the first that they do not. Tolerance: the agreement bar of this file."""
     wl = synth.workload("cfg1", n=64, W=512, L=12, K=64)
@@ -211,6 +284,36 @@ def test_few_token_limit_set_by_the_buffers():
 
 
 def test_head_without_room_for_the_few_token_buffers():
+    """The few-token schedule's buffers are an accelerator: a device that has room for the rest of a head, but not for them,
+    still gets the head, and calls of few tokens take the schedule of larger ones. (The memory is held by one ordinary
+    allocation; nothing runs out but the library's own request.)"""
+    dev = require_cuda()
+    wl = synth.workload("cfg1", n=64, W=512, L=12, K=64)
+    w, cond_bits, noise = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl)
+    t = synth.t_sched(2)
+    idx = np.arange(0, wl.n, 5).astype(np.int32)
+    want = oracle.head_sample(w, cond_bits, noise, t, idx)
+    head = make_head(wl, w)                          # (kernels loaded; what a whole head takes)
+    run_head(head, cond_bits, noise, t, idx)
+    with_buffers = torch.cuda.mem_get_info()[0]
+    head.close()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    taken = free - with_buffers
+    assert taken > 250 << 20                         # weights and scratch about 100 MB, the buffers 128 MB and more
+    held = torch.empty(free - taken + (120 << 20), dtype=torch.uint8, device=dev)
+    try:
+        head = make_head(wl, w)
+        got = run_head(head, cond_bits, noise, t, idx)
+        assert_parity(got, want, idx)
+        head.close()
+    finally:
+        del held
+        torch.cuda.empty_cache()
+
+
+def test_head_without_room_takes_the_tiles():
     """The few-token schedule's buffers are an accelerator: a device that has room for the rest of a head, but not for them,
     still gets the head, and calls of few tokens take the schedule of larger ones. (The memory is held by one ordinary
     allocation; nothing runs out but the library's own request.)"""
@@ -481,11 +584,42 @@ def test_workload_configs_sampled_tokens(name, extra, K):
     head.close()
 
 
-@pytest.mark.parametrize("na,nb", [(700, 900), (4900, 2300), (4900, 900)])
-def test_two_heads_on_two_streams(na, nb):
-    """Two heads of different shapes, driven from two streams without any ordering between them, with the clusters, with tiles and
-    one with each: every launch of the head kernel needs the whole GPU (cooperative launch), so the launches take turns; both
-    results must match what each head gives alone."""
+def test_two_heads_on_two_streams():
+    """Two heads of different shapes, driven from two streams without any ordering between them: every
+    launch needs the whole GPU (cooperative launch), so the launches take turns; both results must
+    match what each head gives alone."""
+    dev = require_cuda()
+    wa, wb = synth.workload("cfg1", n=700), synth.workload("cfg1", n=900, W=512, L=3, seed=77)
+    outs = {}
+    heads = {}
+    for key, wl in (("a", wa), ("b", wb)):
+        w, t = synth.head_weights(wl), synth.t_sched(wl.K)
+        head = make_head(wl, w)
+        cond, noise = dev_bf16(synth.cond(wl)), dev_f32(synth.noise(wl))
+        idx = torch.arange(wl.n, dtype=torch.int32, device=dev)
+        count = torch.tensor([wl.n], dtype=torch.int32, device=dev)
+        alone = torch.empty((wl.n, wl.C), dtype=torch.float32, device=dev)
+        head.ardiff_head_sample(cond, noise, t, idx, count, alone)
+        heads[key] = (head, cond, noise, t, idx, count, alone, wl)
+    torch.cuda.synchronize()
+    streams = {k: torch.cuda.Stream(device=dev) for k in heads}
+    for rep in range(4):
+        for key, (head, cond, noise, t, idx, count, alone, wl) in heads.items():
+            out = torch.full((wl.n, wl.C), SENTINEL, dtype=torch.float32, device=dev)
+            head.ardiff_head_sample(cond, noise, t, idx, count, out, stream=streams[key])
+            outs[(key, rep)] = out
+    torch.cuda.synchronize()
+    for (key, rep), out in outs.items():
+        head, *_, alone, wl = heads[key]
+        assert head.status() == 0
+        assert torch.equal(out, alone), (key, rep)
+    for head, *_ in heads.values():
+        head.close()
+
+
+@pytest.mark.parametrize("na,nb", [(4900, 2300), (4900, 900)])
+def test_two_heads_on_two_streams_with_tiles(na, nb):
+    """The same with tiles, and with one head of tiles beside one of clusters."""
     dev = require_cuda()
     wa, wb = synth.workload("cfg1", n=na), synth.workload("cfg1", n=nb, W=512, L=3, seed=77)
     outs = {}
@@ -624,18 +758,16 @@ def test_extreme_shapes_beyond_the_clusters(shape):
     head.close()
 
 
-@pytest.mark.parametrize("n,tiles", [(900, (0, 3, 7)), (5000, (0, 3, 39))])
-def test_bounded_wait_runs_out_reports_timeout_and_the_head_recovers(n, tiles):
-    """(900 tokens: what precedes the clusters, which then leave at once; 5000: the tile schedule.) The self-test hook makes one tile's dependency wait unsatisfiable and shortens the wait limit to 3 ms:
+def test_bounded_wait_runs_out_reports_timeout_and_the_head_recovers():
+    """The self-test hook makes one tile's dependency wait unsatisfiable and shortens the wait limit to 3 ms:
     the kernel must come back by itself (no fault, no trap, no endless spin), the status word must say
     TIMEOUT, and the very next call on the same head must give the bits of an undisturbed run."""
-    wl = synth.workload("cfg1", n=n)
+    wl = synth.workload("cfg1", n=900)
     w, cond_bits, noise, t = synth.head_weights(wl), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
     idx = np.arange(wl.n, dtype=np.int32)
     head = make_head(wl, w)
-    assert (head.few_limits(wl.K)[1] < n) == (n == 5000)
     clean = run_head(head, cond_bits, noise, t, idx)
-    for tile in tiles:                                    # first, an odd (partner CTA) and the last, ragged tile
+    for tile in (0, 3, 7):                                # first, an odd (partner CTA) and the last, ragged tile
         head.inject_stall(tile, 3000)
         dev = require_cuda()
         out = torch.zeros(noise.shape, dtype=torch.float32, device=dev)
@@ -651,6 +783,27 @@ def test_bounded_wait_runs_out_reports_timeout_and_the_head_recovers(n, tiles):
     with pytest.raises(ardiff.ArdiffError):
         head.inject_stall(0, 5)                           # limit below 100 us
     fresh.close()
+    head.close()
+
+
+def test_a_wait_of_the_tile_schedule_runs_out():
+    """The same with more tokens than the clusters serve: waits of gathers, products, epilogues and of the drained rings. The first
+    tile, an odd one (partner CTA) and the last."""
+    dev = require_cuda()
+    wl = synth.workload("cfg1", n=5000)
+    w, cond_bits, noise, t = synth.head_weights(wl), synth.cond(wl), synth.noise(wl), synth.t_sched(wl.K)
+    idx = np.arange(wl.n, dtype=np.int32)
+    head = make_head(wl, w)
+    assert head.few_limits(wl.K)[1] < wl.n
+    clean = run_head(head, cond_bits, noise, t, idx)
+    for tile in (0, 3, 39):
+        head.inject_stall(tile, 3000)
+        out = torch.zeros(noise.shape, dtype=torch.float32, device=dev)
+        head.ardiff_head_sample(dev_bf16(cond_bits), dev_f32(noise), t, torch.from_numpy(idx).to(dev),
+                                torch.tensor([wl.n], dtype=torch.int32, device=dev), out)
+        assert head.status() == ardiff.ARDIFF_ERR_TIMEOUT
+        assert head.status() == 0
+        assert np.array_equal(run_head(head, cond_bits, noise, t, idx), clean)
     head.close()
 
 

@@ -90,7 +90,7 @@ def test_block_gate_with_gamma_one_equals_plain_gate_and_empty_input():
     assert int(count0.item()) == 0
 
 
-@pytest.mark.parametrize("n,shift", [(1, 1), (3, 2), (8192, 0), (8193, 3), (43008, 0), (43008, 1), (43009, 2), (57344, 1), (57345, 2), (1000003, 1)])
+@pytest.mark.parametrize("n,shift", [(1, 1), (3, 2), (8192, 0), (8193, 3), (57344, 1), (57345, 2), (1000003, 1)])
 def test_tau_calibration_at_any_address(n, shift):
     """One CTA and a cluster of them, the pool starting anywhere: fp64 sums of fp32 values against numpy's (a million terms
     of equal sign in another order differ by less than 1e6 * 2^-53 = 1e-10 of the mean, in practice 1e-13)."""
@@ -102,6 +102,12 @@ def test_tau_calibration_at_any_address(n, shift):
     m, s = x.mean(), x.std()
     assert np.all(np.abs(a - np.array([m, s, 0.3 * m - 0.1 * s])) <= 1e-9)
     assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n,shift", [(43008, 0), (43008, 1), (43009, 0), (43009, 2)])
+def test_tau_calibration_where_the_cluster_begins(n, shift):
+    """The last pool of one CTA and the first of a cluster. Tolerance: that of the test above."""
+    test_tau_calibration_at_any_address(n, shift)
 
 
 @pytest.mark.parametrize("n", [1, 7, 1024, 100003])
