@@ -76,35 +76,40 @@ inline int cluster_units(int W, int C, int rows) {
     return units;
 }
 
-// Survivors up to which the clusters serve a call of K steps: one round of groups. A second round takes as long again, and the
-// tile schedule hardly longer for twice the tokens (W = 1024, 3 blocks, K = 4, 700 / 1434 tokens: clusters 321 / 565 us, tiles
-// 426 / 475). With few layers in all, what the modulations cost (written and read back in fp32) shows in the largest groups, and
-// the round ends earlier. us, clusters / tiles, K = 1: W = 256, 3 blocks, 3848 tokens 89 / 89, 4736 106 / 94, 5 blocks 4440 129 / 126, 4736
-// 131 / 127; 512, 3, 1716 97 / 104, 2112 113 / 106, 4, 1716 125 / 123, 2112 134 / 125; 768, 3, 1408 131 / 121; 1024, 3, 780 141 / 140, 960
-// 144 / 140; K = 2: 256, 2, 3848 118 / 119, 4440 129 / 120; 512, 1, 1980 101 / 104, 2112 108 / 103, 2, 1848 137 / 147, 2112 149 / 144. With one or two
-// layers both take as long (256, 2, 4736 76 / 76), with more layers or steps all of it gains (256, 12, 4736 210 / 233; 512, 3, K = 2, 2112
-// 181 / 186; 512, 1, K = 4, 2112 174 / 179), and so do groups of up to 48 tokens (1280, 4, 528 174 / 193; 1536, 1, 224 66 / 84).
+// Survivors up to which the clusters serve a call of K steps: one round of groups. A second round takes as long again, and
+// the tile schedule hardly longer for twice the tokens (W = 1024, 3 blocks, K = 4, 700 / 1434 tokens: clusters 321 / 565 us,
+// tiles 426 / 475). With few layers in all, what the modulations cost (written and read back in fp32) shows in the largest
+// groups, and the round ends earlier. us, clusters / tiles, K = 1: W = 256, 3 blocks, 3848 tokens 89 / 89, 4736 106 / 94, 5
+// blocks 4440 129 / 126, 4736 131 / 127; 512, 3, 1716 97 / 104, 2112 113 / 106, 4, 1716 125 / 123, 2112 134 / 125; 768, 3,
+// 1408 131 / 121; 1024, 3, 691 120 / 122, 748 132 / 122, 960 143 / 130, 4, 748 159 / 155 (medians over nine heads; groups of
+// 64 tokens leave the ring two stages there); K = 2: 256, 2, 3848 118 / 119, 4440 129 / 120; 512, 1, 1980 101 / 104, 2112
+// 108 / 103, 2, 1848 137 / 147, 2112 149 / 144. With one or two layers both take as long (256, 2, 4736 76 / 76), with more
+// layers or steps all of it gains (256, 12, 4736 210 / 233; 512, 3, K = 2, 2112 181 / 186; 512, 1, K = 4, 2112 174 / 179),
+// and so do groups of up to 48 tokens (1280, 4, 528 174 / 193; 1536, 1, 224 66 / 84).
 inline int64_t cluster_survivors(int W, int clusters, int units, int K, int L) {
     int sixteenths = 16;
-    if (units == 4 && K == 1 && L >= 3 && L <= 6) sixteenths = L <= 4 ? 13 : 15;
+    if (units == 4 && K == 1 && L >= 3 && L <= 6) sixteenths = L > 4 ? 15 : W == 1024 ? 12 : 13;
     if (units == 4 && K == 2 && L <= 2) sixteenths = W == 256 ? 14 : 15;
     return (int64_t)clusters * units * CL_UNIT * sixteenths / 16;
 }
 
-// Survivors up to which the chain (chain.cuh, at most 32 beside the clusters) stays the faster one: it spreads the weights of a
-// layer over W / 16 SMs, a cluster over 16, and has no second launch, but loses time in every step (x goes between the SMs too)
-// and with every token. The more steps and the fewer blocks in each, the fewer: a doubling of K costs 18 tokens with one block, 3 with
-// 12. (Constants for the least loss over widths of 768 to 2048, 1, 3 and 12 blocks, 1 to 8 steps, 1 to 32 tokens: none above 4 %.)
-// us, chain / clusters: W = 768, 12 blocks, K = 1, 16 130 / 131, K = 2, 8 212 / 206; W = 1024, 3 blocks, K = 1, 24 72 / 72, K = 2, 8 98 /
-// 102, 17 101 / 103, K = 4, 1 152 / 166, 8 166 / 166, K = 8, 4 293 / 299, 8 303 / 299; 12 blocks, K = 4, 16 485 / 490, 24 515 / 490, K = 8, 12
-// 901 / 922; 1 block, K = 2, 4 64 / 65, 8 66 / 65; W = 1280, 3 blocks, K = 2, 24 124 / 124, K = 4, 12 206 / 205, 12 blocks, K = 4, 24 609 /
-// 621; W = 1536, 3 blocks, K = 8, 16 443 / 450, 24 462 / 450, 12 blocks, K = 8, 28 1371 / 1407; W = 2048, 1 block, K = 8, 16 276 / 317,
-// 32 325 / 318, all else up to 32. At 512 and below never (1 token, 12 blocks, K = 1: 112 / 97). Clusters of 64 columns a CTA are
-// faster: W = 768, 12 blocks, K = 1, 4 125 / 125, 8 136 / 124; W = 1024, 3 blocks, K = 2, 8 94 / 100, 17 108 / 101, 12 blocks, K = 2, 8 246 / 260,
-// 16 285 / 262, K = 8, 4 837 / 878, 12 922 / 879.
+// Survivors up to which the chain (chain.cuh, at most 32 beside the clusters) stays the faster one: it spreads the weights
+// of a layer over W / 16 SMs, a cluster over 16, and has no second launch, but loses time in every step (x goes between the
+// SMs too) and with every token. The more steps and the fewer blocks in each, the fewer: a doubling of K costs 18 tokens
+// with one block, 3 with 12. (Constants for the least loss over widths of 768 to 2048, 1, 3 and 12 blocks, 1 to 8 steps, 1
+// to 32 tokens: none above 4 %, but 6 % at W = 1792 with one block and K = 4.) us, chain / clusters: W = 768, K = 1, 3
+// blocks, 6 59 / 59, 14 60 / 59, 6 blocks, 6 82 / 82, 14 86 / 81, 12 blocks, 6 124 / 130, 10 127 / 131, 14 135 / 131
+// (medians over nine heads, between which the chain's times differ by up to 10 %), K = 2, 8 212 / 206; W = 1024, 3 blocks, K
+// = 1, 24 72 / 72, K = 2, 8 98 / 102, 17 101 / 103, K = 4, 1 152 / 166, 8 166 / 166, K = 8, 4 293 / 299, 8 303 / 299; 12
+// blocks, K = 4, 16 485 / 490, 24 515 / 490, K = 8, 12 901 / 922; 1 block, K = 2, 4 64 / 65, 8 66 / 65; W = 1280, 3 blocks,
+// K = 2, 24 124 / 124, K = 4, 12 206 / 205, 12 blocks, K = 4, 24 609 / 621; W = 1536, 3 blocks, K = 8, 16 443 / 450, 24 462
+// / 450, 12 blocks, K = 8, 28 1371 / 1407; W = 2048, 1 block, K = 8, 16 276 / 317, 32 325 / 318, all else up to 32. At 512
+// and below never (1 token, 12 blocks, K = 1: 112 / 97). Clusters of 64 columns a CTA are faster: W = 768, 12 blocks, K = 1,
+// 4 125 / 125, 8 136 / 124; W = 1024, 3 blocks, K = 2, 8 94 / 100, 17 108 / 101, 12 blocks, K = 2, 8 246 / 260, 16 285 /
+// 262, K = 8, 4 837 / 878, 12 922 / 879.
 inline int chain_beside_clusters(int W, int rows, int K, int L) {
     if (W < 768 || K < 1) return 0;
-    if (W < 1024) return K > 1 ? 0 : L <= 6 ? 2 * L + 2 : rows == 64 ? 4 : 16;
+    if (W < 1024) return K > 1 ? 0 : L > 6 && rows == 64 ? 4 : L < 4 ? 2 * L + 2 : 10;
     const int most = W >= 1792 ? 76 : W >= 1536 ? 38 : W >= 1280 ? 30 : rows == 64 ? 18 : 23;
     const double per_doubling = rows == 64 ? 6.0 + 10.0 / L : 2.0 + 16.0 / L;
     const int tokens = (int)(most - per_doubling * log2((double)K)), least = L > 1 ? 4 : 1;
