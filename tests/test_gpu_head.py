@@ -178,6 +178,24 @@ def test_few_tokens_at_the_limits_of_every_width(W, n):
     head.close()
 
 
+@pytest.mark.parametrize("L", [1, 3, 12])
+def test_the_chain_at_its_narrowest_width(L):
+    """W = 768, where the chain serves calls of one step only: one token, its last count and the first of the clusters. Tolerance:
+    the agreement bar of this file."""
+    wl = synth.workload("cfg1", n=80, W=768, L=L, K=2, C=32, Dc=192)
+    w, cond_bits, noise, t = synth.head_weights(wl, std=None), synth.cond(wl), synth.noise(wl), synth.t_sched(1)
+    order = np.random.default_rng(L).permutation(wl.n).astype(np.int32)
+    head = make_head(wl, w)
+    chain, clusters = head.few_limits(1)
+    assert 1 < chain < 32 and clusters >= 80 and head.few_limits(2)[0] == 0
+    want = oracle.head_sample(w, cond_bits, noise, t, order[:chain + 1])
+    for count in (1, chain, chain + 1):
+        got = run_head(head, cond_bits, noise, t, order[:count])
+        assert_parity(got, want, order[:count], f"{count} tokens")
+        assert np.array_equal(run_head(head, cond_bits, noise, t, order[:count]), got)
+    head.close()
+
+
 @pytest.mark.parametrize("W,counts", [(256, (80, 81, 2112, 4224, 4225, 4737)), (512, (129, 1600, 2112, 2113)),
                                       (768, (100, 337, 1300)), (1024, (240, 241, 481, 720, 721)),
                                       (1280, (32, 33, 177, 353, 529)), (1536, (32, 33, 112, 113, 224, 225)),
